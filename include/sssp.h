@@ -93,8 +93,10 @@ typedef enum {
 /* L2 queue policies (Section 4.2).  L2V is the bucket queue with one bucket. */
 typedef enum { SSSP_L2_VECTOR = 0, SSSP_L2_BUCKET = 1 } sssp_l2_type;
 
-/* Tunable configuration.  Zero-initialise and call sssp_config_default(),
- * or pass NULL to a solve call to use the graph's tuned (or default)
+/* Tunable configuration of the queue engine.  Zero-initialise and call
+ * sssp_config_default(), or pass NULL to a solve call to leave the choice to
+ * the library: the step-synchronous wavefront kernels where they are the
+ * faster way, else the queue engine in the graph's tuned (or default)
  * configuration.  Fields the paper leaves open (wb, delta, bnum, bmax, NF,
  * F; Sections 3.4 and 4.2) are chosen by sssp_autotune(). */
 typedef struct sssp_config {
@@ -247,8 +249,13 @@ SSSP_API int sssp_graph_features(const sssp_graph *g, sssp_features *out);
  *   src       0 <= src < n.
  *   dist_out  n elements (uint32 or fp32 per the graph), host or device.
  *   pred_out  n int32 or NULL.
- *   cfg       NULL = the graph's tuned configuration, else its default: the feature
- *             prior picked at creation from the Table 2 features (Section 3.5).
+ *   cfg       NULL = the library's choice: the wavefront kernels, unless
+ *             sssp_autotune timed the tuned configuration faster; where they do
+ *             not apply, the graph's tuned configuration, else its default: the
+ *             feature prior picked at creation from the Table 2 features
+ *             (Section 3.5).  The queue engine's counters in sssp_stats are zero
+ *             after a wavefront solve, which counts kernel_ms, relax_arcs,
+ *             improved and rounds (its steps).
  *   stream    cudaStream_t or NULL.
  * Returns after completion.  Errors: SSSP_E_INVAL, SSSP_E_TIMEOUT,
  * SSSP_E_NOMEM (queue could not be grown), SSSP_E_CUDA. */
@@ -261,7 +268,9 @@ SSSP_API int sssp_solve(sssp_graph *g, int32_t src, void *dist_out, int32_t *pre
  *   dist_out  nq * n elements, query-major: dist_out[q * n + v].
  *   pred_out  nq * n int32 or NULL.
  * nq * 2^ceil(log2 n) must not exceed 2^32 (the element key packs the query
- * index above the vertex bits).  With cfg NULL the batch uses the
+ * index above the vertex bits).  With cfg NULL the library picks the kernels
+ * as for sssp_solve (on a small graph or a mesh: a cluster of blocks for every
+ * query); in the queue engine the batch uses the
  * configuration sssp_autotune_batch cached for its size class, if any.
  * Otherwise, when the library picks delta (cfg NULL, or a zero delta), the
  * batch uses delta / min(16, max(1, nq / 32)) with bnum <= 4: the queries
@@ -279,8 +288,9 @@ SSSP_API int sssp_last_stats(const sssp_graph *g, sssp_stats *out);
  * a prior from the Table 2 features and the per-family findings of
  * Section 5.4, refined by timing candidate configurations on up to nsrc of
  * the given sources (host or device int32[nsrc]) within about budget_ms.
- * The winner is cached on the graph (used when cfg == NULL) and copied to
- * *out when out != NULL.  budget_ms <= 0 returns the prior untimed. */
+ * The winner is cached on the graph (used when cfg == NULL and it is faster
+ * than the wavefront kernels, which are timed last) and copied to *out when
+ * out != NULL.  budget_ms <= 0 returns the prior untimed. */
 SSSP_API int sssp_autotune(sssp_graph *g, const int32_t *srcs, int32_t nsrc, int32_t budget_ms,
                   sssp_config *out);
 

@@ -37,6 +37,7 @@ struct Workspace {
     size_t tl_n = 0;
     cudaEvent_t ev0 = nullptr, ev1 = nullptr, ev2 = nullptr;
 
+    int ensure_ctrl(cudaStream_t s);
     int ensure_queue(uint32_t nrings, uint32_t nch, uint32_t margin, cudaStream_t s, int sms);
     void release();
 };
@@ -55,15 +56,19 @@ struct Graph {
     int32_t* row_ptr = nullptr;   // [nv + 1]
     uint2* adj = nullptr;         // [mv] (col, weight bits)
     int32_t* owner = nullptr;     // [nv - n]
+    int2* span = nullptr;         // [n] (begin, end) of a real vertex's arcs in adj (a hub's slices are contiguous)
     sssp_features feat{};
     sssp_config defaults{};
     sssp_config tuned{};
     bool tuned_valid = false;
+    bool tuned_queues = false;    // sssp_autotune timed the tuned queue configuration faster than the wavefront
+    bool wide = false;            // a solve found the front too wide for one cluster
     // multi-query configurations from sssp_autotune_batch, per size class
     // (the number of queries rounded down to a power of two)
     struct BatchTuned {
         int32_t nq_class;
         sssp_config cfg;
+        bool queues;              // timed faster than the wavefront
     };
     std::vector<BatchTuned> batch_tuned;
     sssp_stats last{};
@@ -123,6 +128,27 @@ struct Sampling {
 int run_queries(Graph* g, const int32_t* srcs_host, const int32_t* srcs_dev, int32_t src0, int32_t nq,
                 void* dist_out, int32_t* pred_out, const sssp_config* cfg, cudaStream_t stream,
                 sssp_stats* st_out, bool unit = false, const Sampling* samp = nullptr);
+
+// The wavefront kernels (sssp_wave.cu), for calls that leave the configuration
+// to the library.  kWaveNotRun: the graph or the call is not for them.
+constexpr int kWaveNotRun = 1;
+int run_wave(Graph* g, const int32_t* srcs_host, const int32_t* srcs_dev, int32_t src0, int32_t nq, void* dist_out,
+             int32_t* pred_out, cudaStream_t stream, sssp_stats* st_out, bool unit);
+template <typename T>
+int grow(T** p, size_t* have, size_t want) {
+    if (*have >= want && *p) return SSSP_OK;
+    cudaFree(*p);
+    *p = nullptr;
+    *have = 0;
+    cudaError_t e = cudaMalloc((void**)p, (want > 1 ? want : 1) * sizeof(T));
+    if (e != cudaSuccess) {
+        cudaGetLastError();
+        *p = nullptr;
+        return SSSP_E_NOMEM;
+    }
+    *have = want;
+    return SSSP_OK;
+}
 
 inline uint32_t __float_as_uint_host(float f) {
     uint32_t b;

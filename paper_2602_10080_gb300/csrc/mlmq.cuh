@@ -90,6 +90,7 @@ enum : int {
     kErrOverflow = 2,     // every L2 bucket ring was full
     kErrState = 3,        // queue metadata inconsistent at seeding
     kErrElement = 4,      // a popped element names a vertex or query out of range
+    kErrWide = 5,         // wavefront kernel: the front is too wide for one cluster (the host runs the grid's)
 };
 
 // statistics slots (ctrl.stats)

@@ -326,23 +326,7 @@ void Workspace::release() {
     *this = Workspace();
 }
 
-template <typename T>
-static int grow(T** p, size_t* have, size_t want) {
-    if (*have >= want && *p) return SSSP_OK;
-    cudaFree(*p);
-    *p = nullptr;
-    *have = 0;
-    cudaError_t e = cudaMalloc((void**)p, std::max<size_t>(want, 1) * sizeof(T));
-    if (e != cudaSuccess) {
-        cudaGetLastError();
-        *p = nullptr;
-        return SSSP_E_NOMEM;
-    }
-    *have = want;
-    return SSSP_OK;
-}
-
-int Workspace::ensure_queue(uint32_t nr, uint32_t nch_want, uint32_t margin, cudaStream_t s, int sms) {
+int Workspace::ensure_ctrl(cudaStream_t s) {
     if (!ev0) {
         if (cudaEventCreate(&ev0) != cudaSuccess || cudaEventCreate(&ev1) != cudaSuccess ||
             cudaEventCreate(&ev2) != cudaSuccess)
@@ -355,6 +339,12 @@ int Workspace::ensure_queue(uint32_t nr, uint32_t nch_want, uint32_t margin, cud
         if (cudaMalloc((void**)&ctrl, sizeof(Ctrl)) != cudaSuccess) return SSSP_E_NOMEM;
         cudaMemsetAsync(ctrl, 0, sizeof(Ctrl), s);
     }
+    return SSSP_OK;
+}
+
+int Workspace::ensure_queue(uint32_t nr, uint32_t nch_want, uint32_t margin, cudaStream_t s, int sms) {
+    const int rc = ensure_ctrl(s);
+    if (rc) return rc;
     const bool realloc = !ring_mem || nr != nrings || nch_want > rings.nch;
     if (realloc) {
         const uint32_t nch = std::max(nch_want, nr == nrings ? rings.nch : 0u);
@@ -473,6 +463,13 @@ const sssp_config* batch_tuned_for(const Graph* g, int32_t nq) {
     return nullptr;
 }
 
+static bool batch_prefers_queues(const Graph* g, int32_t nq) {
+    const int32_t k = nq_class(nq);
+    for (const Graph::BatchTuned& b : g->batch_tuned)
+        if (b.nq_class == k) return b.queues;
+    return false;
+}
+
 const sssp_config* batch_tuned_largest(const Graph* g) {
     const Graph::BatchTuned* best = nullptr;
     for (const Graph::BatchTuned& b : g->batch_tuned)
@@ -583,13 +580,33 @@ int plan_launch(const Graph* g, const sssp_config& cfg, int pred_mode, bool mq, 
 
 // ================================================================== solve
 
+// Vertex bits of an element key that also holds one of nq queries, 0 if they
+// do not fit in 32 bits.  2^bits > nv: no key is all ones.
+static int key_bits(const Graph* g, int32_t nq) {
+    int vbits = 1;
+    while (vbits < 31 && (1ll << vbits) <= (long long)g->nv) vbits++;
+    return (unsigned long long)nq << vbits > (1ull << 32) ? 0 : vbits;
+}
+
 int run_queries(Graph* g, const int32_t* srcs_host, const int32_t* srcs_dev, int32_t src0, int32_t nq,
                 void* dist_out, int32_t* pred_out, const sssp_config* cfg_in, cudaStream_t stream,
                 sssp_stats* st_out, bool unit, const Sampling* samp) {
     // a multi-query launch with the library's configuration uses the
     // batch-tuned one of its size class when sssp_autotune_batch made one
+    const bool lib_cfg = !cfg_in;
     if (!cfg_in && nq > 1 && !unit) cfg_in = batch_tuned_for(g, nq);
     sssp_config cfg = cfg_in ? *cfg_in : (g->tuned_valid ? g->tuned : g->defaults);
+    // the library's choice: the wavefront kernels, unless the autotuner timed
+    // the queue engine faster.  They run on any hub layout, but the graph's
+    // own one is restored (or found held by a serving lane) as ever.
+    if (lib_cfg && !samp && (unit || !(nq > 1 ? batch_prefers_queues(g, nq) : g->tuned_queues))) {
+        if (cudaSetDevice(g->device) != cudaSuccess) return SSSP_E_CUDA;
+        const int lrc = ensure_layout(g, cfg.split_arcs ? cfg.split_arcs : kDefaultSplit, stream);
+        if (lrc) return lrc;
+        if (nq > 1 && !key_bits(g, nq)) return SSSP_E_INVAL;
+        const int wrc = run_wave(g, srcs_host, srcs_dev, src0, nq, dist_out, pred_out, stream, st_out, unit);
+        if (wrc != kWaveNotRun) return wrc;
+    }
     // breadth-first: one bucket per level unless the caller chose a delta
     if (unit && (!cfg_in || cfg.delta_u32 == 0)) cfg.delta_u32 = 1;
     const bool lib_delta = !cfg_in || (g->wtype == SSSP_W_F32 ? !(cfg_in->delta_f32 > 0.0f) : cfg_in->delta_u32 == 0);
@@ -602,12 +619,8 @@ int run_queries(Graph* g, const int32_t* srcs_host, const int32_t* srcs_dev, int
     if (rc) return rc;
     const int32_t n = g->n, nv = g->nv;
     const bool mq = nq > 1;
-    int vbits = 0;
-    if (mq) {
-        while (vbits < 31 && (1ll << vbits) <= (long long)nv) vbits++;  // 2^vbits > nv: no key is all ones
-        if (vbits == 0) vbits = 1;
-        if ((unsigned long long)nq << vbits > (1ull << 32)) return SSSP_E_INVAL;
-    }
+    const int vbits = mq ? key_bits(g, nq) : 0;
+    if (mq && !vbits) return SSSP_E_INVAL;
     // unit weights are >= 1: the packed minimum gives the smallest-index parent
     const int pred_mode = pred_out ? (unit ? 1 : pred_mode_for(g)) : 0;
     const bool f32 = g->wtype == SSSP_W_F32 && !unit;
@@ -877,6 +890,24 @@ int run_queries(Graph* g, const int32_t* srcs_host, const int32_t* srcs_dev, int
     }
 }
 
+// Where the arcs of every real vertex lie: its row, or (a split hub, whose row
+// links its shadows) the shadows' rows, which follow one another.
+__global__ void span_kernel(const int32_t* rp, const uint2* adj, int32_t n, int2* span) {
+    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+    for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < n; v += stride) {
+        int32_t b = rp[v], e = rp[v + 1];
+        if (e > b) {
+            const uint32_t first = adj[b].x;
+            if (first >= (uint32_t)n) {
+                const int32_t k = e - b;
+                b = rp[first];
+                e = rp[first + (uint32_t)k];
+            }
+        }
+        span[v] = make_int2(b, e);
+    }
+}
+
 // Builds the device layout with shadow vertices for vertices above `split`
 // arcs.  rp0/adj0 are the validated original arrays (device); on success
 // g->row_ptr / g->adj / g->owner describe the layout (rp0/adj0 are freed
@@ -963,6 +994,16 @@ static int build_layout(Graph* g, int32_t* rp0, uint2* adj0, int32_t split, cuda
     g->mv = mv;
     g->split = split;
     return SSSP_OK;
+}
+
+// g->span for the current layout.
+static int fill_span(Graph* g, cudaStream_t s) {
+    if (!g->span && cudaMalloc((void**)&g->span, sizeof(int2) * (size_t)g->n) != cudaSuccess) {
+        cudaGetLastError();
+        return SSSP_E_NOMEM;
+    }
+    span_kernel<<<grid_for((size_t)g->n, g->sms), 256, 0, s>>>(g->row_ptr, g->adj, g->n, g->span);
+    return cuda_status(cudaStreamSynchronize(s));
 }
 
 // Original arc order from a shadow layout: the arcs of vertex v are its own
@@ -1082,7 +1123,7 @@ int ensure_layout(Graph* g, int32_t split, cudaStream_t s) {
     g->layout_req = split;
     g->feat.shadows = g->nv - g->n;
     g->ws.dirty = true;
-    return SSSP_OK;
+    return fill_span(g, s);
 }
 
 }  // namespace sssp
@@ -1203,6 +1244,7 @@ extern "C" int sssp_graph_create(const int32_t* row_ptr, const int32_t* col_idx,
         if (rc == SSSP_OK) {
             rp0 = nullptr;  // owned by the graph now (or freed by the relayout)
             adj0 = nullptr;
+            rc = fill_span(g, s);
         }
     } while (0);
     cudaFree(col_tmp);
@@ -1213,6 +1255,10 @@ extern "C" int sssp_graph_create(const int32_t* row_ptr, const int32_t* col_idx,
     if (rc != SSSP_OK) {
         cudaFree(rp0);
         cudaFree(adj0);
+        cudaFree(g->row_ptr);
+        cudaFree(g->adj);
+        cudaFree(g->owner);
+        cudaFree(g->span);
         delete g;
         return rc;
     }
@@ -1230,6 +1276,7 @@ extern "C" int sssp_graph_destroy(sssp_graph* gh) {
         cudaFree(g->row_ptr);
         cudaFree(g->adj);
         cudaFree(g->owner);
+        cudaFree(g->span);
     }
     delete g;
     return SSSP_OK;

@@ -143,6 +143,7 @@ extern "C" int sssp_autotune(sssp_graph* gh, const int32_t* srcs, int32_t nsrc, 
     if (budget_ms <= 0 || nsrc <= 0 || !srcs) {
         g->tuned = best;
         g->tuned_valid = true;
+        g->tuned_queues = false;
         if (out) *out = best;
         return SSSP_OK;
     }
@@ -288,6 +289,16 @@ extern "C" int sssp_autotune(sssp_graph* gh, const int32_t* srcs, int32_t nsrc, 
             }
         }
     }
+    // solves without a configuration take the wavefront kernels unless the
+    // queue engine with the tuned configuration is faster
+    std::vector<double> ts;
+    for (int32_t s : hs) {
+        sssp_stats st;
+        const int rc = run_wave(g, nullptr, nullptr, s, 1, dbuf, nullptr, nullptr, &st, false);
+        ts.push_back(rc == SSSP_OK ? st.kernel_ms : INFINITY);
+    }
+    std::sort(ts.begin(), ts.end());
+    g->tuned_queues = best_t < ts[ts.size() / 2];
     cudaFree(dbuf);
     g->tuned = best;
     g->tuned_valid = true;
@@ -317,6 +328,7 @@ extern "C" int sssp_autotune_batch(sssp_graph* gh, const int32_t* srcs, int32_t 
     resolve_auto(g, &base);
     batch_config(g, &base, nq);
     sssp_config best = base;
+    bool queues = false;
     if (budget_ms > 0) {
         void* dbuf = nullptr;
         if (cudaMalloc(&dbuf, sizeof(uint32_t) * (size_t)g->n * (size_t)nq) != cudaSuccess) {
@@ -395,6 +407,9 @@ extern "C" int sssp_autotune_batch(sssp_graph* gh, const int32_t* srcs, int32_t 
                 }
             }
         }
+        sssp_stats st;
+        const int rc = run_wave(g, hs.data(), nullptr, 0, nq, dbuf, nullptr, nullptr, &st, false);
+        queues = rc != SSSP_OK || best_t < st.kernel_ms;
         cudaFree(dbuf);
     }
     const int32_t k = nq_class(nq);
@@ -402,9 +417,10 @@ extern "C" int sssp_autotune_batch(sssp_graph* gh, const int32_t* srcs, int32_t 
     for (Graph::BatchTuned& b : g->batch_tuned)
         if (b.nq_class == k) {
             b.cfg = best;
+            b.queues = queues;
             found = true;
         }
-    if (!found) g->batch_tuned.push_back(Graph::BatchTuned{k, best});
+    if (!found) g->batch_tuned.push_back(Graph::BatchTuned{k, best, queues});
     if (out) *out = best;
     return SSSP_OK;
 }

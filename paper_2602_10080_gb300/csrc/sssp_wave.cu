@@ -1,0 +1,172 @@
+// sssp_wave.cu -- host side of the wavefront kernels (wave.cuh): which calls
+// they take, their launch shape, and one call's launch sequence.
+#include <algorithm>
+#include <cstring>
+
+#include "../../include/sssp.h"
+#include "api_internal.h"
+#include "wave.h"
+
+namespace sssp {
+
+namespace {
+
+struct WavePlan {
+    int log_g = 0;         // log2 of a cluster's blocks
+    int threads = 1024;
+    uint32_t front = 1;
+    double delta = 1.0;
+    int32_t hub_deg = 256;
+    uint32_t wide = kInfU32;
+};
+
+uint32_t pow2_at_least(double x) {
+    uint32_t p = 1;
+    while (p < x && p < (1u << 30)) p <<= 1;
+    return p;
+}
+
+// The kernel and launch shape of a call, from the graph's features; false:
+// the queue engine takes it.
+bool plan_wave(const Graph* g, int32_t nq, WavePlan* w) {
+    const sssp_features& f = g->feat;
+    const double deg = std::max(1.0, f.avg_deg);
+    const bool hubs = f.max_deg > 64.0;
+    // about the average weight over a quarter of the degree: of the widths
+    // 1/2 to 4 times this, meshes and G(n, m) graphs run within 5% of the best
+    w->delta = 4.0 * f.avg_w / deg;
+    // Threads of one cluster: one for eight vertices or 32 arcs, 1024 to
+    // 16384 in 16 blocks (8 for the smallest).  GB300, us a solve: directed
+    // 1000 vertices 8 x 128 76, 1 x 1024 82; grid 256^2 16 x 512 1114, 8 x 512
+    // 1153, 1 x 1024 1800; grid 1024^2 16 x 1024 5670, 8 x 1024 8500.
+    const uint32_t total =
+        std::min(16384u, std::max(1024u, pow2_at_least(std::max((double)g->n / 8.0, (double)g->m / 32.0))));
+    if (nq == 1) {
+        const bool thin = deg <= 6.0 && !hubs && g->n <= (1 << 21);
+        if (g->m <= (1 << 19) || (thin && !g->wide)) {
+            w->log_g = total > 1024u ? 4 : 3;
+            w->threads = (int)(total >> w->log_g);
+            // raise the threshold while there is less than a vertex for every
+            // 16 threads: grid 256^2 1114 us (1088 at a 32nd, 1180 at an
+            // eighth), grid 1024^2 5670 (5740, 5790)
+            w->front = total / 16u;
+            // sparse random graphs look like meshes and have wide fronts, for
+            // which 16 SMs are too few; such a solve starts over in the queues
+            if (g->m > (1 << 19)) w->wide = 24576u;
+            return true;
+        }
+        return false;
+    }
+    // a batch on a small graph or a mesh: one cluster per query, as wide as the
+    // queries leave room for (13 queries on grid 301 x 257: 8 blocks 1690 us,
+    // 4: 1880, 1: 2130)
+    if (g->m > (1 << 21) || (hubs && g->m > (1 << 18))) return false;
+    w->log_g = 4;
+    while (w->log_g > 0 && (nq << w->log_g) > g->sms) w->log_g--;
+    w->threads = (int)std::max(128u, std::min(w->log_g ? 512u : 1024u, total >> w->log_g));
+    w->front = std::max(1u, (uint32_t)(w->threads << w->log_g) / 16u);
+    return true;
+}
+
+}  // namespace
+
+int run_wave(Graph* g, const int32_t* srcs_host, const int32_t* srcs_dev, int32_t src0, int32_t nq, void* dist_out,
+             int32_t* pred_out, cudaStream_t stream, sssp_stats* st_out, bool unit) {
+    WavePlan plan;
+    if (g->device < 0 || g->device >= 64 || !plan_wave(g, nq, &plan)) return kWaveNotRun;
+    if (cudaSetDevice(g->device) != cudaSuccess) return SSSP_E_CUDA;
+    const int32_t n = g->n;
+    const bool f32 = g->wtype == SSSP_W_F32 && !unit;
+    // unit weights are >= 1: the packed minimum gives the smallest-index parent
+    const int pred_mode = pred_out ? (unit ? 1 : pred_mode_for(g)) : 0;
+    WaveParams P;
+    std::memset(&P, 0, sizeof(P));
+    // places: a power of two of at least n, with few bits per word on a small
+    // graph, so that every thread has a word
+    int bits = 0, log_t = 0;
+    while ((1ll << bits) < n) bits++;
+    for (log_t = plan.log_g; (1 << (log_t - plan.log_g)) < plan.threads;) log_t++;
+    P.log_b = std::max(0, std::min(5, bits - log_t));
+    P.mask = (uint32_t)((1ull << bits) - 1);
+    P.log_g = plan.log_g;
+    const uint32_t all_words = 1u << (bits - P.log_b);
+    P.words = (int32_t)std::max(1u, all_words >> P.log_g);
+    const size_t smem = (size_t)P.words * 4 * sizeof(uint32_t);
+    if (smem > 200 * 1024) return kWaveNotRun;
+
+    Workspace& ws = g->ws;
+    int rc = ws.ensure_ctrl(stream);
+    if (rc) return rc;
+    const size_t cells = (size_t)nq * (size_t)n;
+    const bool dist_dev = is_device_ptr(dist_out), pred_dev = pred_out && is_device_ptr(pred_out);
+    uint32_t* dd = (uint32_t*)dist_out;
+    int32_t* pp = pred_out;
+    if (!dist_dev) {
+        if ((rc = grow(&ws.out_d, &ws.out_d_n, cells))) return rc;
+        dd = ws.out_d;
+    }
+    if (pred_out && !pred_dev) {
+        if ((rc = grow(&ws.out_p, &ws.out_p_n, cells))) return rc;
+        pp = ws.out_p;
+    }
+    if (pred_mode && (rc = grow(&ws.d64, &ws.d64_n, cells))) return rc;
+    if (nq > 1) {
+        if ((rc = grow(&ws.srcs, &ws.srcs_n, (size_t)nq))) return rc;
+        cudaMemcpyAsync(ws.srcs, srcs_dev ? srcs_dev : srcs_host, sizeof(int32_t) * nq,
+                        srcs_dev ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice, stream);
+        P.srcs = ws.srcs;
+    }
+    P.span = g->span;
+    P.adj = g->adj;
+    P.n = n;
+    P.src0 = src0;
+    P.work = pred_mode ? (void*)ws.d64 : (void*)dd;
+    P.dist_out = dd;
+    P.pred_out = pp;
+    if (f32) P.delta = __float_as_uint_host((float)std::max(1e-30, plan.delta));
+    else P.delta = (uint32_t)std::min(4.0e9, std::max(1.0, plan.delta));
+    P.front = plan.front;
+    P.wide = plan.wide;
+    P.unit = unit ? 1 : 0;
+    P.hub_deg = plan.hub_deg;
+    P.has_hubs = g->feat.max_deg > (double)P.hub_deg;
+    P.ctrl = ws.ctrl;
+    P.timeout_ns = 20000ull * 1000000ull;
+    cudaMemsetAsync(ws.ctrl, 0, sizeof(Ctrl), stream);
+    cudaEventRecord(ws.ev1, stream);
+    const cudaError_t le = launch_wave(f32 ? 1 : 0, pred_mode, P, nq, plan.threads, smem, stream);
+    if (le != cudaSuccess) {
+        // no room for the cluster on this device
+        cudaGetLastError();
+        return kWaveNotRun;
+    }
+    cudaEventRecord(ws.ev2, stream);
+    if (!dist_dev) cudaMemcpyAsync(dist_out, dd, cells * 4, cudaMemcpyDeviceToHost, stream);
+    if (pred_out && !pred_dev) cudaMemcpyAsync(pred_out, pp, cells * 4, cudaMemcpyDeviceToHost, stream);
+    cudaMemcpyAsync(ws.host_ctrl, ws.ctrl, sizeof(Ctrl), cudaMemcpyDeviceToHost, stream);
+    const cudaError_t ce = cudaStreamSynchronize(stream);
+    if (ce != cudaSuccess) return cuda_status(ce);
+    const Ctrl& hc = *ws.host_ctrl;
+    if (hc.error == kErrWide) {
+        g->wide = true;
+        return run_wave(g, srcs_host, srcs_dev, src0, nq, dist_out, pred_out, stream, st_out, unit);
+    }
+    float ms = 0;
+    cudaEventElapsedTime(&ms, ws.ev1, ws.ev2);
+    sssp_stats st;
+    std::memset(&st, 0, sizeof(st));
+    st.kernel_ms = st.total_ms = ms;
+    st.reached = st.reached_arcs = -1;
+    st.relax_arcs = (int64_t)hc.stats[kStRelax];
+    st.improved = (int64_t)hc.stats[kStImproved];
+    st.rounds = (int64_t)hc.stats[kStIter];
+    st.grid_blocks = nq << P.log_g;
+    st.block_threads = plan.threads;
+    st.attempts = 1;
+    g->last = st;
+    if (st_out) *st_out = st;
+    if (hc.error == kErrNone && hc.finished == nq) return SSSP_OK;
+    return hc.error == kErrTimeout ? SSSP_E_TIMEOUT : SSSP_E_CUDA;
+}
+
+}  // namespace sssp

@@ -1,0 +1,502 @@
+// wave.cuh -- step-synchronous wavefront searches.
+//
+// A search is advanced in steps: the vertices that wait for relaxation are
+// bits, a step relaxes them all, and a barrier ends it.  A push is one OR
+// without an answer, a pop is a word, no queue can overflow, and no element
+// is stale or queued twice.
+//
+//   wave_kernel  one cluster of 1 to 16 blocks per query, its bits in the
+//                cluster's shared memory, the hardware cluster barrier between
+//                steps.  For graphs whose wavefront is thin (meshes, small
+//                graphs), where the latency of a hop is all there is; a batch
+//                is one cluster per query, and no cluster waits for another.
+//
+// Order: vertices below the threshold T wait in `near` and are relaxed in the
+// next step; the others wait in `far`.  When fewer than `front` vertices are
+// waiting in near, T grows by delta and the far bits below it are relaxed in
+// the same step (delta-stepping with a width that follows the parallelism:
+// a step costs the same for one vertex and for one per thread, so a thin
+// front is filled up with speculative work, which saves steps).  Every
+// label-correcting order ends in the same distances.
+#pragma once
+
+#include "mlmq.cuh"
+
+namespace sssp {
+
+constexpr int kWaveMaxCluster = 16;
+constexpr int kWaveHubs = 128;        // hubs one block expands together per step (later ones: by their warp)
+constexpr uint32_t kWaveHash = 0x9E3779B1u;      // odd: v -> v * hash mod 2^bits is one to one
+constexpr uint32_t kWaveHashInv = 0x0E8B2F51u;   // its inverse mod 2^32
+static_assert((uint32_t)(0x9E3779B1ull * 0x0E8B2F51ull) == 1u, "inverse of the vertex hash");
+
+struct WaveParams {
+    const int2* span;         // [n] arcs of a vertex: adj[span.x .. span.y)
+    const uint2* adj;         // (col, weight bits); hubs' slices are contiguous
+    int32_t n;
+    const int32_t* srcs;      // [nq] or null (one query from src0)
+    int32_t src0;
+    void* work;               // DistT[nq * n]
+    uint32_t* dist_out;       // [nq * n], or null when work holds the caller's distances
+    int32_t* pred_out;        // [nq * n] (PRED != 0)
+    uint32_t delta;           // threshold step (u32, or f32 bits)
+    uint32_t front;           // vertices waiting in near below which T grows
+    // Vertex v waits at place p = v * hash mod 2^bits: bit p mod 2^log_b of
+    // word p / 2^log_b.  The hash spreads neighbouring vertices, and so every
+    // front, over the words and their owners.
+    uint32_t mask;            // 2^bits - 1
+    int32_t log_b;            // log2 of the bits used per word (0..5)
+    int32_t log_g;            // log2 of the cluster's blocks: word w lives in block w % G
+    int32_t words;            // words per block
+    int32_t unit;             // breadth-first: every arc weighs 1, no threshold
+    int32_t hub_deg;          // a vertex with more arcs is not left to one warp
+    int32_t has_hubs;
+    uint32_t wide;            // wave: give up (kErrWide) when more vertices than this wait in near
+    Ctrl* ctrl;               // error word, finished queries, statistics
+    unsigned long long timeout_ns;
+};
+
+struct WaveSlot {
+    uint32_t near, fmin, stop, pad;
+};
+
+struct WaveHub {
+    uint32_t v, d;
+    int2 arcs;
+};
+
+struct WaveShared {
+    WaveSlot slot[2][kWaveMaxCluster];  // what every block of the cluster reports at the end of a step
+    uint32_t near[4], fmin[4], nhub[4]; // this block's sums of step s, set s % 4
+    WaveHub hub[kWaveHubs];
+    uint32_t list[32][64];              // per warp: vertices taken from the words (bit 31: from far)
+};
+
+__device__ __forceinline__ uint32_t cluster_rank() {
+    uint32_t r;
+    asm("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+    return r;
+}
+__device__ __forceinline__ void cluster_barrier() {
+    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+__device__ __forceinline__ uint32_t map_rank(uint32_t smem, uint32_t rank) {
+    uint32_t a;
+    asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"(smem), "r"(rank));
+    return a;
+}
+__device__ __forceinline__ void st_cluster(uint32_t a, uint32_t v) {
+    asm volatile("st.relaxed.cluster.shared::cluster.u32 [%0], %1;" ::"r"(a), "r"(v) : "memory");
+}
+
+// T raised above `base` by delta, and at least above `low` (an f32 delta may
+// be absorbed, a u32 sum saturates)
+template <int WT>
+__device__ __forceinline__ uint32_t wave_raise(uint32_t base, uint32_t delta, uint32_t low) {
+    uint32_t t;
+    if (WT == 0) {
+        t = base + delta;
+        if (t < base) t = kInfU32;
+    } else {
+        t = __float_as_uint(__uint_as_float(base) + __uint_as_float(delta));
+        if (t < base) t = base;
+    }
+    return t > low ? t : low + 1u;
+}
+
+// Where the pending bits live: one block's shared memory, a cluster's, or
+// global memory.
+enum WaveMode { kWaveBlock = 0, kWaveCluster = 1, kWaveGrid = 2 };
+
+template <int WT, int PRED, int MODE>
+struct Wave {
+    using DistT = typename std::conditional<PRED == 0, uint32_t, unsigned long long>::type;
+    using A = Arith<WT>;
+    using Addr = typename std::conditional<MODE == kWaveGrid, uint32_t*, uint32_t>::type;
+
+    const WaveParams& P;
+    DistT* dist;
+    uint32_t* list;            // this warp's list
+    uint32_t T, Told;
+    Addr near_w, far_w;        // the words written in this step
+    uint32_t n_imp, fmin;      // this thread's near improvements and smallest far distance of the step
+    uint32_t n_relax;          // arcs relaxed by this thread
+
+    static __device__ __forceinline__ uint32_t dpart(uint32_t w) { return w; }
+    static __device__ __forceinline__ uint32_t dpart(unsigned long long w) { return (uint32_t)(w >> 32); }
+
+    __device__ __forceinline__ Addr bit_addr(Addr base, uint32_t v, uint32_t& mask) const {
+        const uint32_t p = (v * kWaveHash) & P.mask, w = p >> P.log_b;
+        mask = 1u << (p & ((1u << P.log_b) - 1u));
+        if constexpr (MODE == kWaveGrid) return base + w;
+        else if constexpr (MODE == kWaveCluster)
+            return map_rank(base + (w >> P.log_g) * 4u, w & ((1u << P.log_g) - 1u));
+        else return base + w * 4u;
+    }
+    // the vertex of bit b of word w
+    __device__ __forceinline__ uint32_t vertex(uint32_t w, uint32_t b) const {
+        return (((w << P.log_b) | b) * kWaveHashInv) & P.mask;
+    }
+    __device__ __forceinline__ void red_or(Addr a, uint32_t v) const {
+        if constexpr (MODE == kWaveGrid)
+            asm volatile("red.relaxed.gpu.global.or.b32 [%0], %1;" ::"l"(a), "r"(v) : "memory");
+        else if constexpr (MODE == kWaveCluster)
+            asm volatile("red.relaxed.cluster.shared::cluster.or.b32 [%0], %1;" ::"r"(a), "r"(v) : "memory");
+        else asm volatile("red.relaxed.cta.shared::cta.or.b32 [%0], %1;" ::"r"(a), "r"(v) : "memory");
+    }
+
+    // Relaxes K arcs (u at distance du) -> a.x of weight a.y whose distance
+    // words are c: lowers dist[v] without waiting for the answer and marks v
+    // when the distance beat the loaded one (whoever lowers dist[v] saw a
+    // larger value, so the last improvement always marks it).  Straight-line
+    // code with predicated stores: as branches, four arcs took 2200 cycles of
+    // a 9300-cycle step (grid 256^2 on GB300), like this 300.
+    template <int K>
+    __device__ __forceinline__ void relax(const uint32_t (&u)[K], const uint32_t (&du)[K], const uint2 (&a)[K],
+                                          const DistT (&c)[K], const bool (&in)[K]) {
+        uint32_t nd[K], mask[K];
+        Addr ad[K];
+        bool upd[K], imp[K];
+#pragma unroll
+        for (int k = 0; k < K; k++) {
+            nd[k] = A::add(du[k], P.unit ? 1u : a[k].y);
+            if (PRED == 0) {
+                upd[k] = imp[k] = in[k] && nd[k] < (uint32_t)c[k];
+            } else {
+                imp[k] = in[k] && nd[k] < dpart(c[k]);
+                upd[k] = PRED == 2 ? imp[k]
+                                   : in[k] && (((unsigned long long)nd[k] << 32) | u[k]) < (unsigned long long)c[k];
+            }
+            ad[k] = bit_addr(nd[k] < T ? near_w : far_w, a[k].x, mask[k]);
+        }
+#pragma unroll
+        for (int k = 0; k < K; k++) {
+            if (PRED == 0) {
+                if (upd[k]) red_min(reinterpret_cast<uint32_t*>(dist) + a[k].x, nd[k]);
+            } else {
+                unsigned long long* p = reinterpret_cast<unsigned long long*>(dist) + a[k].x;
+                const unsigned long long cand = ((unsigned long long)nd[k] << 32) | u[k];
+                if (PRED == 1) {
+                    if (upd[k]) red_min(p, cand);
+                } else {
+                    unsigned long long x = (unsigned long long)c[k];
+                    while (imp[k]) {
+                        const unsigned long long old = atomicCAS(p, x, cand);
+                        if (old == x) break;
+                        x = old;
+                        imp[k] = nd[k] < (uint32_t)(x >> 32);
+                    }
+                }
+            }
+        }
+#pragma unroll
+        for (int k = 0; k < K; k++) {
+            if (imp[k]) red_or(ad[k], mask[k]);
+            n_imp += imp[k] && nd[k] < T ? 1u : 0u;
+            fmin = imp[k] && nd[k] >= T ? min(fmin, nd[k]) : fmin;
+        }
+    }
+
+    // Up to four arcs of one vertex, `stride` apart, all loads in flight together.
+    __device__ __forceinline__ void arcs4(uint32_t u, uint32_t du, int32_t e, int32_t stride, int32_t end) {
+        uint2 a[4];
+        DistT c[4];
+        uint32_t uu[4], dd[4];
+        bool in[4];
+#pragma unroll
+        for (int k = 0; k < 4; k++) {
+            in[k] = e + k * stride < end;
+            uu[k] = u;
+            dd[k] = du;
+            a[k] = in[k] ? ld_arc(P.adj + e + k * stride) : make_uint2(0u, 0u);
+        }
+#pragma unroll
+        for (int k = 0; k < 4; k++) c[k] = in[k] ? ld_dist(dist + a[k].x) : (DistT)0;
+        relax<4>(uu, dd, a, c, in);
+    }
+
+    // Arcs g0 + lane + 32 k (k < 4) of the warp's concatenated rows (ex: arcs
+    // before this lane's vertex u, row at rs, distance du).
+    __device__ __forceinline__ void arcs_packed(int32_t g0, int32_t total, int32_t ex, int32_t rs, uint32_t du,
+                                                uint32_t u) {
+        uint2 a[4];
+        DistT c[4];
+        uint32_t dj[4], uj[4];
+        bool in[4];
+#pragma unroll
+        for (int k = 0; k < 4; k++) {
+            const int32_t g = g0 + 32 * k + (int32_t)lane_id();
+            int j = 0;
+#pragma unroll
+            for (int s = 16; s >= 1; s >>= 1)
+                if (__shfl_sync(kFull, ex, j + s) <= g) j += s;
+            const int32_t row = __shfl_sync(kFull, rs, j) + (g - __shfl_sync(kFull, ex, j));
+            dj[k] = __shfl_sync(kFull, du, j);
+            uj[k] = PRED != 0 ? __shfl_sync(kFull, u, j) : 0u;
+            in[k] = g < total;
+            a[k] = in[k] ? ld_arc(P.adj + row) : make_uint2(0u, 0u);
+        }
+#pragma unroll
+        for (int k = 0; k < 4; k++) c[k] = in[k] ? ld_dist(dist + a[k].x) : (DistT)0;
+        relax<4>(uj, dj, a, c, in);
+    }
+
+    // Relaxes the k <= 32 vertices list[from ..], one per lane; `hub(v, d,
+    // arcs)` takes those with more than hub_deg arcs (it returns false for
+    // one that the warp has to expand all the same).
+    template <typename Hub>
+    __device__ __forceinline__ void relax_list(uint32_t from, uint32_t k, Hub&& hub) {
+        const uint32_t lane = lane_id();
+        bool have = lane < k;
+        uint32_t v = 0u, d = 0u;
+        int2 sp = make_int2(0, 0);
+        if (have) {
+            v = list[from + lane];
+            const bool is_far = (v >> 31) != 0u;
+            v &= 0x7fffffffu;
+            const DistT dw = ld_dist(dist + v);
+            sp = __ldg(P.span + v);
+            d = dpart(dw);
+            if (is_far) {
+                // below the old threshold: it went through near since
+                if (d < Told) {
+                    have = false;
+                } else if (d >= T) {
+                    have = false;
+                    uint32_t mask;
+                    const Addr a = bit_addr(far_w, v, mask);
+                    red_or(a, mask);
+                    fmin = min(fmin, d);
+                }
+            }
+        }
+        int32_t deg = have ? sp.y - sp.x : 0;
+        n_relax += (uint32_t)deg;
+        if (P.has_hubs) deg = hub(v, d, sp, deg);
+        if (__reduce_max_sync(kFull, (uint32_t)deg) <= 4u) {
+            // few arcs a vertex: each lane its own
+            arcs4(v, d, sp.x, 1, sp.x + deg);
+        } else {
+            // the batch's arcs spread over the lanes, 128 at a time
+            int32_t incl = deg;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const int32_t x = __shfl_up_sync(kFull, incl, o);
+                if (lane >= (uint32_t)o) incl += x;
+            }
+            const int32_t ex = incl - deg, total = __shfl_sync(kFull, incl, 31);
+            for (int32_t g0 = 0; g0 < total; g0 += 128) arcs_packed(g0, total, ex, sp.x, d, v);
+        }
+        __syncwarp();
+    }
+
+    // Empties the words i = first, first + stride, ... below `words` (32 at a
+    // time: this lane's is i + lane) into the list and relaxes the list's
+    // vertices 32 at a time.  `take(i, nb, fb)` reads and clears a lane's word.
+    template <typename Take, typename Vertex, typename Hub>
+    __device__ __forceinline__ void sweep(uint32_t first, uint32_t stride, uint32_t words, Take&& take,
+                                          Vertex&& vertex_of, Hub&& hub) {
+        const uint32_t lane = lane_id();
+        uint32_t held = 0u, nb = 0u, fb = 0u, base = first;
+        bool more = base < words;
+        if (more) take(base + lane, nb, fb);
+        while (more || held) {
+            while (more && held < 32u) {
+                const bool have = (nb | fb) != 0u;
+                const uint32_t m = __ballot_sync(kFull, have);
+                if (!m) {
+                    base += stride;
+                    more = base < words;
+                    if (more) take(base + lane, nb, fb);
+                    continue;
+                }
+                if (have) {
+                    const uint32_t b = (uint32_t)__ffs((int)(nb | fb)) - 1u;
+                    list[held + __popc(m & lanemask_lt())] =
+                        vertex_of(base + lane, b) | ((nb >> b) & 1u ? 0u : 0x80000000u);
+                    nb &= ~(1u << b);
+                    fb &= ~(1u << b);
+                }
+                held += __popc(m);
+                __syncwarp();
+            }
+            if (!held) break;
+            const uint32_t k = held < 32u ? held : 32u;
+            held -= k;
+            relax_list(held, k, hub);
+        }
+    }
+
+    // The results of vertices first, first + stride, ... (packed words only).
+    __device__ __forceinline__ void unpack(size_t out, uint32_t first, uint32_t stride) const {
+        if (PRED == 0) return;
+        for (uint32_t v = first; v < (uint32_t)P.n; v += stride) {
+            const unsigned long long x = __ldcg(reinterpret_cast<const unsigned long long*>(dist) + v);
+            uint32_t dd = (uint32_t)(x >> 32);
+            if (WT == 1 && dd == kInfU32) dd = kInfF32;
+            P.dist_out[out + v] = dd;
+            P.pred_out[out + v] = (int32_t)(uint32_t)x;
+        }
+    }
+
+    __device__ __forceinline__ void init(uint32_t src, uint32_t first, uint32_t stride) const {
+        const DistT inf = PRED != 0 ? (DistT)~0ull : (DistT)(WT == 1 ? kInfF32 : kInfU32);
+        for (uint32_t v = first; v < (uint32_t)P.n; v += stride)
+            dist[v] = v == src ? (DistT)(PRED != 0 ? src : 0u) : inf;
+    }
+
+    // The next step's threshold from this step's sums.  Returns 0: no more
+    // work, 1: near only, 2: near and the far bits below the new T.
+    __device__ __forceinline__ int advance(uint32_t near, uint32_t far_low) {
+        if (near < P.front && far_low != kInfU32) {
+            Told = T;
+            T = near ? wave_raise<WT>(T, P.delta, 0u) : wave_raise<WT>(max(T, far_low), P.delta, far_low);
+            return 2;
+        }
+        return near ? 1 : 0;
+    }
+
+    __device__ __forceinline__ void publish(uint32_t improved) const {
+        unsigned long long r64 = n_relax, i64 = improved;
+        for (int o = 16; o > 0; o >>= 1) {
+            r64 += __shfl_down_sync(kFull, r64, o);
+            i64 += __shfl_down_sync(kFull, i64, o);
+        }
+        if (lane_id() == 0 && r64) {
+            atomicAdd(&P.ctrl->stats[kStRelax], r64);
+            atomicAdd(&P.ctrl->stats[kStImproved], i64);
+        }
+    }
+};
+
+// One cluster (CL) or one block per query.  The blocks exchange a step's sums
+// by writing them into every block's slots; one cluster barrier then makes
+// them and the step's marks visible.  Two slot sets alternate: a block can
+// write set s + 2 only after all blocks passed barrier s + 1, after reading s.
+template <int WT, int PRED, bool CL>
+__global__ void __launch_bounds__(1024, 1) wave_kernel(const __grid_constant__ WaveParams P) {
+    using W = Wave<WT, PRED, CL ? kWaveCluster : kWaveBlock>;
+    using DistT = typename W::DistT;
+    extern __shared__ __align__(16) uint32_t wave_words[];   // near[2], far[2]
+    __shared__ WaveShared S;
+    const uint32_t tid = threadIdx.x, nt = blockDim.x, lane = tid & 31u;
+    const uint32_t G = CL ? 1u << P.log_g : 1u, rank = CL ? cluster_rank() : 0u;
+    const uint32_t q = CL ? blockIdx.x >> P.log_g : blockIdx.x;
+    const uint32_t src = (uint32_t)(P.srcs ? P.srcs[q] : P.src0);
+    const uint32_t words = (uint32_t)P.words;
+    W w{P, reinterpret_cast<DistT*>(P.work) + (size_t)q * (size_t)P.n, S.list[tid >> 5],
+        P.unit ? kInfU32 : wave_raise<WT>(0u, P.delta, 0u), 0u, 0u, 0u, 0u, kInfU32, 0u};
+
+    // every distance to infinity but the source's, and its pending bit
+    w.init(src, rank * nt + tid, G * nt);
+    for (uint32_t i = tid; i < 4u * words; i += nt) wave_words[i] = 0u;
+    if (tid < 4u) {
+        S.near[tid] = S.nhub[tid] = 0u;
+        S.fmin[tid] = kInfU32;
+    }
+    __syncthreads();
+    {
+        const uint32_t p = (src * kWaveHash) & P.mask, sw = p >> P.log_b;
+        if (tid == 0 && (sw & (G - 1u)) == rank) wave_words[sw >> P.log_g] = 1u << (p & ((1u << P.log_b) - 1u));
+    }
+    if (CL) cluster_barrier();
+    else __syncthreads();
+
+    uint32_t cur = 0u, fw = 0u, far_low = kInfU32;   // far_low: no far vertex lies below it
+    uint32_t n_improved = 0, steps = 0;
+    const unsigned long long deadline = gtime() + P.timeout_ns;
+    int error = kErrNone, what = 1;
+    while (what) {
+        const uint32_t par = steps & 1u, set = steps & 3u;
+        const bool scan_far = what == 2;
+        uint32_t* near_r = wave_words + cur * words;
+        uint32_t* far_r = wave_words + (2u + fw) * words;
+        if (scan_far) fw ^= 1u;
+        cur ^= 1u;
+        w.near_w = (uint32_t)__cvta_generic_to_shared(wave_words + cur * words);
+        w.far_w = (uint32_t)__cvta_generic_to_shared(wave_words + (2u + fw) * words);
+        w.n_imp = 0u;
+        w.fmin = kInfU32;
+        w.sweep(
+            tid & ~31u, nt, words,
+            [&](uint32_t i, uint32_t& nb, uint32_t& fb) {
+                nb = fb = 0u;
+                if (i < words) {
+                    nb = near_r[i];
+                    if (nb) near_r[i] = 0u;
+                    if (scan_far) {
+                        fb = far_r[i];
+                        if (fb) far_r[i] = 0u;
+                        fb &= ~nb;
+                    }
+                }
+            },
+            [&](uint32_t i, uint32_t b) { return w.vertex((i << P.log_g) | rank, b); },
+            [&](uint32_t v, uint32_t d, int2 sp, int32_t deg) {
+                if (deg <= P.hub_deg) return deg;
+                const uint32_t h = atomicAdd(&S.nhub[set], 1u);
+                if (h >= (uint32_t)kWaveHubs) return deg;
+                S.hub[h] = WaveHub{v, d, sp};
+                return 0;
+            });
+        if (P.has_hubs) {
+            // a hub is expanded by its whole block
+            __syncthreads();
+            const uint32_t nh = min(S.nhub[set], (uint32_t)kWaveHubs);
+            for (uint32_t h = 0; h < nh; h++) {
+                const WaveHub hb = S.hub[h];
+                for (int32_t e = hb.arcs.x + (int32_t)tid; e < hb.arcs.y; e += 4 * (int32_t)nt)
+                    w.arcs4(hb.v, hb.d, e, (int32_t)nt, hb.arcs.y);
+            }
+        }
+        // the step's sums
+        n_improved += w.n_imp;
+        const uint32_t imp = __reduce_add_sync(kFull, w.n_imp), fm = __reduce_min_sync(kFull, w.fmin);
+        if (lane == 0) {
+            if (imp) atomicAdd(&S.near[set], imp);
+            if (fm != kInfU32) atomicMin(&S.fmin[set], fm);
+        }
+        __syncthreads();
+        // set s + 2 is empty before anyone adds to it: that comes after the
+        // next step's __syncthreads
+        if (tid == 0) {
+            const uint32_t z = (steps + 2u) & 3u;
+            S.near[z] = S.nhub[z] = 0u;
+            S.fmin[z] = kInfU32;
+        }
+        uint32_t near, sfm, stop = 0u;
+        if (CL) {
+            if (tid < G) {
+                const uint32_t a = map_rank((uint32_t)__cvta_generic_to_shared(&S.slot[par][rank]), tid);
+                st_cluster(a, S.near[set]);
+                st_cluster(a + 4u, S.fmin[set]);
+                if (rank == 0) st_cluster(a + 8u, (steps & 255u) == 255u && gtime() > deadline);
+            }
+            cluster_barrier();
+            const bool in = lane < G;
+            near = __reduce_add_sync(kFull, in ? S.slot[par][lane].near : 0u);
+            sfm = __reduce_min_sync(kFull, in ? S.slot[par][lane].fmin : kInfU32);
+            stop = S.slot[par][0].stop;
+        } else {
+            near = S.near[set];
+            sfm = S.fmin[set];
+            if ((steps & 255u) == 255u) stop = __syncthreads_or(gtime() > deadline);
+        }
+        steps++;
+        far_low = scan_far ? sfm : min(far_low, sfm);
+        what = w.advance(near, far_low);
+        if (what && (stop || near > P.wide)) {
+            error = stop ? kErrTimeout : kErrWide;
+            break;
+        }
+    }
+    w.unpack((size_t)q * (size_t)P.n, rank * nt + tid, G * nt);
+    w.publish(n_improved);
+    if (rank == 0 && tid == 0) {
+        atomicAdd(&P.ctrl->stats[kStIter], (unsigned long long)steps);
+        if (error) raise_error(P.ctrl, error, 20, (int)q);
+        else atomicAdd(&P.ctrl->finished, 1);
+    }
+}
+
+}  // namespace sssp

@@ -1,0 +1,148 @@
+"""The wavefront kernels (calls without a configuration) against the oracle
+at the sizes where they can go wrong: around a word, a warp and a block of
+pending bits, one block and clusters, hubs beyond a block's list, a front too
+wide for a cluster, thresholds that saturate or absorb their step, and the
+same answers as the queue engine."""
+import numpy as np
+import pytest
+import torch
+
+import graphgen as gg
+import oracle
+import paper_2602_10080_gb300 as S
+from gpu_util import assert_exact, assert_exact_many, cfg, gpu_batch, gpu_solve, upload
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _built():
+    S.build()
+    S.lib()
+
+
+def path(n, w):
+    return gg.from_edges(n, [(v, v + 1, w(v)) for v in range(n - 1)] + [(v + 1, v, w(v)) for v in range(n - 1)])
+
+
+def hub_graph(hubs, arcs):
+    """0 -> every hub (weight 1); hub h -> `arcs` targets shared by the hubs."""
+    n = 1 + hubs + 2 * arcs
+    e = [(0, 1 + h, 1 + h % 2) for h in range(hubs)]
+    e += [(1 + h, 1 + hubs + (h * 37 + k) % (2 * arcs), 1 + (h * 7 + k * 3) % 50) for h in range(hubs)
+          for k in range(arcs)]
+    return gg.from_edges(n, e)
+
+
+def both(g, src):
+    """With and without predecessors, against the oracle and the queue engine."""
+    G = upload(g)
+    d, p = gpu_solve(G, src, pred=True)
+    assert_exact(g, src, d, p)
+    d2, _ = gpu_solve(G, src, pred=False)
+    np.testing.assert_array_equal(d2, d)
+    d3, p3 = gpu_solve(G, src, pred=True, config=cfg())
+    np.testing.assert_array_equal(d3, d)
+    if g.wtype == "u32" and g.m and int(g.w.min()) >= 1:
+        np.testing.assert_array_equal(p3, p)
+    G.close()
+
+
+@pytest.mark.parametrize("n", [1, 2, 31, 32, 33, 1023, 1024, 1025, 8191, 8193, 20000])
+def test_paths_around_words_and_blocks(n):
+    both(path(n, lambda v: 1 + v * 7919 % 100), n // 2)
+
+
+@pytest.mark.parametrize("wtype", ["u32", "f32"])
+@pytest.mark.parametrize("n,deg", [(300, 3), (5000, 7), (40000, 12)])
+def test_random_directed(n, deg, wtype):
+    for lo in (0, 1):
+        g = gg.random_directed(n, n * deg, lo, 50, seed=n + lo, wtype=wtype)
+        both(g, 1)
+
+
+@pytest.mark.parametrize("hubs,arcs", [(1, 3000), (5, 257), (600, 300)])
+def test_hubs_in_a_cluster(hubs, arcs):
+    both(hub_graph(hubs, arcs), 0)
+
+
+def test_more_hubs_than_a_block_lists():
+    """One block per query, 200 hubs in one step, the list holds 128."""
+    g = hub_graph(200, 257)
+    G = upload(g)
+    srcs = np.array([0, 1, 200, g.n - 1] * 40, np.int32)
+    d, p = gpu_batch(G, srcs, pred=True)
+    assert_exact_many(g, srcs, d, p)
+    G.close()
+
+
+@pytest.mark.parametrize("nq", [2, 9, 10, 19, 38, 77, 153])
+def test_batches_of_clusters(nq):
+    """Every cluster size; repeated sources are independent queries."""
+    g = gg.grid(67, 41, 1, 100, seed=nq)
+    G = upload(g)
+    srcs = (np.arange(nq) * 7919 % (g.n // 2)).astype(np.int32)
+    d, p = gpu_batch(G, srcs, pred=True, host=nq % 2 == 1)
+    assert_exact_many(g, srcs, d, p)
+    G.close()
+
+
+def test_thresholds_at_the_ends():
+    # lengths saturate at 2^32 - 2, and the threshold with them
+    both(path(40, lambda v: 0xFFFFFFFF if v % 3 == 0 else 0x70000000), 0)
+    # the threshold's step is absorbed by the distances it is added to
+    f = gg.from_edges(300, [(v, v + 1, np.float32(1e30 if v < 5 else 1e-6)) for v in range(299)], wtype="f32")
+    both(f, 0)
+    # no arc, and no arc out of the source
+    both(gg.from_edges(700, [(v, v + 1, 5) for v in range(1, 699)]), 0)
+
+
+@pytest.mark.parametrize("n,deg", [(200_000, 4), (130_000, 6)])
+def test_front_too_wide_for_a_cluster(n, deg):
+    """Sparse random graphs begin in one cluster and start over in the queues."""
+    both(gg.random_directed(n, n * deg, 1, 100, seed=deg), 3)
+
+
+def test_levels():
+    for g in (gg.grid(300, 200, 1, 9, seed=1), hub_graph(600, 300)):
+        src = 0
+        G = upload(g)
+        lev = torch.empty(G.n, dtype=torch.int32, device="cuda")
+        par = torch.empty(G.n, dtype=torch.int32, device="cuda")
+        G.bfs(src, lev, par)
+        torch.cuda.synchronize()
+        unit = np.ones(g.m, np.uint32)
+        ref = oracle.dijkstra_u32(g.row_ptr, g.col, unit, src)
+        np.testing.assert_array_equal(lev.cpu().numpy().view(np.uint32), ref)
+        np.testing.assert_array_equal(par.cpu().numpy(), oracle.pred_canonical_u32(g.row_ptr, g.col, unit, src, ref))
+        G.close()
+
+
+def test_layout_of_another_threshold():
+    """The kernels find the arcs of a hub in any layout, and restore the
+    graph's own; a layout held by a serving lane stays refused."""
+    g = gg.rmat(13, 24, seed=4)
+    src = int(gg.giant_sources(g, 1)[0][0])
+    G = upload(g)
+    own = G.features()["shadows"]
+    for split in (32, 300, 0):
+        d, p = gpu_solve(G, src, pred=True, config=cfg(split_arcs=split))
+        assert_exact(g, src, d, p)
+        d, p = gpu_solve(G, src, pred=True)
+        assert_exact(g, src, d, p)
+        assert G.features()["shadows"] == own
+    srv = S.sssp_serve_create()
+    try:
+        gpu_solve(G, src, config=cfg(split_arcs=64))
+        ds = torch.empty(g.n, dtype=torch.int32, device="cuda")
+        t = S.sssp_serve_submit(srv, G.handle, src, ds)
+        assert S.sssp_serve_wait(srv, t)[0] == S.Q_DONE
+        assert_exact(g, src, ds.cpu().numpy().view(np.uint32))
+        with pytest.raises(S.SsspError) as ei:
+            gpu_solve(G, src)
+        assert ei.value.code == S.SSSP_E_BUSY
+    finally:
+        S.sssp_serve_destroy(srv)
+    d, p = gpu_solve(G, src, pred=True)
+    assert_exact(g, src, d, p)
+    G.close()
