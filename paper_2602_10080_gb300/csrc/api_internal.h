@@ -35,6 +35,10 @@ struct Workspace {
     size_t pend_n = 0;
     unsigned long long* tl = nullptr;   // run-time sampling buffer
     size_t tl_n = 0;
+    uint32_t* tide = nullptr;           // whole-grid wavefront: barrier words, then pending bits
+    size_t tide_n = 0;
+    uint4* tide_items = nullptr;        // hub slices of one step
+    size_t tide_items_n = 0;
     cudaEvent_t ev0 = nullptr, ev1 = nullptr, ev2 = nullptr;
 
     int ensure_ctrl(cudaStream_t s);

@@ -319,6 +319,8 @@ void Workspace::release() {
     cudaFree(srcs);
     cudaFree(pend);
     cudaFree(tl);
+    cudaFree(tide);
+    cudaFree(tide_items);
     if (host_ctrl) cudaFreeHost(host_ctrl);
     if (ev0) cudaEventDestroy(ev0);
     if (ev1) cudaEventDestroy(ev1);

@@ -2,6 +2,7 @@
 // they take, their launch shape, and one call's launch sequence.
 #include <algorithm>
 #include <cstring>
+#include <mutex>
 
 #include "../../include/sssp.h"
 #include "api_internal.h"
@@ -12,6 +13,7 @@ namespace sssp {
 namespace {
 
 struct WavePlan {
+    bool grid = false;     // the whole grid (tide) instead of one cluster per query (wave)
     int log_g = 0;         // log2 of a cluster's blocks
     int threads = 1024;
     uint32_t front = 1;
@@ -51,11 +53,31 @@ bool plan_wave(const Graph* g, int32_t nq, WavePlan* w) {
             // eighth), grid 1024^2 5670 (5740, 5790)
             w->front = total / 16u;
             // sparse random graphs look like meshes and have wide fronts, for
-            // which 16 SMs are too few; such a solve starts over in the queues
+            // which 16 SMs are too few: 10^6 vertices of degree 10 take 1370 us
+            // here and 310 us on the whole grid; such a solve starts over there
             if (g->m > (1 << 19)) w->wide = 24576u;
             return true;
         }
-        return false;
+        w->grid = true;
+        if (hubs) {
+            // power law: the arcs of the core are the work, and the order
+            // decides how often they are relaxed, on the large graphs; on the
+            // small ones the number of steps counts.  us at widths 1/4, 1/2
+            // and 1 of the above: R-MAT-22 2380, 1800, 1920; R-MAT-18 757,
+            // 547, 411; R-MAT-16 609, 414, 329
+            const bool large = g->m > (1 << 25);
+            w->delta *= large ? 0.5 : 1.0;
+            w->front = large ? 1u : 256u;
+            // a larger slice saves listing, a smaller one spreads better: R-MAT-22
+            // (and BFS) 2.87 (0.90) ms with 256 arcs, 2.51 (0.79) with 512
+            w->hub_deg = 512;
+        } else {
+            // road 4096^2 9.8 ms at 16384 (13.6 at 4096, 9.4 at 32768); G(2^21, 2^25)
+            // 0.83 ms at 4096 and at 16384
+            w->front = deg <= 6.0 ? 16384u : 4096u;
+            if (deg <= 6.0) w->delta *= 2.0;
+        }
+        return true;
     }
     // a batch on a small graph or a mesh: one cluster per query, as wide as the
     // queries leave room for (13 queries on grid 301 x 257: 8 blocks 1690 us,
@@ -67,6 +89,11 @@ bool plan_wave(const Graph* g, int32_t nq, WavePlan* w) {
     w->front = std::max(1u, (uint32_t)(w->threads << w->log_g) / 16u);
     return true;
 }
+
+// Blocks of a tide kernel wait for one another, so that two of them (of two
+// graphs, on two streams) must not share the device half and half: one runs
+// at a time.  Held from the launch to the end of the call.
+std::mutex g_tide_mu[64];
 
 }  // namespace
 
@@ -83,16 +110,17 @@ int run_wave(Graph* g, const int32_t* srcs_host, const int32_t* srcs_dev, int32_
     std::memset(&P, 0, sizeof(P));
     // places: a power of two of at least n, with few bits per word on a small
     // graph, so that every thread has a word
-    int bits = 0, log_t = 0;
+    int bits = 0, log_t = 17;
     while ((1ll << bits) < n) bits++;
-    for (log_t = plan.log_g; (1 << (log_t - plan.log_g)) < plan.threads;) log_t++;
+    if (!plan.grid)
+        for (log_t = plan.log_g; (1 << (log_t - plan.log_g)) < plan.threads;) log_t++;
     P.log_b = std::max(0, std::min(5, bits - log_t));
     P.mask = (uint32_t)((1ull << bits) - 1);
     P.log_g = plan.log_g;
     const uint32_t all_words = 1u << (bits - P.log_b);
     P.words = (int32_t)std::max(1u, all_words >> P.log_g);
     const size_t smem = (size_t)P.words * 4 * sizeof(uint32_t);
-    if (smem > 200 * 1024) return kWaveNotRun;
+    if (!plan.grid && smem > 200 * 1024) return kWaveNotRun;
 
     Workspace& ws = g->ws;
     int rc = ws.ensure_ctrl(stream);
@@ -132,11 +160,26 @@ int run_wave(Graph* g, const int32_t* srcs_host, const int32_t* srcs_dev, int32_
     P.has_hubs = g->feat.max_deg > (double)P.hub_deg;
     P.ctrl = ws.ctrl;
     P.timeout_ns = 20000ull * 1000000ull;
+    std::unique_lock<std::mutex> tide_lock;
+    if (plan.grid) {
+        if ((rc = grow(&ws.tide, &ws.tide_n, sizeof(TideSync) / 4 + 4 * (size_t)all_words))) return rc;
+        P.sync = (TideSync*)ws.tide;
+        P.bits = ws.tide + sizeof(TideSync) / 4;
+        if (P.has_hubs) {
+            // a hub is listed once a step, in slices of kTideChunk arcs
+            P.items_cap = (uint32_t)(g->m / kTideChunk + g->m / P.hub_deg + 1);
+            if ((rc = grow(&ws.tide_items, &ws.tide_items_n, 2 * (size_t)P.items_cap))) return rc;
+            P.items = ws.tide_items;
+        }
+        tide_lock = std::unique_lock<std::mutex>(g_tide_mu[g->device]);
+        cudaMemsetAsync(ws.tide, 0, sizeof(TideSync), stream);
+    }
     cudaMemsetAsync(ws.ctrl, 0, sizeof(Ctrl), stream);
     cudaEventRecord(ws.ev1, stream);
-    const cudaError_t le = launch_wave(f32 ? 1 : 0, pred_mode, P, nq, plan.threads, smem, stream);
+    const cudaError_t le = plan.grid ? launch_tide(f32 ? 1 : 0, pred_mode, P, g->sms, plan.threads, stream)
+                                     : launch_wave(f32 ? 1 : 0, pred_mode, P, nq, plan.threads, smem, stream);
     if (le != cudaSuccess) {
-        // no room for the cluster on this device
+        // no room for the cluster or the cooperative grid on this device
         cudaGetLastError();
         return kWaveNotRun;
     }
@@ -160,7 +203,7 @@ int run_wave(Graph* g, const int32_t* srcs_host, const int32_t* srcs_dev, int32_
     st.relax_arcs = (int64_t)hc.stats[kStRelax];
     st.improved = (int64_t)hc.stats[kStImproved];
     st.rounds = (int64_t)hc.stats[kStIter];
-    st.grid_blocks = nq << P.log_g;
+    st.grid_blocks = plan.grid ? g->sms : nq << P.log_g;
     st.block_threads = plan.threads;
     st.attempts = 1;
     g->last = st;

@@ -3,13 +3,15 @@
 // A search is advanced in steps: the vertices that wait for relaxation are
 // bits, a step relaxes them all, and a barrier ends it.  A push is one OR
 // without an answer, a pop is a word, no queue can overflow, and no element
-// is stale or queued twice.
+// is stale or queued twice.  Two kernels share the relaxation:
 //
 //   wave_kernel  one cluster of 1 to 16 blocks per query, its bits in the
 //                cluster's shared memory, the hardware cluster barrier between
 //                steps.  For graphs whose wavefront is thin (meshes, small
 //                graphs), where the latency of a hop is all there is; a batch
 //                is one cluster per query, and no cluster waits for another.
+//   tide_kernel  the whole grid on one query, its bits in global memory, a
+//                grid barrier between steps.  For large graphs.
 //
 // Order: vertices below the threshold T wait in `near` and are relaxed in the
 // next step; the others wait in `far`.  When fewer than `front` vertices are
@@ -29,6 +31,7 @@ constexpr int kWaveHubs = 128;        // hubs one block expands together per ste
 constexpr uint32_t kWaveHash = 0x9E3779B1u;      // odd: v -> v * hash mod 2^bits is one to one
 constexpr uint32_t kWaveHashInv = 0x0E8B2F51u;   // its inverse mod 2^32
 static_assert((uint32_t)(0x9E3779B1ull * 0x0E8B2F51ull) == 1u, "inverse of the vertex hash");
+constexpr int32_t kTideChunk = 256;   // arcs of a hub that one warp relaxes at a time
 
 struct WaveParams {
     const int2* span;         // [n] arcs of a vertex: adj[span.x .. span.y)
@@ -47,13 +50,18 @@ struct WaveParams {
     uint32_t mask;            // 2^bits - 1
     int32_t log_b;            // log2 of the bits used per word (0..5)
     int32_t log_g;            // log2 of the cluster's blocks: word w lives in block w % G
-    int32_t words;            // words per block
+    int32_t words;            // words per block (wave), or in all (tide)
     int32_t unit;             // breadth-first: every arc weighs 1, no threshold
     int32_t hub_deg;          // a vertex with more arcs is not left to one warp
     int32_t has_hubs;
     uint32_t wide;            // wave: give up (kErrWide) when more vertices than this wait in near
     Ctrl* ctrl;               // error word, finished queries, statistics
     unsigned long long timeout_ns;
+    // tide only
+    uint32_t* bits;           // near[2], far[2]: `words` words each
+    uint4* items;             // hub slices, two lists of items_cap: (vertex, distance, first arc, end)
+    uint32_t items_cap;
+    struct TideSync* sync;
 };
 
 struct WaveSlot {
@@ -70,6 +78,21 @@ struct WaveShared {
     uint32_t near[4], fmin[4], nhub[4]; // this block's sums of step s, set s % 4
     WaveHub hub[kWaveHubs];
     uint32_t list[32][64];              // per warp: vertices taken from the words (bit 31: from far)
+};
+
+// Grid barriers and the sums of a step (set s % 4).  A block arrives by one
+// addition that carries its near count: arrivals in the low 16 bits.
+struct __align__(128) TideSync {
+    struct __align__(128) {
+        unsigned long long arrived;      // end of the step: near count << 16 | blocks
+        uint32_t far;                    // the complement of the smallest far distance
+        uint32_t pad[29];
+    } set[4];
+    struct __align__(128) {
+        uint32_t count;                  // hub slices listed by the step
+        uint32_t arrived;                // blocks that have listed theirs (breadth-first)
+        uint32_t pad[30];
+    } hub[4];
 };
 
 __device__ __forceinline__ uint32_t cluster_rank() {
@@ -496,6 +519,187 @@ __global__ void __launch_bounds__(1024, 1) wave_kernel(const __grid_constant__ W
         atomicAdd(&P.ctrl->stats[kStIter], (unsigned long long)steps);
         if (error) raise_error(P.ctrl, error, 20, (int)q);
         else atomicAdd(&P.ctrl->finished, 1);
+    }
+}
+
+// One thread's wait until the word's low 16 bits say that all blocks have
+// arrived (launched cooperatively: all are resident); the word, or 0 after
+// the deadline.
+__device__ __forceinline__ unsigned long long tide_wait(const unsigned long long* p, uint32_t blocks,
+                                                        unsigned long long deadline) {
+    for (uint32_t spins = 1;; spins++) {
+        const unsigned long long x = ld_acquire64(p);
+        if ((x & 0xffffull) == blocks) return x;
+        if ((spins & 1023u) == 0 && gtime() > deadline) return 0ull;
+    }
+}
+__device__ __forceinline__ void red_release64(unsigned long long* p, unsigned long long v) {
+    asm volatile("red.release.gpu.global.add.u64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
+}
+
+template <int WT, int PRED>
+__global__ void __launch_bounds__(1024, 1) tide_kernel(const __grid_constant__ WaveParams P) {
+    using W = Wave<WT, PRED, kWaveGrid>;
+    using DistT = typename W::DistT;
+    __shared__ uint32_t lists[32][64];
+    __shared__ uint32_t s_near[4], s_fmin[4], s_out[4];
+    const uint32_t tid = threadIdx.x, nt = blockDim.x, lane = tid & 31u;
+    const uint32_t gt = blockIdx.x * nt + tid, gn = gridDim.x * nt;
+    // consecutive warps of the grid lie in different blocks
+    const uint32_t wid = (tid >> 5) * gridDim.x + blockIdx.x, nw = gn >> 5;
+    const uint32_t words = (uint32_t)P.words;
+    W w{P, reinterpret_cast<DistT*>(P.work), lists[tid >> 5],
+        P.unit ? kInfU32 : wave_raise<WT>(0u, P.delta, 0u), 0u, nullptr, nullptr, 0u, kInfU32, 0u};
+    const unsigned long long deadline = gtime() + P.timeout_ns;
+
+    w.init((uint32_t)P.src0, gt, gn);
+    for (uint32_t i = gt; i < words; i += gn) {
+        const uint32_t p = ((uint32_t)P.src0 * kWaveHash) & P.mask;
+        P.bits[i] = i == p >> P.log_b ? 1u << (p & ((1u << P.log_b) - 1u)) : 0u;
+        P.bits[words + i] = P.bits[2u * words + i] = P.bits[3u * words + i] = 0u;
+    }
+    if (tid < 4u) {
+        s_near[tid] = 0u;
+        s_fmin[tid] = kInfU32;
+    }
+
+    // step 0 ends the preparation; the searching steps follow
+    uint32_t cur = 0u, fw = 0u, far_low = kInfU32, n_improved = 0, steps = 0, near = 0u;
+    int what = 1;
+    bool ok = true;
+    for (;;) {
+        // the step's sums: the block's, then the grid's
+        const uint32_t set = steps & 3u;
+        const bool scanned = what == 2;
+        if (steps) {
+            n_improved += w.n_imp;
+            const uint32_t imp = __reduce_add_sync(kFull, w.n_imp), fm = __reduce_min_sync(kFull, w.fmin);
+            if (lane == 0) {
+                if (imp) atomicAdd(&s_near[set], imp);
+                if (fm != kInfU32) atomicMin(&s_fmin[set], fm);
+            }
+        }
+        __syncthreads();
+        if (tid == 0) {
+            const uint32_t z = (steps + 2u) & 3u;
+            if (s_fmin[set] != kInfU32) atomicMax(&P.sync->set[set].far, ~s_fmin[set]);
+            if (blockIdx.x == 0 && steps) {
+                // nobody touches set s + 2 before the barrier after this one
+                P.sync->set[z].arrived = 0ull;
+                P.sync->set[z].far = P.sync->hub[z].count = P.sync->hub[z].arrived = 0u;
+            }
+            red_release64(&P.sync->set[set].arrived, ((unsigned long long)s_near[set] << 16) | 1ull);
+            s_near[z] = 0u;
+            s_fmin[z] = kInfU32;
+            const unsigned long long x = tide_wait(&P.sync->set[set].arrived, gridDim.x, deadline);
+            s_out[0] = x ? (uint32_t)min(x >> 16, 0xfffffffeull) : kInfU32;
+            s_out[1] = ~ld_relaxed(&P.sync->set[set].far);
+            s_out[2] = ld_relaxed(&P.sync->hub[set].count);
+        }
+        __syncthreads();
+        near = s_out[0];
+        uint32_t items = P.has_hubs && steps && !P.unit ? s_out[2] : 0u;
+        if (near == kInfU32) {
+            ok = false;
+            break;
+        }
+        if (steps == 0) {
+            near = 1u;
+        } else {
+            far_low = scanned ? s_out[1] : min(far_low, s_out[1]);
+            what = w.advance(near + items, far_low);
+            if (!what) break;
+        }
+        const uint32_t prev = set;
+        steps++;
+        const uint32_t now = steps & 3u;
+        const bool scan_far = what == 2;
+        uint32_t* near_r = P.bits + (size_t)cur * words;
+        uint32_t* far_r = P.bits + (size_t)(2u + fw) * words;
+        if (scan_far) fw ^= 1u;
+        cur ^= 1u;
+        w.near_w = P.bits + (size_t)cur * words;
+        w.far_w = P.bits + (size_t)(2u + fw) * words;
+        w.n_imp = 0u;
+        w.fmin = kInfU32;
+        uint4* items_w = P.items + (size_t)(steps & 1u) * P.items_cap;
+        w.sweep(
+            wid * 32u, nw * 32u, words,
+            [&](uint32_t i, uint32_t& nb, uint32_t& fb) {
+                nb = fb = 0u;
+                if (i < words) {
+                    nb = __ldcg(near_r + i);
+                    if (scan_far) fb = __ldcg(far_r + i);
+                    if (nb) near_r[i] = 0u;
+                    if (fb) far_r[i] = 0u;
+                    fb &= ~nb;
+                }
+            },
+            [&](uint32_t i, uint32_t b) { return w.vertex(i, b); },
+            [&](uint32_t v, uint32_t d, int2 sp, int32_t deg) {
+                // hubs are cut into slices for all warps of the grid
+                uint32_t m = __ballot_sync(kFull, deg > P.hub_deg);
+                if (deg > P.hub_deg) deg = 0;
+                while (m) {
+                    const int j = __ffs((int)m) - 1;
+                    m &= m - 1u;
+                    const uint32_t u = __shfl_sync(kFull, v, j), du = __shfl_sync(kFull, d, j);
+                    const int32_t b = __shfl_sync(kFull, sp.x, j), e = __shfl_sync(kFull, sp.y, j);
+                    const int32_t k = (e - b + kTideChunk - 1) / kTideChunk;
+                    uint32_t at = 0;
+                    if (lane == 0) at = atomicAdd(&P.sync->hub[now].count, (uint32_t)k);
+                    at = __shfl_sync(kFull, at, 0);
+                    for (int32_t i = (int32_t)lane; i < k; i += 32) {
+                        const int32_t lo = b + i * kTideChunk;
+                        items_w[at + (uint32_t)i] =
+                            make_uint4(u, du, (uint32_t)lo, (uint32_t)min(e, lo + kTideChunk));
+                    }
+                }
+                return deg;
+            });
+        if (!P.has_hubs) continue;
+        const uint4* items_r;
+        if (P.unit) {
+            // breadth-first: the slices belong to this level
+            __syncthreads();
+            if (tid == 0) {
+                unsigned int x;
+                asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(&P.sync->hub[now].arrived) : "memory");
+                uint32_t spins = 0;
+                ok = true;
+                while ((x = ld_acquire(&P.sync->hub[now].arrived)) != gridDim.x)
+                    if ((++spins & 1023u) == 0 && gtime() > deadline) {
+                        ok = false;
+                        break;
+                    }
+                s_out[2] = ok ? ld_relaxed(&P.sync->hub[now].count) : kInfU32;
+            }
+            __syncthreads();
+            items = s_out[2];
+            items_r = items_w;
+            if (items == kInfU32) {
+                ok = false;
+                break;
+            }
+        } else {
+            // the slices that the last step listed, but for those whose hub
+            // has improved since: it waits again with its new distance
+            items_r = P.items + (size_t)(prev & 1u) * P.items_cap;
+        }
+        for (uint32_t i = wid; i < items; i += nw) {
+            const uint4 it = __ldcg(items_r + i);
+            if (!P.unit && W::dpart(ld_dist(w.dist + it.x)) < it.y) continue;
+            for (int32_t e = (int32_t)it.z + (int32_t)lane; e < (int32_t)it.w; e += 128)
+                w.arcs4(it.x, it.y, e, 32, (int32_t)it.w);
+            __syncwarp();
+        }
+    }
+    if (ok) w.unpack(0, gt, gn);
+    w.publish(n_improved);
+    if (tid == 0 && !ok) raise_error(P.ctrl, kErrTimeout, 21, 0);
+    if (gt == 0) {
+        atomicAdd(&P.ctrl->stats[kStIter], (unsigned long long)steps);
+        atomicAdd(&P.ctrl->finished, 1);
     }
 }
 

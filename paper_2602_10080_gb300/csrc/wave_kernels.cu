@@ -28,6 +28,30 @@ static cudaError_t launch_one(const WaveParams& p, int nq, int threads, size_t s
 }
 
 template <int WT, int PRED>
+static cudaError_t launch_tide_one(const WaveParams& p, int grid, int threads, cudaStream_t stream) {
+    cudaLaunchConfig_t c{};
+    c.gridDim = dim3(grid);
+    c.blockDim = dim3(threads);
+    c.stream = stream;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeCooperative;
+    at[0].val.cooperative = 1;
+    c.attrs = at;
+    c.numAttrs = 1;
+    return cudaLaunchKernelEx(&c, tide_kernel<WT, PRED>, p);
+}
+
+cudaError_t launch_tide(int wt, int pred, const WaveParams& p, int grid, int threads, cudaStream_t stream) {
+    if (wt == 0) {
+        if (pred == 0) return launch_tide_one<0, 0>(p, grid, threads, stream);
+        if (pred == 1) return launch_tide_one<0, 1>(p, grid, threads, stream);
+        return launch_tide_one<0, 2>(p, grid, threads, stream);
+    }
+    return pred == 0 ? launch_tide_one<1, 0>(p, grid, threads, stream)
+                     : launch_tide_one<1, 2>(p, grid, threads, stream);
+}
+
+template <int WT, int PRED>
 static cudaError_t launch_cl(const WaveParams& p, int nq, int threads, size_t smem, cudaStream_t stream) {
     return p.log_g > 0 ? launch_one<WT, PRED, true>(p, nq, threads, smem, stream)
                        : launch_one<WT, PRED, false>(p, nq, threads, smem, stream);

@@ -3,6 +3,8 @@ at the sizes where they can go wrong: around a word, a warp and a block of
 pending bits, one block and clusters, hubs beyond a block's list, a front too
 wide for a cluster, thresholds that saturate or absorb their step, and the
 same answers as the queue engine."""
+import threading
+
 import numpy as np
 import pytest
 import torch
@@ -99,13 +101,24 @@ def test_thresholds_at_the_ends():
 
 @pytest.mark.parametrize("n,deg", [(200_000, 4), (130_000, 6)])
 def test_front_too_wide_for_a_cluster(n, deg):
-    """Sparse random graphs begin in one cluster and start over in the queues."""
+    """Sparse random graphs begin in one cluster and start over on the grid."""
     both(gg.random_directed(n, n * deg, 1, 100, seed=deg), 3)
 
 
-def test_levels():
-    for g in (gg.grid(300, 200, 1, 9, seed=1), hub_graph(600, 300)):
-        src = 0
+@pytest.mark.parametrize("wtype", ["u32", "f32"])
+def test_whole_grid(wtype):
+    """Above 2^19 arcs: with hubs (slices over the grid) and without."""
+    g = gg.rmat(15, 24, seed=8, wtype=wtype)
+    both(g, int(gg.giant_sources(g, 1)[0][0]))
+    both(gg.erdos_renyi(50_000, 400_000, 1, 1000, seed=3, wtype=wtype), 7)
+    if wtype == "u32":
+        both(gg.random_directed(60_000, 900_000, 0, 9, seed=2), 5)
+        both(gg.grid(1500, 1450, 1, 100, seed=5), 1_000_000)   # thin, but more vertices than a cluster takes
+
+
+def test_levels_on_cluster_and_grid():
+    for g in (gg.grid(300, 200, 1, 9, seed=1), gg.rmat(15, 24, seed=8), hub_graph(600, 300)):
+        src = int(gg.giant_sources(g, 1)[0][0]) if g.name.startswith("rmat") else 0
         G = upload(g)
         lev = torch.empty(G.n, dtype=torch.int32, device="cuda")
         par = torch.empty(G.n, dtype=torch.int32, device="cuda")
@@ -116,6 +129,29 @@ def test_levels():
         np.testing.assert_array_equal(lev.cpu().numpy().view(np.uint32), ref)
         np.testing.assert_array_equal(par.cpu().numpy(), oracle.pred_canonical_u32(g.row_ptr, g.col, unit, src, ref))
         G.close()
+
+
+def test_two_threads_two_graphs():
+    """Whole-grid solves of different graphs from two threads and streams."""
+    gs = [gg.rmat(14, 40, seed=s) for s in (1, 2)]
+    srcs = [gg.giant_sources(g, 6)[0] for g in gs]
+    Gs = [upload(g) for g in gs]
+    out = {}
+
+    def work(i):
+        st = torch.cuda.Stream()
+        for k, s in enumerate(srcs[i]):
+            d = torch.empty(Gs[i].n, dtype=torch.int32, device="cuda")
+            Gs[i].solve(int(s), d, None, None, st)
+            out[i, k] = d
+
+    ts = [threading.Thread(target=work, args=(i,)) for i in range(2)]
+    [t.start() for t in ts]
+    [t.join() for t in ts]
+    torch.cuda.synchronize()
+    for (i, k), d in out.items():
+        assert_exact(gs[i], int(srcs[i][k]), d.cpu().numpy().view(np.uint32))
+    [G.close() for G in Gs]
 
 
 def test_layout_of_another_threshold():
