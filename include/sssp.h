@@ -269,9 +269,9 @@ SSSP_API int sssp_solve(sssp_graph *g, int32_t src, void *dist_out, int32_t *pre
  *   pred_out  nq * n int32 or NULL.
  * nq * 2^ceil(log2 n) must not exceed 2^32 (the element key packs the query
  * index above the vertex bits).  With cfg NULL the library picks the kernels
- * as for sssp_solve (on a small graph or a mesh: a cluster of blocks for every
- * query); in the queue engine the batch uses the
- * configuration sssp_autotune_batch cached for its size class, if any.
+ * as for sssp_solve (on a small graph or a mesh a cluster of blocks for every
+ * query, on a larger one groups of 32 queries side by side); in the queue
+ * engine the batch uses the configuration sssp_autotune_batch cached for its size class, if any.
  * Otherwise, when the library picks delta (cfg NULL, or a zero delta), the
  * batch uses delta / min(16, max(1, nq / 32)) with bnum <= 4: the queries
  * supply the parallelism, and narrower buckets cut out-of-order work.

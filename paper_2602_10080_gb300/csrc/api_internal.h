@@ -39,6 +39,10 @@ struct Workspace {
     size_t tide_n = 0;
     uint4* tide_items = nullptr;        // hub slices of one step
     size_t tide_items_n = 0;
+    uint32_t* fan = nullptr;            // multi-source: barrier words, waiting words, distance and predecessor rows
+    size_t fan_n = 0;
+    uint4* fan_slices = nullptr;
+    size_t fan_slices_n = 0;
     cudaEvent_t ev0 = nullptr, ev1 = nullptr, ev2 = nullptr;
 
     int ensure_ctrl(cudaStream_t s);

@@ -419,20 +419,25 @@ __device__ __forceinline__ uint32_t atom_exch_acquire(uint32_t* p, uint32_t v) {
     return old;
 }
 
-// distance minimum whose old value is not needed (a reduction)
+// distance minimum whose old value is not needed: a reduction, spelled out
+// because atomicMin on a generic pointer becomes an atomic that returns
 __device__ __forceinline__ void red_min(uint32_t* p, uint32_t v) {
 #if SSSP_L2_HINTS
     asm volatile("red.relaxed.gpu.global.min.L2::cache_hint.u32 [%0], %1, %2;" ::"l"(p), "r"(v), "l"(pol_keep()));
 #else
-    atomicMin(p, v);
+    asm volatile("red.relaxed.gpu.global.min.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
 #endif
 }
 __device__ __forceinline__ void red_min(unsigned long long* p, unsigned long long v) {
 #if SSSP_L2_HINTS
     asm volatile("red.relaxed.gpu.global.min.L2::cache_hint.u64 [%0], %1, %2;" ::"l"(p), "l"(v), "l"(pol_keep()));
 #else
-    atomicMin(p, v);
+    asm volatile("red.relaxed.gpu.global.min.u64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
 #endif
+}
+// bits set in a word whose old value is not needed
+__device__ __forceinline__ void red_or_global(uint32_t* p, uint32_t v) {
+    asm volatile("red.relaxed.gpu.global.or.b32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
 }
 
 // ------------------------------------------------------------ arithmetic --

@@ -321,6 +321,8 @@ void Workspace::release() {
     cudaFree(tl);
     cudaFree(tide);
     cudaFree(tide_items);
+    cudaFree(fan);
+    cudaFree(fan_slices);
     if (host_ctrl) cudaFreeHost(host_ctrl);
     if (ev0) cudaEventDestroy(ev0);
     if (ev1) cudaEventDestroy(ev1);
@@ -1342,7 +1344,6 @@ extern "C" int sssp_solve_batch(sssp_graph* gh, const int32_t* srcs, int32_t nq,
     std::lock_guard<std::mutex> lk(g->mu);
     try {
         std::vector<int32_t> hs;
-        const int32_t* host = nullptr;
         const int32_t* dev = nullptr;
         if (is_device_ptr(srcs)) {
             hs.resize(nq);
@@ -1351,13 +1352,12 @@ extern "C" int sssp_solve_batch(sssp_graph* gh, const int32_t* srcs, int32_t nq,
             dev = srcs;
         } else {
             hs.assign(srcs, srcs + nq);
-            host = srcs;
         }
         for (int32_t i = 0; i < nq; i++)
             if (hs[i] < 0 || hs[i] >= g->n) return SSSP_E_INVAL;
         if (nq == 1)
             return run_queries(g, nullptr, nullptr, hs[0], 1, dist_out, pred_out, cfg, (cudaStream_t)stream, nullptr);
-        return run_queries(g, host, dev, 0, nq, dist_out, pred_out, cfg, (cudaStream_t)stream, nullptr);
+        return run_queries(g, hs.data(), dev, 0, nq, dist_out, pred_out, cfg, (cudaStream_t)stream, nullptr);
     } catch (...) {
         return SSSP_E_NOMEM;
     }

@@ -6,14 +6,19 @@
 
 #include "../../include/sssp.h"
 #include "api_internal.h"
+#include "fan.h"
 #include "wave.h"
 
 namespace sssp {
 
 namespace {
 
+// One cluster per query (wave), the whole grid on one query (tide), the
+// queries one after the other, or 32 queries side by side (fan).
+enum WaveKind { kOneCluster, kWholeGrid, kInTurn, kSideBySide };
+
 struct WavePlan {
-    bool grid = false;     // the whole grid (tide) instead of one cluster per query (wave)
+    WaveKind kind = kOneCluster;
     int log_g = 0;         // log2 of a cluster's blocks
     int threads = 1024;
     uint32_t front = 1;
@@ -30,7 +35,7 @@ uint32_t pow2_at_least(double x) {
 
 // The kernel and launch shape of a call, from the graph's features; false:
 // the queue engine takes it.
-bool plan_wave(const Graph* g, int32_t nq, WavePlan* w) {
+bool plan_wave(const Graph* g, int32_t nq, int pred_mode, WavePlan* w) {
     const sssp_features& f = g->feat;
     const double deg = std::max(1.0, f.avg_deg);
     const bool hubs = f.max_deg > 64.0;
@@ -58,7 +63,7 @@ bool plan_wave(const Graph* g, int32_t nq, WavePlan* w) {
             if (g->m > (1 << 19)) w->wide = 24576u;
             return true;
         }
-        w->grid = true;
+        w->kind = kWholeGrid;
         if (hubs) {
             // power law: the arcs of the core are the work, and the order
             // decides how often they are relaxed, on the large graphs; on the
@@ -82,7 +87,16 @@ bool plan_wave(const Graph* g, int32_t nq, WavePlan* w) {
     // a batch on a small graph or a mesh: one cluster per query, as wide as the
     // queries leave room for (13 queries on grid 301 x 257: 8 blocks 1690 us,
     // 4: 1880, 1: 2130)
-    if (g->m > (1 << 21) || (hubs && g->m > (1 << 18))) return false;
+    if (g->m > (1 << 21) || (hubs && g->m > (1 << 18))) {
+        // A group of up to 32 queries side by side costs as much as this many
+        // in turn on the whole grid: R-MAT-20 7 (5.7 ms), R-MAT-18 7 (2.7 ms),
+        // G(200K, 2M) 15 (3.1 ms).  Predecessors of the strict-improvement rule
+        // cannot be found after the distances and stay with the queues.
+        if (nq < 12) w->kind = kInTurn;
+        else if (pred_mode != 2 && g->n <= kFanMaxVertices) w->kind = kSideBySide;
+        else return false;
+        return true;
+    }
     w->log_g = 4;
     while (w->log_g > 0 && (nq << w->log_g) > g->sms) w->log_g--;
     w->threads = (int)std::max(128u, std::min(w->log_g ? 512u : 1024u, total >> w->log_g));
@@ -90,29 +104,96 @@ bool plan_wave(const Graph* g, int32_t nq, WavePlan* w) {
     return true;
 }
 
-// Blocks of a tide kernel wait for one another, so that two of them (of two
-// graphs, on two streams) must not share the device half and half: one runs
-// at a time.  Held from the launch to the end of the call.
-std::mutex g_tide_mu[64];
+// The blocks of a whole-grid kernel wait for one another, so that two of them
+// (of two graphs, on two streams) must not share the device half and half:
+// one runs at a time.  Held from the launch to the end of the call.
+std::mutex g_grid_mu[64];
+
+// The batch on the multi-source kernel: groups of up to 32 queries.
+int run_fan(Graph* g, const int32_t* srcs_host, const int32_t* srcs_dev, int32_t nq, uint32_t* dist_out,
+            int32_t* pred_out, cudaStream_t stream) {
+    Workspace& ws = g->ws;
+    const size_t n = (size_t)g->n;
+    uint32_t places = 1;
+    while (places < (uint32_t)g->n) places <<= 1;
+    int rc;
+    if ((rc = grow(&ws.srcs, &ws.srcs_n, (size_t)nq))) return rc;
+    cudaMemcpyAsync(ws.srcs, srcs_dev ? srcs_dev : srcs_host, sizeof(int32_t) * nq,
+                    srcs_dev ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice, stream);
+    const size_t sync_words = sizeof(FanSync) / 4, rows = 32 * n;
+    if ((rc = grow(&ws.fan, &ws.fan_n, sync_words + 2 * (size_t)places + rows * (pred_out ? 2 : 1) + 32))) return rc;
+    // a row of more than kFanShort arcs is cut into slices of kFanChunk
+    const size_t slices = (size_t)(g->m / kFanChunk + g->m / kFanShort + 1);
+    if ((rc = grow(&ws.fan_slices, &ws.fan_slices_n, slices + (n + 1) / 2))) return rc;
+    FanParams P;
+    std::memset(&P, 0, sizeof(P));
+    P.span = g->span;
+    P.adj = g->adj;
+    P.n = g->n;
+    P.sync = (FanSync*)ws.fan;
+    // the rows on their own 128-byte lines
+    P.dist = ws.fan + sync_words + (((2 * (size_t)places) + 31) & ~size_t(31));
+    P.wait = ws.fan + sync_words;
+    P.pred = pred_out ? P.dist + rows : nullptr;
+    P.mask = places - 1u;
+    P.slices = ws.fan_slices;
+    P.rows = (uint2*)(ws.fan_slices + slices);
+    P.ctrl = ws.ctrl;
+    P.timeout_ns = 20000ull * 1000000ull;
+    const int32_t groups = (nq + 31) / 32, per = (nq + groups - 1) / groups;
+    for (int32_t q0 = 0; q0 < nq; q0 += per) {
+        P.nq = std::min(per, nq - q0);
+        P.srcs = ws.srcs + q0;
+        cudaMemsetAsync(P.sync, 0, sizeof(FanSync), stream);
+        if (launch_fan(g->wtype == SSSP_W_F32 ? 1 : 0, P, g->sms, stream) != cudaSuccess) {
+            cudaGetLastError();
+            return kWaveNotRun;
+        }
+        launch_fan_out(P.dist, g->n, P.nq, dist_out + (size_t)q0 * n, g->sms, stream);
+        if (pred_out) launch_fan_out(P.pred, g->n, P.nq, (uint32_t*)pred_out + (size_t)q0 * n, g->sms, stream);
+    }
+    return cuda_status(cudaGetLastError());
+}
 
 }  // namespace
 
 int run_wave(Graph* g, const int32_t* srcs_host, const int32_t* srcs_dev, int32_t src0, int32_t nq, void* dist_out,
              int32_t* pred_out, cudaStream_t stream, sssp_stats* st_out, bool unit) {
+    // unit weights are >= 1: the packed minimum gives the smallest-index parent
+    const int pred_mode = pred_out ? (unit ? 1 : pred_mode_for(g)) : 0;
     WavePlan plan;
-    if (g->device < 0 || g->device >= 64 || !plan_wave(g, nq, &plan)) return kWaveNotRun;
+    if (g->device < 0 || g->device >= 64 || !plan_wave(g, nq, pred_mode, &plan)) return kWaveNotRun;
     if (cudaSetDevice(g->device) != cudaSuccess) return SSSP_E_CUDA;
     const int32_t n = g->n;
     const bool f32 = g->wtype == SSSP_W_F32 && !unit;
-    // unit weights are >= 1: the packed minimum gives the smallest-index parent
-    const int pred_mode = pred_out ? (unit ? 1 : pred_mode_for(g)) : 0;
+    const bool grid = plan.kind == kWholeGrid;
+    if (plan.kind == kInTurn) {
+        sssp_stats sum;
+        std::memset(&sum, 0, sizeof(sum));
+        for (int32_t q = 0; q < nq; q++) {
+            sssp_stats one;
+            const size_t at = (size_t)q * (size_t)n;
+            const int rc = run_wave(g, nullptr, nullptr, srcs_host[q], 1, (uint32_t*)dist_out + at,
+                                    pred_out ? pred_out + at : nullptr, stream, &one, unit);
+            if (rc) return rc;
+            one.kernel_ms += sum.kernel_ms;
+            one.total_ms += sum.total_ms;
+            one.relax_arcs += sum.relax_arcs;
+            one.improved += sum.improved;
+            one.rounds += sum.rounds;
+            sum = one;
+        }
+        g->last = sum;
+        if (st_out) *st_out = sum;
+        return SSSP_OK;
+    }
     WaveParams P;
     std::memset(&P, 0, sizeof(P));
     // places: a power of two of at least n, with few bits per word on a small
     // graph, so that every thread has a word
     int bits = 0, log_t = 17;
     while ((1ll << bits) < n) bits++;
-    if (!plan.grid)
+    if (!grid)
         for (log_t = plan.log_g; (1 << (log_t - plan.log_g)) < plan.threads;) log_t++;
     P.log_b = std::max(0, std::min(5, bits - log_t));
     P.mask = (uint32_t)((1ull << bits) - 1);
@@ -120,7 +201,7 @@ int run_wave(Graph* g, const int32_t* srcs_host, const int32_t* srcs_dev, int32_
     const uint32_t all_words = 1u << (bits - P.log_b);
     P.words = (int32_t)std::max(1u, all_words >> P.log_g);
     const size_t smem = (size_t)P.words * 4 * sizeof(uint32_t);
-    if (!plan.grid && smem > 200 * 1024) return kWaveNotRun;
+    if (plan.kind == kOneCluster && smem > 200 * 1024) return kWaveNotRun;
 
     Workspace& ws = g->ws;
     int rc = ws.ensure_ctrl(stream);
@@ -137,51 +218,56 @@ int run_wave(Graph* g, const int32_t* srcs_host, const int32_t* srcs_dev, int32_
         if ((rc = grow(&ws.out_p, &ws.out_p_n, cells))) return rc;
         pp = ws.out_p;
     }
-    if (pred_mode && (rc = grow(&ws.d64, &ws.d64_n, cells))) return rc;
-    if (nq > 1) {
-        if ((rc = grow(&ws.srcs, &ws.srcs_n, (size_t)nq))) return rc;
-        cudaMemcpyAsync(ws.srcs, srcs_dev ? srcs_dev : srcs_host, sizeof(int32_t) * nq,
-                        srcs_dev ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice, stream);
-        P.srcs = ws.srcs;
-    }
-    P.span = g->span;
-    P.adj = g->adj;
-    P.n = n;
-    P.src0 = src0;
-    P.work = pred_mode ? (void*)ws.d64 : (void*)dd;
-    P.dist_out = dd;
-    P.pred_out = pp;
-    if (f32) P.delta = __float_as_uint_host((float)std::max(1e-30, plan.delta));
-    else P.delta = (uint32_t)std::min(4.0e9, std::max(1.0, plan.delta));
-    P.front = plan.front;
-    P.wide = plan.wide;
-    P.unit = unit ? 1 : 0;
-    P.hub_deg = plan.hub_deg;
-    P.has_hubs = g->feat.max_deg > (double)P.hub_deg;
-    P.ctrl = ws.ctrl;
-    P.timeout_ns = 20000ull * 1000000ull;
-    std::unique_lock<std::mutex> tide_lock;
-    if (plan.grid) {
-        if ((rc = grow(&ws.tide, &ws.tide_n, sizeof(TideSync) / 4 + 4 * (size_t)all_words))) return rc;
-        P.sync = (TideSync*)ws.tide;
-        P.bits = ws.tide + sizeof(TideSync) / 4;
-        if (P.has_hubs) {
-            // a hub is listed once a step, in slices of kTideChunk arcs
-            P.items_cap = (uint32_t)(g->m / kTideChunk + g->m / P.hub_deg + 1);
-            if ((rc = grow(&ws.tide_items, &ws.tide_items_n, 2 * (size_t)P.items_cap))) return rc;
-            P.items = ws.tide_items;
-        }
-        tide_lock = std::unique_lock<std::mutex>(g_tide_mu[g->device]);
-        cudaMemsetAsync(ws.tide, 0, sizeof(TideSync), stream);
-    }
+    std::unique_lock<std::mutex> grid_lock;
+    if (plan.kind != kOneCluster) grid_lock = std::unique_lock<std::mutex>(g_grid_mu[g->device]);
     cudaMemsetAsync(ws.ctrl, 0, sizeof(Ctrl), stream);
-    cudaEventRecord(ws.ev1, stream);
-    const cudaError_t le = plan.grid ? launch_tide(f32 ? 1 : 0, pred_mode, P, g->sms, plan.threads, stream)
-                                     : launch_wave(f32 ? 1 : 0, pred_mode, P, nq, plan.threads, smem, stream);
-    if (le != cudaSuccess) {
-        // no room for the cluster or the cooperative grid on this device
-        cudaGetLastError();
-        return kWaveNotRun;
+    if (plan.kind == kSideBySide) {
+        cudaEventRecord(ws.ev1, stream);
+        if ((rc = run_fan(g, srcs_host, srcs_dev, nq, dd, pp, stream))) return rc;
+    } else {
+        if (pred_mode && (rc = grow(&ws.d64, &ws.d64_n, cells))) return rc;
+        if (nq > 1) {
+            if ((rc = grow(&ws.srcs, &ws.srcs_n, (size_t)nq))) return rc;
+            cudaMemcpyAsync(ws.srcs, srcs_dev ? srcs_dev : srcs_host, sizeof(int32_t) * nq,
+                            srcs_dev ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice, stream);
+            P.srcs = ws.srcs;
+        }
+        P.span = g->span;
+        P.adj = g->adj;
+        P.n = n;
+        P.src0 = src0;
+        P.work = pred_mode ? (void*)ws.d64 : (void*)dd;
+        P.dist_out = dd;
+        P.pred_out = pp;
+        if (f32) P.delta = __float_as_uint_host((float)std::max(1e-30, plan.delta));
+        else P.delta = (uint32_t)std::min(4.0e9, std::max(1.0, plan.delta));
+        P.front = plan.front;
+        P.wide = plan.wide;
+        P.unit = unit ? 1 : 0;
+        P.hub_deg = plan.hub_deg;
+        P.has_hubs = g->feat.max_deg > (double)P.hub_deg;
+        P.ctrl = ws.ctrl;
+        P.timeout_ns = 20000ull * 1000000ull;
+        if (grid) {
+            if ((rc = grow(&ws.tide, &ws.tide_n, sizeof(TideSync) / 4 + 4 * (size_t)all_words))) return rc;
+            P.sync = (TideSync*)ws.tide;
+            P.bits = ws.tide + sizeof(TideSync) / 4;
+            if (P.has_hubs) {
+                // a hub is listed once a step, in slices of kTideChunk arcs
+                P.items_cap = (uint32_t)(g->m / kTideChunk + g->m / P.hub_deg + 1);
+                if ((rc = grow(&ws.tide_items, &ws.tide_items_n, 2 * (size_t)P.items_cap))) return rc;
+                P.items = ws.tide_items;
+            }
+            cudaMemsetAsync(ws.tide, 0, sizeof(TideSync), stream);
+        }
+        cudaEventRecord(ws.ev1, stream);
+        const cudaError_t le = grid ? launch_tide(f32 ? 1 : 0, pred_mode, P, g->sms, plan.threads, stream)
+                                    : launch_wave(f32 ? 1 : 0, pred_mode, P, nq, plan.threads, smem, stream);
+        if (le != cudaSuccess) {
+            // no room for the cluster or the cooperative grid on this device
+            cudaGetLastError();
+            return kWaveNotRun;
+        }
     }
     cudaEventRecord(ws.ev2, stream);
     if (!dist_dev) cudaMemcpyAsync(dist_out, dd, cells * 4, cudaMemcpyDeviceToHost, stream);
@@ -203,7 +289,7 @@ int run_wave(Graph* g, const int32_t* srcs_host, const int32_t* srcs_dev, int32_
     st.relax_arcs = (int64_t)hc.stats[kStRelax];
     st.improved = (int64_t)hc.stats[kStImproved];
     st.rounds = (int64_t)hc.stats[kStIter];
-    st.grid_blocks = plan.grid ? g->sms : nq << P.log_g;
+    st.grid_blocks = plan.kind == kOneCluster ? nq << P.log_g : g->sms;
     st.block_threads = plan.threads;
     st.attempts = 1;
     g->last = st;

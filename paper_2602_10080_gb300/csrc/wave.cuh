@@ -162,7 +162,7 @@ struct Wave {
     }
     __device__ __forceinline__ void red_or(Addr a, uint32_t v) const {
         if constexpr (MODE == kWaveGrid)
-            asm volatile("red.relaxed.gpu.global.or.b32 [%0], %1;" ::"l"(a), "r"(v) : "memory");
+            red_or_global(a, v);
         else if constexpr (MODE == kWaveCluster)
             asm volatile("red.relaxed.cluster.shared::cluster.or.b32 [%0], %1;" ::"r"(a), "r"(v) : "memory");
         else asm volatile("red.relaxed.cta.shared::cta.or.b32 [%0], %1;" ::"r"(a), "r"(v) : "memory");

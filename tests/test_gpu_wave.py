@@ -116,6 +116,51 @@ def test_whole_grid(wtype):
         both(gg.grid(1500, 1450, 1, 100, seed=5), 1_000_000)   # thin, but more vertices than a cluster takes
 
 
+def side_by_side(g, srcs, pred=True):
+    G = upload(g)
+    srcs = np.asarray(srcs, np.int32)
+    for host in (False, True):
+        d, p = gpu_batch(G, srcs, pred=pred, host=host)
+        assert_exact_many(g, srcs, d, p)
+    d2, _ = gpu_batch(G, srcs, pred=False)
+    np.testing.assert_array_equal(d2, d)
+    G.close()
+
+
+@pytest.mark.parametrize("nq", [2, 11, 12, 31, 32, 33, 64, 70])
+def test_batch_side_by_side(nq):
+    """Groups of 32 queries on a graph with hubs, in turn below 12 queries;
+    repeated sources, sources without arcs."""
+    g = gg.rmat(13, 24, seed=nq)
+    srcs = gg.giant_sources(g, nq)[0]
+    srcs[nq // 2] = srcs[0]
+    srcs[nq - 1] = int(np.flatnonzero(np.diff(g.row_ptr) == 0)[0])
+    side_by_side(g, srcs)
+
+
+@pytest.mark.parametrize("nq", [3, 40])
+def test_batch_side_by_side_f32(nq):
+    g = gg.rmat(13, 24, seed=5, wtype="f32")
+    side_by_side(g, gg.giant_sources(g, nq)[0], pred=nq == 3)
+    if nq == 40:   # strict-improvement predecessors
+        G = upload(g)
+        srcs = gg.giant_sources(g, nq)[0]
+        d, p = gpu_batch(G, srcs, pred=True)
+        assert_exact_many(g, srcs, d, p)
+        G.close()
+
+
+def test_batch_rows_of_every_length():
+    """Rows at the ends of the short list and of the slices, and lengths that
+    saturate."""
+    arcs = [0, 1, 7, 8, 9, 15, 16, 17, 31, 32, 33, 127, 128, 129, 255, 256, 257, 700]
+    n = 4000
+    e = [(v, (v * 31 + k * 97 + 1) % n, 1 + (v * k) % 60) for v in range(n) for k in range(arcs[v % len(arcs)])]
+    side_by_side(gg.from_edges(n, e), np.arange(40) * 97)
+    side_by_side(gg.random_directed(4000, 300_000, 1, 0xFFFFFFFF, seed=3), np.arange(20) * 7)
+    side_by_side(gg.erdos_renyi(130_000, 1_300_000, 1, 99, seed=4, wtype="u32"), np.arange(13) * 9999)
+
+
 def test_levels_on_cluster_and_grid():
     for g in (gg.grid(300, 200, 1, 9, seed=1), gg.rmat(15, 24, seed=8), hub_graph(600, 300)):
         src = int(gg.giant_sources(g, 1)[0][0]) if g.name.startswith("rmat") else 0
