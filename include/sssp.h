@@ -324,15 +324,14 @@ SSSP_API int sssp_autotune_batch(sssp_graph *g, const int32_t *srcs, int32_t nq,
  * latency-critical paths that must not call cudaMalloc/cudaFree because
  * those calls can synchronise the device.
  *
- * It runs the same persistent relaxation kernel as sssp_solve with a fixed
- * configuration (L1 filter queue, 8-bucket L2, no hub splitting), keeping
- * every piece of scratch state (control block, L2 rings, packed
+ * It runs the wavefront kernels of sssp_solve, keeping every piece of scratch
+ * state (control block, pending bits, hub slices, packed
  * distance/predecessor words) in one array of about 25 MiB that is part of
  * the library image: every GPU that loads the library holds it until the
  * process exits.  The first call on a device resolves that array's device
  * address.  All calls share the array and it keeps the last call's contents;
- * every call first re-initialises what must start empty (queue metadata,
- * control block, distance words), so a call does not depend on how the
+ * every call first re-initialises what must start empty (control block,
+ * pending bits, distance words), so a call does not depend on how the
  * previous one ended.  Calls serialise on a process-wide lock and return only
  * after the GPU work has finished; two calls that overlapped on the GPU would
  * race on the array.  Every call reads a status back and synchronises its
@@ -349,9 +348,8 @@ SSSP_API int sssp_autotune_batch(sssp_graph *g, const int32_t *srcs, int32_t nq,
  * The CSR is validated on the device (SSSP_E_BADGRAPH).  Distances and
  * predecessors follow the conventions of sssp_solve.  An fp32 weight of
  * -0.0 is accepted and adds like +0.0, but the arcs are used as given (not
- * normalised), so such an arc is routed like a weight above the light-arc
- * bound; results are the same.  SSSP_E_NOMEM if the
- * fixed L2 rings overflow; host pointers are rejected with SSSP_E_INVAL. */
+ * normalised); results are the same.  Host pointers are rejected with
+ * SSSP_E_INVAL. */
 SSSP_API int sssp_solve_noalloc(const int32_t *row_ptr, const uint32_t *arcs, int32_t n, int64_t m,
                                 int32_t wtype, int32_t src, void *dist_out, int32_t *pred_out,
                                 void *stream);

@@ -13,44 +13,29 @@ namespace sssp {
 
 namespace {
 
-// One cluster per query (wave), the whole grid on one query (tide), the
-// queries one after the other, or 32 queries side by side (fan).
-enum WaveKind { kOneCluster, kWholeGrid, kInTurn, kSideBySide };
-
-struct WavePlan {
-    WaveKind kind = kOneCluster;
-    int log_g = 0;         // log2 of a cluster's blocks
-    int threads = 1024;
-    uint32_t front = 1;
-    double delta = 1.0;
-    int32_t hub_deg = 256;
-    uint32_t wide = kInfU32;
-};
-
 uint32_t pow2_at_least(double x) {
     uint32_t p = 1;
     while (p < x && p < (1u << 30)) p <<= 1;
     return p;
 }
 
-// The kernel and launch shape of a call, from the graph's features; false:
-// the queue engine takes it.
-bool plan_wave(const Graph* g, int32_t nq, int pred_mode, WavePlan* w) {
-    const sssp_features& f = g->feat;
-    const double deg = std::max(1.0, f.avg_deg);
-    const bool hubs = f.max_deg > 64.0;
+}  // namespace
+
+bool plan_wave(const WaveGraph& g, int32_t nq, int pred_mode, WavePlan* w) {
+    const double deg = std::max(1.0, (double)g.m / (double)g.n);
+    const bool hubs = g.max_deg > 64.0;
     // about the average weight over a quarter of the degree: of the widths
     // 1/2 to 4 times this, meshes and G(n, m) graphs run within 5% of the best
-    w->delta = 4.0 * f.avg_w / deg;
+    w->delta = 4.0 * g.avg_w / deg;
     // Threads of one cluster: one for eight vertices or 32 arcs, 1024 to
     // 16384 in 16 blocks (8 for the smallest).  GB300, us a solve: directed
     // 1000 vertices 8 x 128 76, 1 x 1024 82; grid 256^2 16 x 512 1114, 8 x 512
     // 1153, 1 x 1024 1800; grid 1024^2 16 x 1024 5670, 8 x 1024 8500.
     const uint32_t total =
-        std::min(16384u, std::max(1024u, pow2_at_least(std::max((double)g->n / 8.0, (double)g->m / 32.0))));
+        std::min(16384u, std::max(1024u, pow2_at_least(std::max((double)g.n / 8.0, (double)g.m / 32.0))));
     if (nq == 1) {
-        const bool thin = deg <= 6.0 && !hubs && g->n <= (1 << 21);
-        if (g->m <= (1 << 19) || (thin && !g->wide)) {
+        const bool thin = deg <= 6.0 && !hubs && g.n <= (1 << 21);
+        if (g.m <= (1 << 19) || (thin && !g.wide)) {
             w->log_g = total > 1024u ? 4 : 3;
             w->threads = (int)(total >> w->log_g);
             // raise the threshold while there is less than a vertex for every
@@ -60,7 +45,7 @@ bool plan_wave(const Graph* g, int32_t nq, int pred_mode, WavePlan* w) {
             // sparse random graphs look like meshes and have wide fronts, for
             // which 16 SMs are too few: 10^6 vertices of degree 10 take 1370 us
             // here and 310 us on the whole grid; such a solve starts over there
-            if (g->m > (1 << 19)) w->wide = 24576u;
+            if (g.m > (1 << 19)) w->wide = 24576u;
             return true;
         }
         w->kind = kWholeGrid;
@@ -70,7 +55,7 @@ bool plan_wave(const Graph* g, int32_t nq, int pred_mode, WavePlan* w) {
             // small ones the number of steps counts.  us at widths 1/4, 1/2
             // and 1 of the above: R-MAT-22 2380, 1800, 1920; R-MAT-18 757,
             // 547, 411; R-MAT-16 609, 414, 329
-            const bool large = g->m > (1 << 25);
+            const bool large = g.m > (1 << 25);
             w->delta *= large ? 0.5 : 1.0;
             w->front = large ? 1u : 256u;
             // a larger slice saves listing, a smaller one spreads better: R-MAT-22
@@ -87,27 +72,54 @@ bool plan_wave(const Graph* g, int32_t nq, int pred_mode, WavePlan* w) {
     // a batch on a small graph or a mesh: one cluster per query, as wide as the
     // queries leave room for (13 queries on grid 301 x 257: 8 blocks 1690 us,
     // 4: 1880, 1: 2130)
-    if (g->m > (1 << 21) || (hubs && g->m > (1 << 18))) {
+    if (g.m > (1 << 21) || (hubs && g.m > (1 << 18))) {
         // A group of up to 32 queries side by side costs as much as this many
         // in turn on the whole grid: R-MAT-20 7 (5.7 ms), R-MAT-18 7 (2.7 ms),
         // G(200K, 2M) 15 (3.1 ms).  Predecessors of the strict-improvement rule
         // cannot be found after the distances and stay with the queues.
         if (nq < 12) w->kind = kInTurn;
-        else if (pred_mode != 2 && g->n <= kFanMaxVertices) w->kind = kSideBySide;
+        else if (pred_mode != 2 && g.n <= kFanMaxVertices) w->kind = kSideBySide;
         else return false;
         return true;
     }
     w->log_g = 4;
-    while (w->log_g > 0 && (nq << w->log_g) > g->sms) w->log_g--;
+    while (w->log_g > 0 && (nq << w->log_g) > g.sms) w->log_g--;
     w->threads = (int)std::max(128u, std::min(w->log_g ? 512u : 1024u, total >> w->log_g));
     w->front = std::max(1u, (uint32_t)(w->threads << w->log_g) / 16u);
     return true;
 }
 
-// The blocks of a whole-grid kernel wait for one another, so that two of them
-// (of two graphs, on two streams) must not share the device half and half:
-// one runs at a time.  Held from the launch to the end of the call.
-std::mutex g_grid_mu[64];
+size_t wave_params(const WavePlan& w, const WaveGraph& g, bool f32, bool unit, WaveParams* p) {
+    // places: a power of two of at least n, with few bits per word on a small
+    // graph, so that every thread has a word
+    int bits = 0, log_t = kTideLogWords;
+    while ((1ll << bits) < g.n) bits++;
+    if (w.kind == kOneCluster)
+        for (log_t = w.log_g; (1 << (log_t - w.log_g)) < w.threads;) log_t++;
+    p->log_b = std::max(0, std::min(5, bits - log_t));
+    p->mask = (uint32_t)((1ull << bits) - 1);
+    p->log_g = w.log_g;
+    p->words = (int32_t)std::max(1u, (1u << (bits - p->log_b)) >> p->log_g);
+    p->n = g.n;
+    if (f32) p->delta = __float_as_uint_host((float)std::max(1e-30, w.delta));
+    else p->delta = (uint32_t)std::min(4.0e9, std::max(1.0, w.delta));
+    p->front = w.front;
+    p->wide = w.wide;
+    p->unit = unit ? 1 : 0;
+    p->hub_deg = w.hub_deg;
+    p->has_hubs = g.max_deg > (double)w.hub_deg;
+    p->timeout_ns = 20000ull * 1000000ull;
+    return w.kind == kOneCluster ? (size_t)p->words * 4 * sizeof(uint32_t) : 0;
+}
+
+uint32_t tide_slices(int64_t m, int32_t hub_deg) { return (uint32_t)(m / kTideChunk + m / hub_deg + 1); }
+
+std::mutex& grid_mutex(int device) {
+    static std::mutex mu[64];
+    return mu[device & 63];
+}
+
+namespace {
 
 // The batch on the multi-source kernel: groups of up to 32 queries.
 int run_fan(Graph* g, const int32_t* srcs_host, const int32_t* srcs_dev, int32_t nq, uint32_t* dist_out,
@@ -162,7 +174,8 @@ int run_wave(Graph* g, const int32_t* srcs_host, const int32_t* srcs_dev, int32_
     // unit weights are >= 1: the packed minimum gives the smallest-index parent
     const int pred_mode = pred_out ? (unit ? 1 : pred_mode_for(g)) : 0;
     WavePlan plan;
-    if (g->device < 0 || g->device >= 64 || !plan_wave(g, nq, pred_mode, &plan)) return kWaveNotRun;
+    const WaveGraph wg{g->n, g->m, g->feat.avg_w, g->feat.max_deg, g->sms, g->wide};
+    if (!plan_wave(wg, nq, pred_mode, &plan)) return kWaveNotRun;
     if (cudaSetDevice(g->device) != cudaSuccess) return SSSP_E_CUDA;
     const int32_t n = g->n;
     const bool f32 = g->wtype == SSSP_W_F32 && !unit;
@@ -189,19 +202,8 @@ int run_wave(Graph* g, const int32_t* srcs_host, const int32_t* srcs_dev, int32_
     }
     WaveParams P;
     std::memset(&P, 0, sizeof(P));
-    // places: a power of two of at least n, with few bits per word on a small
-    // graph, so that every thread has a word
-    int bits = 0, log_t = 17;
-    while ((1ll << bits) < n) bits++;
-    if (!grid)
-        for (log_t = plan.log_g; (1 << (log_t - plan.log_g)) < plan.threads;) log_t++;
-    P.log_b = std::max(0, std::min(5, bits - log_t));
-    P.mask = (uint32_t)((1ull << bits) - 1);
-    P.log_g = plan.log_g;
-    const uint32_t all_words = 1u << (bits - P.log_b);
-    P.words = (int32_t)std::max(1u, all_words >> P.log_g);
-    const size_t smem = (size_t)P.words * 4 * sizeof(uint32_t);
-    if (plan.kind == kOneCluster && smem > 200 * 1024) return kWaveNotRun;
+    const size_t smem = wave_params(plan, wg, f32, unit, &P);
+    if (smem > kWaveMaxShared) return kWaveNotRun;
 
     Workspace& ws = g->ws;
     int rc = ws.ensure_ctrl(stream);
@@ -219,7 +221,7 @@ int run_wave(Graph* g, const int32_t* srcs_host, const int32_t* srcs_dev, int32_
         pp = ws.out_p;
     }
     std::unique_lock<std::mutex> grid_lock;
-    if (plan.kind != kOneCluster) grid_lock = std::unique_lock<std::mutex>(g_grid_mu[g->device]);
+    if (plan.kind != kOneCluster) grid_lock = std::unique_lock<std::mutex>(grid_mutex(g->device));
     cudaMemsetAsync(ws.ctrl, 0, sizeof(Ctrl), stream);
     if (plan.kind == kSideBySide) {
         cudaEventRecord(ws.ev1, stream);
@@ -234,27 +236,17 @@ int run_wave(Graph* g, const int32_t* srcs_host, const int32_t* srcs_dev, int32_
         }
         P.span = g->span;
         P.adj = g->adj;
-        P.n = n;
         P.src0 = src0;
         P.work = pred_mode ? (void*)ws.d64 : (void*)dd;
         P.dist_out = dd;
         P.pred_out = pp;
-        if (f32) P.delta = __float_as_uint_host((float)std::max(1e-30, plan.delta));
-        else P.delta = (uint32_t)std::min(4.0e9, std::max(1.0, plan.delta));
-        P.front = plan.front;
-        P.wide = plan.wide;
-        P.unit = unit ? 1 : 0;
-        P.hub_deg = plan.hub_deg;
-        P.has_hubs = g->feat.max_deg > (double)P.hub_deg;
         P.ctrl = ws.ctrl;
-        P.timeout_ns = 20000ull * 1000000ull;
         if (grid) {
-            if ((rc = grow(&ws.tide, &ws.tide_n, sizeof(TideSync) / 4 + 4 * (size_t)all_words))) return rc;
+            if ((rc = grow(&ws.tide, &ws.tide_n, sizeof(TideSync) / 4 + 4 * (size_t)P.words))) return rc;
             P.sync = (TideSync*)ws.tide;
             P.bits = ws.tide + sizeof(TideSync) / 4;
             if (P.has_hubs) {
-                // a hub is listed once a step, in slices of kTideChunk arcs
-                P.items_cap = (uint32_t)(g->m / kTideChunk + g->m / P.hub_deg + 1);
+                P.items_cap = tide_slices(g->m, P.hub_deg);
                 if ((rc = grow(&ws.tide_items, &ws.tide_items_n, 2 * (size_t)P.items_cap))) return rc;
                 P.items = ws.tide_items;
             }

@@ -34,7 +34,8 @@ static_assert((uint32_t)(0x9E3779B1ull * 0x0E8B2F51ull) == 1u, "inverse of the v
 constexpr int32_t kTideChunk = 256;   // arcs of a hub that one warp relaxes at a time
 
 struct WaveParams {
-    const int2* span;         // [n] arcs of a vertex: adj[span.x .. span.y)
+    const int2* span;         // [n] arcs of a vertex: adj[span.x .. span.y); null: from row
+    const int32_t* row;       // [n + 1] row offsets (span null)
     const uint2* adj;         // (col, weight bits); hubs' slices are contiguous
     int32_t n;
     const int32_t* srcs;      // [nq] or null (one query from src0)
@@ -278,7 +279,7 @@ struct Wave {
             const bool is_far = (v >> 31) != 0u;
             v &= 0x7fffffffu;
             const DistT dw = ld_dist(dist + v);
-            sp = __ldg(P.span + v);
+            sp = P.span ? __ldg(P.span + v) : make_int2(__ldg(P.row + v), __ldg(P.row + v + 1));
             d = dpart(dw);
             if (is_far) {
                 // below the old threshold: it went through near since

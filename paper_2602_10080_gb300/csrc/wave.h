@@ -1,9 +1,53 @@
 // wave.h -- host-side declarations of the cluster wavefront kernel (wave.cuh).
 #pragma once
 
+#include <cstddef>
+#include <mutex>
+
 #include "wave.cuh"
 
 namespace sssp {
+
+// How a call without a configuration is run: one cluster per query (wave),
+// the whole grid on one query (tide), the queries one after the other, or 32
+// queries side by side (fan).
+enum WaveKind { kOneCluster, kWholeGrid, kInTurn, kSideBySide };
+
+struct WavePlan {
+    WaveKind kind = kOneCluster;
+    int log_g = 0;         // log2 of a cluster's blocks
+    int threads = 1024;
+    uint32_t front = 1;
+    double delta = 1.0;
+    int32_t hub_deg = 256;
+    uint32_t wide = kInfU32;
+};
+
+// What the plan depends on.  wide: a solve found the front too wide for one
+// cluster.
+struct WaveGraph {
+    int32_t n;
+    int64_t m;
+    double avg_w, max_deg;
+    int sms;
+    bool wide;
+};
+
+constexpr int kTideLogWords = 17;               // the grid kernel spreads the places over at least 2^17 words
+constexpr size_t kWaveMaxShared = 200 * 1024;   // pending words of one block
+
+// The kernel and launch shape of a call; false: the queue engine takes it.
+bool plan_wave(const WaveGraph& g, int32_t nq, int pred_mode, WavePlan* w);
+// The fields of the parameters that follow from the plan; returns the dynamic
+// shared memory of a block.
+size_t wave_params(const WavePlan& w, const WaveGraph& g, bool f32, bool unit, WaveParams* p);
+// The most hub slices of one step: a hub is listed once, in slices of
+// kTideChunk arcs.
+uint32_t tide_slices(int64_t m, int32_t hub_deg);
+// The blocks of a whole-grid kernel wait for one another, so that two of them
+// (of two graphs, on two streams) must not share the device half and half:
+// one runs at a time.  Held from the launch to the end of the call.
+std::mutex& grid_mutex(int device);
 
 // Launches one cluster of 1 << p.log_g blocks per query.
 cudaError_t launch_wave(int wt, int pred, const WaveParams& p, int nq, int threads, size_t smem,

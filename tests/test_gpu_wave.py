@@ -227,3 +227,20 @@ def test_layout_of_another_threshold():
     d, p = gpu_solve(G, src, pred=True)
     assert_exact(g, src, d, p)
     G.close()
+
+
+def test_noalloc_on_cluster_and_grid():
+    """The fixed scratch serves every kernel and size: one cluster, a front
+    that outgrows it, the grid with hubs, and the largest vertex count."""
+    for g in (gg.random_directed(200_000, 800_000, 1, 100, seed=4), gg.rmat(16, 16, seed=3),
+              gg.erdos_renyi(50_000, 400_000, 1, 99, seed=3, wtype="f32"),
+              gg.random_directed(S.SSSP_NOALLOC_MAX_VERTICES, 6_000_000, 0, 9, seed=6)):
+        src = int(gg.giant_sources(g, 1)[0][0])
+        rp = torch.from_numpy(g.row_ptr).cuda()
+        arcs = torch.from_numpy(np.stack([g.col.view(np.uint32), g.w_bits], 1).view(np.int32).copy()).cuda()
+        d = torch.empty(g.n, dtype=torch.int32, device="cuda")
+        p = torch.empty(g.n, dtype=torch.int32, device="cuda")
+        for pred in (p, None):
+            S.sssp_solve_noalloc(rp, arcs, g.n, g.m, S.SSSP_W_F32 if g.wtype == "f32" else S.SSSP_W_U32, src, d, pred)
+            torch.cuda.synchronize()
+            assert_exact(g, src, d.cpu().numpy().view(np.uint32), None if pred is None else p.cpu().numpy())
