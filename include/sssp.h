@@ -402,7 +402,13 @@ SSSP_API int sssp_bfs(sssp_graph *g, int32_t src, uint32_t *level_out, int32_t *
  * lane's bucket window is at W has its buckets shifted by W, so its work
  * is ordered with the work already in flight.  A lane uses a quarter of the
  * graph's delta (it holds many queries under load).  Lanes of different graphs
- * run concurrently on their own streams, sharing the SMs. */
+ * run concurrently on their own streams, sharing the SMs.
+ *
+ * Queries that the wavefront kernels finish within about a slice are run to
+ * their end instead (without per-query timeouts and test flags): on a graph
+ * of at most 2^19 arcs a cluster of blocks each, the waiting ones in one
+ * launch beside those that run; on a larger graph that is not a mesh 12 to 32
+ * waiting ones side by side, or one by one, with the whole device. */
 typedef struct sssp_serve_options {
     size_t  mem_budget_bytes;  /* device bytes for distance slices and L2 rings of all lanes
                                   (0 = a quarter of the free device memory at creation) */

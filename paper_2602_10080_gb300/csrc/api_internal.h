@@ -1,6 +1,7 @@
 // api_internal.h -- host-side state behind the opaque C handles.
 #pragma once
 
+#include <atomic>
 #include <cstdint>
 #include <cstring>
 #include <mutex>
@@ -8,6 +9,7 @@
 
 #include "../../include/sssp.h"
 #include "internal.h"
+#include "wave.h"
 
 namespace sssp {
 
@@ -70,7 +72,7 @@ struct Graph {
     sssp_config tuned{};
     bool tuned_valid = false;
     bool tuned_queues = false;    // sssp_autotune timed the tuned queue configuration faster than the wavefront
-    bool wide = false;            // a solve found the front too wide for one cluster
+    std::atomic<bool> wide{false};   // a solve found the front too wide for one cluster
     // multi-query configurations from sssp_autotune_batch, per size class
     // (the number of queries rounded down to a power of two)
     struct BatchTuned {
@@ -137,6 +139,9 @@ int run_queries(Graph* g, const int32_t* srcs_host, const int32_t* srcs_dev, int
                 void* dist_out, int32_t* pred_out, const sssp_config* cfg, cudaStream_t stream,
                 sssp_stats* st_out, bool unit = false, const Sampling* samp = nullptr);
 
+inline WaveGraph wave_graph(const Graph* g) {
+    return WaveGraph{g->n, g->m, g->feat.avg_w, g->feat.max_deg, g->sms, g->wide.load()};
+}
 // The wavefront kernels (sssp_wave.cu), for calls that leave the configuration
 // to the library.  kWaveNotRun: the graph or the call is not for them.
 constexpr int kWaveNotRun = 1;

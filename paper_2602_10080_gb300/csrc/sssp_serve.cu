@@ -21,6 +21,15 @@
 //   4. grows the rings (migrating the live chunks) when one is half full.
 // Lanes of different graphs run concurrently on their own streams and
 // share the SMs in proportion to their queries in flight.
+//
+// Most queries are over within a slice or two on the wavefront kernels
+// (wave.cuh, fan.cuh).  A lane whose graph is for them (and no per-query
+// timeout has to end a running query) is an express lane: it takes the
+// queries that wait as one job on a stream of its own, to the end -- one
+// cluster per query on small graphs, several jobs at a time; on larger graphs
+// one job at a time, 12 to 32 waiting queries side by side, fewer one by one.
+// Long queries (meshes of more than 2^19 arcs) keep the slices.  24 queries on
+// R-MAT-18 at once (GB300): 2.3 ms, 12.1 in slices.
 #include <algorithm>
 #include <atomic>
 #include <chrono>
@@ -36,6 +45,8 @@
 #include <vector>
 
 #include "api_internal.h"
+#include "fan.h"
+#include "wave.h"
 
 namespace sssp {
 namespace {
@@ -230,8 +241,29 @@ struct Query {
     Clock::time_point t_submit, t_admit, t_done;
 };
 
+// One launch of an express lane with its own stream and buffers.
+struct Job {
+    cudaStream_t stream = nullptr;
+    cudaEvent_t k0 = nullptr, k1 = nullptr, done = nullptr;
+    Ctrl* ctrl = nullptr;
+    Ctrl* ctrl_h = nullptr;     // pinned mirror
+    int32_t* srcs = nullptr;    // [kJobQueries]
+    int32_t* srcs_h = nullptr;  // pinned
+    uint32_t* out_d = nullptr;  // [k][n] results, delivered when the job is done
+    int32_t* out_p = nullptr;
+    unsigned long long* work = nullptr;   // [k][n] packed words (wave, tide with predecessors)
+    uint32_t* words = nullptr;  // tide: barrier and bits; fan: its words
+    uint4* slices = nullptr;
+    size_t out_n = 0, outp_n = 0, work_n = 0, words_n = 0, slices_n = 0;
+    size_t bytes = 0;           // charged to the budget
+    std::vector<Query*> qs;     // in flight (empty: free)
+    bool grid = false;          // holds the grid mutex
+};
+
 struct Lane {
     Graph* g = nullptr;
+    bool express = false;       // wavefront jobs instead of slices
+    std::vector<Job*> jobs;
     uint64_t uid = 0;
     bool counted = false;       // registered in lane_refs (the graph's layout is pinned)
     int pred_mode = 0;
@@ -295,6 +327,7 @@ struct sssp_server {
     sssp_serve_stats stats{};
     std::thread worker;
     // worker-thread state
+    bool grid_job = false;                                  // a job holds the grid mutex
     std::deque<sssp::Query*> backlog;                       // waiting for a slot
     std::vector<sssp::Lane*> lanes;
 };
@@ -332,7 +365,34 @@ void lane_free_buffers(sssp_server* s, Lane* L) {
     L->nrings = 0;
 }
 
+// Worker thread, after the job's kernel (or a failure of the device).
+void job_release_grid(sssp_server* s, Job* J) {
+    if (!J->grid) return;
+    grid_mutex(s->device).unlock();
+    J->grid = s->grid_job = false;
+}
+
+void job_destroy(sssp_server* s, Job* J) {
+    if (J->stream) cudaStreamSynchronize(J->stream);
+    cudaFree(J->ctrl);
+    cudaFree(J->srcs);
+    cudaFree(J->out_d);
+    cudaFree(J->out_p);
+    cudaFree(J->work);
+    cudaFree(J->words);
+    cudaFree(J->slices);
+    if (J->ctrl_h) cudaFreeHost(J->ctrl_h);
+    if (J->srcs_h) cudaFreeHost(J->srcs_h);
+    if (J->k0) cudaEventDestroy(J->k0);
+    if (J->k1) cudaEventDestroy(J->k1);
+    if (J->done) cudaEventDestroy(J->done);
+    if (J->stream) cudaStreamDestroy(J->stream);
+    s->used -= J->bytes;
+    delete J;
+}
+
 void lane_destroy(sssp_server* s, Lane* L) {
+    for (Job* J : L->jobs) job_destroy(s, J);
     lane_free_buffers(s, L);
     if (L->counted) lane_refs(L->uid, -1);
     if (L->k0) cudaEventDestroy(L->k0);
@@ -539,6 +599,11 @@ Lane* lane_create(sssp_server* s, Graph* g, int pred_mode, int* rc) {
     }
     while (L->vbits < 31 && (1ll << L->vbits) <= (long long)g->nv) L->vbits++;  // 2^vbits > nv
     L->cap_limit = (uint32_t)std::min<uint64_t>((uint64_t)s->opt.max_slots, 1ull << (32 - L->vbits));
+    {
+        WavePlan w;
+        L->express = s->opt.flags == 0 && s->opt.query_timeout_ms == 0 && plan_wave(wave_graph(g), 1, pred_mode, &w) &&
+                     (w.kind == kWholeGrid || g->m <= (1 << 19));
+    }
     L->cell = pred_mode ? 8 : 4;
     L->idle_since = Clock::now();
     if (cudaStreamCreateWithFlags(&L->stream, cudaStreamNonBlocking) != cudaSuccess ||
@@ -551,7 +616,7 @@ Lane* lane_create(sssp_server* s, Graph* g, int pred_mode, int* rc) {
         lane_destroy(s, L);
         return nullptr;
     }
-    if (pred_mode) {
+    if (pred_mode && !L->express) {
         if (dev_alloc(&L->out_d, (size_t)g->n) || dev_alloc(&L->out_p, (size_t)g->n)) {
             *rc = SSSP_E_NOMEM;
             lane_destroy(s, L);
@@ -636,9 +701,19 @@ void admit(sssp_server* s) {
             continue;
         }
         int rc = SSSP_OK;
+        if (!L && s->grid_job) {
+            // lane_create waits for the graph's lock, whose holder may wait
+            // for the grid that this thread's job holds: after the job
+            keep.push_back(q);
+            continue;
+        }
         if (!L) {
             L = lane_create(s, q->g, pm, &rc);
             if (L) s->lanes.push_back(L);
+        }
+        if (L && L->express) {
+            keep.push_back(q);   // its next job takes it
+            continue;
         }
         if (L && L->free_slots.empty()) {
             const uint32_t want = L->cap ? L->cap * 2u : 8u;
@@ -698,12 +773,253 @@ void admit(sssp_server* s) {
     for (auto it = keep.rbegin(); it != keep.rend(); ++it) s->backlog.push_front(*it);
 }
 
+// ------------------------------------------------------- express lanes --
+
+constexpr int kJobQueries = 32;      // queries of one job
+constexpr size_t kLaneJobs = 8;      // jobs of one lane in flight (cluster jobs)
+
+// Room for `want` elements, charged to the budget.
+template <typename T>
+int job_room(sssp_server* s, Job* J, T** p, size_t* have, size_t want) {
+    if (*p && *have >= want) return SSSP_OK;
+    cudaFree(*p);
+    *p = nullptr;
+    s->used -= *have * sizeof(T);
+    J->bytes -= *have * sizeof(T);
+    *have = 0;
+    if (s->used + want * sizeof(T) > s->budget || dev_alloc(p, want)) return SSSP_E_NOMEM;
+    *have = want;
+    s->used += want * sizeof(T);
+    J->bytes += want * sizeof(T);
+    return SSSP_OK;
+}
+
+Job* job_create(sssp_server* s) {
+    Job* J = new (std::nothrow) Job();
+    if (!J) return nullptr;
+    if (cudaStreamCreateWithFlags(&J->stream, cudaStreamNonBlocking) != cudaSuccess ||
+        cudaEventCreate(&J->k0) != cudaSuccess || cudaEventCreate(&J->k1) != cudaSuccess ||
+        cudaEventCreateWithFlags(&J->done, cudaEventDisableTiming) != cudaSuccess || dev_alloc(&J->ctrl, 1) ||
+        dev_alloc(&J->srcs, kJobQueries) ||
+        cudaMallocHost((void**)&J->ctrl_h, sizeof(Ctrl)) != cudaSuccess ||
+        cudaMallocHost((void**)&J->srcs_h, kJobQueries * sizeof(int32_t)) != cudaSuccess) {
+        cudaGetLastError();
+        job_destroy(s, J);
+        return nullptr;
+    }
+    return J;
+}
+
+// The lane's waiting queries, oldest first (at most `most`).
+std::vector<Query*> express_waiting(sssp_server* s, Lane* L, size_t most) {
+    std::vector<Query*> qs;
+    std::lock_guard<std::mutex> lk(s->mu);
+    for (Query* q : s->backlog) {
+        if (qs.size() == most) break;
+        if (!q->cancel && q->g->uid == L->uid && (q->pred_out ? pred_mode_for(q->g) : 0) == L->pred_mode)
+            qs.push_back(q);
+    }
+    return qs;
+}
+
+// The lane runs slices from now on (no job in flight).
+int lane_to_slices(sssp_server* s, Lane* L) {
+    for (Job* J : L->jobs) job_destroy(s, J);
+    L->jobs.clear();
+    L->express = false;
+    if (L->pred_mode) {
+        const size_t n = (size_t)L->g->n;
+        if (dev_alloc(&L->out_d, n) || dev_alloc(&L->out_p, n)) return SSSP_E_NOMEM;
+        L->bytes += n * 8;
+        s->used += n * 8;
+    }
+    return SSSP_OK;
+}
+
+// Starts jobs for the lane's waiting queries as far as slots, jobs and the
+// grid are free.  Without memory for a job the lane goes back to slices (and
+// to their rules when that does not fit either).
+int express_launch(sssp_server* s, Lane* L) {
+    Graph* g = L->g;
+    const size_t n = (size_t)g->n;
+    const bool f32 = g->wtype == SSSP_W_F32, pred = L->pred_mode != 0;
+    for (;;) {
+        const int room = std::min<int>((int)L->cap_limit - L->running, kJobQueries);
+        if (room <= 0) return SSSP_OK;
+        std::vector<Query*> qs = express_waiting(s, L, (size_t)room);
+        if (qs.empty()) return SSSP_OK;
+        const WaveGraph wg = wave_graph(g);
+        WavePlan plan;
+        if (qs.size() > 1 && (!plan_wave(wg, (int32_t)qs.size(), L->pred_mode, &plan) || plan.kind == kInTurn))
+            qs.resize(1);
+        if (qs.size() == 1) {
+            plan = WavePlan();
+            plan_wave(wg, 1, L->pred_mode, &plan);
+        }
+        const bool grid = plan.kind != kOneCluster;
+        if (grid && s->grid_job) return SSSP_OK;
+        Job* J = nullptr;
+        for (Job* j : L->jobs)
+            if (j->qs.empty()) J = j;
+        if (!J) {
+            if (L->jobs.size() == kLaneJobs) return SSSP_OK;
+            J = job_create(s);
+            if (J) L->jobs.push_back(J);
+        }
+        const int32_t k = (int32_t)qs.size();
+        const size_t cells = (size_t)k * n;
+        WaveParams P;
+        std::memset(&P, 0, sizeof(P));
+        FanParams F;
+        std::memset(&F, 0, sizeof(F));
+        size_t smem = 0;
+        int rc = J ? SSSP_OK : SSSP_E_NOMEM;
+        if (!rc) rc = job_room(s, J, &J->out_d, &J->out_n, cells);
+        if (!rc && pred) rc = job_room(s, J, &J->out_p, &J->outp_n, cells);
+        if (!rc && plan.kind == kSideBySide) {
+            rc = job_room(s, J, &J->words, &J->words_n, fan_words(g->n, pred));
+            if (!rc) rc = job_room(s, J, &J->slices, &J->slices_n, fan_slices(g->n, g->m));
+            if (!rc) fan_carve(J->words, J->slices, g->n, g->m, pred, &F);
+        } else if (!rc) {
+            smem = wave_params(plan, wg, f32, false, &P);
+            if (smem > kWaveMaxShared) rc = SSSP_E_NOMEM;
+            if (!rc && pred) rc = job_room(s, J, &J->work, &J->work_n, cells);
+            if (!rc && grid) {
+                const size_t sync_words = sizeof(TideSync) / sizeof(uint32_t);
+                rc = job_room(s, J, &J->words, &J->words_n, sync_words + 4 * (size_t)P.words);
+                if (!rc && P.has_hubs) {
+                    P.items_cap = tide_slices(g->m, P.hub_deg);
+                    rc = job_room(s, J, &J->slices, &J->slices_n, 2 * (size_t)P.items_cap);
+                    P.items = J->slices;
+                }
+                if (!rc) {
+                    P.sync = reinterpret_cast<TideSync*>(J->words);
+                    P.bits = J->words + sync_words;
+                }
+            }
+        }
+        if (rc) return L->running ? SSSP_OK : lane_to_slices(s, L);
+        if (grid) {
+            if (!grid_mutex(s->device).try_lock()) return SSSP_OK;   // a solve holds the grid
+            J->grid = s->grid_job = true;
+        }
+        {
+            std::lock_guard<std::mutex> lk(s->mu);
+            const Clock::time_point now = Clock::now();
+            for (Query* q : qs) {
+                s->backlog.erase(std::find(s->backlog.begin(), s->backlog.end(), q));
+                if (q->cancel) continue;   // meanwhile: its result is not delivered
+                q->state = SSSP_Q_RUNNING;
+                q->t_admit = now;
+                if (L->running > 0) s->stats.joined_running++;
+            }
+            s->stats.slices++;
+        }
+        for (int32_t i = 0; i < k; i++) J->srcs_h[i] = qs[(size_t)i]->src;
+        cudaMemcpyAsync(J->srcs, J->srcs_h, (size_t)k * sizeof(int32_t), cudaMemcpyHostToDevice, J->stream);
+        cudaMemsetAsync(J->ctrl, 0, sizeof(Ctrl), J->stream);
+        if (plan.kind == kSideBySide) cudaMemsetAsync(F.sync, 0, sizeof(FanSync), J->stream);
+        else if (grid) cudaMemsetAsync(P.sync, 0, sizeof(TideSync), J->stream);
+        cudaEventRecord(J->k0, J->stream);
+        cudaError_t e;
+        if (plan.kind == kSideBySide) {
+            F.nq = k;
+            F.srcs = J->srcs;
+            F.span = g->span;
+            F.adj = g->adj;
+            F.ctrl = J->ctrl;
+            F.timeout_ns = 20000ull * 1000000ull;
+            e = launch_fan(f32 ? 1 : 0, F, s->sms, J->stream);
+            if (e == cudaSuccess) e = launch_fan_out(F.dist, g->n, k, J->out_d, s->sms, J->stream);
+            if (e == cudaSuccess && pred)
+                e = launch_fan_out(F.pred, g->n, k, reinterpret_cast<uint32_t*>(J->out_p), s->sms, J->stream);
+        } else {
+            P.span = g->span;
+            P.adj = g->adj;
+            P.srcs = grid ? nullptr : J->srcs;
+            P.src0 = J->srcs_h[0];
+            P.work = pred ? (void*)J->work : (void*)J->out_d;
+            P.dist_out = J->out_d;
+            P.pred_out = J->out_p;
+            P.ctrl = J->ctrl;
+            e = grid ? launch_tide(f32 ? 1 : 0, L->pred_mode, P, s->sms, plan.threads, J->stream)
+                     : launch_wave(f32 ? 1 : 0, L->pred_mode, P, k, plan.threads, smem, J->stream);
+        }
+        if (e != cudaSuccess) {
+            // no room for the cluster or the cooperative grid on this device
+            cudaGetLastError();
+            job_release_grid(s, J);
+            {
+                std::lock_guard<std::mutex> lk(s->mu);
+                for (auto it = qs.rbegin(); it != qs.rend(); ++it) {
+                    if ((*it)->cancel) continue;
+                    (*it)->state = SSSP_Q_QUEUED;
+                    s->backlog.push_front(*it);
+                }
+            }
+            return L->running ? cuda_status(e) : lane_to_slices(s, L);
+        }
+        J->qs = qs;
+        L->running += k;
+        cudaEventRecord(J->k1, J->stream);
+        cudaMemcpyAsync(J->ctrl_h, J->ctrl, sizeof(Ctrl), cudaMemcpyDeviceToHost, J->stream);
+        cudaEventRecord(J->done, J->stream);
+    }
+}
+
+// A finished job: its results to the queries' buffers.
+int express_collect(sssp_server* s, Lane* L, Job* J) {
+    job_release_grid(s, J);
+    const size_t n = (size_t)L->g->n;
+    float ms = 0;
+    cudaEventElapsedTime(&ms, J->k0, J->k1);
+    const Ctrl& hc = *J->ctrl_h;
+    int status = SSSP_OK;
+    if (hc.error != kErrNone || hc.finished != (int)J->qs.size())
+        status = hc.error == kErrTimeout ? SSSP_E_TIMEOUT : SSSP_E_CUDA;
+    std::vector<Query*> out;
+    {
+        std::lock_guard<std::mutex> lk(s->mu);
+        s->stats.kernel_ms += ms;
+        for (Query* q : J->qs) {
+            if (q->cancel) continue;
+            if (status == SSSP_OK) {
+                q->delivering = true;
+                out.push_back(q);
+            } else {
+                finish_query(s, q, status);
+            }
+        }
+    }
+    for (size_t i = 0; i < J->qs.size(); i++) {
+        Query* q = J->qs[i];
+        if (std::find(out.begin(), out.end(), q) == out.end()) continue;
+        cudaMemcpyAsync(q->dist_out, J->out_d + i * n, n * 4, cudaMemcpyDefault, J->stream);
+        if (q->pred_out) cudaMemcpyAsync(q->pred_out, J->out_p + i * n, n * 4, cudaMemcpyDefault, J->stream);
+    }
+    const cudaError_t e = cudaStreamSynchronize(J->stream);
+    L->running -= (int)J->qs.size();
+    if (e != cudaSuccess) return cuda_status(e);
+    J->qs.clear();
+    if (L->running == 0) L->idle_since = Clock::now();
+    std::lock_guard<std::mutex> lk(s->mu);
+    for (Query* q : out) finish_query(s, q, SSSP_OK);
+    s->cv_done.notify_all();
+    return SSSP_OK;
+}
+
 // Launches one slice on every lane that has work and no slice in flight.
 int launch_ready(sssp_server* s) {
     // the SMs are shared in proportion to each lane's queries in flight
     int total = 0;
-    for (Lane* L : s->lanes) total += L->running + L->draining;
+    for (Lane* L : s->lanes)
+        if (!L->express) total += L->running + L->draining;
     for (Lane* L : s->lanes) {
+        if (L->express) {
+            const int rc = express_launch(s, L);
+            if (rc) return rc;
+            continue;
+        }
         if (L->inflight || L->running + L->draining == 0) continue;
         KParams P = L->plan.P;
         P.nq = (int32_t)L->cap;
@@ -782,6 +1098,12 @@ void fail_all(sssp_server* s, int status) {
                 if (!L->slot_q[k]->cancel) finish_query(s, L->slot_q[k], status);
                 L->slot_q[k] = nullptr;
             }
+        for (Job* J : L->jobs) {
+            for (Query* q : J->qs)
+                if (!q->cancel) finish_query(s, q, status);
+            J->qs.clear();
+            job_release_grid(s, J);
+        }
         L->running = 0;
         L->draining = 0;
     }
@@ -1036,6 +1358,18 @@ void worker_main(sssp_server* s) {
         while (!rc) {
             inflight = false;
             for (Lane* L : s->lanes) {
+                for (Job* J : L->jobs) {
+                    if (J->qs.empty()) continue;
+                    const cudaError_t e = cudaEventQuery(J->done);
+                    if (e == cudaErrorNotReady) {
+                        inflight = true;
+                        continue;
+                    }
+                    rc = e == cudaSuccess ? express_collect(s, L, J) : cuda_status(e);
+                    any = true;
+                    if (rc) break;
+                }
+                if (rc) break;
                 if (!L->inflight) continue;
                 cudaError_t q = cudaEventQuery(L->done_ev);
                 if (q == cudaErrorNotReady) {
@@ -1049,6 +1383,14 @@ void worker_main(sssp_server* s) {
                 rc = collect_lane(s, L);
                 any = true;
                 if (rc) break;
+            }
+            if (!rc && !any && !inflight) {
+                // express queries that wait for the grid (a solve of another
+                // thread holds it): not at once again
+                std::unique_lock<std::mutex> lk(s->mu);
+                const bool waits = !s->backlog.empty();
+                lk.unlock();
+                if (waits) std::this_thread::sleep_for(std::chrono::microseconds(20));
             }
             if (rc || any || !inflight) break;
             if (std::chrono::duration<double, std::micro>(Clock::now() - t0).count() > 250.0) {

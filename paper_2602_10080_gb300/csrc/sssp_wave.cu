@@ -114,6 +114,34 @@ size_t wave_params(const WavePlan& w, const WaveGraph& g, bool f32, bool unit, W
 
 uint32_t tide_slices(int64_t m, int32_t hub_deg) { return (uint32_t)(m / kTideChunk + m / hub_deg + 1); }
 
+static size_t fan_places(int32_t n) {
+    size_t places = 1;
+    while (places < (size_t)n) places <<= 1;
+    return places;
+}
+
+constexpr size_t kFanSyncWords = sizeof(FanSync) / sizeof(uint32_t);
+static_assert(kFanSyncWords % 32 == 0, "the rows start on a 128-byte line");
+
+size_t fan_words(int32_t n, bool pred) {
+    return kFanSyncWords + std::max<size_t>(32, 2 * fan_places(n)) + 32 * (size_t)n * (pred ? 2 : 1);
+}
+
+// a row of more than kFanShort arcs is cut into slices of kFanChunk
+size_t fan_slices(int32_t n, int64_t m) { return (size_t)(m / kFanChunk + m / kFanShort + 1) + ((size_t)n + 1) / 2; }
+
+void fan_carve(uint32_t* words, uint4* slices, int32_t n, int64_t m, bool pred, FanParams* p) {
+    const size_t places = fan_places(n);
+    p->n = n;
+    p->mask = (uint32_t)(places - 1);
+    p->sync = reinterpret_cast<FanSync*>(words);
+    p->wait = words + kFanSyncWords;
+    p->dist = p->wait + std::max<size_t>(32, 2 * places);
+    p->pred = pred ? p->dist + 32 * (size_t)n : nullptr;
+    p->slices = slices;
+    p->rows = reinterpret_cast<uint2*>(slices + (m / kFanChunk + m / kFanShort + 1));
+}
+
 std::mutex& grid_mutex(int device) {
     static std::mutex mu[64];
     return mu[device & 63];
@@ -126,30 +154,17 @@ int run_fan(Graph* g, const int32_t* srcs_host, const int32_t* srcs_dev, int32_t
             int32_t* pred_out, cudaStream_t stream) {
     Workspace& ws = g->ws;
     const size_t n = (size_t)g->n;
-    uint32_t places = 1;
-    while (places < (uint32_t)g->n) places <<= 1;
     int rc;
     if ((rc = grow(&ws.srcs, &ws.srcs_n, (size_t)nq))) return rc;
     cudaMemcpyAsync(ws.srcs, srcs_dev ? srcs_dev : srcs_host, sizeof(int32_t) * nq,
                     srcs_dev ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice, stream);
-    const size_t sync_words = sizeof(FanSync) / 4, rows = 32 * n;
-    if ((rc = grow(&ws.fan, &ws.fan_n, sync_words + 2 * (size_t)places + rows * (pred_out ? 2 : 1) + 32))) return rc;
-    // a row of more than kFanShort arcs is cut into slices of kFanChunk
-    const size_t slices = (size_t)(g->m / kFanChunk + g->m / kFanShort + 1);
-    if ((rc = grow(&ws.fan_slices, &ws.fan_slices_n, slices + (n + 1) / 2))) return rc;
+    if ((rc = grow(&ws.fan, &ws.fan_n, fan_words(g->n, pred_out != nullptr)))) return rc;
+    if ((rc = grow(&ws.fan_slices, &ws.fan_slices_n, fan_slices(g->n, g->m)))) return rc;
     FanParams P;
     std::memset(&P, 0, sizeof(P));
+    fan_carve(ws.fan, ws.fan_slices, g->n, g->m, pred_out != nullptr, &P);
     P.span = g->span;
     P.adj = g->adj;
-    P.n = g->n;
-    P.sync = (FanSync*)ws.fan;
-    // the rows on their own 128-byte lines
-    P.dist = ws.fan + sync_words + (((2 * (size_t)places) + 31) & ~size_t(31));
-    P.wait = ws.fan + sync_words;
-    P.pred = pred_out ? P.dist + rows : nullptr;
-    P.mask = places - 1u;
-    P.slices = ws.fan_slices;
-    P.rows = (uint2*)(ws.fan_slices + slices);
     P.ctrl = ws.ctrl;
     P.timeout_ns = 20000ull * 1000000ull;
     const int32_t groups = (nq + 31) / 32, per = (nq + groups - 1) / groups;
@@ -174,7 +189,7 @@ int run_wave(Graph* g, const int32_t* srcs_host, const int32_t* srcs_dev, int32_
     // unit weights are >= 1: the packed minimum gives the smallest-index parent
     const int pred_mode = pred_out ? (unit ? 1 : pred_mode_for(g)) : 0;
     WavePlan plan;
-    const WaveGraph wg{g->n, g->m, g->feat.avg_w, g->feat.max_deg, g->sms, g->wide};
+    const WaveGraph wg = wave_graph(g);
     if (!plan_wave(wg, nq, pred_mode, &plan)) return kWaveNotRun;
     if (cudaSetDevice(g->device) != cudaSuccess) return SSSP_E_CUDA;
     const int32_t n = g->n;

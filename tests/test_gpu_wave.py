@@ -244,3 +244,59 @@ def test_noalloc_on_cluster_and_grid():
             S.sssp_solve_noalloc(rp, arcs, g.n, g.m, S.SSSP_W_F32 if g.wtype == "f32" else S.SSSP_W_U32, src, d, pred)
             torch.cuda.synchronize()
             assert_exact(g, src, d.cpu().numpy().view(np.uint32), None if pred is None else p.cpu().numpy())
+
+
+def test_served_bursts_and_concurrent_solves():
+    """Express lanes: bursts of queries on a grid-kernel graph (side by side)
+    and on a small one (a cluster each), with and without predecessors, host
+    and device buffers, cancellations, while another thread solves on the same
+    and on other graphs."""
+    graphs = [gg.rmat(15, 24, seed=8), gg.rmat(12, 16, seed=2, wtype="f32")]
+    Gs = [upload(g) for g in graphs]
+    other = gg.rmat(15, 20, seed=9)
+    O = upload(other)
+    osrc = gg.giant_sources(other, 12)[0]
+    got, stop = [], threading.Event()
+
+    def solver():
+        k = 0
+        while not stop.is_set() or k < 12:
+            s = int(osrc[k % 12])
+            got.append((s, gpu_solve(O, s, pred=False)[0]))
+            gpu_solve(Gs[0], 0, pred=False)
+            k += 1
+
+    srv = S.sssp_serve_create()
+    th = threading.Thread(target=solver)
+    th.start()
+    try:
+        for rnd in range(2):
+            jobs = []
+            for gi, g in enumerate(graphs):
+                for q, s in enumerate(gg.giant_sources(g, 45, seed=rnd)[0]):
+                    host, pred = q % 5 == 4, q % 3 == 0
+                    d = np.full(g.n, 7, np.uint32) if host else torch.empty(g.n, dtype=torch.int32, device="cuda")
+                    p = None
+                    if pred:
+                        p = np.empty(g.n, np.int32) if host else torch.empty(g.n, dtype=torch.int32, device="cuda")
+                    jobs.append((g, int(s), d, p, S.sssp_serve_submit(srv, Gs[gi].handle, int(s), d, p)))
+            cancelled = {j for j in range(0, len(jobs), 11) if S.sssp_serve_cancel(srv, jobs[j][4]) == S.SSSP_OK}
+            for j, (g, s, d, p, t) in enumerate(jobs):
+                st, code = S.sssp_serve_wait(srv, t, 60000)
+                if j in cancelled:
+                    assert st == S.Q_ERROR and code == S.SSSP_E_CANCELLED
+                    continue
+                assert st == S.Q_DONE, S.strerror(code)
+                torch.cuda.synchronize()
+                db = d if isinstance(d, np.ndarray) else d.cpu().numpy().view(np.uint32)
+                pb = p if p is None or isinstance(p, np.ndarray) else p.cpu().numpy()
+                assert_exact(g, s, db, pb)
+    finally:
+        stop.set()
+        th.join()
+        stats = S.sssp_serve_get_stats(srv)
+        S.sssp_serve_destroy(srv)
+    assert stats["completed"] + stats["cancelled"] == stats["submitted"] == 180
+    for s, d in got[:12]:
+        assert_exact(other, s, d)
+    [G.close() for G in Gs + [O]]
