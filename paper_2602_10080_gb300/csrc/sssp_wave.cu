@@ -21,30 +21,49 @@ uint32_t pow2_at_least(double x) {
 
 }  // namespace
 
+// The pending bits of a cluster: four sets of a bit for every vertex, rounded
+// up to a power of two.
+constexpr int32_t kClusterVertices = 1 << 21;
+static_assert((size_t)kClusterVertices / 2 / 16 <= kWaveMaxShared, "pending bits of 16 blocks");
+
 bool plan_wave(const WaveGraph& g, int32_t nq, int pred_mode, WavePlan* w) {
     const double deg = std::max(1.0, (double)g.m / (double)g.n);
     const bool hubs = g.max_deg > 64.0;
     // about the average weight over a quarter of the degree: of the widths
-    // 1/2 to 4 times this, meshes and G(n, m) graphs run within 5% of the best
+    // 1/2 to 4 times this, G(n, m) graphs run within 5% of the best at one hop
+    // a step
     w->delta = 4.0 * g.avg_w / deg;
     // Threads of one cluster: one for eight vertices or 32 arcs, 1024 to
-    // 16384 in 16 blocks (8 for the smallest).  GB300, us a solve: directed
-    // 1000 vertices 8 x 128 76, 1 x 1024 82; grid 256^2 16 x 512 1114, 8 x 512
-    // 1153, 1 x 1024 1800; grid 1024^2 16 x 1024 5670, 8 x 1024 8500.
+    // 16384 in 16 blocks (8 for the smallest).  GB300, us a solve at one hop a
+    // step: directed 1000 vertices 8 x 128 76, 1 x 1024 82; grid 256^2 16 x 512
+    // 1114, 8 x 512 1153, 1 x 1024 1800; grid 1024^2 16 x 1024 5670, 8 x 1024 8500.
     const uint32_t total =
         std::min(16384u, std::max(1024u, pow2_at_least(std::max((double)g.n / 8.0, (double)g.m / 32.0))));
+    // On a mesh or a road map the front is thin and the hops are all there is
+    // (few arcs a vertex, and none with many more: in a sparse random graph
+    // some vertex has over twice the average).  There a warp goes on for several
+    // hops a step with the vertices that it improved itself, and the threshold
+    // moves as far.  us at 1, 4, 6 and 8 hops (width x4): grid 256^2 1132, 825,
+    // 797, 775; grid 1024^2 6150, 4139, 4021, 3835; road 900 x 777 1893, 1378,
+    // 1414, 1404; grid 64 x 60 285, 220, -, 215.  Elsewhere a second hop may pay
+    // (directed 60000 vertices of degree 6 174, 150 at 2, 255 at 8; G(10^4, 10^5)
+    // 128, 115 at 2) but not on the smallest graphs (directed 10^4 vertices 102,
+    // 114 at 2), nor with hubs (R-MAT-13 164, 189 at 2).
+    const bool thin = deg <= 6.5 && g.max_deg <= std::min(2.0 * deg + 1.5, 11.5);
+    const int32_t hops = thin ? 8 : !hubs && g.m > (1 << 16) ? 2 : 1;
     if (nq == 1) {
-        const bool thin = deg <= 6.0 && !hubs && g.n <= (1 << 21);
-        if (g.m <= (1 << 19) || (thin && !g.wide)) {
+        if (g.n <= kClusterVertices && (g.m <= (1 << 19) || (thin && !g.wide))) {
+            w->hops = hops;
+            w->delta *= thin ? 4.0 : 1.0;
             w->log_g = total > 1024u ? 4 : 3;
             w->threads = (int)(total >> w->log_g);
             // raise the threshold while there is less than a vertex for every
-            // 16 threads: grid 256^2 1114 us (1088 at a 32nd, 1180 at an
-            // eighth), grid 1024^2 5670 (5740, 5790)
+            // 16 threads: grid 256^2 775 us (800 at a 32nd), grid 1024^2 3835
+            // (4134; 3800 at an eighth)
             w->front = total / 16u;
-            // sparse random graphs look like meshes and have wide fronts, for
-            // which 16 SMs are too few: 10^6 vertices of degree 10 take 1370 us
-            // here and 310 us on the whole grid; such a solve starts over there
+            // a random graph of equal degrees looks like a mesh and has a wide
+            // front, for which 16 SMs are too few: 10^6 vertices of degree 10 take
+            // 1370 us here and 310 us on the whole grid; it starts over there
             if (g.m > (1 << 19)) w->wide = 24576u;
             return true;
         }
@@ -62,17 +81,19 @@ bool plan_wave(const WaveGraph& g, int32_t nq, int pred_mode, WavePlan* w) {
             // (and BFS) 2.87 (0.90) ms with 256 arcs, 2.51 (0.79) with 512
             w->hub_deg = 512;
         } else {
-            // road 4096^2 9.8 ms at 16384 (13.6 at 4096, 9.4 at 32768); G(2^21, 2^25)
-            // 0.83 ms at 4096 and at 16384
-            w->front = deg <= 6.0 ? 16384u : 4096u;
-            if (deg <= 6.0) w->delta *= 2.0;
+            // road 4096^2, ms at 1, 3, 4, 5 and 6 hops: 9.49 (width x2), 6.13, 5.90,
+            // 5.80, 5.84 (x3), 6.46 at 4 hops with a front of 16384; G(2^21, 2^25)
+            // 0.79 ms at one hop, 0.81 at two, 0.83 with a front of 16384
+            w->front = thin ? 32768u : 4096u;
+            w->hops = thin ? 5 : 1;
+            if (thin) w->delta *= 3.0;
         }
         return true;
     }
     // a batch on a small graph or a mesh: one cluster per query, as wide as the
     // queries leave room for (13 queries on grid 301 x 257: 8 blocks 1690 us,
     // 4: 1880, 1: 2130)
-    if (g.m > (1 << 21) || (hubs && g.m > (1 << 18))) {
+    if (g.n > kClusterVertices || g.m > (1 << 21) || (hubs && g.m > (1 << 18))) {
         // A group of up to 32 queries side by side costs as much as this many
         // in turn on the whole grid: R-MAT-20 7 (5.7 ms), R-MAT-18 7 (2.7 ms),
         // G(200K, 2M) 15 (3.1 ms).  Predecessors of the strict-improvement rule
@@ -83,9 +104,12 @@ bool plan_wave(const WaveGraph& g, int32_t nq, int pred_mode, WavePlan* w) {
         return true;
     }
     w->log_g = 4;
-    while (w->log_g > 0 && (nq << w->log_g) > g.sms) w->log_g--;
+    const size_t pending = pow2_at_least((double)g.n) / 2;
+    while (w->log_g > 0 && (nq << w->log_g) > g.sms && pending >> (w->log_g - 1) <= kWaveMaxShared) w->log_g--;
     w->threads = (int)std::max(128u, std::min(w->log_g ? 512u : 1024u, total >> w->log_g));
     w->front = std::max(1u, (uint32_t)(w->threads << w->log_g) / 16u);
+    w->hops = hops;
+    w->delta *= thin ? 4.0 : 1.0;
     return true;
 }
 
@@ -101,11 +125,16 @@ size_t wave_params(const WavePlan& w, const WaveGraph& g, bool f32, bool unit, W
     p->log_g = w.log_g;
     p->words = (int32_t)std::max(1u, (1u << (bits - p->log_b)) >> p->log_g);
     p->n = g.n;
-    if (f32) p->delta = __float_as_uint_host((float)std::max(1e-30, w.delta));
+    if (unit) {
+        // breadth-first: level by level; on a mesh as many levels a step as hops
+        p->delta = w.hops > 2 ? (uint32_t)w.hops : kInfU32;
+        p->hops = w.hops > 2 ? w.hops : 1;
+    } else if (f32) p->delta = __float_as_uint_host((float)std::max(1e-30, w.delta));
     else p->delta = (uint32_t)std::min(4.0e9, std::max(1.0, w.delta));
     p->front = w.front;
     p->wide = w.wide;
     p->unit = unit ? 1 : 0;
+    if (!unit) p->hops = w.hops;
     p->hub_deg = w.hub_deg;
     p->has_hubs = g.max_deg > (double)w.hub_deg;
     p->timeout_ns = 20000ull * 1000000ull;

@@ -52,7 +52,8 @@ struct WaveParams {
     int32_t log_b;            // log2 of the bits used per word (0..5)
     int32_t log_g;            // log2 of the cluster's blocks: word w lives in block w % G
     int32_t words;            // words per block (wave), or in all (tide)
-    int32_t unit;             // breadth-first: every arc weighs 1, no threshold
+    int32_t hops;             // hops of a warp per step
+    int32_t unit;             // breadth-first: every arc weighs 1, hub slices belong to the step that lists them
     int32_t hub_deg;          // a vertex with more arcs is not left to one warp
     int32_t has_hubs;
     uint32_t wide;            // wave: give up (kErrWide) when more vertices than this wait in near
@@ -63,6 +64,14 @@ struct WaveParams {
     uint4* items;             // hub slices, two lists of items_cap: (vertex, distance, first arc, end)
     uint32_t items_cap;
     struct TideSync* sync;
+};
+
+constexpr uint32_t kWaveOwn = 64;      // improved vertices that a warp keeps for its own next hop
+
+template <bool HOPS>
+struct WaveLists {
+    uint32_t list[64];                 // vertices taken from the words (bit 31: from far)
+    uint2 own[2][HOPS ? kWaveOwn : 1]; // (vertex, distance) of this hop and the next
 };
 
 struct WaveSlot {
@@ -78,7 +87,6 @@ struct WaveShared {
     WaveSlot slot[2][kWaveMaxCluster];  // what every block of the cluster reports at the end of a step
     uint32_t near[4], fmin[4], nhub[4]; // this block's sums of step s, set s % 4
     WaveHub hub[kWaveHubs];
-    uint32_t list[32][64];              // per warp: vertices taken from the words (bit 31: from far)
 };
 
 // Grid barriers and the sums of a step (set s % 4).  A block arrives by one
@@ -132,7 +140,9 @@ __device__ __forceinline__ uint32_t wave_raise(uint32_t base, uint32_t delta, ui
 // global memory.
 enum WaveMode { kWaveBlock = 0, kWaveCluster = 1, kWaveGrid = 2 };
 
-template <int WT, int PRED, int MODE>
+// HOPS: a warp may have more than one hop a step (compiled out otherwise: with
+// it R-MAT-22 took 8% and R-MAT-13 12% longer at one hop).
+template <int WT, int PRED, int MODE, bool HOPS>
 struct Wave {
     using DistT = typename std::conditional<PRED == 0, uint32_t, unsigned long long>::type;
     using A = Arith<WT>;
@@ -140,11 +150,13 @@ struct Wave {
 
     const WaveParams& P;
     DistT* dist;
-    uint32_t* list;            // this warp's list
+    WaveLists<HOPS>* lists;    // this warp's
     uint32_t T, Told;
     Addr near_w, far_w;        // the words written in this step
     uint32_t n_imp, fmin;      // this thread's near improvements and smallest far distance of the step
     uint32_t n_relax;          // arcs relaxed by this thread
+    uint32_t n_own, own_w;     // entries kept for the next hop, and which half they are in
+    bool keep;                 // the warp has another hop in this step
 
     static __device__ __forceinline__ uint32_t dpart(uint32_t w) { return w; }
     static __device__ __forceinline__ uint32_t dpart(unsigned long long w) { return (uint32_t)(w >> 32); }
@@ -175,7 +187,7 @@ struct Wave {
     // larger value, so the last improvement always marks it).  Straight-line
     // code with predicated stores: as branches, four arcs took 2200 cycles of
     // a 9300-cycle step (grid 256^2 on GB300), like this 300.
-    template <int K>
+    template <int K, bool OWN>
     __device__ __forceinline__ void relax(const uint32_t (&u)[K], const uint32_t (&du)[K], const uint2 (&a)[K],
                                           const DistT (&c)[K], const bool (&in)[K]) {
         uint32_t nd[K], mask[K];
@@ -215,13 +227,23 @@ struct Wave {
         }
 #pragma unroll
         for (int k = 0; k < K; k++) {
+            bool near = imp[k] && nd[k] < T;
+            fmin = imp[k] && !near ? min(fmin, nd[k]) : fmin;
+            if (OWN && HOPS && keep) {
+                const uint32_t b = __ballot_sync(kFull, near), at = n_own + __popc(b & lanemask_lt());
+                n_own = min(kWaveOwn, n_own + (uint32_t)__popc(b));
+                if (near && at < kWaveOwn) {
+                    lists->own[own_w][at] = make_uint2(a[k].x, nd[k]);
+                    near = imp[k] = false;
+                }
+            }
             if (imp[k]) red_or(ad[k], mask[k]);
-            n_imp += imp[k] && nd[k] < T ? 1u : 0u;
-            fmin = imp[k] && nd[k] >= T ? min(fmin, nd[k]) : fmin;
+            n_imp += near ? 1u : 0u;
         }
     }
 
     // Up to four arcs of one vertex, `stride` apart, all loads in flight together.
+    template <bool OWN>
     __device__ __forceinline__ void arcs4(uint32_t u, uint32_t du, int32_t e, int32_t stride, int32_t end) {
         uint2 a[4];
         DistT c[4];
@@ -236,7 +258,7 @@ struct Wave {
         }
 #pragma unroll
         for (int k = 0; k < 4; k++) c[k] = in[k] ? ld_dist(dist + a[k].x) : (DistT)0;
-        relax<4>(uu, dd, a, c, in);
+        relax<4, OWN>(uu, dd, a, c, in);
     }
 
     // Arcs g0 + lane + 32 k (k < 4) of the warp's concatenated rows (ex: arcs
@@ -262,25 +284,23 @@ struct Wave {
         }
 #pragma unroll
         for (int k = 0; k < 4; k++) c[k] = in[k] ? ld_dist(dist + a[k].x) : (DistT)0;
-        relax<4>(uj, dj, a, c, in);
+        relax<4, true>(uj, dj, a, c, in);
     }
 
-    // Relaxes the k <= 32 vertices list[from ..], one per lane; `hub(v, d,
-    // arcs)` takes those with more than hub_deg arcs (it returns false for
-    // one that the warp has to expand all the same).
+    // Relaxes up to 32 vertices, one per lane (`have`): from the words
+    // (is_far: from the far ones) or, with their distance d, from the warp's
+    // last hop.  `hub(v, d, arcs, deg)` takes those with more than hub_deg arcs
+    // (it returns the arcs that are left to the warp).
     template <typename Hub>
-    __device__ __forceinline__ void relax_list(uint32_t from, uint32_t k, Hub&& hub) {
+    __device__ __forceinline__ void relax_batch(bool have, uint32_t v, bool is_far, uint32_t d, Hub&& hub) {
         const uint32_t lane = lane_id();
-        bool have = lane < k;
-        uint32_t v = 0u, d = 0u;
         int2 sp = make_int2(0, 0);
         if (have) {
-            v = list[from + lane];
-            const bool is_far = (v >> 31) != 0u;
-            v &= 0x7fffffffu;
-            const DistT dw = ld_dist(dist + v);
+            const uint32_t now = dpart(ld_dist(dist + v));
             sp = P.span ? __ldg(P.span + v) : make_int2(__ldg(P.row + v), __ldg(P.row + v + 1));
-            d = dpart(dw);
+            // improved meanwhile: whoever did marked it again
+            if (d != kInfU32) have = now >= d;
+            else d = now;
             if (is_far) {
                 // below the old threshold: it went through near since
                 if (d < Told) {
@@ -299,7 +319,7 @@ struct Wave {
         if (P.has_hubs) deg = hub(v, d, sp, deg);
         if (__reduce_max_sync(kFull, (uint32_t)deg) <= 4u) {
             // few arcs a vertex: each lane its own
-            arcs4(v, d, sp.x, 1, sp.x + deg);
+            arcs4<true>(v, d, sp.x, 1, sp.x + deg);
         } else {
             // the batch's arcs spread over the lanes, 128 at a time
             int32_t incl = deg;
@@ -314,29 +334,37 @@ struct Wave {
         __syncwarp();
     }
 
-    // Empties the words i = first, first + stride, ... below `words` (32 at a
-    // time: this lane's is i + lane) into the list and relaxes the list's
-    // vertices 32 at a time.  `take(i, nb, fb)` reads and clears a lane's word.
+    // The warp's part of a step.  Hop 0: empties the words i = first,
+    // first + stride, ... below `words` (32 at a time: this lane's is i + lane)
+    // into the list and relaxes the list's vertices 32 at a time; `take(i, nb,
+    // fb)` reads and clears a lane's word.  Then P.hops - 1 hops over the near
+    // vertices that the warp itself improved: a hop without the barrier and the
+    // words costs half, and a vertex relaxed too early only costs its arcs.
     template <typename Take, typename Vertex, typename Hub>
     __device__ __forceinline__ void sweep(uint32_t first, uint32_t stride, uint32_t words, Take&& take,
                                           Vertex&& vertex_of, Hub&& hub) {
         const uint32_t lane = lane_id();
-        uint32_t held = 0u, nb = 0u, fb = 0u, base = first;
+        uint32_t held = 0u, nb = 0u, fb = 0u, base = first, own = 0u, pos = 0u;
+        int32_t hop = 0;
         bool more = base < words;
+        n_own = own_w = 0u;
+        keep = HOPS && P.hops > 1;
         if (more) take(base + lane, nb, fb);
-        while (more || held) {
+        for (;;) {
+            uint32_t v = 0u, d = kInfU32;
+            bool have = false, is_far = false;
             while (more && held < 32u) {
-                const bool have = (nb | fb) != 0u;
-                const uint32_t m = __ballot_sync(kFull, have);
+                const bool got = (nb | fb) != 0u;
+                const uint32_t m = __ballot_sync(kFull, got);
                 if (!m) {
                     base += stride;
                     more = base < words;
                     if (more) take(base + lane, nb, fb);
                     continue;
                 }
-                if (have) {
+                if (got) {
                     const uint32_t b = (uint32_t)__ffs((int)(nb | fb)) - 1u;
-                    list[held + __popc(m & lanemask_lt())] =
+                    lists->list[held + __popc(m & lanemask_lt())] =
                         vertex_of(base + lane, b) | ((nb >> b) & 1u ? 0u : 0x80000000u);
                     nb &= ~(1u << b);
                     fb &= ~(1u << b);
@@ -344,10 +372,32 @@ struct Wave {
                 held += __popc(m);
                 __syncwarp();
             }
-            if (!held) break;
-            const uint32_t k = held < 32u ? held : 32u;
-            held -= k;
-            relax_list(held, k, hub);
+            if (held) {
+                const uint32_t k = held < 32u ? held : 32u;
+                held -= k;
+                have = lane < k;
+                if (have) v = lists->list[held + lane];
+                is_far = (v >> 31) != 0u;
+                v &= 0x7fffffffu;
+            } else if (HOPS && pos < own) {
+                have = pos + lane < own;
+                if (have) {
+                    const uint2 e = lists->own[own_w ^ 1u][pos + lane];
+                    v = e.x;
+                    d = e.y;
+                }
+                pos += 32u;
+            } else {
+                if (!HOPS || n_own == 0u) break;
+                hop++;
+                keep = hop + 1 < P.hops;
+                own = n_own;
+                pos = n_own = 0u;
+                own_w ^= 1u;
+                __syncwarp();
+                continue;
+            }
+            relax_batch(have, v, is_far, d, hub);
         }
     }
 
@@ -397,19 +447,20 @@ struct Wave {
 // by writing them into every block's slots; one cluster barrier then makes
 // them and the step's marks visible.  Two slot sets alternate: a block can
 // write set s + 2 only after all blocks passed barrier s + 1, after reading s.
-template <int WT, int PRED, bool CL>
+template <int WT, int PRED, bool CL, bool HOPS>
 __global__ void __launch_bounds__(1024, 1) wave_kernel(const __grid_constant__ WaveParams P) {
-    using W = Wave<WT, PRED, CL ? kWaveCluster : kWaveBlock>;
+    using W = Wave<WT, PRED, CL ? kWaveCluster : kWaveBlock, HOPS>;
     using DistT = typename W::DistT;
     extern __shared__ __align__(16) uint32_t wave_words[];   // near[2], far[2]
     __shared__ WaveShared S;
+    __shared__ WaveLists<HOPS> lists[32];
     const uint32_t tid = threadIdx.x, nt = blockDim.x, lane = tid & 31u;
     const uint32_t G = CL ? 1u << P.log_g : 1u, rank = CL ? cluster_rank() : 0u;
     const uint32_t q = CL ? blockIdx.x >> P.log_g : blockIdx.x;
     const uint32_t src = (uint32_t)(P.srcs ? P.srcs[q] : P.src0);
     const uint32_t words = (uint32_t)P.words;
-    W w{P, reinterpret_cast<DistT*>(P.work) + (size_t)q * (size_t)P.n, S.list[tid >> 5],
-        P.unit ? kInfU32 : wave_raise<WT>(0u, P.delta, 0u), 0u, 0u, 0u, 0u, kInfU32, 0u};
+    W w{P, reinterpret_cast<DistT*>(P.work) + (size_t)q * (size_t)P.n, &lists[tid >> 5],
+        wave_raise<WT>(0u, P.delta, 0u), 0u, 0u, 0u, 0u, kInfU32, 0u, 0u, 0u, false};
 
     // every distance to infinity but the source's, and its pending bit
     w.init(src, rank * nt + tid, G * nt);
@@ -470,7 +521,7 @@ __global__ void __launch_bounds__(1024, 1) wave_kernel(const __grid_constant__ W
             for (uint32_t h = 0; h < nh; h++) {
                 const WaveHub hb = S.hub[h];
                 for (int32_t e = hb.arcs.x + (int32_t)tid; e < hb.arcs.y; e += 4 * (int32_t)nt)
-                    w.arcs4(hb.v, hb.d, e, (int32_t)nt, hb.arcs.y);
+                    w.template arcs4<false>(hb.v, hb.d, e, (int32_t)nt, hb.arcs.y);
             }
         }
         // the step's sums
@@ -538,19 +589,19 @@ __device__ __forceinline__ void red_release64(unsigned long long* p, unsigned lo
     asm volatile("red.release.gpu.global.add.u64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
 }
 
-template <int WT, int PRED>
+template <int WT, int PRED, bool HOPS>
 __global__ void __launch_bounds__(1024, 1) tide_kernel(const __grid_constant__ WaveParams P) {
-    using W = Wave<WT, PRED, kWaveGrid>;
+    using W = Wave<WT, PRED, kWaveGrid, HOPS>;
     using DistT = typename W::DistT;
-    __shared__ uint32_t lists[32][64];
+    __shared__ WaveLists<HOPS> lists[32];
     __shared__ uint32_t s_near[4], s_fmin[4], s_out[4];
     const uint32_t tid = threadIdx.x, nt = blockDim.x, lane = tid & 31u;
     const uint32_t gt = blockIdx.x * nt + tid, gn = gridDim.x * nt;
     // consecutive warps of the grid lie in different blocks
     const uint32_t wid = (tid >> 5) * gridDim.x + blockIdx.x, nw = gn >> 5;
     const uint32_t words = (uint32_t)P.words;
-    W w{P, reinterpret_cast<DistT*>(P.work), lists[tid >> 5],
-        P.unit ? kInfU32 : wave_raise<WT>(0u, P.delta, 0u), 0u, nullptr, nullptr, 0u, kInfU32, 0u};
+    W w{P, reinterpret_cast<DistT*>(P.work), &lists[tid >> 5],
+        wave_raise<WT>(0u, P.delta, 0u), 0u, nullptr, nullptr, 0u, kInfU32, 0u, 0u, 0u, false};
     const unsigned long long deadline = gtime() + P.timeout_ns;
 
     w.init((uint32_t)P.src0, gt, gn);
@@ -691,7 +742,7 @@ __global__ void __launch_bounds__(1024, 1) tide_kernel(const __grid_constant__ W
             const uint4 it = __ldcg(items_r + i);
             if (!P.unit && W::dpart(ld_dist(w.dist + it.x)) < it.y) continue;
             for (int32_t e = (int32_t)it.z + (int32_t)lane; e < (int32_t)it.w; e += 128)
-                w.arcs4(it.x, it.y, e, 32, (int32_t)it.w);
+                w.template arcs4<false>(it.x, it.y, e, 32, (int32_t)it.w);
             __syncwarp();
         }
     }

@@ -19,6 +19,7 @@ struct WavePlan {
     int threads = 1024;
     uint32_t front = 1;
     double delta = 1.0;
+    int32_t hops = 1;
     int32_t hub_deg = 256;
     uint32_t wide = kInfU32;
 };
@@ -34,7 +35,7 @@ struct WaveGraph {
 };
 
 constexpr int kTideLogWords = 17;               // the grid kernel spreads the places over at least 2^17 words
-constexpr size_t kWaveMaxShared = 200 * 1024;   // pending words of one block
+constexpr size_t kWaveMaxShared = 176 * 1024;   // pending words of one block (beside WaveShared)
 
 // The kernel and launch shape of a call; false: the queue engine takes it.
 bool plan_wave(const WaveGraph& g, int32_t nq, int pred_mode, WavePlan* w);

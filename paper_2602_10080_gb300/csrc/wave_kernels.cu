@@ -3,9 +3,9 @@
 
 namespace sssp {
 
-template <int WT, int PRED, bool CL>
-static cudaError_t launch_one(const WaveParams& p, int nq, int threads, size_t smem, cudaStream_t stream) {
-    auto fn = wave_kernel<WT, PRED, CL>;
+template <int WT, int PRED, bool CL, bool HOPS>
+static cudaError_t launch_hops(const WaveParams& p, int nq, int threads, size_t smem, cudaStream_t stream) {
+    auto fn = wave_kernel<WT, PRED, CL, HOPS>;
     cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     cudaLaunchConfig_t c{};
@@ -27,6 +27,12 @@ static cudaError_t launch_one(const WaveParams& p, int nq, int threads, size_t s
     return cudaLaunchKernelEx(&c, fn, p);
 }
 
+template <int WT, int PRED, bool CL>
+static cudaError_t launch_one(const WaveParams& p, int nq, int threads, size_t smem, cudaStream_t stream) {
+    return p.hops > 1 ? launch_hops<WT, PRED, CL, true>(p, nq, threads, smem, stream)
+                      : launch_hops<WT, PRED, CL, false>(p, nq, threads, smem, stream);
+}
+
 template <int WT, int PRED>
 static cudaError_t launch_tide_one(const WaveParams& p, int grid, int threads, cudaStream_t stream) {
     cudaLaunchConfig_t c{};
@@ -38,7 +44,8 @@ static cudaError_t launch_tide_one(const WaveParams& p, int grid, int threads, c
     at[0].val.cooperative = 1;
     c.attrs = at;
     c.numAttrs = 1;
-    return cudaLaunchKernelEx(&c, tide_kernel<WT, PRED>, p);
+    return p.hops > 1 ? cudaLaunchKernelEx(&c, tide_kernel<WT, PRED, true>, p)
+                      : cudaLaunchKernelEx(&c, tide_kernel<WT, PRED, false>, p);
 }
 
 cudaError_t launch_tide(int wt, int pred, const WaveParams& p, int grid, int threads, cudaStream_t stream) {

@@ -99,9 +99,17 @@ def test_thresholds_at_the_ends():
     both(gg.from_edges(700, [(v, v + 1, 5) for v in range(1, 699)]), 0)
 
 
+def regular(n, deg, seed):
+    """`deg` random arcs from every vertex: by its degrees a mesh, by its front not."""
+    rng = np.random.default_rng(seed)
+    return gg.Graph("regular", n, n * deg, np.arange(n + 1, dtype=np.int32) * deg,
+                    rng.integers(0, n, n * deg).astype(np.int32), rng.integers(1, 100, n * deg).astype(np.uint32), "u32")
+
+
 @pytest.mark.parametrize("n,deg", [(200_000, 4), (130_000, 6)])
 def test_front_too_wide_for_a_cluster(n, deg):
-    """Sparse random graphs begin in one cluster and start over on the grid."""
+    """Sparse graphs begin in one cluster and start over on the grid."""
+    both(regular(n, deg, deg), 3)
     both(gg.random_directed(n, n * deg, 1, 100, seed=deg), 3)
 
 
@@ -232,7 +240,7 @@ def test_layout_of_another_threshold():
 def test_noalloc_on_cluster_and_grid():
     """The fixed scratch serves every kernel and size: one cluster, a front
     that outgrows it, the grid with hubs, and the largest vertex count."""
-    for g in (gg.random_directed(200_000, 800_000, 1, 100, seed=4), gg.rmat(16, 16, seed=3),
+    for g in (regular(200_000, 4, 4), gg.rmat(16, 16, seed=3),
               gg.erdos_renyi(50_000, 400_000, 1, 99, seed=3, wtype="f32"),
               gg.random_directed(S.SSSP_NOALLOC_MAX_VERTICES, 6_000_000, 0, 9, seed=6)):
         src = int(gg.giant_sources(g, 1)[0][0])
@@ -300,3 +308,31 @@ def test_served_bursts_and_concurrent_solves():
     for s, d in got[:12]:
         assert_exact(other, s, d)
     [G.close() for G in Gs + [O]]
+
+
+def test_hops_of_a_warp():
+    """Several hops a step: more improved vertices than a warp keeps, breadth
+    first by several levels a step, and a batch of one block per query on a mesh
+    whose bits just fit."""
+    g = gg.grid(700, 3, 1, 3, seed=2)
+    both(g, 900)
+    star = gg.from_edges(4097, [(0, v, 1) for v in range(1, 4)] +
+                         [(v, 4 * v + k, 1 + k % 2) for v in range(1, 1024) for k in range(4)], name="tree")
+    both(star, 0)
+    for g in (gg.grid(500, 333, 1, 9, seed=1), gg.road(300, 200, seed=3)):
+        G = upload(g)
+        lev = torch.empty(G.n, dtype=torch.int32, device="cuda")
+        par = torch.empty(G.n, dtype=torch.int32, device="cuda")
+        G.bfs(77, lev, par)
+        torch.cuda.synchronize()
+        unit = np.ones(g.m, np.uint32)
+        ref = oracle.dijkstra_u32(g.row_ptr, g.col, unit, 77)
+        np.testing.assert_array_equal(lev.cpu().numpy().view(np.uint32), ref)
+        np.testing.assert_array_equal(par.cpu().numpy(), oracle.pred_canonical_u32(g.row_ptr, g.col, unit, 77, ref))
+        G.close()
+    g = gg.grid(600, 560, 1, 100, seed=4)   # 2^19 places: two blocks a query
+    G = upload(g)
+    srcs = (np.arange(160) * 1999).astype(np.int32)
+    d, p = gpu_batch(G, srcs, pred=True)
+    assert_exact_many(g, srcs[::16], d[::16], p[::16])
+    G.close()
