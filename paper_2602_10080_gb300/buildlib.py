@@ -18,7 +18,7 @@ OBJ = os.path.join(HERE, "_build")
 
 SOURCES = ["kernels_u32.cu", "kernels_u32x.cu", "kernels_f32.cu", "kernels_f32x.cu", "sssp_api.cu",
            "sssp_autotune.cu", "sssp_serve.cu", "sssp_noalloc.cu", "wave_kernels.cu", "fan_kernels.cu",
-           "sssp_wave.cu"]
+           "sssp_wave.cu", "sssp_layout.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 FLAGS = ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC", "-Xcompiler", "-fvisibility=hidden",
          "-I", os.path.join(ROOT, "include")]

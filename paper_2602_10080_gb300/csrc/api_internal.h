@@ -67,6 +67,13 @@ struct Graph {
     uint2* adj = nullptr;         // [mv] (col, weight bits)
     int32_t* owner = nullptr;     // [nv - n]
     int2* span = nullptr;         // [n] (begin, end) of a real vertex's arcs in adj (a hub's slices are contiguous)
+    // hubs of symmetric graphs (see check_symmetry): rows are laid out with
+    // their light arcs first (weight bits <= light_w), mid[v] ends them
+    bool symmetric = false;       // every arc has its reverse of equal weight (shown arc by arc)
+    bool light_first = false;     // the current layout's rows are partitioned
+    uint32_t light_w = 0;
+    double light_share = 0.0;     // of the arcs
+    int32_t* mid = nullptr;       // [n] (light_first)
     sssp_features feat{};
     sssp_config defaults{};
     sssp_config tuned{};
@@ -107,6 +114,17 @@ int lane_refs(uint64_t uid, int delta);
 // Makes the graph's layout the one for hub split threshold `split` (caller
 // holds g->mu); SSSP_E_BUSY while a serving lane uses the graph.
 int ensure_layout(Graph* g, int32_t split, cudaStream_t s);
+// The layout (sssp_layout.cu): hubs split into shadow vertices of `split`
+// arcs.  rp0 / adj0 are the validated original arrays (device); on success
+// g->row_ptr / adj / owner describe the layout (rp0 / adj0 are freed when new
+// arrays replaced them), on failure the graph is untouched.
+int build_layout(Graph* g, int32_t* rp0, uint2* adj0, int32_t split, cudaStream_t s);
+// g->span (and g->mid) for the current layout.
+int fill_span(Graph* g, cudaStream_t s);
+// Original arc order from a split layout: row v of rp0 from adj[src_start[v] ..].
+void launch_unsplit(const Graph* g, const int32_t* src_start, const int32_t* rp0, uint2* adj0, cudaStream_t s);
+// Whether the graph is symmetric, for graphs that profit (g->symmetric).
+int check_symmetry(Graph* g, const int32_t* rp0, const uint2* adj0, cudaStream_t s);
 sssp_config prior_config(const Graph* g);   // the feature prior (sssp_autotune.cu)
 int pred_mode_for(const Graph* g);
 int plan_launch(const Graph* g, const sssp_config& cfg, int pred_mode, bool mq, LaunchPlan* out,

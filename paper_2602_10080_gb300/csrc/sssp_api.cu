@@ -228,33 +228,6 @@ __global__ void pack_kernel(const int32_t* col, const uint32_t* w, int64_t m, in
     }
 }
 
-// Shadow layout: vertex v with sfirst[v] >= 0 gets arcs to its shadows
-// sfirst[v] .. sfirst[v] + k - 1 (weight 0), and shadow j owns the arc slice
-// [j * split, (j + 1) * split) of v.  One warp per vertex.
-__global__ void relayout_kernel(const int32_t* rp0, const uint2* adj0, int32_t n, const int32_t* rp1,
-                                const int32_t* sfirst, int32_t split, uint2* adj1) {
-    const int64_t wid = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
-    const uint32_t lane = threadIdx.x & 31u;
-    for (int64_t v = wid; v < n; v += nw) {
-        const int32_t b0 = rp0[v], e0 = rp0[v + 1];
-        const int32_t s0 = sfirst[v];
-        if (s0 < 0) {
-            const int32_t b1 = rp1[v];
-            for (int32_t e = b0 + (int32_t)lane; e < e0; e += 32) adj1[b1 + (e - b0)] = adj0[e];
-        } else {
-            const int32_t k = (e0 - b0 + split - 1) / split;
-            const int32_t b1 = rp1[v];
-            for (int32_t j = (int32_t)lane; j < k; j += 32) adj1[b1 + j] = make_uint2((uint32_t)(s0 + j), 0u);
-            for (int32_t j = 0; j < k; j++) {
-                const int32_t lo = b0 + j * split, hi = min(e0, lo + split);
-                const int32_t d1 = rp1[s0 + j];
-                for (int32_t e = lo + (int32_t)lane; e < hi; e += 32) adj1[d1 + (e - lo)] = adj0[e];
-            }
-        }
-    }
-}
-
 // Table 2 features: sums for degree and weight moments.
 struct FeatAcc {
     double sdeg, sdeg2, sw, sw2;
@@ -894,136 +867,6 @@ int run_queries(Graph* g, const int32_t* srcs_host, const int32_t* srcs_dev, int
     }
 }
 
-// Where the arcs of every real vertex lie: its row, or (a split hub, whose row
-// links its shadows) the shadows' rows, which follow one another.
-__global__ void span_kernel(const int32_t* rp, const uint2* adj, int32_t n, int2* span) {
-    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < n; v += stride) {
-        int32_t b = rp[v], e = rp[v + 1];
-        if (e > b) {
-            const uint32_t first = adj[b].x;
-            if (first >= (uint32_t)n) {
-                const int32_t k = e - b;
-                b = rp[first];
-                e = rp[first + (uint32_t)k];
-            }
-        }
-        span[v] = make_int2(b, e);
-    }
-}
-
-// Builds the device layout with shadow vertices for vertices above `split`
-// arcs.  rp0/adj0 are the validated original arrays (device); on success
-// g->row_ptr / g->adj / g->owner describe the layout (rp0/adj0 are freed
-// when new arrays replaced them).
-static int build_layout(Graph* g, int32_t* rp0, uint2* adj0, int32_t split, cudaStream_t s) {
-    const int32_t n = g->n;
-    std::vector<int32_t> h(n + 1);
-    if (cudaMemcpyAsync(h.data(), rp0, sizeof(int32_t) * (n + 1), cudaMemcpyDeviceToHost, s) != cudaSuccess ||
-        cudaStreamSynchronize(s) != cudaSuccess)
-        return SSSP_E_CUDA;
-    int64_t ns = 0;
-    for (int32_t v = 0; v < n; v++) {
-        int64_t d = h[v + 1] - h[v];
-        if (split > 0 && d > split) ns += (d + split - 1) / split;
-    }
-    if (ns == 0 || (int64_t)n + ns > 2147483647LL || g->m + ns > 2147483647LL) {
-        g->row_ptr = rp0;
-        g->adj = adj0;
-        g->owner = nullptr;
-        g->nv = n;
-        g->mv = g->m;
-        g->split = 0;
-        return SSSP_OK;
-    }
-    const int32_t nv = (int32_t)(n + ns);
-    std::vector<int32_t> rp1((size_t)nv + 1), sfirst(n, -1), owner((size_t)ns);
-    // real vertices first, then the shadows in vertex order
-    int64_t pos = 0;
-    int32_t next_shadow = n;
-    std::vector<int32_t> sdeg;
-    sdeg.reserve((size_t)ns);
-    for (int32_t v = 0; v < n; v++) {
-        rp1[v] = (int32_t)pos;
-        int64_t d = h[v + 1] - h[v];
-        if (split > 0 && d > split) {
-            int32_t k = (int32_t)((d + split - 1) / split);
-            sfirst[v] = next_shadow;
-            for (int32_t j = 0; j < k; j++) {
-                owner[(size_t)(next_shadow - n) + j] = v;
-                sdeg.push_back((int32_t)std::min<int64_t>(split, d - (int64_t)j * split));
-            }
-            next_shadow += k;
-            pos += k;
-        } else {
-            pos += d;
-        }
-    }
-    for (int64_t i = 0; i < ns; i++) {
-        rp1[(size_t)n + i] = (int32_t)pos;
-        pos += sdeg[(size_t)i];
-    }
-    rp1[nv] = (int32_t)pos;
-    const int64_t mv = pos;
-    int32_t *d_rp1 = nullptr, *d_sfirst = nullptr, *d_owner = nullptr;
-    uint2* d_adj1 = nullptr;
-    int rc = SSSP_OK;
-    if (cudaMalloc(&d_rp1, sizeof(int32_t) * ((size_t)nv + 1)) != cudaSuccess ||
-        cudaMalloc(&d_sfirst, sizeof(int32_t) * (size_t)n) != cudaSuccess ||
-        cudaMalloc(&d_owner, sizeof(int32_t) * (size_t)ns) != cudaSuccess ||
-        cudaMalloc(&d_adj1, sizeof(uint2) * (size_t)mv) != cudaSuccess) {
-        cudaGetLastError();
-        rc = SSSP_E_NOMEM;
-    }
-    if (rc == SSSP_OK) {
-        cudaMemcpyAsync(d_rp1, rp1.data(), sizeof(int32_t) * ((size_t)nv + 1), cudaMemcpyHostToDevice, s);
-        cudaMemcpyAsync(d_sfirst, sfirst.data(), sizeof(int32_t) * (size_t)n, cudaMemcpyHostToDevice, s);
-        cudaMemcpyAsync(d_owner, owner.data(), sizeof(int32_t) * (size_t)ns, cudaMemcpyHostToDevice, s);
-        relayout_kernel<<<g->sms * 8, 256, 0, s>>>(rp0, adj0, n, d_rp1, d_sfirst, split, d_adj1);
-        if (cudaStreamSynchronize(s) != cudaSuccess) rc = SSSP_E_CUDA;
-    }
-    cudaFree(d_sfirst);
-    if (rc != SSSP_OK) {
-        cudaFree(d_rp1);
-        cudaFree(d_owner);
-        cudaFree(d_adj1);
-        return rc;
-    }
-    cudaFree(rp0);
-    cudaFree(adj0);
-    g->row_ptr = d_rp1;
-    g->adj = d_adj1;
-    g->owner = d_owner;
-    g->nv = nv;
-    g->mv = mv;
-    g->split = split;
-    return SSSP_OK;
-}
-
-// g->span for the current layout.
-static int fill_span(Graph* g, cudaStream_t s) {
-    if (!g->span && cudaMalloc((void**)&g->span, sizeof(int2) * (size_t)g->n) != cudaSuccess) {
-        cudaGetLastError();
-        return SSSP_E_NOMEM;
-    }
-    span_kernel<<<grid_for((size_t)g->n, g->sms), 256, 0, s>>>(g->row_ptr, g->adj, g->n, g->span);
-    return cuda_status(cudaStreamSynchronize(s));
-}
-
-// Original arc order from a shadow layout: the arcs of vertex v are its own
-// row, or (a split hub) the rows of its shadows, which are consecutive.  One
-// warp per vertex copies them to their place in the original CSR.
-__global__ void unsplit_kernel(const uint2* adj1, const int32_t* src_start, const int32_t* rp0, int32_t n,
-                               uint2* adj0) {
-    const int64_t wid = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
-    const uint32_t lane = threadIdx.x & 31u;
-    for (int64_t v = wid; v < n; v += nw) {
-        const int32_t b = rp0[v], e = rp0[v + 1], src = src_start[v];
-        for (int32_t i = (int32_t)lane; i < e - b; i += 32) adj0[b + i] = adj1[src + i];
-    }
-}
-
 int lane_refs(uint64_t uid, int delta) {
     static std::mutex mu;
     static std::vector<std::pair<uint64_t, int>> refs;
@@ -1098,7 +941,7 @@ int ensure_layout(Graph* g, int32_t split, cudaStream_t s) {
         }
         cudaMemcpyAsync(rp0, h0.data(), sizeof(int32_t) * ((size_t)n + 1), cudaMemcpyHostToDevice, s);
         cudaMemcpyAsync(d_src, src.data(), sizeof(int32_t) * (size_t)n, cudaMemcpyHostToDevice, s);
-        unsplit_kernel<<<g->sms * 8, 256, 0, s>>>(g->adj, d_src, rp0, n, adj0);
+        launch_unsplit(g, d_src, rp0, adj0, s);
         const cudaError_t e = cudaStreamSynchronize(s);
         cudaFree(d_src);
         if (e != cudaSuccess) {
@@ -1242,6 +1085,8 @@ extern "C" int sssp_graph_create(const int32_t* row_ptr, const int32_t* col_idx,
         // split threshold gives the initial layout
         g->defaults = prior_config(g);
         const int32_t split0 = g->defaults.split_arcs ? g->defaults.split_arcs : kDefaultSplit;
+        rc = check_symmetry(g, rp0, adj0, s);
+        if (rc) break;
         rc = build_layout(g, rp0, adj0, split0, s);
         g->layout_req = split0;
         f.shadows = g->nv - g->n;
@@ -1263,6 +1108,7 @@ extern "C" int sssp_graph_create(const int32_t* row_ptr, const int32_t* col_idx,
         cudaFree(g->adj);
         cudaFree(g->owner);
         cudaFree(g->span);
+        cudaFree(g->mid);
         delete g;
         return rc;
     }
@@ -1281,6 +1127,7 @@ extern "C" int sssp_graph_destroy(sssp_graph* gh) {
         cudaFree(g->adj);
         cudaFree(g->owner);
         cudaFree(g->span);
+        cudaFree(g->mid);
     }
     delete g;
     return SSSP_OK;

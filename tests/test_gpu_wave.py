@@ -336,3 +336,25 @@ def test_hops_of_a_warp():
     d, p = gpu_batch(G, srcs, pred=True)
     assert_exact_many(g, srcs[::16], d[::16], p[::16])
     G.close()
+
+
+@pytest.mark.parametrize("n", [1, 2047, 2048, 2049, 6000])
+def test_layout_around_tiles(n):
+    """Split layouts at the edges of the scan's tiles, with hubs at the ends,
+    rows above and below the block's limit, and thresholds back and forth."""
+    deg = np.arange(n) % 7
+    deg[[0, n // 2, n - 1]] = 33, 2049, 700
+    if n == 1:
+        deg[:] = 0
+    rp = np.concatenate([[0], np.cumsum(deg)]).astype(np.int32)
+    m = int(rp[-1])
+    rng = np.random.default_rng(n)
+    g = gg.Graph("rows", n, m, rp, rng.integers(0, n, m).astype(np.int32), rng.integers(1, 50, m).astype(np.uint32), "u32")
+    G = upload(g)
+    for split in (32, 100, 2048, 1 << 20, 33):
+        d, p = gpu_solve(G, n // 2, config=cfg(split_arcs=split))
+        assert_exact(g, n // 2, d, p)
+        assert G.features()["shadows"] == int(sum(-(-int(x) // split) for x in deg if x > split))
+        d, p = gpu_solve(G, n // 2)
+        assert_exact(g, n // 2, d, p)
+    G.close()
