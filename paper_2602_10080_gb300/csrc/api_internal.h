@@ -158,7 +158,8 @@ int run_queries(Graph* g, const int32_t* srcs_host, const int32_t* srcs_dev, int
                 sssp_stats* st_out, bool unit = false, const Sampling* samp = nullptr);
 
 inline WaveGraph wave_graph(const Graph* g) {
-    return WaveGraph{g->n, g->m, g->feat.avg_w, g->feat.max_deg, g->sms, g->wide.load()};
+    return WaveGraph{g->n, g->m, g->feat.avg_w, g->feat.max_deg, g->sms, g->wide.load(),
+                     g->light_first && g->light_share >= 0.02 && g->light_share <= 0.4};
 }
 // The wavefront kernels (sssp_wave.cu), for calls that leave the configuration
 // to the library.  kWaveNotRun: the graph or the call is not for them.

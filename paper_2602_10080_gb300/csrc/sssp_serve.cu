@@ -936,6 +936,10 @@ int express_launch(sssp_server* s, Lane* L) {
         } else {
             P.span = g->span;
             P.adj = g->adj;
+            if (plan.core) {
+                P.mid = g->mid;
+                P.light_w = g->light_w;
+            }
             P.srcs = grid ? nullptr : J->srcs;
             P.src0 = J->srcs_h[0];
             P.work = pred ? (void*)J->work : (void*)J->out_d;

@@ -69,14 +69,15 @@ bool plan_wave(const WaveGraph& g, int32_t nq, int pred_mode, WavePlan* w) {
         }
         w->kind = kWholeGrid;
         if (hubs) {
-            // power law: the arcs of the core are the work, and the order
-            // decides how often they are relaxed, on the large graphs; on the
-            // small ones the number of steps counts.  us at widths 1/4, 1/2
-            // and 1 of the above: R-MAT-22 2380, 1800, 1920; R-MAT-18 757,
-            // 547, 411; R-MAT-16 609, 414, 329
-            const bool large = g.m > (1 << 25);
-            w->delta *= large ? 0.5 : 1.0;
-            w->front = large ? 1u : 256u;
+            // power law: the arcs of the core are the work.  Without them the
+            // steps count on all but the largest graphs, us with (without) the
+            // core's heavy arcs: R-MAT-22 675 (1786), at width 1 773, 1/4 710;
+            // R-MAT-20 344 (920), a front of 256 363; R-MAT-18 190 (378), a front
+            // of 1 202; R-MAT-16 155 (303); R-MAT-19 f32 312 (626).  A graph whose
+            // core does not settle in time (weights up to 15) loses 8%
+            w->core = g.core;
+            w->delta *= g.m > (1 << 25) ? 0.5 : 1.0;
+            w->front = g.m > (w->core ? 1 << 24 : 1 << 25) ? 1u : 256u;
             // a larger slice saves listing, a smaller one spreads better: R-MAT-22
             // (and BFS) 2.87 (0.90) ms with 256 arcs, 2.51 (0.79) with 512
             w->hub_deg = 512;
@@ -132,6 +133,10 @@ size_t wave_params(const WavePlan& w, const WaveGraph& g, bool f32, bool unit, W
     } else if (f32) p->delta = __float_as_uint_host((float)std::max(1e-30, w.delta));
     else p->delta = (uint32_t)std::min(4.0e9, std::max(1.0, w.delta));
     p->front = w.front;
+    if (w.core && !unit) {
+        p->core_deg = w.core_deg;
+        p->arcs = g.m;
+    }
     p->wide = w.wide;
     p->unit = unit ? 1 : 0;
     if (!unit) p->hops = w.hops;
@@ -280,6 +285,10 @@ int run_wave(Graph* g, const int32_t* srcs_host, const int32_t* srcs_dev, int32_
         }
         P.span = g->span;
         P.adj = g->adj;
+        if (plan.core && !unit) {
+            P.mid = g->mid;
+            P.light_w = g->light_w;
+        }
         P.src0 = src0;
         P.work = pred_mode ? (void*)ws.d64 : (void*)dd;
         P.dist_out = dd;

@@ -60,6 +60,10 @@ struct WaveParams {
     Ctrl* ctrl;               // error word, finished queries, statistics
     unsigned long long timeout_ns;
     // tide only
+    const int32_t* mid;       // [n] end of a row's light arcs (core search), or null
+    uint32_t light_w;         // weights of light arcs: at most this
+    int32_t core_deg;         // a vertex with as many arcs belongs to the core
+    int64_t arcs;             // of the graph
     uint32_t* bits;           // near[2], far[2]: `words` words each
     uint4* items;             // hub slices, two lists of items_cap: (vertex, distance, first arc, end)
     uint32_t items_cap;
@@ -95,8 +99,13 @@ struct __align__(128) TideSync {
     struct __align__(128) {
         unsigned long long arrived;      // end of the step: near count << 16 | blocks
         uint32_t far;                    // the complement of the smallest far distance
-        uint32_t pad[29];
+        uint32_t core;                   // the complement of the smallest distance that left heavy arcs out
+        uint32_t pad[28];
     } set[4];
+    struct __align__(128) {
+        unsigned long long arcs;         // left out by the core
+        unsigned long long pad[15];
+    } left;
     struct __align__(128) {
         uint32_t count;                  // hub slices listed by the step
         uint32_t arrived;                // blocks that have listed theirs (breadth-first)
@@ -142,7 +151,8 @@ enum WaveMode { kWaveBlock = 0, kWaveCluster = 1, kWaveGrid = 2 };
 
 // HOPS: a warp may have more than one hop a step (compiled out otherwise: with
 // it R-MAT-22 took 8% and R-MAT-13 12% longer at one hop).
-template <int WT, int PRED, int MODE, bool HOPS>
+// CORE: rows may be relaxed without their heavy arcs (see tide_kernel).
+template <int WT, int PRED, int MODE, bool HOPS, bool CORE = false>
 struct Wave {
     using DistT = typename std::conditional<PRED == 0, uint32_t, unsigned long long>::type;
     using A = Arith<WT>;
@@ -157,6 +167,12 @@ struct Wave {
     uint32_t n_relax;          // arcs relaxed by this thread
     uint32_t n_own, own_w;     // entries kept for the next hop, and which half they are in
     bool keep;                 // the warp has another hop in this step
+    uint32_t delta;            // of P, or infinite after the pull
+    // CORE: the smallest distance that left heavy arcs out, so far and in this
+    // step, the arcs that this thread left out in this step, and the bound from
+    // which on distances are of no use
+    uint32_t core, left, left_arcs, bound;
+    bool skip;                 // CORE: heavy arcs of the core are left out
 
     static __device__ __forceinline__ uint32_t dpart(uint32_t w) { return w; }
     static __device__ __forceinline__ uint32_t dpart(unsigned long long w) { return (uint32_t)(w >> 32); }
@@ -196,12 +212,13 @@ struct Wave {
 #pragma unroll
         for (int k = 0; k < K; k++) {
             nd[k] = A::add(du[k], P.unit ? 1u : a[k].y);
+            const bool use = in[k] && (!CORE || nd[k] < bound);
             if (PRED == 0) {
-                upd[k] = imp[k] = in[k] && nd[k] < (uint32_t)c[k];
+                upd[k] = imp[k] = use && nd[k] < (uint32_t)c[k];
             } else {
-                imp[k] = in[k] && nd[k] < dpart(c[k]);
+                imp[k] = use && nd[k] < dpart(c[k]);
                 upd[k] = PRED == 2 ? imp[k]
-                                   : in[k] && (((unsigned long long)nd[k] << 32) | u[k]) < (unsigned long long)c[k];
+                                   : use && (((unsigned long long)nd[k] << 32) | u[k]) < (unsigned long long)c[k];
             }
             ad[k] = bit_addr(nd[k] < T ? near_w : far_w, a[k].x, mask[k]);
         }
@@ -314,6 +331,12 @@ struct Wave {
                 }
             }
         }
+        if (CORE && skip && have && (sp.y - sp.x >= P.core_deg || d >= core)) {
+            const int32_t m = __ldg(P.mid + v);
+            if (m < sp.y) left = min(left, d);
+            left_arcs += (uint32_t)(sp.y - m);
+            sp.y = m;
+        }
         int32_t deg = have ? sp.y - sp.x : 0;
         n_relax += (uint32_t)deg;
         if (P.has_hubs) deg = hub(v, d, sp, deg);
@@ -424,10 +447,84 @@ struct Wave {
     __device__ __forceinline__ int advance(uint32_t near, uint32_t far_low) {
         if (near < P.front && far_low != kInfU32) {
             Told = T;
-            T = near ? wave_raise<WT>(T, P.delta, 0u) : wave_raise<WT>(max(T, far_low), P.delta, far_low);
+            T = near ? wave_raise<WT>(T, delta, 0u) : wave_raise<WT>(max(T, far_low), delta, far_low);
             return 2;
         }
         return near ? 1 : 0;
+    }
+
+    // The same while heavy arcs are left out: the threshold stops at `settled`,
+    // below which distances are final.  3: they are, and the others are to be
+    // pulled.
+    __device__ __forceinline__ int advance_core(uint32_t near, uint32_t far_low, uint32_t settled) {
+        if (core == kInfU32) return advance(near, far_low);
+        if (T >= settled) return near ? 1 : 3;
+        const int what = advance(near, far_low);
+        T = min(T, settled);
+        return what ? what : 3;
+    }
+
+    // Vertex v (distance word cur, arcs sp; deg arcs to look at, all of them
+    // or none) takes the best of its in-neighbours, its own arcs' ends.  The
+    // whole warp is here.  Returns its distance after that.
+    __device__ __forceinline__ uint32_t pull(uint32_t v, DistT cur, int2 sp, int32_t deg) {
+        constexpr uint32_t none = PRED == 0 && WT == 1 ? kInfF32 : kInfU32;
+        const uint32_t lane = lane_id();
+        uint32_t best = none, from = kInfU32;
+        auto offer = [&](uint2 a, DistT c) {
+            const uint32_t du = dpart(c);
+            if (du == none) return;
+            const uint32_t nd = A::add(du, a.y);
+            if (nd < best || (nd == best && a.x < from)) {
+                best = nd;
+                from = a.x;
+            }
+        };
+        const bool by_warp = deg > 64;
+        for (int32_t e = 0; !by_warp && e < deg; e += 4) {
+            uint2 a[4];
+            DistT c[4];
+#pragma unroll
+            for (int k = 0; k < 4; k++) a[k] = ld_arc(P.adj + sp.x + min(e + k, deg - 1));
+#pragma unroll
+            for (int k = 0; k < 4; k++) c[k] = ld_dist(dist + a[k].x);
+#pragma unroll
+            for (int k = 0; k < 4; k++) offer(a[k], c[k]);
+        }
+        uint32_t m = __ballot_sync(kFull, by_warp);
+        while (m) {
+            const int j = __ffs((int)m) - 1;
+            m &= m - 1u;
+            const uint32_t keep_b = best, keep_f = from;
+            const int32_t b = __shfl_sync(kFull, sp.x, j), end = b + __shfl_sync(kFull, deg, j);
+            best = none;
+            from = kInfU32;
+            for (int32_t e = b; e < end; e += 128) {
+                uint2 a[4];
+                DistT c[4];
+#pragma unroll
+                for (int k = 0; k < 4; k++) a[k] = ld_arc(P.adj + min(e + 32 * k + (int32_t)lane, end - 1));
+#pragma unroll
+                for (int k = 0; k < 4; k++) c[k] = ld_dist(dist + a[k].x);
+#pragma unroll
+                for (int k = 0; k < 4; k++) offer(a[k], c[k]);
+            }
+            const uint32_t mb = __reduce_min_sync(kFull, best);
+            const uint32_t mf = __reduce_min_sync(kFull, best == mb ? from : kInfU32);
+            best = (int)lane == j ? mb : keep_b;
+            from = (int)lane == j ? mf : keep_f;
+        }
+        const uint32_t d = dpart(cur);
+        if (deg > 0 && best != none) {
+            if (PRED == 0) {
+                if (best < d) reinterpret_cast<volatile uint32_t*>(dist)[v] = best;
+            } else {
+                const unsigned long long cand = ((unsigned long long)best << 32) | from;
+                if (PRED == 1 ? cand < (unsigned long long)cur : best < d)
+                    reinterpret_cast<volatile unsigned long long*>(dist)[v] = cand;
+            }
+        }
+        return deg > 0 ? min(d, best) : d;
     }
 
     __device__ __forceinline__ void publish(uint32_t improved) const {
@@ -460,7 +557,7 @@ __global__ void __launch_bounds__(1024, 1) wave_kernel(const __grid_constant__ W
     const uint32_t src = (uint32_t)(P.srcs ? P.srcs[q] : P.src0);
     const uint32_t words = (uint32_t)P.words;
     W w{P, reinterpret_cast<DistT*>(P.work) + (size_t)q * (size_t)P.n, &lists[tid >> 5],
-        wave_raise<WT>(0u, P.delta, 0u), 0u, 0u, 0u, 0u, kInfU32, 0u, 0u, 0u, false};
+        wave_raise<WT>(0u, P.delta, 0u), 0u, 0u, 0u, 0u, kInfU32, 0u, 0u, 0u, false, P.delta, kInfU32, kInfU32, 0u, kInfU32, false};
 
     // every distance to infinity but the source's, and its pending bit
     w.init(src, rank * nt + tid, G * nt);
@@ -589,19 +686,32 @@ __device__ __forceinline__ void red_release64(unsigned long long* p, unsigned lo
     asm volatile("red.release.gpu.global.add.u64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
 }
 
-template <int WT, int PRED, bool HOPS>
+// The whole grid on one query.
+//
+// CORE (symmetric graphs with hubs, light arcs first in every row): most arcs
+// belong to hubs that lie close together, and most of those lead to vertices
+// that are nearer by other ways.  So vertices of core_deg arcs or more relax
+// only their light arcs, and, from the first of them on (at distance `core`),
+// all vertices.  What is left out reaches no vertex below core + light_w: up
+// to there the search goes on as ever, and what it finds is final.  Then every
+// other vertex with arcs looks at all its in-neighbours once (its own arcs,
+// reversed), which covers all that was left out, and the search ends among
+// these vertices with all their arcs.  On R-MAT-22 from a source of the giant
+// component 5% of the arcs are below the bound, 12% light, and the other
+// vertices have 4 to 6% of the arcs.
+template <int WT, int PRED, bool HOPS, bool CORE>
 __global__ void __launch_bounds__(1024, 1) tide_kernel(const __grid_constant__ WaveParams P) {
-    using W = Wave<WT, PRED, kWaveGrid, HOPS>;
+    using W = Wave<WT, PRED, kWaveGrid, HOPS, CORE>;
     using DistT = typename W::DistT;
     __shared__ WaveLists<HOPS> lists[32];
-    __shared__ uint32_t s_near[4], s_fmin[4], s_out[4];
+    __shared__ uint32_t s_near[4], s_fmin[4], s_left[4], s_arcs[4], s_out[4];
     const uint32_t tid = threadIdx.x, nt = blockDim.x, lane = tid & 31u;
     const uint32_t gt = blockIdx.x * nt + tid, gn = gridDim.x * nt;
     // consecutive warps of the grid lie in different blocks
     const uint32_t wid = (tid >> 5) * gridDim.x + blockIdx.x, nw = gn >> 5;
     const uint32_t words = (uint32_t)P.words;
     W w{P, reinterpret_cast<DistT*>(P.work), &lists[tid >> 5],
-        wave_raise<WT>(0u, P.delta, 0u), 0u, nullptr, nullptr, 0u, kInfU32, 0u, 0u, 0u, false};
+        wave_raise<WT>(0u, P.delta, 0u), 0u, nullptr, nullptr, 0u, kInfU32, 0u, 0u, 0u, false, P.delta, kInfU32, kInfU32, 0u, kInfU32, false};
     const unsigned long long deadline = gtime() + P.timeout_ns;
 
     w.init((uint32_t)P.src0, gt, gn);
@@ -612,11 +722,13 @@ __global__ void __launch_bounds__(1024, 1) tide_kernel(const __grid_constant__ W
     }
     if (tid < 4u) {
         s_near[tid] = 0u;
-        s_fmin[tid] = kInfU32;
+        s_fmin[tid] = s_left[tid] = kInfU32;
+        s_arcs[tid] = 0u;
     }
+    w.skip = CORE;
 
     // step 0 ends the preparation; the searching steps follow
-    uint32_t cur = 0u, fw = 0u, far_low = kInfU32, n_improved = 0, steps = 0, near = 0u;
+    uint32_t cur = 0u, fw = 0u, far_low = kInfU32, n_improved = 0, steps = 0, near = 0u, settled = kInfU32;
     int what = 1;
     bool ok = true;
     for (;;) {
@@ -630,23 +742,35 @@ __global__ void __launch_bounds__(1024, 1) tide_kernel(const __grid_constant__ W
                 if (imp) atomicAdd(&s_near[set], imp);
                 if (fm != kInfU32) atomicMin(&s_fmin[set], fm);
             }
+            if (CORE && w.skip) {
+                const uint32_t left = __reduce_min_sync(kFull, w.left);
+                const uint32_t arcs = __reduce_add_sync(kFull, w.left_arcs);
+                if (lane == 0 && left != kInfU32) atomicMin(&s_left[set], left);
+                if (lane == 0 && arcs) atomicAdd(&s_arcs[set], arcs);
+            }
         }
         __syncthreads();
         if (tid == 0) {
             const uint32_t z = (steps + 2u) & 3u;
+            if (CORE && s_left[set] != kInfU32) {
+                atomicMax(&P.sync->set[set].core, ~s_left[set]);
+                atomicAdd(&P.sync->left.arcs, (unsigned long long)s_arcs[set]);
+            }
             if (s_fmin[set] != kInfU32) atomicMax(&P.sync->set[set].far, ~s_fmin[set]);
             if (blockIdx.x == 0 && steps) {
                 // nobody touches set s + 2 before the barrier after this one
                 P.sync->set[z].arrived = 0ull;
-                P.sync->set[z].far = P.sync->hub[z].count = P.sync->hub[z].arrived = 0u;
+                P.sync->set[z].far = P.sync->set[z].core = P.sync->hub[z].count = P.sync->hub[z].arrived = 0u;
             }
             red_release64(&P.sync->set[set].arrived, ((unsigned long long)s_near[set] << 16) | 1ull);
             s_near[z] = 0u;
-            s_fmin[z] = kInfU32;
+            s_fmin[z] = s_left[z] = kInfU32;
+            s_arcs[z] = 0u;
             const unsigned long long x = tide_wait(&P.sync->set[set].arrived, gridDim.x, deadline);
             s_out[0] = x ? (uint32_t)min(x >> 16, 0xfffffffeull) : kInfU32;
             s_out[1] = ~ld_relaxed(&P.sync->set[set].far);
             s_out[2] = ld_relaxed(&P.sync->hub[set].count);
+            if (CORE) s_out[3] = ~ld_relaxed(&P.sync->set[set].core);
         }
         __syncthreads();
         near = s_out[0];
@@ -659,12 +783,62 @@ __global__ void __launch_bounds__(1024, 1) tide_kernel(const __grid_constant__ W
             near = 1u;
         } else {
             far_low = scanned ? s_out[1] : min(far_low, s_out[1]);
-            what = w.advance(near + items, far_low);
+            if (CORE && w.skip) {
+                w.core = min(w.core, s_out[3]);
+                w.bound = settled = w.core != kInfU32 ? Arith<WT>::add(w.core, P.light_w) : kInfU32;
+                what = w.advance_core(near + items, far_low, settled);
+            } else {
+                what = w.advance(near + items, far_low);
+            }
             if (!what) break;
         }
         const uint32_t prev = set;
         steps++;
         const uint32_t now = steps & 3u;
+        if (CORE && what == 3) {
+            // nobody waits below `settled`: the others pull, and wait.  Where
+            // the core has not settled yet (less than half of the arcs left
+            // out) pulling would cost more than relaxing everything again.
+            const bool pulls = ld_relaxed64(&P.sync->left.arcs) * 2ull >= (unsigned long long)P.arcs;
+            w.skip = false;
+            w.bound = kInfU32;
+            // little is left after the pull: no order among it any more
+            if (pulls) w.delta = WT == 1 ? kInfF32 : kInfU32;
+            w.near_w = P.bits + (size_t)cur * words;
+            w.far_w = P.bits + (size_t)(2u + fw) * words;
+            w.n_imp = 0u;
+            w.fmin = kInfU32;
+            uint32_t v = wid * 32u + lane;
+            DistT dv_next = 0;
+            int2 sp_next = make_int2(0, 0);
+            auto fetch = [&](uint32_t u) {
+                if (u < (uint32_t)P.n) {
+                    dv_next = ld_dist(w.dist + u);
+                    sp_next = __ldg(P.span + u);
+                }
+            };
+            fetch(v);
+            for (uint32_t base = wid * 32u; base < (uint32_t)P.n; base += nw * 32u, v += nw * 32u) {
+                const bool in = v < (uint32_t)P.n;
+                const DistT dv = dv_next;
+                const int2 sp = sp_next;
+                fetch(v + nw * 32u);
+                const int32_t deg = in ? sp.y - sp.x : 0;
+                const int32_t look = pulls && W::dpart(dv) >= settled ? deg : 0;
+                if (!__any_sync(kFull, pulls ? look > 0 : deg > 0)) continue;
+                w.n_relax += (uint32_t)look;
+                const uint32_t d = w.pull(v, dv, sp, look);
+                // (a vertex with one arc has nobody to tell but its source)
+                if ((pulls ? look > 1 : deg > 0) && d != (PRED == 0 && WT == 1 ? kInfF32 : kInfU32)) {
+                    uint32_t mask;
+                    uint32_t* const a = w.bit_addr(d < w.T ? w.near_w : w.far_w, v, mask);
+                    w.red_or(a, mask);
+                    if (d < w.T) w.n_imp++;
+                    else w.fmin = min(w.fmin, d);
+                }
+            }
+            continue;
+        }
         const bool scan_far = what == 2;
         uint32_t* near_r = P.bits + (size_t)cur * words;
         uint32_t* far_r = P.bits + (size_t)(2u + fw) * words;
@@ -673,7 +847,8 @@ __global__ void __launch_bounds__(1024, 1) tide_kernel(const __grid_constant__ W
         w.near_w = P.bits + (size_t)cur * words;
         w.far_w = P.bits + (size_t)(2u + fw) * words;
         w.n_imp = 0u;
-        w.fmin = kInfU32;
+        w.fmin = w.left = kInfU32;
+        w.left_arcs = 0u;
         uint4* items_w = P.items + (size_t)(steps & 1u) * P.items_cap;
         w.sweep(
             wid * 32u, nw * 32u, words,

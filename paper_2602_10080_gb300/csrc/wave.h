@@ -22,6 +22,8 @@ struct WavePlan {
     int32_t hops = 1;
     int32_t hub_deg = 256;
     uint32_t wide = kInfU32;
+    bool core = false;     // tide: leave the core's heavy arcs out (WaveGraph::core)
+    int32_t core_deg = 256;
 };
 
 // What the plan depends on.  wide: a solve found the front too wide for one
@@ -32,6 +34,7 @@ struct WaveGraph {
     double avg_w, max_deg;
     int sms;
     bool wide;
+    bool core;             // symmetric, hubs, rows with their light arcs (a fair share of all) first
 };
 
 constexpr int kTideLogWords = 17;               // the grid kernel spreads the places over at least 2^17 words

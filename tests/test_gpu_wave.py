@@ -358,3 +358,71 @@ def test_layout_around_tiles(n):
         d, p = gpu_solve(G, n // 2)
         assert_exact(g, n // 2, d, p)
     G.close()
+
+
+def symmetric(n, u, v, w, wtype="u32"):
+    key, at = np.unique(np.concatenate([u * n + v, v * n + u]), return_index=True)
+    w2 = np.concatenate([w, w])[at]
+    # one weight for both directions of a repeated pair: that of the smaller arc
+    lo, hi = np.minimum(key // n, key % n), np.maximum(key // n, key % n)
+    order = np.lexsort((key, hi, lo))
+    first = np.concatenate([[True], (lo[order][1:] != lo[order][:-1]) | (hi[order][1:] != hi[order][:-1])])
+    w2[order] = w2[order][np.flatnonzero(first)[np.cumsum(first) - 1]]
+    rp = np.concatenate([[0], np.cumsum(np.bincount(key // n, minlength=n))]).astype(np.int32)
+    return gg.Graph("sym", n, len(key), rp, (key % n).astype(np.int32), w2, wtype)
+
+
+def hubs_and_leaves(n, hubs, arcs, lo, hi, seed, wtype="u32"):
+    """A few hubs that reach everything, leaves and self-loops, weights lo..hi."""
+    rng = np.random.default_rng(seed)
+    u = np.concatenate([rng.integers(0, hubs, arcs), np.arange(n), np.arange(0, n, 97)])
+    v = np.concatenate([rng.integers(0, n, arcs), rng.integers(0, n, n), np.arange(0, n, 97)])
+    w = rng.integers(lo, hi + 1, len(u))
+    w = (w / 64.0).astype(np.float32) if wtype == "f32" else w.astype(np.uint32)
+    return symmetric(n, u.astype(np.int64), v.astype(np.int64), w, wtype)
+
+
+@pytest.mark.parametrize("wtype", ["u32", "f32"])
+@pytest.mark.parametrize("lo,hi", [(1, 255), (0, 255), (1, 9), (7, 7), (200, 255)])
+def test_core_and_pull(wtype, lo, hi):
+    """Symmetric graphs with hubs: heavy arcs left out and pulled, or relaxed
+    after all where the core does not settle; no light arcs; sources in the
+    core, at its edge, and alone."""
+    g = hubs_and_leaves(60_000, 40, 400_000, lo, hi, seed=hi + lo, wtype=wtype)
+    G = upload(g)
+    deg = np.diff(g.row_ptr)
+    for src in (0, int(np.argmax(deg)), int(np.argmin(deg)), 59_999):
+        d, p = gpu_solve(G, src, pred=True)
+        assert_exact(g, src, d, p)
+        d2, _ = gpu_solve(G, src, pred=False)
+        np.testing.assert_array_equal(d2, d)
+    G.close()
+
+
+def test_core_needs_symmetry():
+    """One arc, one weight or one order that spoils the symmetry, parallel arcs,
+    and lengths that saturate: the same answers as ever."""
+    g = hubs_and_leaves(50_000, 30, 400_000, 1, 255, seed=1)
+    src = 12345
+    variants = []
+    for k in range(5):
+        rp, col, w = g.row_ptr.copy(), g.col.copy(), g.w.copy()
+        e = int(rp[40_000])
+        if k == 0:
+            w[e] = 1 + (int(w[e]) + 7) % 255
+        elif k == 1:
+            col[e] = (int(col[e]) + 1) % g.n
+        elif k == 2:
+            hub = int(np.argmax(np.diff(rp)))
+            a, b = int(rp[hub]), int(rp[hub + 1])
+            col[a:b], w[a:b] = col[a:b][::-1].copy(), w[a:b][::-1].copy()
+        elif k == 3:
+            col[e + 1], w[e + 1] = col[e], w[e]
+        else:
+            w[:] = w * 0x1000000 + 0x00FFFFFF
+        variants.append(gg.Graph("v%d" % k, g.n, g.m, rp, col, w, "u32"))
+    for h in variants:
+        G = upload(h)
+        d, p = gpu_solve(G, src, pred=True)
+        assert_exact(h, src, d, p)
+        G.close()
