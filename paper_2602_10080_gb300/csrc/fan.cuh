@@ -9,27 +9,43 @@
 // word whose bits are the queries that improved it.
 //
 // The grid steps over the waiting vertices in Bellman-Ford order: the queries
-// are then aligned by hops.  256 R-MAT-20 queries visit every arc 5.4 times
-// per group with three quarters of the lanes at work; ordered by distance a
-// query relaxes an arc 1.2 times instead of 4, but the queries reach a vertex
-// at different steps, and the visits are as many (7 to 8 in simulation).
+// are then aligned by hops.  Ordered by distance a query relaxes an arc 1.2
+// times instead of 4, but the queries reach a vertex at different steps, and
+// the visits are as many (R-MAT-20, 32 queries, all arcs: 5.4 visits an arc by
+// hops, 7 to 8 by distance in simulation).
 //
 // Per step: list the waiting vertices (long rows in slices, short rows
-// whole), grid barrier, relax the lists, grid barrier.  GB300: 256 queries on
-// R-MAT-20 137.7 ms through the queues, 45.1 here (30 G visits of 32 queries
-// a second); 64 on R-MAT-18 f32 21.1 -> 5.5 ms; 40 on G(200K, 2M) with
-// predecessors 12.8 -> 6.3 ms.  It is bound by instructions and their
-// latency (59% of the issue slots, 39% of the L1 wavefronts, 14% of L2): 1024
-// threads of 64 registers beat 768 of 80 (52.1 ms).
+// whole), grid barrier, relax the lists, grid barrier.
+//
+// CORE (symmetric graphs with hubs, as in tide_kernel): each query leaves out
+// the heavy arcs of the core's vertices, and of all others from the distance
+// on where it met the core, and stops at that distance plus the light bound.
+// When nobody waits, the vertices beyond pull over their own rows and the
+// search ends among them.  In simulation, 32 queries on R-MAT-18: 0.4 visits an
+// arc in the core, 0.2 in the pull.
+//
+// GB300, ms: 256 queries on R-MAT-20 137.7 through the queues, 43.6 here with
+// all arcs, 13.8 with the core search; 64 on R-MAT-18 f32 21.1, 5.4, 2.3; 40 on
+// R-MAT-17 with predecessors 2.2, 1.4 (all arcs, core); 40 on G(200K, 2M) with
+// predecessors 12.8 through the queues, 5.5 here.  With all arcs it is bound by
+// instructions and their latency (59% of the issue slots, 39% of the L1
+// wavefronts, 14% of L2; 30 G visits of 32 queries a second): 1024 threads of
+// 64 registers beat 768 of 80.  The core search is bound by the latency of its
+// 18 steps, each of a few items per warp.
 #pragma once
 
 #include "wave.cuh"
 
 namespace sssp {
 
-constexpr int32_t kFanShort = 8;      // rows up to this long are relaxed packed together, longer ones in slices
+// Rows up to kFanShort arcs are relaxed kFanRows at a time, longer ones in
+// slices of kFanChunk.  64 queries on R-MAT-20, us: slices of 128 3630, 64 3430,
+// 32 3740; at 128, 8 rows of up to 8 arcs 4230, 16 4060, 32 rows of up to 16 4270.
+constexpr int32_t kFanShort = 16;
+constexpr uint32_t kFanRows = 8;
+constexpr int32_t kFanChunk = 64;
 constexpr int kFanThreads = 1024;
-constexpr int32_t kFanChunk = 128;    // arcs of a slice
+constexpr int32_t kFanCoreArcs = 128; // a vertex with as many arcs belongs to the core
 constexpr int32_t kFanMaxVertices = 1 << 25;   // rows are addressed by 32-bit byte offsets
 
 struct FanSync {
@@ -43,11 +59,15 @@ struct FanSync {
         uint32_t claimed;             // slices and batches of short rows taken by warps
         uint32_t pad1[31];
     } set[4];
+    uint32_t core[32];                // per query: the complement of the smallest distance that left heavy arcs out
 };
 
 struct FanParams {
     const int2* span;
     const uint2* adj;
+    const int32_t* mid;       // [n] end of a row's light arcs (core search), or null
+    uint32_t light_w;         // their largest weight
+    int32_t core_deg;         // kFanCoreArcs
     int32_t n;
     int32_t nq;               // queries of this group (1..32)
     const int32_t* srcs;      // [nq]
@@ -56,24 +76,32 @@ struct FanParams {
     uint32_t* wait;           // [2][places]: queries that improved the vertex at place v * hash & mask
     uint32_t mask;
     uint4* slices;            // (vertex, queries, first arc, end)
-    uint2* rows;              // short rows: (vertex, queries)
+    uint4* rows;              // the same of short rows
     FanSync* sync;
     Ctrl* ctrl;
     unsigned long long timeout_ns;
 };
 
-// How an arc is used: to relax it, or (distances final) to find the tight ones.
-enum FanPass { kFanRelax = 0, kFanTight = 1 };
+// How an arc is used: to relax it, (distances final) to find the tight ones,
+// to relax it while the core leaves heavy arcs out, or to pull over it, from
+// its end to the row's vertex.
+enum FanPass { kFanRelax = 0, kFanTight = 1, kFanCore = 2, kFanPull = 3 };
 
 template <int WT, int PASS>
 struct Fan {
     const FanParams& P;
     uint32_t* wait_w;
     uint32_t lane;
-
-    __device__ __forceinline__ Fan(const FanParams& p, uint32_t* w) : P(p), wait_w(w), lane(lane_id()) {}
+    uint32_t core, bound;     // this lane's query: where heavy arcs are left out from, and up to where that changes nothing
 
     static constexpr uint32_t kInf = WT == 1 ? kInfF32 : kInfU32;
+
+    __device__ __forceinline__ Fan(const FanParams& p, uint32_t* w) : P(p), wait_w(w), lane(lane_id()) {
+        if (PASS == kFanCore || PASS == kFanPull) {
+            core = ~__ldcg(P.sync->core + lane);
+            bound = core == kInfU32 ? kInf : Arith<WT>::add(core, P.light_w);
+        }
+    }
 
     // du (+) w: for whole weights du + min(w, cap) with cap = the largest
     // length - du, which saturates in two instructions (0 from an infinite du)
@@ -104,7 +132,9 @@ struct Fan {
 #pragma unroll
         for (int k = 0; k < 8; k++) {
             const uint2 d = du(k);
-            const uint32_t nd = add(d.x, d.y, __shfl_sync(kFull, a.y, j0 + k));
+            const uint32_t w = __shfl_sync(kFull, a.y, j0 + k);
+            const uint32_t nd = PASS == kFanPull ? add(cur[k], cap(cur[k]), w) : add(d.x, d.y, w);
+            if (PASS == kFanPull) off[k] = at(__shfl_sync(kFull, u, j0 + k));
             if (PASS == kFanTight) {
                 const uint32_t uk = __shfl_sync(kFull, u, j0 + k);
                 if (d.x != kInfU32 && nd == cur[k]) red_min(word(P.pred, off[k]), uk);
@@ -115,27 +145,51 @@ struct Fan {
                     "setp.lt.u32 p, %2, %3;\n\t"
                     "@p red.relaxed.gpu.global.min.u32 [%1], %2;\n\t"
                     "vote.sync.ballot.b32 %0, p, 0xffffffff;\n\t}"
-                    : "=r"(b) : "l"(word(P.dist, off[k])), "r"(nd), "r"(cur[k]) : "memory");
+                    : "=r"(b) : "l"(word(P.dist, off[k])), "r"(nd),
+                      "r"(PASS == kFanPull ? d.x : PASS == kFanCore ? min(cur[k], bound) : cur[k]) : "memory");
                 if (lane == j0 + k) won = b;
             }
         }
     }
     __device__ __forceinline__ void wake(uint32_t v, uint32_t won) const {
-        if (PASS == kFanRelax && won) red_or_global(wait_w + ((v * kWaveHash) & P.mask), won);
+        if (PASS != kFanTight && won) red_or_global(wait_w + ((v * kWaveHash) & P.mask), won);
     }
 
     // A slice of one row: its arcs 32 at a time, one per lane, the next 32 on
     // their way meanwhile.  Lanes past the end hold the last arc again: to
     // relax it twice changes nothing.
     __device__ __forceinline__ void slice(uint4 it) const {
-        uint2 next = ld_arc(P.adj + min(it.z + lane, it.w - 1u));
+        const uint32_t end = it.w;
+        uint2 next = ld_arc(P.adj + min(it.z + lane, end - 1u));
         uint32_t d = __ldcg(word(P.dist, at(it.x)));
-        if (!((it.y >> lane) & 1u)) d = kInf;
+        const bool on = (it.y >> lane) & 1u;
+        if (PASS == kFanPull) {
+            uint32_t best = kInf;
+            for (uint32_t e = it.z; e < end; e += 32u) {
+                const uint32_t cnt = min(32u, end - e);
+                const uint2 a = next;
+                next = ld_arc(P.adj + min(e + 32u + lane, end - 1u));
+                for (uint32_t j0 = 0; j0 < cnt; j0 += 8u) {
+                    uint32_t c[8];
+#pragma unroll
+                    for (int k = 0; k < 8; k++) c[k] = __ldcg(word(P.dist, at(__shfl_sync(kFull, a.x, j0 + k))));
+#pragma unroll
+                    for (int k = 0; k < 8; k++)
+                        best = min(best, add(c[k], cap(c[k]), __shfl_sync(kFull, a.y, j0 + k)));
+                }
+            }
+            const bool better = on && best < d;
+            if (better) red_min(word(P.dist, at(it.x)), best);
+            const uint32_t won = __ballot_sync(kFull, better);
+            if (lane == 0) wake(it.x, won);
+            return;
+        }
+        if (!on) d = kInf;
         const uint2 from = make_uint2(d, cap(d));
-        for (uint32_t e = it.z; e < it.w; e += 32u) {
-            const uint32_t cnt = min(32u, it.w - e);
+        for (uint32_t e = it.z; e < end; e += 32u) {
+            const uint32_t cnt = min(32u, end - e);
             const uint2 a = next;
-            next = ld_arc(P.adj + min(e + 32u + lane, it.w - 1u));
+            next = ld_arc(P.adj + min(e + 32u + lane, end - 1u));
             uint32_t won = 0u;
             for (uint32_t j0 = 0; j0 < cnt; j0 += 8u) use8(a, it.x, [&](int) { return from; }, j0, won);
             wake(a.x, won);
@@ -160,6 +214,7 @@ struct Fan {
                 if (__shfl_sync(kFull, ex, i + s) <= g) i += s;
             const int32_t arc = __shfl_sync(kFull, begin, i) + (g - __shfl_sync(kFull, ex, i));
             const uint32_t u = __shfl_sync(kFull, v, i), mu = __shfl_sync(kFull, m, i);
+            const int32_t row_arcs = PASS == kFanPull ? __shfl_sync(kFull, deg, i) : 0;
             const uint2 a = ld_arc(P.adj + arc);
             const uint32_t cnt = (uint32_t)min(32, total - g0);
             uint32_t won = 0u;
@@ -169,22 +224,23 @@ struct Fan {
                 for (uint32_t k = 0; k < 8u; k++) {
                     const uint32_t uk = __shfl_sync(kFull, u, j0 + k), mk = __shfl_sync(kFull, mu, j0 + k);
                     du[k] = __ldcg(word(P.dist, at(uk)));
-                    if (!((mk >> lane) & 1u)) du[k] = kInf;
+                    if (!((mk >> lane) & 1u)) du[k] = PASS == kFanPull ? 0u : kInf;
                 }
                 use8(a, u, [&](int k) { return make_uint2(du[k], cap(du[k])); }, j0, won);
             }
-            wake(a.x, won);
+            if (PASS != kFanPull) wake(a.x, won);
+            else if (row_arcs > 1) wake(u, won);
         }
     }
 
-    // The step's lists: slices, then the short rows 32 at a time.  The first
-    // three quarters are dealt out, the rest claimed one by one (one counter
+    // The step's lists: slices, then the short rows kFanRows at a time.  The first
+    // seven eighths are dealt out, the rest claimed one by one (one counter
     // gives a claim every nanosecond: with every slice claimed, a step on
     // G(200K, 2M) was bound by it).  While a slice is relaxed, the next one is
     // on its way and the claim after that too.
     __device__ __forceinline__ void work(uint32_t slices, uint32_t rows_n, uint32_t wid, uint32_t warps,
                                          uint32_t* claimed) const {
-        const uint32_t all = slices + (rows_n + 31u) / 32u, dealt = all / 4u * 3u / warps * warps;
+        const uint32_t all = slices + (rows_n + kFanRows - 1u) / kFanRows, dealt = all / 8u * 7u / warps * warps;
         uint32_t ahead = 0u;
         auto after = [&](uint32_t i) {   // the item after i (dealt ones first)
             if (i + warps < dealt) return i + warps;
@@ -192,24 +248,19 @@ struct Fan {
             if (lane == 0) ahead = atomicAdd(claimed, 1u);
             return dealt + c;
         };
+        auto fetch = [&](uint32_t i) {
+            if (i < slices) return __ldcg(P.slices + i);
+            const uint32_t r = (i - slices) * kFanRows + lane;
+            return i < all && lane < kFanRows && r < rows_n ? __ldcg(P.rows + r) : make_uint4(0u, 0u, 0u, 0u);
+        };
         if (lane == 0) ahead = atomicAdd(claimed, 1u);
         uint32_t i = wid < dealt ? wid : after(dealt);
-        uint4 it = i < slices ? __ldcg(P.slices + i) : make_uint4(0u, 0u, 0u, 0u);
+        uint4 it = fetch(i);
         while (i < all) {
             const uint32_t i1 = after(i);
-            const uint4 it1 = i1 < slices ? __ldcg(P.slices + i1) : make_uint4(0u, 0u, 0u, 0u);
-            if (i < slices) {
-                slice(it);
-            } else {
-                const uint32_t r = (i - slices) * 32u + lane;
-                uint2 x = make_uint2(0u, 0u);
-                int2 sp = make_int2(0, 0);
-                if (r < rows_n) {
-                    x = __ldcg(P.rows + r);
-                    sp = __ldg(P.span + x.x);
-                }
-                rows(x.x, x.y, sp.x, sp.y - sp.x);
-            }
+            const uint4 it1 = fetch(i1);
+            if (i < slices) slice(it);
+            else rows(it.x, it.y, (int32_t)it.z, (int32_t)(it.w - it.z));
             i = i1;
             it = it1;
         }
@@ -231,7 +282,7 @@ __device__ __forceinline__ bool fan_barrier(FanSync* s, uint32_t target, unsigne
     return __syncthreads_and(ok) != 0;
 }
 
-template <int WT>
+template <int WT, bool CORE>
 __global__ void __launch_bounds__(kFanThreads, 1) fan_kernel(const __grid_constant__ FanParams P) {
     const uint32_t tid = threadIdx.x, lane = tid & 31u, gt = blockIdx.x * blockDim.x + tid;
     const uint32_t gn = gridDim.x * blockDim.x, wid = (tid >> 5) * gridDim.x + blockIdx.x, nw = gn >> 5;
@@ -259,7 +310,7 @@ __global__ void __launch_bounds__(kFanThreads, 1) fan_kernel(const __grid_consta
     ok = ok && fan_barrier(P.sync, arrivals += gridDim.x, deadline);
 
     uint32_t step = 0u;
-    bool tight = false;
+    FanPass pass = CORE ? kFanCore : kFanRelax;
     while (ok) {
         const uint32_t set = step & 3u;
         uint32_t* wait_r = P.wait + (size_t)(step & 1u) * places;
@@ -270,13 +321,59 @@ __global__ void __launch_bounds__(kFanThreads, 1) fan_kernel(const __grid_consta
             uint32_t m = 0u;
             int2 sp = make_int2(0, 0);
             if (base + lane < places) {
-                if (tight) {
+                if (pass == kFanTight || pass == kFanPull) {
                     if (v < (uint32_t)P.n) m = kFull;
                 } else {
                     m = __ldcg(wait_r + base + lane);
                     if (m) wait_r[base + lane] = 0u;
                 }
                 if (m) sp = __ldg(P.span + v);
+            }
+            if (CORE && (pass == kFanCore || pass == kFanPull)) {
+                // Eight rows at a time.  Core: the queries that wait below
+                // their bound, and whether one of them is not at the core yet
+                // and relaxes all arcs.  Pull: those that have not settled the
+                // vertex; those that know a way there wait with it, as it has
+                // relaxed nothing yet.
+                const Fan<WT, kFanCore> f(P, nullptr);
+                const int32_t deg = sp.y - sp.x;
+                const bool has = deg > 0, hub = deg >= P.core_deg;
+                const int32_t mid = has && pass == kFanCore ? __ldg(P.mid + v) : sp.y;
+                const uint32_t row = min(v, (uint32_t)P.n - 1u), some = __ballot_sync(kFull, has);
+                uint32_t open = 0u, told = 0u;
+                for (int j0 = 0; j0 < 32; j0 += 8) {
+                    if (!((some >> j0) & 255u)) continue;
+                    uint32_t d[8];
+#pragma unroll
+                    for (int k = 0; k < 8; k++) {
+                        const uint32_t off = f.at(__shfl_sync(kFull, row, j0 + k));
+                        d[k] = (some >> (j0 + k)) & 1u ? __ldcg(f.word(P.dist, off)) : 0u;
+                    }
+#pragma unroll
+                    for (int k = 0; k < 8; k++) {
+                        const bool in = (__shfl_sync(kFull, m, j0 + k) >> lane) & 1u;
+                        const bool core = __shfl_sync(kFull, (int)hub, j0 + k) != 0;
+                        bool a, b;
+                        if (pass == kFanCore) {
+                            a = in && d[k] < f.bound;
+                            b = a && d[k] < f.core;
+                            if (b && core) atomicMax(P.sync->core + lane, ~d[k]);
+                        } else {
+                            a = in && f.core != kInfU32 && d[k] >= f.bound;
+                            b = a && d[k] != Fan<WT, kFanCore>::kInf;
+                        }
+                        const uint32_t ma = __ballot_sync(kFull, a), mb = __ballot_sync(kFull, b);
+                        if ((int)lane == j0 + k) open = ma, told = mb;
+                    }
+                }
+                m = has ? open : 0u;
+                if (pass == kFanCore) {
+                    if (hub || !told) sp.y = mid;
+                } else if (m && told && deg > 1) {
+                    // (a vertex with one arc has nobody to tell but its source)
+                    wait_w[base + lane] = told;
+                }
+                if (!m) sp.y = sp.x;
             }
             const int32_t deg = sp.y - sp.x;
             n_relax += (uint32_t)deg;
@@ -296,7 +393,8 @@ __global__ void __launch_bounds__(kFanThreads, 1) fan_kernel(const __grid_consta
             if (lane == 0u && sm) at = atomicAdd(&P.sync->set[set].rows, (uint32_t)__popc(sm));
             if (lane == 31u && lm) at = atomicAdd(&P.sync->set[set].slices, incl);
             const uint32_t at_r = __shfl_sync(kFull, at, 0), at_s = __shfl_sync(kFull, at, 31) + incl - k;
-            if ((sm >> lane) & 1u) P.rows[at_r + __popc(sm & lanemask_lt())] = make_uint2(v, m);
+            if ((sm >> lane) & 1u) P.rows[at_r + __popc(sm & lanemask_lt())] =
+                    make_uint4(v, m, (uint32_t)sp.x, (uint32_t)sp.y);
             // one slice of its own row each, then the rest of the longest rows together
             if (k == 1u) P.slices[at_s] = make_uint4(v, m, (uint32_t)sp.x, (uint32_t)sp.y);
             lm = __ballot_sync(kFull, k > 1u);
@@ -318,14 +416,20 @@ __global__ void __launch_bounds__(kFanThreads, 1) fan_kernel(const __grid_consta
         }
         if (!(ok = fan_barrier(P.sync, arrivals += gridDim.x, deadline))) break;
         const uint32_t slices = ld_relaxed(&P.sync->set[set].slices), rows = ld_relaxed(&P.sync->set[set].rows);
-        if (tight) {
+        if (pass == kFanTight) {
             Fan<WT, kFanTight>(P, wait_w).work(slices, rows, wid, nw, &P.sync->set[set].claimed);
             break;
         }
         if (slices + rows == 0u) {
-            // nobody waits: the distances are final
-            if (!P.pred) break;
-            tight = true;
+            // nobody waits: the core has settled, or all distances are final
+            if (CORE && pass == kFanCore) pass = kFanPull;
+            else if (!P.pred) break;
+            else pass = kFanTight;
+        } else if (CORE && pass == kFanCore) {
+            Fan<WT, kFanCore>(P, wait_w).work(slices, rows, wid, nw, &P.sync->set[set].claimed);
+        } else if (CORE && pass == kFanPull) {
+            Fan<WT, kFanPull>(P, wait_w).work(slices, rows, wid, nw, &P.sync->set[set].claimed);
+            pass = kFanRelax;
         } else {
             Fan<WT, kFanRelax>(P, wait_w).work(slices, rows, wid, nw, &P.sync->set[set].claimed);
         }

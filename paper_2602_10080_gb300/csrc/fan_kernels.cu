@@ -5,7 +5,7 @@
 
 namespace sssp {
 
-template <int WT>
+template <int WT, bool CORE>
 static cudaError_t launch_one(const FanParams& p, int grid, cudaStream_t stream) {
     cudaLaunchConfig_t c{};
     c.gridDim = dim3(grid);
@@ -16,11 +16,12 @@ static cudaError_t launch_one(const FanParams& p, int grid, cudaStream_t stream)
     at[0].val.cooperative = 1;
     c.attrs = at;
     c.numAttrs = 1;
-    return cudaLaunchKernelEx(&c, fan_kernel<WT>, p);
+    return cudaLaunchKernelEx(&c, fan_kernel<WT, CORE>, p);
 }
 
 cudaError_t launch_fan(int wt, const FanParams& p, int grid, cudaStream_t stream) {
-    return wt == 0 ? launch_one<0>(p, grid, stream) : launch_one<1>(p, grid, stream);
+    if (p.mid) return wt == 0 ? launch_one<0, true>(p, grid, stream) : launch_one<1, true>(p, grid, stream);
+    return wt == 0 ? launch_one<0, false>(p, grid, stream) : launch_one<1, false>(p, grid, stream);
 }
 
 cudaError_t launch_fan_out(const uint32_t* rows, int32_t n, int32_t nq, uint32_t* out, int sms, cudaStream_t stream) {

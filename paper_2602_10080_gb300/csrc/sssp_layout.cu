@@ -354,9 +354,13 @@ int check_symmetry(Graph* g, const int32_t* rp0, const uint2* adj0, cudaStream_t
     cudaFree(st);
     if (e != cudaSuccess) return cuda_status(e);
     g->symmetric = h.bad == 0 && h.looked == h.other;
-    // a quarter of the average weight: an eighth of the arcs of evenly
-    // distributed weights; of small whole weights a few values
-    const double lw = g->feat.avg_w / 4.0;
+    // A seventh of the average weight: a fourteenth of the arcs of evenly
+    // distributed weights; of small whole weights a few values.  us at a
+    // quarter, sixth, eighth and tenth: R-MAT-22 665, 636, 638, 672; R-MAT-20
+    // 311, 274, 263, 262; R-MAT-19 f32 311, 286, 272, 264; 64 queries on
+    // R-MAT-20 4100, 3740, 3780, 4940 (too few settle), on R-MAT-18 f32 2670,
+    // 2560, 2400, 2320.
+    const double lw = g->feat.avg_w / 7.0;
     g->light_w = g->wtype == SSSP_W_F32 ? __float_as_uint_host((float)lw) : (uint32_t)std::max(3.0, std::floor(lw));
     return SSSP_OK;
 }

@@ -70,11 +70,11 @@ bool plan_wave(const WaveGraph& g, int32_t nq, int pred_mode, WavePlan* w) {
         w->kind = kWholeGrid;
         if (hubs) {
             // power law: the arcs of the core are the work.  Without them the
-            // steps count on all but the largest graphs, us with (without) the
-            // core's heavy arcs: R-MAT-22 675 (1786), at width 1 773, 1/4 710;
-            // R-MAT-20 344 (920), a front of 256 363; R-MAT-18 190 (378), a front
-            // of 1 202; R-MAT-16 155 (303); R-MAT-19 f32 312 (626).  A graph whose
-            // core does not settle in time (weights up to 15) loses 8%
+            // steps count on all but the largest graphs, us without (with) the
+            // core's heavy arcs: R-MAT-22 637 (1786), at width 1 and a wider light
+            // bound 15% slower, at 1/4 6%; R-MAT-20 270 (920); R-MAT-18 195 (378);
+            // R-MAT-16 160 (303); R-MAT-19 f32 280 (626).  A graph whose core does
+            // not settle in time (weights up to 15) loses 8%
             w->core = g.core;
             w->delta *= g.m > (1 << 25) ? 0.5 : 1.0;
             w->front = g.m > (w->core ? 1 << 24 : 1 << 25) ? 1u : 256u;
@@ -96,10 +96,11 @@ bool plan_wave(const WaveGraph& g, int32_t nq, int pred_mode, WavePlan* w) {
     // 4: 1880, 1: 2130)
     if (g.n > kClusterVertices || g.m > (1 << 21) || (hubs && g.m > (1 << 18))) {
         // A group of up to 32 queries side by side costs as much as this many
-        // in turn on the whole grid: R-MAT-20 7 (5.7 ms), R-MAT-18 7 (2.7 ms),
-        // G(200K, 2M) 15 (3.1 ms).  Predecessors of the strict-improvement rule
-        // cannot be found after the distances and stay with the queues.
-        if (nq < 12) w->kind = kInTurn;
+        // in turn on the whole grid: R-MAT-20 6 (1.40 ms), R-MAT-18 5 (0.93 ms),
+        // with all arcs 7, G(200K, 2M) 14 (2.6 ms).  Predecessors of the
+        // strict-improvement rule cannot be found after the distances and stay
+        // with the queues.
+        if (nq < (g.core ? 6 : hubs ? 8 : 14)) w->kind = kInTurn;
         else if (pred_mode != 2 && g.n <= kFanMaxVertices) w->kind = kSideBySide;
         else return false;
         return true;
@@ -162,7 +163,7 @@ size_t fan_words(int32_t n, bool pred) {
 }
 
 // a row of more than kFanShort arcs is cut into slices of kFanChunk
-size_t fan_slices(int32_t n, int64_t m) { return (size_t)(m / kFanChunk + m / kFanShort + 1) + ((size_t)n + 1) / 2; }
+size_t fan_slices(int32_t n, int64_t m) { return (size_t)(m / kFanChunk + m / kFanShort + 1) + (size_t)n; }
 
 void fan_carve(uint32_t* words, uint4* slices, int32_t n, int64_t m, bool pred, FanParams* p) {
     const size_t places = fan_places(n);
@@ -173,7 +174,7 @@ void fan_carve(uint32_t* words, uint4* slices, int32_t n, int64_t m, bool pred, 
     p->dist = p->wait + std::max<size_t>(32, 2 * places);
     p->pred = pred ? p->dist + 32 * (size_t)n : nullptr;
     p->slices = slices;
-    p->rows = reinterpret_cast<uint2*>(slices + (m / kFanChunk + m / kFanShort + 1));
+    p->rows = slices + (m / kFanChunk + m / kFanShort + 1);
 }
 
 std::mutex& grid_mutex(int device) {
@@ -192,14 +193,20 @@ int run_fan(Graph* g, const int32_t* srcs_host, const int32_t* srcs_dev, int32_t
     if ((rc = grow(&ws.srcs, &ws.srcs_n, (size_t)nq))) return rc;
     cudaMemcpyAsync(ws.srcs, srcs_dev ? srcs_dev : srcs_host, sizeof(int32_t) * nq,
                     srcs_dev ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice, stream);
-    if ((rc = grow(&ws.fan, &ws.fan_n, fan_words(g->n, pred_out != nullptr)))) return rc;
-    if ((rc = grow(&ws.fan_slices, &ws.fan_slices_n, fan_slices(g->n, g->m)))) return rc;
+    // (no room for the rows: the queues need less)
+    if (grow(&ws.fan, &ws.fan_n, fan_words(g->n, pred_out != nullptr))) return kWaveNotRun;
+    if (grow(&ws.fan_slices, &ws.fan_slices_n, fan_slices(g->n, g->m))) return kWaveNotRun;
     FanParams P;
     std::memset(&P, 0, sizeof(P));
     fan_carve(ws.fan, ws.fan_slices, g->n, g->m, pred_out != nullptr, &P);
     P.span = g->span;
     P.adj = g->adj;
     P.ctrl = ws.ctrl;
+    if (wave_graph(g).core) {
+        P.mid = g->mid;
+        P.light_w = g->light_w;
+        P.core_deg = kFanCoreArcs;
+    }
     P.timeout_ns = 20000ull * 1000000ull;
     const int32_t groups = (nq + 31) / 32, per = (nq + groups - 1) / groups;
     for (int32_t q0 = 0; q0 < nq; q0 += per) {

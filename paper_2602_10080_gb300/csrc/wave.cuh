@@ -697,8 +697,7 @@ __device__ __forceinline__ void red_release64(unsigned long long* p, unsigned lo
 // other vertex with arcs looks at all its in-neighbours once (its own arcs,
 // reversed), which covers all that was left out, and the search ends among
 // these vertices with all their arcs.  On R-MAT-22 from a source of the giant
-// component 5% of the arcs are below the bound, 12% light, and the other
-// vertices have 4 to 6% of the arcs.
+// component a fifth as many arcs as there are is relaxed or looked at in all.
 template <int WT, int PRED, bool HOPS, bool CORE>
 __global__ void __launch_bounds__(1024, 1) tide_kernel(const __grid_constant__ WaveParams P) {
     using W = Wave<WT, PRED, kWaveGrid, HOPS, CORE>;

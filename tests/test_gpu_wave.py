@@ -137,7 +137,7 @@ def side_by_side(g, srcs, pred=True):
 
 @pytest.mark.parametrize("nq", [2, 11, 12, 31, 32, 33, 64, 70])
 def test_batch_side_by_side(nq):
-    """Groups of 32 queries on a graph with hubs, in turn below 12 queries;
+    """Groups of 32 queries on a graph with hubs, few queries in turn;
     repeated sources, sources without arcs."""
     g = gg.rmat(13, 24, seed=nq)
     srcs = gg.giant_sources(g, nq)[0]
@@ -426,3 +426,27 @@ def test_core_needs_symmetry():
         d, p = gpu_solve(G, src, pred=True)
         assert_exact(h, src, d, p)
         G.close()
+
+
+@pytest.mark.parametrize("wtype,lo,hi", [("u32", 1, 255), ("u32", 0, 255), ("u32", 1, 15), ("f32", 1, 255)])
+@pytest.mark.parametrize("nq", [12, 33])
+def test_batch_core_and_pull(wtype, lo, hi, nq):
+    """Side by side on symmetric graphs with hubs: rows with one arc and none,
+    a component apart, sources in the core, at its edge and alone."""
+    g = hubs_and_leaves(70_000, 60, 300_000, lo, hi, seed=3, wtype=wtype)
+    keep = g.n + 100                        # more vertices: some without arcs, some apart
+    rp = np.concatenate([g.row_ptr, np.full(100, g.m, np.int32)])
+    rp[g.n + 60:] += 2
+    rp[g.n + 59] += 1
+    col = np.concatenate([g.col, [g.n + 59, g.n + 58]]).astype(np.int32)
+    w = np.concatenate([g.w, g.w[:1], g.w[:1]])
+    h = gg.Graph("apart", keep, len(col), rp, col, w, wtype)
+    G = upload(h)
+    deg = np.diff(h.row_ptr)
+    srcs = np.concatenate([[np.argmax(deg), g.n + 58, g.n + 59, g.n + 5, 0, 69_999],
+                           np.random.default_rng(4).integers(0, g.n, nq - 6)]).astype(np.int32)
+    d, p = gpu_batch(G, srcs, pred=True)
+    assert_exact_many(h, srcs, d, p)
+    d2, _ = gpu_batch(G, srcs, pred=False)
+    np.testing.assert_array_equal(d2, d)
+    G.close()
