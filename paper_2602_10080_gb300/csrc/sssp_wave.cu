@@ -292,6 +292,7 @@ int run_wave(Graph* g, const int32_t* srcs_host, const int32_t* srcs_dev, int32_
         }
         P.span = g->span;
         P.adj = g->adj;
+        P.pull = unit && g->symmetric;
         if (plan.core && !unit) {
             P.mid = g->mid;
             P.light_w = g->light_w;

@@ -53,6 +53,7 @@ struct WaveParams {
     int32_t log_g;            // log2 of the cluster's blocks: word w lives in block w % G
     int32_t words;            // words per block (wave), or in all (tide)
     int32_t hops;             // hops of a warp per step
+    int32_t pull;             // breadth-first on a symmetric graph: wide levels are pulled
     int32_t unit;             // breadth-first: every arc weighs 1, hub slices belong to the step that lists them
     int32_t hub_deg;          // a vertex with more arcs is not left to one warp
     int32_t has_hubs;
@@ -465,23 +466,25 @@ struct Wave {
     }
 
     // Vertex v (distance word cur, arcs sp; deg arcs to look at, all of them
-    // or none) takes the best of its in-neighbours, its own arcs' ends.  The
-    // whole warp is here.  Returns its distance after that.
-    __device__ __forceinline__ uint32_t pull(uint32_t v, DistT cur, int2 sp, int32_t deg) {
+    // or none) takes the best of its in-neighbours, its own arcs' ends, of
+    // those nearer than `limit`.  The whole warp is here.  Returns its distance
+    // after that.
+    __device__ __forceinline__ uint32_t pull(uint32_t v, DistT cur, int2 sp, int32_t deg, uint32_t limit) {
         constexpr uint32_t none = PRED == 0 && WT == 1 ? kInfF32 : kInfU32;
         const uint32_t lane = lane_id();
         uint32_t best = none, from = kInfU32;
         auto offer = [&](uint2 a, DistT c) {
             const uint32_t du = dpart(c);
-            if (du == none) return;
-            const uint32_t nd = A::add(du, a.y);
+            if (du >= limit) return;
+            const uint32_t nd = A::add(du, P.unit ? 1u : a.y);
             if (nd < best || (nd == best && a.x < from)) {
                 best = nd;
                 from = a.x;
             }
         };
         const bool by_warp = deg > 64;
-        for (int32_t e = 0; !by_warp && e < deg; e += 4) {
+        // (of a level, any parent gives the distance)
+        for (int32_t e = 0; !by_warp && e < deg && !(PRED == 0 && P.unit && best != none); e += 4) {
             uint2 a[4];
             DistT c[4];
 #pragma unroll
@@ -686,6 +689,15 @@ __device__ __forceinline__ void red_release64(unsigned long long* p, unsigned lo
     asm volatile("red.release.gpu.global.add.u64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
 }
 
+// Breadth-first on a symmetric graph, a level of more vertices than these
+// fractions of those not reached yet and of all is pulled: every vertex not
+// reached looks for the level in its own row.  On power-law graphs nearly all
+// arcs belong to the level before the widest, and lead back.  R-MAT-22 us, with
+// parents 783 -> 312, levels only 725 -> 238; R-MAT-20 290 -> 200 (231 at a
+// 14th of those not reached; at 1000ths R-MAT-22 pulls too early, 1104), R-MAT-16
+// 106 -> 89.
+constexpr uint32_t kPullUnreached = 50u, kPullAll = 64u;
+
 // The whole grid on one query.
 //
 // CORE (symmetric graphs with hubs, light arcs first in every row): most arcs
@@ -724,10 +736,10 @@ __global__ void __launch_bounds__(1024, 1) tide_kernel(const __grid_constant__ W
         s_fmin[tid] = s_left[tid] = kInfU32;
         s_arcs[tid] = 0u;
     }
-    w.skip = CORE;
+    w.skip = CORE && !P.unit;
 
     // step 0 ends the preparation; the searching steps follow
-    uint32_t cur = 0u, fw = 0u, far_low = kInfU32, n_improved = 0, steps = 0, near = 0u, settled = kInfU32;
+    uint32_t cur = 0u, fw = 0u, far_low = kInfU32, n_improved = 0, steps = 0, near = 0u, settled = kInfU32, reached = 1u;
     int what = 1;
     bool ok = true;
     for (;;) {
@@ -790,6 +802,10 @@ __global__ void __launch_bounds__(1024, 1) tide_kernel(const __grid_constant__ W
                 what = w.advance(near + items, far_low);
             }
             if (!what) break;
+            if (CORE && P.pull) {
+                reached = min((uint32_t)P.n, reached + near);
+                if (near >= max(((uint32_t)P.n - reached) / kPullUnreached, (uint32_t)P.n / kPullAll)) what = 3;
+            }
         }
         const uint32_t prev = set;
         steps++;
@@ -798,9 +814,17 @@ __global__ void __launch_bounds__(1024, 1) tide_kernel(const __grid_constant__ W
             // nobody waits below `settled`: the others pull, and wait.  Where
             // the core has not settled yet (less than half of the arcs left
             // out) pulling would cost more than relaxing everything again.
-            const bool pulls = ld_relaxed64(&P.sync->left.arcs) * 2ull >= (unsigned long long)P.arcs;
+            // A wide level: those not reached yet look for a parent in it.
+            const bool level = P.unit != 0;
+            const bool pulls = level || ld_relaxed64(&P.sync->left.arcs) * 2ull >= (unsigned long long)P.arcs;
+            const uint32_t limit = level ? steps : PRED == 0 && WT == 1 ? kInfF32 : kInfU32;
             w.skip = false;
             w.bound = kInfU32;
+            if (level) {
+                for (uint32_t i = gt; i < words; i += gn) P.bits[(size_t)cur * words + i] = 0u;
+                cur ^= 1u;
+                settled = PRED == 0 && WT == 1 ? kInfF32 : kInfU32;
+            }
             // little is left after the pull: no order among it any more
             if (pulls) w.delta = WT == 1 ? kInfF32 : kInfU32;
             w.near_w = P.bits + (size_t)cur * words;
@@ -826,7 +850,7 @@ __global__ void __launch_bounds__(1024, 1) tide_kernel(const __grid_constant__ W
                 const int32_t look = pulls && W::dpart(dv) >= settled ? deg : 0;
                 if (!__any_sync(kFull, pulls ? look > 0 : deg > 0)) continue;
                 w.n_relax += (uint32_t)look;
-                const uint32_t d = w.pull(v, dv, sp, look);
+                const uint32_t d = w.pull(v, dv, sp, look, limit);
                 // (a vertex with one arc has nobody to tell but its source)
                 if ((pulls ? look > 1 : deg > 0) && d != (PRED == 0 && WT == 1 ? kInfF32 : kInfU32)) {
                     uint32_t mask;

@@ -44,7 +44,7 @@ static cudaError_t launch_tide_one(const WaveParams& p, int grid, int threads, c
     at[0].val.cooperative = 1;
     c.attrs = at;
     c.numAttrs = 1;
-    if (p.mid) return cudaLaunchKernelEx(&c, tide_kernel<WT, PRED, false, true>, p);
+    if (p.mid || p.pull) return cudaLaunchKernelEx(&c, tide_kernel<WT, PRED, false, true>, p);
     return p.hops > 1 ? cudaLaunchKernelEx(&c, tide_kernel<WT, PRED, true, false>, p)
                       : cudaLaunchKernelEx(&c, tide_kernel<WT, PRED, false, false>, p);
 }

@@ -450,3 +450,45 @@ def test_batch_core_and_pull(wtype, lo, hi, nq):
     d2, _ = gpu_batch(G, srcs, pred=False)
     np.testing.assert_array_equal(d2, d)
     G.close()
+
+
+@pytest.mark.parametrize("kind", ["leaves", "star", "rmat", "apart", "directed"])
+def test_levels_pulled(kind):
+    """Wide levels on symmetric graphs with hubs (and on one that is not
+    symmetric): rows beyond a warp's, self-loops, leaves, vertices without
+    arcs, a component apart; with and without parents."""
+    if kind == "star":
+        n = 600_000
+        leaf = np.arange(1, n)
+        g = symmetric(n, np.zeros(n - 1, np.int64), leaf, np.ones(n - 1, np.uint32))
+        srcs = (0, 1, n - 1)
+    elif kind == "rmat":
+        g = gg.rmat(17, 16, seed=5)
+        srcs = [int(x) for x in gg.giant_sources(g, 3)[0]] + [int(np.flatnonzero(np.diff(g.row_ptr) == 0)[0])]
+    else:
+        g = hubs_and_leaves(90_000, 20, 500_000, 1, 99, seed=6)
+        if kind == "apart":
+            e = np.arange(g.n, g.n + 300_000, 2)
+            rp = np.concatenate([g.row_ptr, g.m + 1 + np.arange(300_000)]).astype(np.int32)
+            col = np.concatenate([g.col, np.stack([e + 1, e], 1).ravel()]).astype(np.int32)
+            g = gg.Graph("apart", g.n + 300_000, len(col), rp, col, np.concatenate([g.w, np.ones(300_000, np.uint32)]), "u32")
+        if kind == "directed":
+            col = g.col.copy()
+            col[::1001] = (col[::1001] + 1) % g.n
+            g = gg.Graph("directed", g.n, g.m, g.row_ptr, col, g.w, "u32")
+        srcs = (0, int(np.argmax(np.diff(g.row_ptr))), 77_777, g.n - 1)
+    G = upload(g)
+    unit = np.ones(g.m, np.uint32)
+    for src in srcs:
+        lev = torch.empty(G.n, dtype=torch.int32, device="cuda")
+        par = torch.empty(G.n, dtype=torch.int32, device="cuda")
+        G.bfs(src, lev, par)
+        torch.cuda.synchronize()
+        ref = oracle.dijkstra_u32(g.row_ptr, g.col, unit, src)
+        np.testing.assert_array_equal(lev.cpu().numpy().view(np.uint32), ref)
+        np.testing.assert_array_equal(par.cpu().numpy(), oracle.pred_canonical_u32(g.row_ptr, g.col, unit, src, ref))
+        lev2 = torch.empty(G.n, dtype=torch.int32, device="cuda")
+        G.bfs(src, lev2, None)
+        torch.cuda.synchronize()
+        assert torch.equal(lev, lev2)
+    G.close()
