@@ -74,6 +74,7 @@ struct Graph {
     uint32_t light_w = 0;
     double light_share = 0.0;     // of the arcs
     int32_t* mid = nullptr;       // [n] (light_first)
+    uint4* quads = nullptr;       // [n][2] the first four arcs of every vertex of a thin graph (see WaveParams)
     sssp_features feat{};
     sssp_config defaults{};
     sssp_config tuned{};
@@ -119,7 +120,7 @@ int ensure_layout(Graph* g, int32_t split, cudaStream_t s);
 // g->row_ptr / adj / owner describe the layout (rp0 / adj0 are freed when new
 // arrays replaced them), on failure the graph is untouched.
 int build_layout(Graph* g, int32_t* rp0, uint2* adj0, int32_t split, cudaStream_t s);
-// g->span (and g->mid) for the current layout.
+// g->span (and g->mid, g->quads) for the current layout.
 int fill_span(Graph* g, cudaStream_t s);
 // Original arc order from a split layout: row v of rp0 from adj[src_start[v] ..].
 void launch_unsplit(const Graph* g, const int32_t* src_start, const int32_t* rp0, uint2* adj0, cudaStream_t s);

@@ -1109,6 +1109,7 @@ extern "C" int sssp_graph_create(const int32_t* row_ptr, const int32_t* col_idx,
         cudaFree(g->owner);
         cudaFree(g->span);
         cudaFree(g->mid);
+        cudaFree(g->quads);
         delete g;
         return rc;
     }
@@ -1128,6 +1129,7 @@ extern "C" int sssp_graph_destroy(sssp_graph* gh) {
         cudaFree(g->owner);
         cudaFree(g->span);
         cudaFree(g->mid);
+        cudaFree(g->quads);
     }
     delete g;
     return SSSP_OK;

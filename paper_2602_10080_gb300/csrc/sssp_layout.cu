@@ -229,6 +229,20 @@ __global__ void span_kernel(const int32_t* rp, const uint2* adj, int32_t n, int2
     if (lane_id() == 0 && count) atomicAdd(lights, count);
 }
 
+// The first four arcs of every vertex at a fixed place.
+__global__ void quads_kernel(const int2* span, const uint2* adj, int32_t n, uint4* quads) {
+    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+    for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < n; v += stride) {
+        const int2 sp = span[v];
+        uint2 a[4];
+#pragma unroll
+        for (int k = 0; k < 4; k++) a[k] = sp.x + k < sp.y ? adj[sp.x + k] : make_uint2(kNoArc, 0u);
+        if (sp.y - sp.x > 4) a[0].x |= 0x80000000u;
+        quads[2 * v] = make_uint4(a[0].x, a[0].y, a[1].x, a[1].y);
+        quads[2 * v + 1] = make_uint4(a[2].x, a[2].y, a[3].x, a[3].y);
+    }
+}
+
 // Original arc order from a split layout: the arcs of vertex v lie from
 // src_start[v] on.  One warp per vertex.
 __global__ void unsplit_kernel(const uint2* adj1, const int32_t* src_start, const int32_t* rp0, int32_t n,
@@ -457,6 +471,11 @@ int fill_span(Graph* g, cudaStream_t s) {
     const int64_t blocks = std::min<int64_t>(((int64_t)g->n + 255) / 256, (int64_t)g->sms * 8);
     span_kernel<<<(int)std::max<int64_t>(1, blocks), 256, 0, s>>>(g->row_ptr, g->adj, g->n, g->span, g->light_w,
                                                                   g->light_first ? g->mid : nullptr, lights);
+    // (the quads of a mesh only save time: without room for them, without them)
+    if (thin_graph(g->feat.avg_deg, g->feat.max_deg) &&
+        (g->quads || cudaMalloc((void**)&g->quads, 2 * sizeof(uint4) * (size_t)g->n) == cudaSuccess))
+        quads_kernel<<<(int)std::max<int64_t>(1, blocks), 256, 0, s>>>(g->span, g->adj, g->n, g->quads);
+    else cudaGetLastError();
     if (lights) cudaMemcpyAsync(&h, lights, sizeof(h), cudaMemcpyDeviceToHost, s);
     const cudaError_t e = cudaStreamSynchronize(s);
     cudaFree(lights);

@@ -936,6 +936,7 @@ int express_launch(sssp_server* s, Lane* L) {
         } else {
             P.span = g->span;
             P.adj = g->adj;
+            P.quads = g->quads;
             if (plan.core) {
                 P.mid = g->mid;
                 P.light_w = g->light_w;

@@ -49,7 +49,7 @@ bool plan_wave(const WaveGraph& g, int32_t nq, int pred_mode, WavePlan* w) {
     // (directed 60000 vertices of degree 6 174, 150 at 2, 255 at 8; G(10^4, 10^5)
     // 128, 115 at 2) but not on the smallest graphs (directed 10^4 vertices 102,
     // 114 at 2), nor with hubs (R-MAT-13 164, 189 at 2).
-    const bool thin = deg <= 6.5 && g.max_deg <= std::min(2.0 * deg + 1.5, 11.5);
+    const bool thin = thin_graph(deg, g.max_deg);
     const int32_t hops = thin ? 8 : !hubs && g.m > (1 << 16) ? 2 : 1;
     if (nq == 1) {
         if (g.n <= kClusterVertices && (g.m <= (1 << 19) || (thin && !g.wide))) {
@@ -292,6 +292,7 @@ int run_wave(Graph* g, const int32_t* srcs_host, const int32_t* srcs_dev, int32_
         }
         P.span = g->span;
         P.adj = g->adj;
+        P.quads = g->quads;
         P.pull = unit && g->symmetric;
         if (plan.core && !unit) {
             P.mid = g->mid;

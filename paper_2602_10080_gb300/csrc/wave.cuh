@@ -62,6 +62,7 @@ struct WaveParams {
     unsigned long long timeout_ns;
     // tide only
     const int32_t* mid;       // [n] end of a row's light arcs (core search), or null
+    const uint4* quads;       // [n][2] the first four arcs of every vertex (kNoArc: none; bit 31 of the first: more), or null
     uint32_t light_w;         // weights of light arcs: at most this
     int32_t core_deg;         // a vertex with as many arcs belongs to the core
     int64_t arcs;             // of the graph
@@ -73,7 +74,10 @@ struct WaveParams {
 
 constexpr uint32_t kWaveOwn = 64;      // improved vertices that a warp keeps for its own next hop
 
-template <bool HOPS>
+constexpr uint32_t kNoArc = 0x7fffffffu;
+constexpr int kHopsQuads = 2;          // several hops a step, on graphs with quads
+
+template <int HOPS>
 struct WaveLists {
     uint32_t list[64];                 // vertices taken from the words (bit 31: from far)
     uint2 own[2][HOPS ? kWaveOwn : 1]; // (vertex, distance) of this hop and the next
@@ -153,7 +157,7 @@ enum WaveMode { kWaveBlock = 0, kWaveCluster = 1, kWaveGrid = 2 };
 // HOPS: a warp may have more than one hop a step (compiled out otherwise: with
 // it R-MAT-22 took 8% and R-MAT-13 12% longer at one hop).
 // CORE: rows may be relaxed without their heavy arcs (see tide_kernel).
-template <int WT, int PRED, int MODE, bool HOPS, bool CORE = false>
+template <int WT, int PRED, int MODE, int HOPS, bool CORE = false>
 struct Wave {
     using DistT = typename std::conditional<PRED == 0, uint32_t, unsigned long long>::type;
     using A = Arith<WT>;
@@ -305,6 +309,62 @@ struct Wave {
         relax<4, true>(uj, dj, a, c, in);
     }
 
+    // Whether vertex v, of the last hop at distance d or from the words (d
+    // infinite), is still to be relaxed, and d: its distance `now`.
+    __device__ __forceinline__ bool claim(uint32_t v, bool is_far, uint32_t now, uint32_t& d) {
+        // improved meanwhile: whoever did marked it again
+        if (d != kInfU32) return now >= d;
+        d = now;
+        if (!is_far) return true;
+        // below the old threshold: it went through near since
+        if (d < Told) return false;
+        if (d < T) return true;
+        uint32_t mask;
+        const Addr a = bit_addr(far_w, v, mask);
+        red_or(a, mask);
+        fmin = min(fmin, d);
+        return false;
+    }
+
+    // A batch of relax_batch whose first four arcs lie at a fixed place: two
+    // dependent loads (arcs, their ends' distances) instead of three.  The
+    // check of the vertex itself comes back meanwhile.  GB300, us: grid 256^2 864
+    // -> 768, grid 1024^2 4006 -> 3600, 13 queries on grid 301 x 257 1122 -> 1000;
+    // road 4096^2 6006, 5987.
+    __device__ __forceinline__ void relax_quads(bool have, uint32_t v, bool is_far, uint32_t d) {
+        uint4 x = make_uint4(kNoArc, 0u, kNoArc, 0u), y = x;
+        uint32_t now = kInfU32;
+        if (have) {
+            x = __ldg(P.quads + 2 * (size_t)v);
+            y = __ldg(P.quads + 2 * (size_t)v + 1);
+            now = dpart(ld_dist(dist + v));
+        }
+        const bool more = (x.x >> 31) != 0u;
+        const uint2 a[4] = {make_uint2(x.x & kNoArc, x.y), make_uint2(x.z, x.w), make_uint2(y.x, y.y), make_uint2(y.z, y.w)};
+        DistT c[4];
+        bool in[4];
+#pragma unroll
+        for (int k = 0; k < 4; k++) {
+            in[k] = a[k].x != kNoArc;
+            c[k] = in[k] ? ld_dist(dist + a[k].x) : (DistT)0;
+        }
+        if (have) have = claim(v, is_far, now, d);
+        const uint32_t uu[4] = {v, v, v, v}, dd[4] = {d, d, d, d};
+#pragma unroll
+        for (int k = 0; k < 4; k++) {
+            in[k] = in[k] && have;
+            n_relax += in[k] ? 1u : 0u;
+        }
+        relax<4, true>(uu, dd, a, c, in);
+        if (__any_sync(kFull, have && more)) {
+            int2 sp = have && more ? __ldg(P.span + v) : make_int2(0, 0);
+            sp.x = min(sp.x + 4, sp.y);
+            n_relax += (uint32_t)(sp.y - sp.x);
+            for (; __any_sync(kFull, sp.x < sp.y); sp.x += 4) arcs4<true>(v, d, sp.x, 1, sp.y);
+        }
+        __syncwarp();
+    }
+
     // Relaxes up to 32 vertices, one per lane (`have`): from the words
     // (is_far: from the far ones) or, with their distance d, from the warp's
     // last hop.  `hub(v, d, arcs, deg)` takes those with more than hub_deg arcs
@@ -312,25 +372,15 @@ struct Wave {
     template <typename Hub>
     __device__ __forceinline__ void relax_batch(bool have, uint32_t v, bool is_far, uint32_t d, Hub&& hub) {
         const uint32_t lane = lane_id();
+        if constexpr (HOPS == kHopsQuads) {
+            relax_quads(have, v, is_far, d);
+            return;
+        }
         int2 sp = make_int2(0, 0);
         if (have) {
             const uint32_t now = dpart(ld_dist(dist + v));
             sp = P.span ? __ldg(P.span + v) : make_int2(__ldg(P.row + v), __ldg(P.row + v + 1));
-            // improved meanwhile: whoever did marked it again
-            if (d != kInfU32) have = now >= d;
-            else d = now;
-            if (is_far) {
-                // below the old threshold: it went through near since
-                if (d < Told) {
-                    have = false;
-                } else if (d >= T) {
-                    have = false;
-                    uint32_t mask;
-                    const Addr a = bit_addr(far_w, v, mask);
-                    red_or(a, mask);
-                    fmin = min(fmin, d);
-                }
-            }
+            have = claim(v, is_far, now, d);
         }
         if (CORE && skip && have && (sp.y - sp.x >= P.core_deg || d >= core)) {
             const int32_t m = __ldg(P.mid + v);
@@ -547,7 +597,7 @@ struct Wave {
 // by writing them into every block's slots; one cluster barrier then makes
 // them and the step's marks visible.  Two slot sets alternate: a block can
 // write set s + 2 only after all blocks passed barrier s + 1, after reading s.
-template <int WT, int PRED, bool CL, bool HOPS>
+template <int WT, int PRED, bool CL, int HOPS>
 __global__ void __launch_bounds__(1024, 1) wave_kernel(const __grid_constant__ WaveParams P) {
     using W = Wave<WT, PRED, CL ? kWaveCluster : kWaveBlock, HOPS>;
     using DistT = typename W::DistT;
@@ -710,7 +760,7 @@ constexpr uint32_t kPullUnreached = 50u, kPullAll = 64u;
 // reversed), which covers all that was left out, and the search ends among
 // these vertices with all their arcs.  On R-MAT-22 from a source of the giant
 // component a fifth as many arcs as there are is relaxed or looked at in all.
-template <int WT, int PRED, bool HOPS, bool CORE>
+template <int WT, int PRED, int HOPS, bool CORE>
 __global__ void __launch_bounds__(1024, 1) tide_kernel(const __grid_constant__ WaveParams P) {
     using W = Wave<WT, PRED, kWaveGrid, HOPS, CORE>;
     using DistT = typename W::DistT;

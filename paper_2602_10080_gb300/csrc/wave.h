@@ -41,6 +41,10 @@ constexpr int kTideLogWords = 17;               // the grid kernel spreads the p
 constexpr size_t kWaveMaxShared = 176 * 1024;   // pending words of one block (beside WaveShared)
 
 // The kernel and launch shape of a call; false: the queue engine takes it.
+// A mesh or a road map: few arcs a vertex, and none with many more.
+inline bool thin_graph(double deg, double max_deg) {
+    return deg <= 6.5 && max_deg <= (2.0 * deg + 1.5 < 11.5 ? 2.0 * deg + 1.5 : 11.5);
+}
 bool plan_wave(const WaveGraph& g, int32_t nq, int pred_mode, WavePlan* w);
 // The fields of the parameters that follow from the plan; returns the dynamic
 // shared memory of a block.

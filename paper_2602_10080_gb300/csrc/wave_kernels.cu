@@ -3,7 +3,7 @@
 
 namespace sssp {
 
-template <int WT, int PRED, bool CL, bool HOPS>
+template <int WT, int PRED, bool CL, int HOPS>
 static cudaError_t launch_hops(const WaveParams& p, int nq, int threads, size_t smem, cudaStream_t stream) {
     auto fn = wave_kernel<WT, PRED, CL, HOPS>;
     cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
@@ -29,8 +29,9 @@ static cudaError_t launch_hops(const WaveParams& p, int nq, int threads, size_t 
 
 template <int WT, int PRED, bool CL>
 static cudaError_t launch_one(const WaveParams& p, int nq, int threads, size_t smem, cudaStream_t stream) {
-    return p.hops > 1 ? launch_hops<WT, PRED, CL, true>(p, nq, threads, smem, stream)
-                      : launch_hops<WT, PRED, CL, false>(p, nq, threads, smem, stream);
+    if (p.quads && p.hops > 1) return launch_hops<WT, PRED, CL, kHopsQuads>(p, nq, threads, smem, stream);
+    return p.hops > 1 ? launch_hops<WT, PRED, CL, 1>(p, nq, threads, smem, stream)
+                      : launch_hops<WT, PRED, CL, 0>(p, nq, threads, smem, stream);
 }
 
 template <int WT, int PRED>
@@ -44,9 +45,10 @@ static cudaError_t launch_tide_one(const WaveParams& p, int grid, int threads, c
     at[0].val.cooperative = 1;
     c.attrs = at;
     c.numAttrs = 1;
-    if (p.mid || p.pull) return cudaLaunchKernelEx(&c, tide_kernel<WT, PRED, false, true>, p);
-    return p.hops > 1 ? cudaLaunchKernelEx(&c, tide_kernel<WT, PRED, true, false>, p)
-                      : cudaLaunchKernelEx(&c, tide_kernel<WT, PRED, false, false>, p);
+    if (p.mid || p.pull) return cudaLaunchKernelEx(&c, tide_kernel<WT, PRED, 0, true>, p);
+    if (p.quads && p.hops > 1) return cudaLaunchKernelEx(&c, tide_kernel<WT, PRED, kHopsQuads, false>, p);
+    return p.hops > 1 ? cudaLaunchKernelEx(&c, tide_kernel<WT, PRED, 1, false>, p)
+                      : cudaLaunchKernelEx(&c, tide_kernel<WT, PRED, 0, false>, p);
 }
 
 cudaError_t launch_tide(int wt, int pred, const WaveParams& p, int grid, int threads, cudaStream_t stream) {

@@ -492,3 +492,31 @@ def test_levels_pulled(kind):
         torch.cuda.synchronize()
         assert torch.equal(lev, lev2)
     G.close()
+
+
+@pytest.mark.parametrize("n", [33, 5000, 1_100_000])
+@pytest.mark.parametrize("wtype", ["u32", "f32"])
+def test_thin_rows_around_four(n, wtype):
+    """Meshes whose rows have none to nine arcs, four of them at a fixed place:
+    one cluster and the whole grid, one query and a batch, levels."""
+    rng = np.random.default_rng(n)
+    deg = np.where(rng.random(n) < 0.9, 4, rng.integers(0, 10, n))
+    deg[[0, n - 1]] = 5, 9
+    rp = np.concatenate([[0], np.cumsum(deg)]).astype(np.int32)
+    m = int(rp[-1])
+    u = np.repeat(np.arange(n), deg)
+    col = ((u + rng.choice([-40, -2, -1, 1, 3, 40], m)) % n).astype(np.int32)
+    w = rng.integers(1, 60, m)
+    g = gg.Graph("mesh", n, m, rp, col, (w / 8.0).astype(np.float32) if wtype == "f32" else w.astype(np.uint32), wtype)
+    both(g, n // 2)
+    G = upload(g)
+    srcs = np.array([0, n - 1, n // 3], np.int32)
+    if n <= 5000:
+        d, p = gpu_batch(G, srcs, pred=True)
+        assert_exact_many(g, srcs, d, p)
+    lev = torch.empty(n, dtype=torch.int32, device="cuda")
+    G.bfs(0, lev, None)
+    torch.cuda.synchronize()
+    ref = oracle.dijkstra_u32(rp, col, np.ones(m, np.uint32), 0)
+    np.testing.assert_array_equal(lev.cpu().numpy().view(np.uint32), ref)
+    G.close()
