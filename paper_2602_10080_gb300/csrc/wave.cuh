@@ -135,6 +135,26 @@ __device__ __forceinline__ void st_cluster(uint32_t a, uint32_t v) {
     asm volatile("st.relaxed.cluster.shared::cluster.u32 [%0], %1;" ::"r"(a), "r"(v) : "memory");
 }
 
+// Stores of a batch, predicated by hand where most of them happen (thin fronts:
+// a branch around each costs more than the store) or behind a branch where
+// few arcs improve anything (R-MAT-22 loses 6% without it).
+template <bool PREDICATED, typename V>
+__device__ __forceinline__ void red_min_if(bool on, V* p, V v) {
+    if constexpr (!PREDICATED) {
+        if (on) red_min(p, v);
+    } else if constexpr (sizeof(V) == 4) {
+        asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %2, 0;\n\t@p red.relaxed.gpu.global.min.u32 [%0], %1;\n\t}"
+                     ::"l"(p), "r"(v), "r"((uint32_t)on) : "memory");
+    } else {
+        asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %2, 0;\n\t@p red.relaxed.gpu.global.min.u64 [%0], %1;\n\t}"
+                     ::"l"(p), "l"(v), "r"((uint32_t)on) : "memory");
+    }
+}
+__device__ __forceinline__ void st_shared_if(bool on, uint32_t a, uint32_t x, uint32_t y) {
+    asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %3, 0;\n\t@p st.shared.v2.u32 [%0], {%1, %2};\n\t}"
+                 ::"r"(a), "r"(x), "r"(y), "r"((uint32_t)on) : "memory");
+}
+
 // T raised above `base` by delta, and at least above `low` (an f32 delta may
 // be absorbed, a u32 sum saturates)
 template <int WT>
@@ -202,6 +222,20 @@ struct Wave {
         else asm volatile("red.relaxed.cta.shared::cta.or.b32 [%0], %1;" ::"r"(a), "r"(v) : "memory");
     }
 
+    __device__ __forceinline__ void red_or_if(bool on, Addr a, uint32_t v) const {
+        if constexpr (MODE == kWaveGrid)
+            asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %2, 0;\n\t@p red.relaxed.gpu.global.or.b32 [%0], %1;\n\t}"
+                         ::"l"(a), "r"(v), "r"((uint32_t)on) : "memory");
+        else if constexpr (MODE == kWaveCluster)
+            asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %2, 0;\n\t"
+                         "@p red.relaxed.cluster.shared::cluster.or.b32 [%0], %1;\n\t}"
+                         ::"r"(a), "r"(v), "r"((uint32_t)on) : "memory");
+        else
+            asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %2, 0;\n\t"
+                         "@p red.relaxed.cta.shared::cta.or.b32 [%0], %1;\n\t}"
+                         ::"r"(a), "r"(v), "r"((uint32_t)on) : "memory");
+    }
+
     // Relaxes K arcs (u at distance du) -> a.x of weight a.y whose distance
     // words are c: lowers dist[v] without waiting for the answer and marks v
     // when the distance beat the loaded one (whoever lowers dist[v] saw a
@@ -230,12 +264,12 @@ struct Wave {
 #pragma unroll
         for (int k = 0; k < K; k++) {
             if (PRED == 0) {
-                if (upd[k]) red_min(reinterpret_cast<uint32_t*>(dist) + a[k].x, nd[k]);
+                red_min_if<HOPS != 0>(upd[k], reinterpret_cast<uint32_t*>(dist) + a[k].x, nd[k]);
             } else {
                 unsigned long long* p = reinterpret_cast<unsigned long long*>(dist) + a[k].x;
                 const unsigned long long cand = ((unsigned long long)nd[k] << 32) | u[k];
                 if (PRED == 1) {
-                    if (upd[k]) red_min(p, cand);
+                    red_min_if<HOPS != 0>(upd[k], p, cand);
                 } else {
                     unsigned long long x = (unsigned long long)c[k];
                     while (imp[k]) {
@@ -247,20 +281,49 @@ struct Wave {
                 }
             }
         }
+        if constexpr (!(OWN && HOPS != 0)) {
+#pragma unroll
+            for (int k = 0; k < K; k++) {
+                const bool near = imp[k] && nd[k] < T;
+                fmin = imp[k] && !near ? min(fmin, nd[k]) : fmin;
+                if (imp[k]) red_or(ad[k], mask[k]);
+                n_imp += near ? 1u : 0u;
+            }
+            return;
+        }
+        bool near[K], mark[K];
+        uint32_t b[K];
 #pragma unroll
         for (int k = 0; k < K; k++) {
-            bool near = imp[k] && nd[k] < T;
-            fmin = imp[k] && !near ? min(fmin, nd[k]) : fmin;
-            if (OWN && HOPS && keep) {
-                const uint32_t b = __ballot_sync(kFull, near), at = n_own + __popc(b & lanemask_lt());
-                n_own = min(kWaveOwn, n_own + (uint32_t)__popc(b));
-                if (near && at < kWaveOwn) {
-                    lists->own[own_w][at] = make_uint2(a[k].x, nd[k]);
-                    near = imp[k] = false;
-                }
+            near[k] = imp[k] && nd[k] < T;
+            mark[k] = imp[k];
+            fmin = imp[k] && !near[k] ? min(fmin, nd[k]) : fmin;
+            b[k] = __ballot_sync(kFull, near[k]);
+        }
+        if (keep) {
+            // what the warp keeps for its next hop is not marked
+            const uint32_t list = (uint32_t)__cvta_generic_to_shared(lists->own[own_w]), lt = lanemask_lt();
+            uint32_t at[K], room[K];
+#pragma unroll
+            for (int k = 0; k < K; k++) {
+                at[k] = __popc(b[k] & lt);
+                room[k] = __popc(b[k]);
             }
-            if (imp[k]) red_or(ad[k], mask[k]);
-            n_imp += near ? 1u : 0u;
+#pragma unroll
+            for (int k = 0; k < K; k++) {
+                at[k] += n_own;
+                n_own += room[k];
+                const bool kept = near[k] && at[k] < kWaveOwn;
+                st_shared_if(kept, list + at[k] * 8u, a[k].x, nd[k]);
+                near[k] = near[k] && !kept;
+                mark[k] = mark[k] && !kept;
+            }
+            n_own = min(n_own, kWaveOwn);
+        }
+#pragma unroll
+        for (int k = 0; k < K; k++) {
+            red_or_if(mark[k], ad[k], mask[k]);
+            n_imp += near[k] ? 1u : 0u;
         }
     }
 
@@ -283,16 +346,17 @@ struct Wave {
         relax<4, OWN>(uu, dd, a, c, in);
     }
 
-    // Arcs g0 + lane + 32 k (k < 4) of the warp's concatenated rows (ex: arcs
+    // Arcs g0 + lane + 32 k (k < K) of the warp's concatenated rows (ex: arcs
     // before this lane's vertex u, row at rs, distance du).
+    template <int K>
     __device__ __forceinline__ void arcs_packed(int32_t g0, int32_t total, int32_t ex, int32_t rs, uint32_t du,
                                                 uint32_t u) {
-        uint2 a[4];
-        DistT c[4];
-        uint32_t dj[4], uj[4];
-        bool in[4];
+        uint2 a[K];
+        DistT c[K];
+        uint32_t dj[K], uj[K];
+        bool in[K];
 #pragma unroll
-        for (int k = 0; k < 4; k++) {
+        for (int k = 0; k < K; k++) {
             const int32_t g = g0 + 32 * k + (int32_t)lane_id();
             int j = 0;
 #pragma unroll
@@ -305,13 +369,13 @@ struct Wave {
             a[k] = in[k] ? ld_arc(P.adj + row) : make_uint2(0u, 0u);
         }
 #pragma unroll
-        for (int k = 0; k < 4; k++) c[k] = in[k] ? ld_dist(dist + a[k].x) : (DistT)0;
-        relax<4, true>(uj, dj, a, c, in);
+        for (int k = 0; k < K; k++) c[k] = in[k] ? ld_dist(dist + a[k].x) : (DistT)0;
+        relax<K, true>(uj, dj, a, c, in);
     }
 
     // Whether vertex v, of the last hop at distance d or from the words (d
     // infinite), is still to be relaxed, and d: its distance `now`.
-    __device__ __forceinline__ bool claim(uint32_t v, bool is_far, uint32_t now, uint32_t& d) {
+    __device__ __forceinline__ bool claim(uint32_t v, bool is_far, uint32_t now, uint32_t& d, bool marks = true) {
         // improved meanwhile: whoever did marked it again
         if (d != kInfU32) return now >= d;
         d = now;
@@ -321,9 +385,42 @@ struct Wave {
         if (d < T) return true;
         uint32_t mask;
         const Addr a = bit_addr(far_w, v, mask);
-        red_or(a, mask);
+        if (marks) red_or(a, mask);
         fmin = min(fmin, d);
         return false;
+    }
+
+    // A batch of up to eight vertices, an arc a lane (lanes 4 j to 4 j + 3 have
+    // vertex j): on a thin front a batch has three on average, and the chain of
+    // instructions from the answers to the next hop is a third as long.
+    __device__ __forceinline__ void relax_narrow(bool have, uint32_t v, bool is_far, uint32_t d) {
+        const uint32_t k = lane_id() & 3u;
+        uint2 a[1] = {make_uint2(kNoArc, 0u)};
+        uint32_t now = kInfU32;
+        if (have) {
+            a[0] = ld_arc(reinterpret_cast<const uint2*>(P.quads) + 4 * (size_t)v + k);
+            now = dpart(ld_dist(dist + v));
+        }
+        const bool more = k == 0u && (a[0].x >> 31) != 0u;
+        a[0].x &= kNoArc;
+        bool in[1] = {a[0].x != kNoArc};
+        const DistT c[1] = {in[0] ? ld_dist(dist + a[0].x) : (DistT)0};
+        if (have) have = claim(v, is_far, now, d, k == 0u);
+        in[0] = in[0] && have;
+        n_relax += in[0] ? 1u : 0u;
+        const uint32_t uu[1] = {v}, dd[1] = {d};
+        relax<1, true>(uu, dd, a, c, in);
+        rest_of(v, d, have && more);
+    }
+    // The arcs after the fourth of the vertices of lanes `more`.
+    __device__ __forceinline__ void rest_of(uint32_t v, uint32_t d, bool more) {
+        if (__any_sync(kFull, more)) {
+            int2 sp = more ? __ldg(P.span + v) : make_int2(0, 0);
+            sp.x = min(sp.x + 4, sp.y);
+            n_relax += (uint32_t)(sp.y - sp.x);
+            for (; __any_sync(kFull, sp.x < sp.y); sp.x += 4) arcs4<true>(v, d, sp.x, 1, sp.y);
+        }
+        __syncwarp();
     }
 
     // A batch of relax_batch whose first four arcs lie at a fixed place: two
@@ -356,13 +453,7 @@ struct Wave {
             n_relax += in[k] ? 1u : 0u;
         }
         relax<4, true>(uu, dd, a, c, in);
-        if (__any_sync(kFull, have && more)) {
-            int2 sp = have && more ? __ldg(P.span + v) : make_int2(0, 0);
-            sp.x = min(sp.x + 4, sp.y);
-            n_relax += (uint32_t)(sp.y - sp.x);
-            for (; __any_sync(kFull, sp.x < sp.y); sp.x += 4) arcs4<true>(v, d, sp.x, 1, sp.y);
-        }
-        __syncwarp();
+        rest_of(v, d, have && more);
     }
 
     // Relaxes up to 32 vertices, one per lane (`have`): from the words
@@ -370,10 +461,11 @@ struct Wave {
     // last hop.  `hub(v, d, arcs, deg)` takes those with more than hub_deg arcs
     // (it returns the arcs that are left to the warp).
     template <typename Hub>
-    __device__ __forceinline__ void relax_batch(bool have, uint32_t v, bool is_far, uint32_t d, Hub&& hub) {
+    __device__ __forceinline__ void relax_batch(bool have, uint32_t v, bool is_far, uint32_t d, bool narrow, Hub&& hub) {
         const uint32_t lane = lane_id();
         if constexpr (HOPS == kHopsQuads) {
-            relax_quads(have, v, is_far, d);
+            if (narrow) relax_narrow(have, v, is_far, d);
+            else relax_quads(have, v, is_far, d);
             return;
         }
         int2 sp = make_int2(0, 0);
@@ -403,7 +495,8 @@ struct Wave {
                 if (lane >= (uint32_t)o) incl += x;
             }
             const int32_t ex = incl - deg, total = __shfl_sync(kFull, incl, 31);
-            for (int32_t g0 = 0; g0 < total; g0 += 128) arcs_packed(g0, total, ex, sp.x, d, v);
+            if (!P.has_hubs && total <= 32) arcs_packed<1>(0, total, ex, sp.x, d, v);
+            else for (int32_t g0 = 0; g0 < total; g0 += 128) arcs_packed<4>(g0, total, ex, sp.x, d, v);
         }
         __syncwarp();
     }
@@ -426,7 +519,7 @@ struct Wave {
         if (more) take(base + lane, nb, fb);
         for (;;) {
             uint32_t v = 0u, d = kInfU32;
-            bool have = false, is_far = false;
+            bool have = false, is_far = false, narrow = false;
             while (more && held < 32u) {
                 const bool got = (nb | fb) != 0u;
                 const uint32_t m = __ballot_sync(kFull, got);
@@ -449,14 +542,18 @@ struct Wave {
             if (held) {
                 const uint32_t k = held < 32u ? held : 32u;
                 held -= k;
-                have = lane < k;
-                if (have) v = lists->list[held + lane];
+                narrow = HOPS == kHopsQuads && k <= 8u;
+                const uint32_t j = narrow ? lane >> 2 : lane;
+                have = j < k;
+                if (have) v = lists->list[held + j];
                 is_far = (v >> 31) != 0u;
                 v &= 0x7fffffffu;
             } else if (HOPS && pos < own) {
-                have = pos + lane < own;
+                narrow = HOPS == kHopsQuads && own - pos <= 8u;
+                const uint32_t j = pos + (narrow ? lane >> 2 : lane);
+                have = j < own;
                 if (have) {
-                    const uint2 e = lists->own[own_w ^ 1u][pos + lane];
+                    const uint2 e = lists->own[own_w ^ 1u][j];
                     v = e.x;
                     d = e.y;
                 }
@@ -471,7 +568,7 @@ struct Wave {
                 __syncwarp();
                 continue;
             }
-            relax_batch(have, v, is_far, d, hub);
+            relax_batch(have, v, is_far, d, narrow, hub);
         }
     }
 
