@@ -629,7 +629,9 @@ struct Wave {
                 from = a.x;
             }
         };
-        const bool by_warp = deg > 64;
+        // (longer rows by the whole warp: R-MAT-22 us at 64, 32, 16, 8 622, 607, 576,
+        // 598; R-MAT-20 274, 262, 255, 262)
+        const bool by_warp = deg > 16;
         // (of a level, any parent gives the distance)
         for (int32_t e = 0; !by_warp && e < deg && !(PRED == 0 && P.unit && best != none); e += 4) {
             uint2 a[4];
