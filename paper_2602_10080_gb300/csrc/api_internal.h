@@ -162,6 +162,9 @@ inline WaveGraph wave_graph(const Graph* g) {
     return WaveGraph{g->n, g->m, g->feat.avg_w, g->feat.max_deg, g->sms, g->wide.load(),
                      g->light_first && g->light_share >= 0.02 && g->light_share <= 0.4};
 }
+// The graph's part of the multi-source kernel's parameters.
+struct FanParams;
+void fan_graph(const Graph* g, FanParams* p);
 // The wavefront kernels (sssp_wave.cu), for calls that leave the configuration
 // to the library.  kWaveNotRun: the graph or the call is not for them.
 constexpr int kWaveNotRun = 1;

@@ -925,8 +925,7 @@ int express_launch(sssp_server* s, Lane* L) {
         if (plan.kind == kSideBySide) {
             F.nq = k;
             F.srcs = J->srcs;
-            F.span = g->span;
-            F.adj = g->adj;
+            fan_graph(g, &F);
             F.ctrl = J->ctrl;
             F.timeout_ns = 20000ull * 1000000ull;
             e = launch_fan(f32 ? 1 : 0, F, s->sms, J->stream);

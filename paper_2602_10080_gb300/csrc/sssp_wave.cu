@@ -177,6 +177,16 @@ void fan_carve(uint32_t* words, uint4* slices, int32_t n, int64_t m, bool pred, 
     p->rows = slices + (m / kFanChunk + m / kFanShort + 1);
 }
 
+void fan_graph(const Graph* g, FanParams* p) {
+    p->span = g->span;
+    p->adj = g->adj;
+    if (wave_graph(g).core) {
+        p->mid = g->mid;
+        p->light_w = g->light_w;
+        p->core_deg = kFanCoreArcs;
+    }
+}
+
 std::mutex& grid_mutex(int device) {
     static std::mutex mu[64];
     return mu[device & 63];
@@ -199,14 +209,8 @@ int run_fan(Graph* g, const int32_t* srcs_host, const int32_t* srcs_dev, int32_t
     FanParams P;
     std::memset(&P, 0, sizeof(P));
     fan_carve(ws.fan, ws.fan_slices, g->n, g->m, pred_out != nullptr, &P);
-    P.span = g->span;
-    P.adj = g->adj;
+    fan_graph(g, &P);
     P.ctrl = ws.ctrl;
-    if (wave_graph(g).core) {
-        P.mid = g->mid;
-        P.light_w = g->light_w;
-        P.core_deg = kFanCoreArcs;
-    }
     P.timeout_ns = 20000ull * 1000000ull;
     const int32_t groups = (nq + 31) / 32, per = (nq + groups - 1) / groups;
     for (int32_t q0 = 0; q0 < nq; q0 += per) {
