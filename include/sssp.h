@@ -404,11 +404,12 @@ SSSP_API int sssp_bfs(sssp_graph *g, int32_t src, uint32_t *level_out, int32_t *
  * graph's delta (it holds many queries under load).  Lanes of different graphs
  * run concurrently on their own streams, sharing the SMs.
  *
- * Queries that the wavefront kernels finish within about a slice are run to
+ * Queries that the wavefront kernels finish within a few slices are run to
  * their end instead (without per-query timeouts and test flags): on a graph
- * of at most 2^19 arcs a cluster of blocks each, the waiting ones in one
- * launch beside those that run; on a larger graph that is not a mesh 12 to 32
- * waiting ones side by side, or one by one, with the whole device. */
+ * of at most 2^19 arcs, and on a mesh unless slice_us is below its default, a
+ * cluster of blocks each, the waiting ones in one launch beside those that
+ * run; on a larger graph up to 32 waiting ones side by side, or one by one,
+ * with the whole device. */
 typedef struct sssp_serve_options {
     size_t  mem_budget_bytes;  /* device bytes for distance slices and L2 rings of all lanes
                                   (0 = a quarter of the free device memory at creation) */

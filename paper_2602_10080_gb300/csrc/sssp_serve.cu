@@ -27,9 +27,11 @@
 // timeout has to end a running query) is an express lane: it takes the
 // queries that wait as one job on a stream of its own, to the end -- one
 // cluster per query on small graphs, several jobs at a time; on larger graphs
-// one job at a time, 12 to 32 waiting queries side by side, fewer one by one.
-// Long queries (meshes of more than 2^19 arcs) keep the slices.  24 queries on
-// R-MAT-18 at once (GB300): 2.3 ms, 12.1 in slices.
+// one job at a time, several waiting queries side by side (plan_wave), few one by one.
+// A mesh of more than 2^19 arcs holds its cluster for milliseconds (grid 1024^2
+// 3.0): where the server asks for shorter slices than the usual ones, it keeps
+// the slices.  GB300, queries at once: 24 on R-MAT-18 1.4 ms, 12.1 in slices;
+// 24 on grid 500 x 512 2.9, 42; 4 on grid 400 x 500 1.6, 20.
 #include <algorithm>
 #include <atomic>
 #include <chrono>
@@ -52,6 +54,8 @@ namespace sssp {
 namespace {
 
 using Clock = std::chrono::steady_clock;
+
+constexpr int32_t kSliceUs = 1000;   // sssp_serve_options_default
 
 // ------------------------------------------------------------- kernels --
 
@@ -559,6 +563,15 @@ int lane_grow_slots(sssp_server* s, Lane* L, uint32_t want) {
     return SSSP_OK;
 }
 
+// Whether the budget holds a new lane's first slots, rings and results.
+bool lane_slices_fit(const sssp_server* s, const Lane* L) {
+    const uint32_t slots = std::min<uint32_t>(8, L->cap_limit);
+    const size_t work = (size_t)slots * ((size_t)L->g->nv * L->cell + 4 + 8 + 4) + 8;
+    const size_t rings = ring_bytes_for((uint32_t)(L->plan.P.bmax * L->plan.P.shards), lane_initial_nch(s, L, slots));
+    const size_t results = L->pred_mode ? (size_t)L->g->n * 8 : 0;
+    return s->used + work + rings + results <= s->budget;
+}
+
 Lane* lane_create(sssp_server* s, Graph* g, int pred_mode, int* rc) {
     Lane* L = new (std::nothrow) Lane();
     if (!L) {
@@ -599,12 +612,13 @@ Lane* lane_create(sssp_server* s, Graph* g, int pred_mode, int* rc) {
     }
     while (L->vbits < 31 && (1ll << L->vbits) <= (long long)g->nv) L->vbits++;  // 2^vbits > nv
     L->cap_limit = (uint32_t)std::min<uint64_t>((uint64_t)s->opt.max_slots, 1ull << (32 - L->vbits));
-    {
-        WavePlan w;
-        L->express = s->opt.flags == 0 && s->opt.query_timeout_ms == 0 && plan_wave(wave_graph(g), 1, pred_mode, &w) &&
-                     (w.kind == kWholeGrid || g->m <= (1 << 19));
-    }
     L->cell = pred_mode ? 8 : 4;
+    {
+        // (a budget that refuses the lane's slices refuses the lane)
+        WavePlan w;
+        L->express = lane_slices_fit(s, L) && s->opt.flags == 0 && s->opt.query_timeout_ms == 0 && plan_wave(wave_graph(g), 1, pred_mode, &w) &&
+                     (w.kind == kWholeGrid || g->m <= (1 << 19) || s->opt.slice_us >= kSliceUs);
+    }
     L->idle_since = Clock::now();
     if (cudaStreamCreateWithFlags(&L->stream, cudaStreamNonBlocking) != cudaSuccess ||
         cudaEventCreate(&L->k0) != cudaSuccess || cudaEventCreate(&L->k1) != cudaSuccess ||
@@ -882,6 +896,7 @@ int express_launch(sssp_server* s, Lane* L) {
             if (!rc) fan_carve(J->words, J->slices, g->n, g->m, pred, &F);
         } else if (!rc) {
             smem = wave_params(plan, wg, f32, false, &P);
+            P.wide = kInfU32;   // (a job does not start over)
             if (smem > kWaveMaxShared) rc = SSSP_E_NOMEM;
             if (!rc && pred) rc = job_room(s, J, &J->work, &J->work_n, cells);
             if (!rc && grid) {
@@ -1417,7 +1432,7 @@ extern "C" int sssp_serve_options_default(sssp_serve_options* opt) {
     std::memset(opt, 0, sizeof(*opt));
     opt->mem_budget_bytes = 0;
     opt->max_slots = 128;
-    opt->slice_us = 1000;
+    opt->slice_us = sssp::kSliceUs;
     opt->max_queued = 65536;
     opt->ring_shift = 4;
     opt->query_timeout_ms = 0;

@@ -520,3 +520,32 @@ def test_thin_rows_around_four(n, wtype):
     ref = oracle.dijkstra_u32(rp, col, np.ones(m, np.uint32), 0)
     np.testing.assert_array_equal(lev.cpu().numpy().view(np.uint32), ref)
     G.close()
+
+
+@pytest.mark.parametrize("slice_us", [1000, 100])
+@pytest.mark.parametrize("kind", ["grid", "ring"])
+def test_served_meshes(kind, slice_us):
+    """Meshes of more than 2^19 arcs: as jobs, and in slices where the server
+    asks for short ones; a random graph of equal degrees, whose front is wide."""
+    if kind == "grid":
+        g = gg.grid(401, 390, 1, 100, seed=2)
+    else:
+        rng = np.random.default_rng(5)
+        n, k = 150_000, 4
+        col = np.concatenate([rng.permutation(n) for _ in range(k)]).reshape(k, n).T.ravel().astype(np.int32)
+        g = gg.Graph("ring", n, n * k, (np.arange(n + 1) * k).astype(np.int32), col,
+                     rng.integers(1, 100, n * k).astype(np.uint32), "u32")
+    assert g.m > 1 << 19
+    G = upload(g)
+    srcs = [0, 77, g.n - 1, g.n // 2, 77]
+    srv = S.sssp_serve_create(slice_us=slice_us)
+    try:
+        d = torch.empty((len(srcs), g.n), dtype=torch.int32, device="cuda")
+        p = torch.empty((len(srcs), g.n), dtype=torch.int32, device="cuda")
+        tickets = [S.sssp_serve_submit(srv, G.handle, s, d[i], p[i]) for i, s in enumerate(srcs)]
+        for t in tickets:
+            assert S.sssp_serve_wait(srv, t, 60000)[0] == S.Q_DONE
+    finally:
+        S.sssp_serve_destroy(srv)
+    assert_exact_many(g, np.array(srcs), d.cpu().numpy().view(np.uint32), p.cpu().numpy())
+    G.close()
