@@ -461,21 +461,27 @@ int fill_span(Graph* g, cudaStream_t s) {
     unsigned long long* lights = nullptr;
     unsigned long long h = 0;
     if (g->light_first) {
+        // (without room for them the share of light arcs stays 0, which turns
+        // the core search off)
         if ((!g->mid && cudaMalloc((void**)&g->mid, sizeof(int32_t) * (size_t)g->n) != cudaSuccess) ||
             cudaMalloc((void**)&lights, sizeof(*lights)) != cudaSuccess) {
             cudaGetLastError();
-            return SSSP_E_NOMEM;
+            lights = nullptr;
+        } else {
+            cudaMemsetAsync(lights, 0, sizeof(*lights), s);
         }
-        cudaMemsetAsync(lights, 0, sizeof(*lights), s);
     }
     const int64_t blocks = std::min<int64_t>(((int64_t)g->n + 255) / 256, (int64_t)g->sms * 8);
     span_kernel<<<(int)std::max<int64_t>(1, blocks), 256, 0, s>>>(g->row_ptr, g->adj, g->n, g->span, g->light_w,
-                                                                  g->light_first ? g->mid : nullptr, lights);
-    // (the quads of a mesh only save time: without room for them, without them)
-    if (thin_graph(g->feat.avg_deg, g->feat.max_deg) &&
-        (g->quads || cudaMalloc((void**)&g->quads, 2 * sizeof(uint4) * (size_t)g->n) == cudaSuccess))
-        quads_kernel<<<(int)std::max<int64_t>(1, blocks), 256, 0, s>>>(g->span, g->adj, g->n, g->quads);
-    else cudaGetLastError();
+                                                                  lights ? g->mid : nullptr, lights);
+    if (thin_graph(g->feat.avg_deg, g->feat.max_deg)) {
+        if (!g->quads && cudaMalloc((void**)&g->quads, 2 * sizeof(uint4) * (size_t)g->n) != cudaSuccess) {
+            // they only save time: without room for them, without them
+            cudaGetLastError();
+            g->quads = nullptr;
+        }
+        if (g->quads) quads_kernel<<<(int)std::max<int64_t>(1, blocks), 256, 0, s>>>(g->span, g->adj, g->n, g->quads);
+    }
     if (lights) cudaMemcpyAsync(&h, lights, sizeof(h), cudaMemcpyDeviceToHost, s);
     const cudaError_t e = cudaStreamSynchronize(s);
     cudaFree(lights);
