@@ -160,7 +160,8 @@ int run_queries(Graph* g, const int32_t* srcs_host, const int32_t* srcs_dev, int
 
 inline WaveGraph wave_graph(const Graph* g) {
     return WaveGraph{g->n, g->m, g->feat.avg_w, g->feat.max_deg, g->sms, g->wide.load(),
-                     g->light_first && g->light_share >= 0.02 && g->light_share <= 0.4};
+                     g->light_first && g->light_share >= 0.02 && g->light_share <= 0.4,
+                     g->light_first && g->light_share >= 0.02 && g->light_share <= 0.15};
 }
 // The graph's part of the multi-source kernel's parameters.
 struct FanParams;

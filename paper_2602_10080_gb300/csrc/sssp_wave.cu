@@ -43,9 +43,10 @@ bool plan_wave(const WaveGraph& g, int32_t nq, int pred_mode, WavePlan* w) {
     // (few arcs a vertex, and none with many more: in a sparse random graph
     // some vertex has over twice the average).  There a warp goes on for several
     // hops a step with the vertices that it improved itself, and the threshold
-    // moves as far.  us at 1, 4, 6 and 8 hops (width x4): grid 256^2 1132, 825,
-    // 797, 775; grid 1024^2 6150, 4139, 4021, 3835; road 900 x 777 1893, 1378,
-    // 1414, 1404; grid 64 x 60 285, 220, -, 215.  Elsewhere a second hop may pay
+    // moves as far.  us at 1, 4, 6 and 8 hops (width x4) before the quads: grid
+    // 256^2 1132, 825, 797, 775; grid 1024^2 6150, 4139, 4021, 3835; road 900 x 777
+    // 1893, 1378, 1414, 1404; grid 64 x 60 285, 220, -, 215; with them, at 6, 8 and
+    // 12: grid 256^2 586, 577, 625; grid 1024^2 -, 2960, 3240.  Elsewhere a second hop may pay
     // (directed 60000 vertices of degree 6 174, 150 at 2, 255 at 8; G(10^4, 10^5)
     // 128, 115 at 2) but not on the smallest graphs (directed 10^4 vertices 102,
     // 114 at 2), nor with hubs (R-MAT-13 164, 189 at 2).
@@ -71,11 +72,12 @@ bool plan_wave(const WaveGraph& g, int32_t nq, int pred_mode, WavePlan* w) {
         if (hubs) {
             // power law: the arcs of the core are the work.  Without them the
             // steps count on all but the largest graphs, us without (with) the
-            // core's heavy arcs: R-MAT-22 637 (1786), at width 1 and a wider light
-            // bound 15% slower, at 1/4 6%; R-MAT-20 270 (920); R-MAT-18 195 (378);
-            // R-MAT-16 160 (303); R-MAT-19 f32 280 (626).  A graph whose core does
-            // not settle in time (weights up to 15) loses 8%
-            w->core = g.core;
+            // core's heavy arcs: R-MAT-22 565 (1786), at width 1 and a wider light
+            // bound 15% slower, at 1/4 6%; R-MAT-20 255 (920); R-MAT-18 188 (378);
+            // R-MAT-16 160 (303); R-MAT-19 f32 275 (626).  With a fifth of the arcs
+            // light (weights up to 15) the core does not settle in time: R-MAT-21
+            // 588 (556), R-MAT-18 299 (263), so it is left out above 15%
+            w->core = g.core_one;
             w->delta *= g.m > (1 << 25) ? 0.5 : 1.0;
             w->front = g.m > (w->core ? 1 << 24 : 1 << 25) ? 1u : 256u;
             // a larger slice saves listing, a smaller one spreads better: R-MAT-22

@@ -34,7 +34,9 @@ struct WaveGraph {
     double avg_w, max_deg;
     int sms;
     bool wide;
-    bool core;             // symmetric, hubs, rows with their light arcs (a fair share of all) first
+    // symmetric, hubs, rows with their light arcs first: for a batch side by
+    // side, and (few light arcs) for one query
+    bool core, core_one;
 };
 
 constexpr int kTideLogWords = 17;               // the grid kernel spreads the places over at least 2^17 words
