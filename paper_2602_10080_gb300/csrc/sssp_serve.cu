@@ -1363,13 +1363,13 @@ void worker_main(sssp_server* s) {
             }
         }
         admit(s);
+        int rc = launch_ready(s);
         {
-            int resident = 0;
+            int resident = 0;   // those of jobs just launched too
             for (Lane* L : s->lanes) resident += L->running;
             std::lock_guard<std::mutex> lk(s->mu);
             s->stats.max_resident = std::max<int64_t>(s->stats.max_resident, resident);
         }
-        int rc = launch_ready(s);
         // wait for any lane's slice (lanes run on their own streams); come
         // back now and then for new submissions to idle lanes
         const Clock::time_point t0 = Clock::now();

@@ -95,18 +95,22 @@ bool plan_wave(const WaveGraph& g, int32_t nq, int pred_mode, WavePlan* w) {
     }
     // a batch on a small graph or a mesh: one cluster per query, as wide as the
     // queries leave room for (13 queries on grid 301 x 257: 8 blocks 1690 us,
-    // 4: 1880, 1: 2130)
-    if (g.n > kClusterVertices || g.m > (1 << 21) || (hubs && g.m > (1 << 18))) {
+    // 4: 1880, 1: 2130; 20 queries on grid 900 x 1000 16: 8465, 8: 5820, 4: 6030).
+    // A mesh too large for that goes one by one: side by side, by hops, 20 queries
+    // on grid 900 x 1000 take 167 ms.
+    const bool mesh = thin && !g.wide;
+    if (g.n > kClusterVertices || (!mesh && (g.m > (1 << 21) || (hubs && g.m > (1 << 18))))) {
         // A group of up to 32 queries side by side costs as much as this many
         // in turn on the whole grid: R-MAT-20 6 (1.40 ms), R-MAT-18 5 (0.93 ms),
         // with all arcs 7, G(200K, 2M) 14 (2.6 ms).  Predecessors of the
         // strict-improvement rule cannot be found after the distances and stay
         // with the queues.
-        if (nq < (g.core ? 6 : hubs ? 8 : 14)) w->kind = kInTurn;
+        if (mesh || nq < (g.core ? 6 : hubs ? 8 : 14)) w->kind = kInTurn;
         else if (pred_mode != 2 && g.n <= kFanMaxVertices) w->kind = kSideBySide;
         else return false;
         return true;
     }
+    if (g.m > (1 << 21)) w->wide = 24576u;
     w->log_g = 4;
     const size_t pending = pow2_at_least((double)g.n) / 2;
     while (w->log_g > 0 && (nq << w->log_g) > g.sms && pending >> (w->log_g - 1) <= kWaveMaxShared) w->log_g--;

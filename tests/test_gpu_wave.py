@@ -549,3 +549,30 @@ def test_served_meshes(kind, slice_us):
         S.sssp_serve_destroy(srv)
     assert_exact_many(g, np.array(srcs), d.cpu().numpy().view(np.uint32), p.cpu().numpy())
     G.close()
+
+
+def test_batches_on_large_meshes():
+    """A cluster per query on a mesh of more than 2^21 arcs, and one by one
+    beyond a cluster's vertices; a random graph of equal degrees starts over."""
+    g = gg.grid(760, 740, 1, 50, seed=3)
+    assert g.m > 1 << 21
+    srcs = np.arange(15) * 37_000
+    G = upload(g)
+    d, p = gpu_batch(G, srcs, pred=True)
+    assert_exact_many(g, srcs, d, p)
+    G.close()
+    rng = np.random.default_rng(5)
+    n, k = 560_000, 4
+    col = np.concatenate([rng.permutation(n) for _ in range(k)]).reshape(k, n).T.ravel().astype(np.int32)
+    w = rng.integers(1, 100, n * k).astype(np.uint32)
+    h = gg.Graph("regular", n, n * k, (np.arange(n + 1) * k).astype(np.int32), col, w, "u32")
+    G = upload(h)
+    for _ in range(2):
+        d, p = gpu_batch(G, srcs, pred=True)
+        assert_exact_many(h, srcs, d, p)
+    G.close()
+    big = gg.grid(1100, 1000, 1, 50, seed=4)
+    G = upload(big)
+    d, _ = gpu_batch(G, srcs, pred=False)
+    assert_exact_many(big, srcs, d, None)
+    G.close()
