@@ -58,9 +58,9 @@ def _strip_comments(src: str) -> str:
     return "\n".join(lines)
 
 
-def kernel_source_hash() -> str:
+def kernel_source_hash(files=("mlmq.cuh", "kernels_inst.cuh", "kernels_u32.cu")) -> str:
     h = hashlib.sha256()
-    for f in ("mlmq.cuh", "kernels_inst.cuh", "kernels_u32.cu"):
+    for f in files:
         text = open(os.path.join(ROOT, "paper_2602_10080_gb300", "csrc", f), encoding="utf-8").read()
         h.update(_strip_comments(text).encode())
     return h.hexdigest()[:16]
@@ -75,11 +75,11 @@ def config_signature(cfg) -> str:
     return ",".join(f"{k}={d[k]}" for k in TRAFFIC_CONFIG_KEYS)
 
 
-def profiled_traffic(signature=None):
+def profiled_traffic(signature=None, kernel="mlmq_kernel"):
     """Per-launch DRAM bytes of the relaxation kernel from the committed ncu
     summary, or None if the kernel source or the configuration changed
-    since it was captured."""
-    p = os.path.join(ROOT, "profiles", "mlmq_kernel_rmat22_traffic.txt")
+    since it was captured (the wavefront kernel has no configuration)."""
+    p = os.path.join(ROOT, "profiles", f"{kernel}_rmat22_traffic.txt")
     if not os.path.exists(p):
         return None
     vals = {}
@@ -87,7 +87,8 @@ def profiled_traffic(signature=None):
         if ":" in line and not line.startswith("#"):
             k, v = line.split(":", 1)
             vals[k.strip()] = v.strip()
-    if vals.get("kernel_source_hash") != kernel_source_hash():
+    files = {"tide_kernel": ("wave.cuh", "wave_kernels.cu")}
+    if vals.get("kernel_source_hash") != (kernel_source_hash(files[kernel]) if kernel in files else kernel_source_hash()):
         return None
     if signature is not None and vals.get("config") != signature:
         return None
@@ -264,7 +265,7 @@ def run_reference(args):
 
 
 def batch_leg(S, gg, torch, wtype: str = "u32", nq: int = 256, seq_sample: int = 32, tune_ms: int = 8000):
-    """Batched throughput: nq sources of R-MAT 20 in one persistent launch
+    """Batched throughput: nq sources of R-MAT 20 in one call
     (sssp_solve_batch, dist nq x n on the device) against one-at-a-time
     sssp_solve calls on the same sources (a timed sample of them), first
     with the library's multi-query heuristic, then with the configuration
@@ -339,8 +340,9 @@ def bfs_leg(S, G, g, srcs, torch, nsrc: int = 4):
 
 def road_leg(S, gg, torch, nsrc: int = 4, tune_ms: int = 3000):
     """Road-shaped high-diameter graph (4096^2 grid, 5% of edges dropped,
-    0.5% long-range edges): the prior configuration against the autotuned
-    one on the same sources (distances and predecessors)."""
+    0.5% long-range edges): the library's choice against the queues' prior
+    configuration and the autotuned one on the same sources (distances and
+    predecessors)."""
     g = gg.workload("road4096")
     srcs, _ = gg.giant_sources(g, 16, seed=2)
     G = S.Graph(torch.from_numpy(g.row_ptr).cuda(), torch.from_numpy(g.col).cuda(),
@@ -352,7 +354,7 @@ def road_leg(S, gg, torch, nsrc: int = 4, tune_ms: int = 3000):
         prior = S.sssp_autotune(G.handle, None, 0)
         tuned = G.autotune(torch.from_numpy(srcs[:2].astype(np.int32)).cuda(), tune_ms)
         out = {"workload": f"road4096 (n={g.n}, m={g.m}), {nsrc} giant-component sources"}
-        for name, cfg in (("prior", prior), ("autotuned", tuned)):
+        for name, cfg in (("default", None), ("prior", prior), ("autotuned", tuned)):
             G.solve(int(srcs[0]), d, p, cfg)
             ms, arcs = [], 0
             for s in srcs[2:2 + nsrc]:
@@ -363,7 +365,7 @@ def road_leg(S, gg, torch, nsrc: int = 4, tune_ms: int = 3000):
                          "gteps": round(arcs / (sum(ms) / 1e3) / 1e9, 3),
                          "config": {k: v for k, v in cfg.as_dict().items()
                                     if k not in ("delta_f32", "l0_rows", "timeout_ms", "pending_marks",
-                                                 "dedup", "l2_only")}}
+                                                 "dedup", "l2_only")} if cfg else "library's choice"}
         return out
     finally:
         G.close()
@@ -605,10 +607,15 @@ def main():
     # roofline of the relaxation kernel: algorithmic bytes per launch / kernel time
     alg_bytes = (BYTES_PER_ARC * arcs + BYTES_PER_VERTEX * verts) / (args.steps * ws)
     kms = float(np.mean(kernel_ms))
+    # which kernel ran: the queue engine counts its queue operations, the
+    # whole-grid wavefront kernel has none
+    waves = work_sum["rounds"] > 0 and work_sum["pops_l0"] + work_sum["pops_l1"] + work_sum["pops_l2"] == 0
+    kernel = "tide_kernel" if waves else "mlmq_kernel"
     achieved = alg_bytes / (kms / 1e3) / 1e9
     roof = {"bound": "hbm", "achieved": round(achieved, 1), "peak": peaks["hbm_gbs"], "unit": "GB/s",
-            "frac": round(achieved / peaks["hbm_gbs"], 4), "traffic": profiled_traffic(config_signature(tuned)),
-            "peak_source": peaks["source"], "kernel": "mlmq_kernel", "kernel_ms_mean": round(kms, 4),
+            "frac": round(achieved / peaks["hbm_gbs"], 4),
+            "traffic": profiled_traffic(None if waves else config_signature(tuned), kernel),
+            "peak_source": peaks["source"], "kernel": kernel, "kernel_ms_mean": round(kms, 4),
             "alg_bytes_per_launch": int(alg_bytes)}
 
     line = {
@@ -627,8 +634,9 @@ def main():
                    "parallelism": f"replicas x{ws}"},
         "e2e": {"value": round(e2e_value, 3), "unit": "GTEPS", "h2d_bytes_per_step": 4,
                 "d2h_bytes_per_step": 8 * g.n},
-        # per solve: distance fill, [pending-mark fill], seed, relaxation, unpack
-        "gpu_launches": (4 + int(tuned.pending_marks)) * args.steps,
+        # per solve: the wavefront kernel alone, or distance fill, [pending-mark
+        # fill], seed, relaxation, unpack
+        "gpu_launches": (1 if waves else 4 + int(tuned.pending_marks)) * args.steps,
         "roofline": roof,
         "clocks": clk.summary(),
         "per_source": {"kernel_ms": percentiles(kernel_ms),
