@@ -43,7 +43,7 @@ namespace sssp {
 // 32 3740; at 128, 8 rows of up to 8 arcs 4230, 16 4060, 32 rows of up to 16 4270.
 constexpr int32_t kFanShort = 16;
 constexpr uint32_t kFanRows = 8;
-constexpr int32_t kFanChunk = 64;
+constexpr uint32_t kFanChunk = 64;
 constexpr int kFanThreads = 1024;
 constexpr int32_t kFanCoreArcs = 128; // a vertex with as many arcs belongs to the core
 constexpr int32_t kFanMaxVertices = 1 << 25;   // rows are addressed by 32-bit byte offsets
@@ -380,7 +380,7 @@ __global__ void __launch_bounds__(kFanThreads, 1) fan_kernel(const __grid_consta
             const uint32_t sm = __ballot_sync(kFull, deg > 0 && deg <= kFanShort);
             uint32_t lm = __ballot_sync(kFull, deg > kFanShort);
             if (!(sm | lm)) continue;
-            uint32_t k = deg > kFanShort ? (uint32_t)((deg + kFanChunk - 1) / kFanChunk) : 0u, incl = k;
+            uint32_t k = deg > kFanShort ? ((uint32_t)deg + kFanChunk - 1u) / kFanChunk : 0u, incl = k;
             if (lm) {
 #pragma unroll
                 for (int o = 1; o < 32; o <<= 1) {
@@ -403,10 +403,10 @@ __global__ void __launch_bounds__(kFanThreads, 1) fan_kernel(const __grid_consta
                 lm &= lm - 1u;
                 const uint32_t vj = __shfl_sync(kFull, v, j), mj = __shfl_sync(kFull, m, j);
                 const uint32_t kj = __shfl_sync(kFull, k, j), aj = __shfl_sync(kFull, at_s, j);
-                const int32_t b = __shfl_sync(kFull, sp.x, j), e = __shfl_sync(kFull, sp.y, j);
+                const uint32_t b = (uint32_t)__shfl_sync(kFull, sp.x, j), e = (uint32_t)__shfl_sync(kFull, sp.y, j);
                 for (uint32_t i = lane; i < kj; i += 32u) {
-                    const int32_t lo = b + (int32_t)i * kFanChunk;
-                    P.slices[aj + i] = make_uint4(vj, mj, (uint32_t)lo, (uint32_t)min(e, lo + kFanChunk));
+                    const uint32_t lo = b + i * kFanChunk;
+                    P.slices[aj + i] = make_uint4(vj, mj, lo, min(e, lo + kFanChunk));
                 }
             }
         }

@@ -17,10 +17,11 @@ constexpr int kScanThreads = 256, kScanItems = 8, kScanTile = kScanThreads * kSc
 constexpr int32_t kBigRow = 2048;   // rows above this are copied and checked by a block, not a warp
 constexpr int kBigThreads = 1024;
 
-// Shadow vertices of a row and the arcs that move to them.
+// Shadow vertices of a row and the arcs that move to them.  (Arc numbers and
+// degrees end at 2^31 - 1: sums beyond a row are formed unsigned.)
 __device__ __forceinline__ uint2 split_of(int32_t deg, int32_t split) {
     if (deg <= split) return make_uint2(0u, 0u);
-    return make_uint2((uint32_t)((deg + split - 1) / split), (uint32_t)deg);
+    return make_uint2(((uint32_t)deg + (uint32_t)split - 1u) / (uint32_t)split, (uint32_t)deg);
 }
 
 __device__ __forceinline__ uint2 warp_scan(uint2 x, uint2& total) {   // inclusive
@@ -151,7 +152,7 @@ __global__ void relayout_kernel(const int32_t* rp0, const uint2* adj0, int32_t n
     for (int64_t v = wid; v < n; v += nw) {
         const int32_t b = rp0[v], deg = rp0[v + 1] - b, s0 = first[v];
         if (s0 >= 0) {
-            const int32_t k = (deg + split - 1) / split, at = rp1[v];
+            const int32_t k = (int32_t)split_of(deg, split).x, at = rp1[v];
             for (int32_t j = (int32_t)lane; j < k; j += 32) adj1[at + j] = make_uint2((uint32_t)(s0 + j), 0u);
         }
         if (deg > 0 && deg <= kBigRow) copy_row_warp(adj0 + b, adj1 + (s0 >= 0 ? rp1[s0] : rp1[v]), deg, light);
@@ -172,15 +173,16 @@ __global__ void __launch_bounds__(kBigThreads) relayout_big_kernel(const int32_t
         if (v < n && rp0[v + 1] - rp0[v] > kBigRow) list[atomicAdd(&listed, 1)] = (int32_t)v;
         __syncthreads();
         for (int i = 0; i < listed; i++) {
-            const int32_t u = list[i], b = rp0[u], deg = rp0[u + 1] - b;
+            const int32_t u = list[i], b = rp0[u];
+            const uint32_t deg = (uint32_t)(rp0[u + 1] - b);
             const uint2* from = adj0 + b;
             uint2* to = adj1 + (first[u] >= 0 ? rp1[first[u]] : rp1[u]);
             uint2 mine = make_uint2(0u, 0u), total;
-            for (int32_t e = (int32_t)threadIdx.x; e < deg; e += kBigThreads) mine.x += from[e].y <= light;
+            for (uint32_t e = threadIdx.x; e < deg; e += kBigThreads) mine.x += from[e].y <= light;
             block_scan(mine, total);
             uint32_t l = 0u, h = total.x;
-            for (int32_t e0 = 0; e0 < deg; e0 += kBigThreads) {
-                const int32_t e = e0 + (int32_t)threadIdx.x;
+            for (uint32_t e0 = 0; e0 < deg; e0 += kBigThreads) {
+                const uint32_t e = e0 + threadIdx.x;
                 const bool in = e < deg;
                 const uint2 a = in ? from[e] : make_uint2(0u, 0u);
                 const bool lt = in && a.y <= light;
@@ -236,7 +238,7 @@ __global__ void quads_kernel(const int2* span, const uint2* adj, int32_t n, uint
         const int2 sp = span[v];
         uint2 a[4];
 #pragma unroll
-        for (int k = 0; k < 4; k++) a[k] = sp.x + k < sp.y ? adj[sp.x + k] : make_uint2(kNoArc, 0u);
+        for (int k = 0; k < 4; k++) a[k] = k < sp.y - sp.x ? adj[sp.x + k] : make_uint2(kNoArc, 0u);
         if (sp.y - sp.x > 4) a[0].x |= 0x80000000u;
         quads[2 * v] = make_uint4(a[0].x, a[0].y, a[1].x, a[1].y);
         quads[2 * v + 1] = make_uint4(a[2].x, a[2].y, a[3].x, a[3].y);
@@ -266,10 +268,10 @@ struct SymState {
 };
 
 __device__ __forceinline__ void check_arc(const int32_t* rp, const uint2* adj, int32_t u, int32_t du, int32_t first,
-                                          int32_t e, int& bad, unsigned long long& looked,
+                                          uint32_t e, int& bad, unsigned long long& looked,
                                           unsigned long long& other) {
     const uint2 a = adj[e];
-    if (e > first && adj[e - 1].x >= a.x) bad = 1;
+    if (e > (uint32_t)first && adj[e - 1u].x >= a.x) bad = 1;
     const int32_t v = (int32_t)a.x;
     if (v == u) return;
     int32_t lo = rp[v], hi = rp[v + 1];
@@ -316,7 +318,7 @@ __global__ void symmetry_kernel(const int32_t* rp, const uint2* adj, int32_t n, 
         }
         const int32_t b = rp[v], e = rp[v + 1];
         if (e - b > kBigRow) continue;
-        for (int32_t i = b + (int32_t)lane; i < e; i += 32)
+        for (uint32_t i = (uint32_t)b + lane; i < (uint32_t)e; i += 32u)
             check_arc(rp, adj, (int32_t)v, e - b, b, i, bad, looked, other);
         __syncwarp();
     }
@@ -338,7 +340,7 @@ __global__ void __launch_bounds__(kBigThreads) symmetry_big_kernel(const int32_t
         __syncthreads();
         for (int i = 0; i < listed; i++) {
             const int32_t u = list[i], b = rp[u], e = rp[u + 1];
-            for (int32_t j = b + (int32_t)threadIdx.x; j < e; j += kBigThreads)
+            for (uint32_t j = (uint32_t)b + threadIdx.x; j < (uint32_t)e; j += kBigThreads)
                 check_arc(rp, adj, u, e - b, b, j, bad, looked, other);
         }
         __syncthreads();

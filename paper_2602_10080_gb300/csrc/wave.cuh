@@ -39,7 +39,7 @@ constexpr int kWaveHubs = 128;        // hubs one block expands together per ste
 constexpr uint32_t kWaveHash = 0x9E3779B1u;      // odd: v -> v * hash mod 2^bits is one to one
 constexpr uint32_t kWaveHashInv = 0x0E8B2F51u;   // its inverse mod 2^32
 static_assert((uint32_t)(0x9E3779B1ull * 0x0E8B2F51ull) == 1u, "inverse of the vertex hash");
-constexpr int32_t kTideChunk = 256;   // arcs of a hub that one warp relaxes at a time
+constexpr uint32_t kTideChunk = 256;  // arcs of a hub that one warp relaxes at a time
 
 struct WaveParams {
     const int2* span;         // [n] arcs of a vertex: adj[span.x .. span.y); null: from row
@@ -336,8 +336,9 @@ struct Wave {
     }
 
     // Up to four arcs of one vertex, `stride` apart, all loads in flight together.
+    // (Arc numbers end at 2^31 - 1: those past a row's end are formed unsigned.)
     template <bool OWN>
-    __device__ __forceinline__ void arcs4(uint32_t u, uint32_t du, int32_t e, int32_t stride, int32_t end) {
+    __device__ __forceinline__ void arcs4(uint32_t u, uint32_t du, uint32_t e, uint32_t stride, uint32_t end) {
         uint2 a[4];
         DistT c[4];
         uint32_t uu[4], dd[4];
@@ -357,7 +358,7 @@ struct Wave {
     // Arcs g0 + lane + 32 k (k < K) of the warp's concatenated rows (ex: arcs
     // before this lane's vertex u, row at rs, distance du).
     template <int K>
-    __device__ __forceinline__ void arcs_packed(int32_t g0, int32_t total, int32_t ex, int32_t rs, uint32_t du,
+    __device__ __forceinline__ void arcs_packed(uint32_t g0, uint32_t total, uint32_t ex, uint32_t rs, uint32_t du,
                                                 uint32_t u) {
         uint2 a[K];
         DistT c[K];
@@ -365,12 +366,12 @@ struct Wave {
         bool in[K];
 #pragma unroll
         for (int k = 0; k < K; k++) {
-            const int32_t g = g0 + 32 * k + (int32_t)lane_id();
+            const uint32_t g = g0 + 32u * k + lane_id();
             int j = 0;
 #pragma unroll
             for (int s = 16; s >= 1; s >>= 1)
                 if (__shfl_sync(kFull, ex, j + s) <= g) j += s;
-            const int32_t row = __shfl_sync(kFull, rs, j) + (g - __shfl_sync(kFull, ex, j));
+            const uint32_t row = __shfl_sync(kFull, rs, j) + (g - __shfl_sync(kFull, ex, j));
             dj[k] = __shfl_sync(kFull, du, j);
             uj[k] = PRED != 0 ? __shfl_sync(kFull, u, j) : 0u;
             in[k] = g < total;
@@ -423,10 +424,11 @@ struct Wave {
     // The arcs after the fourth of the vertices of lanes `more`.
     __device__ __forceinline__ void rest_of(uint32_t v, uint32_t d, bool more) {
         if (__any_sync(kFull, more)) {
-            int2 sp = more ? __ldg(P.span + v) : make_int2(0, 0);
-            sp.x = min(sp.x + 4, sp.y);
-            n_relax += (uint32_t)(sp.y - sp.x);
-            for (; __any_sync(kFull, sp.x < sp.y); sp.x += 4) arcs4<true>(v, d, sp.x, 1, sp.y);
+            const int2 sp = more ? __ldg(P.span + v) : make_int2(0, 0);
+            const uint32_t end = (uint32_t)sp.y;
+            uint32_t e = min((uint32_t)sp.x + 4u, end);
+            n_relax += end - e;
+            for (; __any_sync(kFull, e < end); e += 4u) arcs4<true>(v, d, e, 1u, end);
         }
         __syncwarp();
     }
@@ -493,18 +495,18 @@ struct Wave {
         if (P.has_hubs) deg = hub(v, d, sp, deg);
         if (__reduce_max_sync(kFull, (uint32_t)deg) <= 4u) {
             // few arcs a vertex: each lane its own
-            arcs4<true>(v, d, sp.x, 1, sp.x + deg);
+            arcs4<true>(v, d, (uint32_t)sp.x, 1u, (uint32_t)(sp.x + deg));
         } else {
             // the batch's arcs spread over the lanes, 128 at a time
-            int32_t incl = deg;
+            uint32_t incl = (uint32_t)deg;
 #pragma unroll
             for (int o = 1; o < 32; o <<= 1) {
-                const int32_t x = __shfl_up_sync(kFull, incl, o);
+                const uint32_t x = __shfl_up_sync(kFull, incl, o);
                 if (lane >= (uint32_t)o) incl += x;
             }
-            const int32_t ex = incl - deg, total = __shfl_sync(kFull, incl, 31);
-            if (!P.has_hubs && total <= 32) arcs_packed<1>(0, total, ex, sp.x, d, v);
-            else for (int32_t g0 = 0; g0 < total; g0 += 128) arcs_packed<4>(g0, total, ex, sp.x, d, v);
+            const uint32_t ex = incl - (uint32_t)deg, total = __shfl_sync(kFull, incl, 31);
+            if (!P.has_hubs && total <= 32u) arcs_packed<1>(0u, total, ex, (uint32_t)sp.x, d, v);
+            else for (uint32_t g0 = 0u; g0 < total; g0 += 128u) arcs_packed<4>(g0, total, ex, (uint32_t)sp.x, d, v);
         }
         __syncwarp();
     }
@@ -656,14 +658,14 @@ struct Wave {
             const int j = __ffs((int)m) - 1;
             m &= m - 1u;
             const uint32_t keep_b = best, keep_f = from;
-            const int32_t b = __shfl_sync(kFull, sp.x, j), end = b + __shfl_sync(kFull, deg, j);
+            const uint32_t b = (uint32_t)__shfl_sync(kFull, sp.x, j), end = b + (uint32_t)__shfl_sync(kFull, deg, j);
             best = none;
             from = kInfU32;
-            for (int32_t e = b; e < end; e += 128) {
+            for (uint32_t e = b; e < end; e += 128u) {
                 uint2 a[4];
                 DistT c[4];
 #pragma unroll
-                for (int k = 0; k < 4; k++) a[k] = ld_arc(P.adj + min(e + 32 * k + (int32_t)lane, end - 1));
+                for (int k = 0; k < 4; k++) a[k] = ld_arc(P.adj + min(e + 32u * k + lane, end - 1u));
 #pragma unroll
                 for (int k = 0; k < 4; k++) c[k] = ld_dist(dist + a[k].x);
 #pragma unroll
@@ -777,8 +779,9 @@ __global__ void __launch_bounds__(1024, 1) wave_kernel(const __grid_constant__ W
             const uint32_t nh = min(S.nhub[set], (uint32_t)kWaveHubs);
             for (uint32_t h = 0; h < nh; h++) {
                 const WaveHub hb = S.hub[h];
-                for (int32_t e = hb.arcs.x + (int32_t)tid; e < hb.arcs.y; e += 4 * (int32_t)nt)
-                    w.template arcs4<false>(hb.v, hb.d, e, (int32_t)nt, hb.arcs.y);
+                const uint32_t end = (uint32_t)hb.arcs.y;
+                for (uint32_t e = (uint32_t)hb.arcs.x + tid; e < end; e += 4u * nt)
+                    w.template arcs4<false>(hb.v, hb.d, e, nt, end);
             }
         }
         // the step's sums
@@ -1051,15 +1054,14 @@ __global__ void __launch_bounds__(1024, 1) tide_kernel(const __grid_constant__ W
                     const int j = __ffs((int)m) - 1;
                     m &= m - 1u;
                     const uint32_t u = __shfl_sync(kFull, v, j), du = __shfl_sync(kFull, d, j);
-                    const int32_t b = __shfl_sync(kFull, sp.x, j), e = __shfl_sync(kFull, sp.y, j);
-                    const int32_t k = (e - b + kTideChunk - 1) / kTideChunk;
+                    const uint32_t b = (uint32_t)__shfl_sync(kFull, sp.x, j), e = (uint32_t)__shfl_sync(kFull, sp.y, j);
+                    const uint32_t k = (e - b + kTideChunk - 1u) / kTideChunk;
                     uint32_t at = 0;
-                    if (lane == 0) at = atomicAdd(&P.sync->hub[now].count, (uint32_t)k);
+                    if (lane == 0) at = atomicAdd(&P.sync->hub[now].count, k);
                     at = __shfl_sync(kFull, at, 0);
-                    for (int32_t i = (int32_t)lane; i < k; i += 32) {
-                        const int32_t lo = b + i * kTideChunk;
-                        items_w[at + (uint32_t)i] =
-                            make_uint4(u, du, (uint32_t)lo, (uint32_t)min(e, lo + kTideChunk));
+                    for (uint32_t i = lane; i < k; i += 32u) {
+                        const uint32_t lo = b + i * kTideChunk;
+                        items_w[at + i] = make_uint4(u, du, lo, min(e, lo + kTideChunk));
                     }
                 }
                 return deg;
@@ -1096,8 +1098,7 @@ __global__ void __launch_bounds__(1024, 1) tide_kernel(const __grid_constant__ W
         for (uint32_t i = wid; i < items; i += nw) {
             const uint4 it = __ldcg(items_r + i);
             if (!P.unit && W::dpart(ld_dist(w.dist + it.x)) < it.y) continue;
-            for (int32_t e = (int32_t)it.z + (int32_t)lane; e < (int32_t)it.w; e += 128)
-                w.template arcs4<false>(it.x, it.y, e, 32, (int32_t)it.w);
+            for (uint32_t e = it.z + lane; e < it.w; e += 128u) w.template arcs4<false>(it.x, it.y, e, 32u, it.w);
             __syncwarp();
         }
     }
