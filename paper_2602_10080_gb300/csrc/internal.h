@@ -2,6 +2,7 @@
 // units (not part of the public C ABI).
 #pragma once
 
+#include <atomic>
 #include <cstdint>
 #include <cuda_runtime.h>
 
@@ -50,6 +51,31 @@ inline cudaError_t launch_mlmq(const KernelKey& key, dim3 grid, dim3 block, size
 inline cudaError_t occupancy_mlmq(const KernelKey& key, int threads, size_t smem, int* blocks) {
     return key.wt == 0 ? occupancy_mlmq_u32x(key, threads, smem, blocks)
                        : occupancy_mlmq_f32x(key, threads, smem, blocks);
+}
+
+constexpr int kMaxDevices = 64;
+
+// Opens all of a block's shared memory to the kernel; the launch says how much
+// of it a block takes.  The limit belongs to the function and not to a call: set
+// to one call's own size it would refuse the larger one of another thread that
+// launches at the same time.  room: of this function, what is left beside its
+// static shared memory by device (0: not asked yet).
+template <typename F>
+cudaError_t open_shared(F* fn, size_t smem, std::atomic<int> (&room)[kMaxDevices]) {
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    int most = dev < kMaxDevices ? room[dev].load(std::memory_order_relaxed) : 0;
+    if (!most) {
+        cudaFuncAttributes fa;
+        if ((e = cudaDeviceGetAttribute(&most, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev)) != cudaSuccess ||
+            (e = cudaFuncGetAttributes(&fa, fn)) != cudaSuccess)
+            return e;
+        most -= (int)fa.sharedSizeBytes;
+        if (dev < kMaxDevices) room[dev].store(most, std::memory_order_relaxed);
+    }
+    if (smem > (size_t)most) return cudaErrorInvalidValue;
+    return cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
 }
 
 constexpr int kL0Rows = 2;  // L0 ring rows per warp compiled into the kernels

@@ -12,9 +12,14 @@ namespace sssp {
 template <int WT, bool X>
 struct MlmqInstances {
     template <int PRED, bool MQ>
+    static cudaError_t open(size_t smem) {
+        static std::atomic<int> room[kMaxDevices];
+        return open_shared(mlmq_kernel<WT, PRED, MQ, kL0Rows, X>, smem, room);
+    }
+    template <int PRED, bool MQ>
     static cudaError_t launch_one(dim3 grid, dim3 block, size_t smem, cudaStream_t stream, const KParams& p) {
         auto fn = mlmq_kernel<WT, PRED, MQ, kL0Rows, X>;
-        cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        const cudaError_t e = open<PRED, MQ>(smem);
         if (e != cudaSuccess) return e;
         fn<<<grid, block, smem, stream>>>(p);
         return cudaGetLastError();
@@ -22,7 +27,7 @@ struct MlmqInstances {
     template <int PRED, bool MQ>
     static cudaError_t occ_one(int threads, size_t smem, int* blocks) {
         auto fn = mlmq_kernel<WT, PRED, MQ, kL0Rows, X>;
-        cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        const cudaError_t e = open<PRED, MQ>(smem);
         if (e != cudaSuccess) return e;
         return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks, fn, threads, smem);
     }

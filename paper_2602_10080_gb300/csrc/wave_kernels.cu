@@ -1,4 +1,5 @@
 // wave_kernels.cu -- instantiations of the cluster wavefront kernel and their launch.
+#include "internal.h"
 #include "wave.h"
 
 namespace sssp {
@@ -6,7 +7,8 @@ namespace sssp {
 template <int WT, int PRED, bool CL, int HOPS>
 static cudaError_t launch_hops(const WaveParams& p, int nq, int threads, size_t smem, cudaStream_t stream) {
     auto fn = wave_kernel<WT, PRED, CL, HOPS>;
-    cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    static std::atomic<int> room[kMaxDevices];
+    cudaError_t e = open_shared(fn, smem, room);
     if (e != cudaSuccess) return e;
     cudaLaunchConfig_t c{};
     c.gridDim = dim3((unsigned)nq << p.log_g);
