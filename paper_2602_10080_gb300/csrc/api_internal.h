@@ -81,6 +81,8 @@ struct Graph {
     bool tuned_valid = false;
     bool tuned_queues = false;    // sssp_autotune timed the tuned queue configuration faster than the wavefront
     std::atomic<bool> wide{false};   // a solve found the front too wide for one cluster
+    std::atomic<bool> deep{false};   // a batch side by side gave up: too many steps
+    std::atomic<int64_t> steps{0};   // the most that a single query has taken on the wavefront kernels
     // multi-query configurations from sssp_autotune_batch, per size class
     // (the number of queries rounded down to a power of two)
     struct BatchTuned {
@@ -161,16 +163,22 @@ int run_queries(Graph* g, const int32_t* srcs_host, const int32_t* srcs_dev, int
 inline WaveGraph wave_graph(const Graph* g) {
     return WaveGraph{g->n, g->m, g->feat.avg_w, g->feat.max_deg, g->sms, g->wide.load(),
                      g->light_first && g->light_share >= 0.02 && g->light_share <= 0.4,
-                     g->light_first && g->light_share >= 0.02 && g->light_share <= 0.15};
+                     g->light_first && g->light_share >= 0.02 && g->light_share <= 0.15,
+                     g->deep.load(), g->steps.load()};
+}
+inline void note_steps(Graph* g, int64_t steps) {
+    int64_t had = g->steps.load();
+    while (had < steps && !g->steps.compare_exchange_weak(had, steps)) {}
 }
 // The graph's part of the multi-source kernel's parameters.
 struct FanParams;
 void fan_graph(const Graph* g, FanParams* p);
 // The wavefront kernels (sssp_wave.cu), for calls that leave the configuration
 // to the library.  kWaveNotRun: the graph or the call is not for them.
+// *done (or null): the first queries of the batch that are finished all the same.
 constexpr int kWaveNotRun = 1;
 int run_wave(Graph* g, const int32_t* srcs_host, const int32_t* srcs_dev, int32_t src0, int32_t nq, void* dist_out,
-             int32_t* pred_out, cudaStream_t stream, sssp_stats* st_out, bool unit);
+             int32_t* pred_out, cudaStream_t stream, sssp_stats* st_out, bool unit, int32_t* done = nullptr);
 template <typename T>
 int grow(T** p, size_t* have, size_t want) {
     if (*have >= want && *p) return SSSP_OK;

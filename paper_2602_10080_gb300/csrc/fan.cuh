@@ -80,7 +80,13 @@ struct FanParams {
     FanSync* sync;
     Ctrl* ctrl;
     unsigned long long timeout_ns;
+    // From step max_steps on the search gives up (kErrDeep) where more wait than a
+    // tail that the bulk left behind, whose steps cost 12 us (a power-law graph
+    // with a chain of 300 arcs: 3.5 ms, 0.9 with 50), or after 16 times as many.
+    uint32_t max_steps;
 };
+
+constexpr uint32_t kFanTail = 1024;   // slices and short rows of a step
 
 // How an arc is used: to relax it, (distances final) to find the tight ones,
 // to relax it while the core leaves heavy arcs out, or to pull over it, from
@@ -287,6 +293,9 @@ __global__ void __launch_bounds__(kFanThreads, 1) fan_kernel(const __grid_consta
     const uint32_t tid = threadIdx.x, lane = tid & 31u, gt = blockIdx.x * blockDim.x + tid;
     const uint32_t gn = gridDim.x * blockDim.x, wid = (tid >> 5) * gridDim.x + blockIdx.x, nw = gn >> 5;
     const unsigned long long deadline = gtime() + P.timeout_ns;
+    // the group before gave up (set by an earlier kernel of the stream, so that
+    // every block finds the same)
+    if (ld_volatile_int(&P.ctrl->error) != kErrNone) return;
     const uint32_t places = P.mask + 1u;
     uint32_t arrivals = 0u;
     unsigned long long n_relax = 0ull;
@@ -311,6 +320,7 @@ __global__ void __launch_bounds__(kFanThreads, 1) fan_kernel(const __grid_consta
 
     uint32_t step = 0u;
     FanPass pass = CORE ? kFanCore : kFanRelax;
+    bool deep = false;
     while (ok) {
         const uint32_t set = step & 3u;
         uint32_t* wait_r = P.wait + (size_t)(step & 1u) * places;
@@ -420,6 +430,10 @@ __global__ void __launch_bounds__(kFanThreads, 1) fan_kernel(const __grid_consta
             Fan<WT, kFanTight>(P, wait_w).work(slices, rows, wid, nw, &P.sync->set[set].claimed);
             break;
         }
+        if ((pass == kFanCore || pass == kFanRelax) && step >= P.max_steps) {
+            deep = slices + rows > kFanTail || (slices + rows != 0u && step >= 16u * P.max_steps);
+            if (deep) break;
+        }
         if (slices + rows == 0u) {
             // nobody waits: the core has settled, or all distances are final
             if (CORE && pass == kFanCore) pass = kFanPull;
@@ -441,7 +455,8 @@ __global__ void __launch_bounds__(kFanThreads, 1) fan_kernel(const __grid_consta
     if (tid == 0 && !ok) raise_error(P.ctrl, kErrTimeout, 22, 0);
     if (gt == 0) {
         atomicAdd(&P.ctrl->stats[kStIter], (unsigned long long)step);
-        atomicAdd(&P.ctrl->finished, P.nq);
+        if (deep) raise_error(P.ctrl, kErrDeep, 23, (int)step);
+        else atomicAdd(&P.ctrl->finished, P.nq);
     }
 }
 

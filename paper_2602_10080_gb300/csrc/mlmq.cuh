@@ -91,6 +91,7 @@ enum : int {
     kErrState = 3,        // queue metadata inconsistent at seeding
     kErrElement = 4,      // a popped element names a vertex or query out of range
     kErrWide = 5,         // wavefront kernel: the front is too wide for one cluster (the host runs the grid's)
+    kErrDeep = 6,         // multi-source kernel: more steps than it pays for (the host takes another way)
 };
 
 // statistics slots (ctrl.stats)

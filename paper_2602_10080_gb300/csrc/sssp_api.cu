@@ -581,8 +581,15 @@ int run_queries(Graph* g, const int32_t* srcs_host, const int32_t* srcs_dev, int
         const int lrc = ensure_layout(g, cfg.split_arcs ? cfg.split_arcs : kDefaultSplit, stream);
         if (lrc) return lrc;
         if (nq > 1 && !key_bits(g, nq)) return SSSP_E_INVAL;
-        const int wrc = run_wave(g, srcs_host, srcs_dev, src0, nq, dist_out, pred_out, stream, st_out, unit);
+        int32_t done = 0;
+        const int wrc = run_wave(g, srcs_host, srcs_dev, src0, nq, dist_out, pred_out, stream, st_out, unit, &done);
         if (wrc != kWaveNotRun) return wrc;
+        // the queues take the others (two of them or more)
+        srcs_host += done;
+        if (srcs_dev) srcs_dev += done;
+        nq -= done;
+        dist_out = (uint32_t*)dist_out + (size_t)done * (size_t)g->n;
+        if (pred_out) pred_out += (size_t)done * (size_t)g->n;
     }
     // breadth-first: one bucket per level unless the caller chose a delta
     if (unit && (!cfg_in || cfg.delta_u32 == 0)) cfg.delta_u32 = 1;

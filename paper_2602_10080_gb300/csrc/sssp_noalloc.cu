@@ -197,7 +197,7 @@ extern "C" int sssp_solve_noalloc(const int32_t* row_ptr, const uint32_t* arcs, 
 
     const int pred_mode = pred_out ? ((!f32 && m > 0 && ~hf.min_not >= 1u) ? 1 : 2) : 0;
     const double avg_w = m > 0 ? hf.sum_w / (double)m : 1.0;
-    WaveGraph wg{n, m, avg_w, (double)hf.max_deg, sms, false, false, false};
+    WaveGraph wg{n, m, avg_w, (double)hf.max_deg, sms, false, false, false, false, 0};
     Ctrl hc;
     for (;;) {
         WavePlan plan;

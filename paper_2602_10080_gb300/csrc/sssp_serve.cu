@@ -267,6 +267,7 @@ struct Job {
 struct Lane {
     Graph* g = nullptr;
     bool express = false;       // wavefront jobs instead of slices
+    bool many = false;          // slices while many queries wait (see express_launch)
     std::vector<Job*> jobs;
     uint64_t uid = 0;
     bool counted = false;       // registered in lane_refs (the graph's layout is pinned)
@@ -824,16 +825,28 @@ Job* job_create(sssp_server* s) {
     return J;
 }
 
-// The lane's waiting queries, oldest first (at most `most`).
-std::vector<Query*> express_waiting(sssp_server* s, Lane* L, size_t most) {
+// The lane's waiting queries, oldest first (at most `most`); *all: how many wait.
+std::vector<Query*> express_waiting(sssp_server* s, Lane* L, size_t most, size_t* all) {
     std::vector<Query*> qs;
+    *all = 0;
     std::lock_guard<std::mutex> lk(s->mu);
     for (Query* q : s->backlog) {
-        if (qs.size() == most) break;
-        if (!q->cancel && q->g->uid == L->uid && (q->pred_out ? pred_mode_for(q->g) : 0) == L->pred_mode)
-            qs.push_back(q);
+        if (q->cancel || q->g->uid != L->uid || (q->pred_out ? pred_mode_for(q->g) : 0) != L->pred_mode) continue;
+        if (qs.size() < most) qs.push_back(q);
+        ++*all;
     }
     return qs;
+}
+
+// A job's queries to the front of the backlog again (the job has ended, or was
+// not launched).
+void job_requeue(sssp_server* s, const std::vector<Query*>& qs) {
+    std::lock_guard<std::mutex> lk(s->mu);
+    for (auto it = qs.rbegin(); it != qs.rend(); ++it) {
+        if ((*it)->cancel) continue;
+        (*it)->state = SSSP_Q_QUEUED;
+        s->backlog.push_front(*it);
+    }
 }
 
 // The lane runs slices from now on (no job in flight).
@@ -841,7 +854,7 @@ int lane_to_slices(sssp_server* s, Lane* L) {
     for (Job* J : L->jobs) job_destroy(s, J);
     L->jobs.clear();
     L->express = false;
-    if (L->pred_mode) {
+    if (L->pred_mode && !L->out_d) {
         const size_t n = (size_t)L->g->n;
         if (dev_alloc(&L->out_d, n) || dev_alloc(&L->out_p, n)) return SSSP_E_NOMEM;
         L->bytes += n * 8;
@@ -852,7 +865,12 @@ int lane_to_slices(sssp_server* s, Lane* L) {
 
 // Starts jobs for the lane's waiting queries as far as slots, jobs and the
 // grid are free.  Without memory for a job the lane goes back to slices (and
-// to their rules when that does not fit either).
+// to their rules when that does not fit either).  Where a graph takes many steps,
+// so that queries are taken in turn, and many wait, slices are faster: three
+// times as many as in a batch, since slices are slower than a batch.  ms one by
+// one (slices): eight-neighbour grid 1000^2 4 queries 25 (71), 20 140 (94);
+// road map 1500^2 4 41 (87), 20 220 (131); grid 1500 x 1450 20 108 (162), grid
+// 4000^2 20 356 (441).
 int express_launch(sssp_server* s, Lane* L) {
     Graph* g = L->g;
     const size_t n = (size_t)g->n;
@@ -860,10 +878,19 @@ int express_launch(sssp_server* s, Lane* L) {
     for (;;) {
         const int room = std::min<int>((int)L->cap_limit - L->running, kJobQueries);
         if (room <= 0) return SSSP_OK;
-        std::vector<Query*> qs = express_waiting(s, L, (size_t)room);
+        size_t waiting = 0;
+        std::vector<Query*> qs = express_waiting(s, L, (size_t)room, &waiting);
         if (qs.empty()) return SSSP_OK;
         const WaveGraph wg = wave_graph(g);
         WavePlan plan;
+        const bool steps = wg.deep || (wg.steps > (int64_t)deep_steps(wg.m) && wg.m < 100000 * wg.steps);
+        if (steps && (int64_t)waiting > 3ll * in_turn_limit(wg) &&
+            (!plan_wave(wg, (int32_t)qs.size(), L->pred_mode, &plan) || plan.kind == kInTurn)) {
+            if (L->running) return SSSP_OK;
+            L->many = true;
+            return lane_to_slices(s, L);
+        }
+        plan = WavePlan();
         if (qs.size() > 1 && (!plan_wave(wg, (int32_t)qs.size(), L->pred_mode, &plan) || plan.kind == kInTurn))
             qs.resize(1);
         if (qs.size() == 1) {
@@ -968,14 +995,7 @@ int express_launch(sssp_server* s, Lane* L) {
             // no room for the cluster or the cooperative grid on this device
             cudaGetLastError();
             job_release_grid(s, J);
-            {
-                std::lock_guard<std::mutex> lk(s->mu);
-                for (auto it = qs.rbegin(); it != qs.rend(); ++it) {
-                    if ((*it)->cancel) continue;
-                    (*it)->state = SSSP_Q_QUEUED;
-                    s->backlog.push_front(*it);
-                }
-            }
+            job_requeue(s, qs);
             return L->running ? cuda_status(e) : lane_to_slices(s, L);
         }
         J->qs = qs;
@@ -994,6 +1014,18 @@ int express_collect(sssp_server* s, Lane* L, Job* J) {
     cudaEventElapsedTime(&ms, J->k0, J->k1);
     const Ctrl& hc = *J->ctrl_h;
     int status = SSSP_OK;
+    if (hc.error == kErrDeep) {
+        // too many steps side by side: the queries take another way
+        {
+            std::lock_guard<std::mutex> lk(s->mu);
+            for (Query* q : J->qs)
+                if (!q->cancel) q->g->deep = true;
+        }
+        L->running -= (int)J->qs.size();
+        job_requeue(s, J->qs);
+        J->qs.clear();
+        return SSSP_OK;
+    }
     if (hc.error != kErrNone || hc.finished != (int)J->qs.size())
         status = hc.error == kErrTimeout ? SSSP_E_TIMEOUT : SSSP_E_CUDA;
     std::vector<Query*> out;
@@ -1003,6 +1035,7 @@ int express_collect(sssp_server* s, Lane* L, Job* J) {
         for (Query* q : J->qs) {
             if (q->cancel) continue;
             if (status == SSSP_OK) {
+                if (J->qs.size() == 1) note_steps(q->g, (int64_t)hc.stats[kStIter]);
                 q->delivering = true;
                 out.push_back(q);
             } else {
@@ -1034,6 +1067,10 @@ int launch_ready(sssp_server* s) {
     for (Lane* L : s->lanes)
         if (!L->express) total += L->running + L->draining;
     for (Lane* L : s->lanes) {
+        if (L->many && !L->inflight && L->running + L->draining + L->nadm == 0) {
+            L->express = true;   // those many are done
+            L->many = false;
+        }
         if (L->express) {
             const int rc = express_launch(s, L);
             if (rc) return rc;

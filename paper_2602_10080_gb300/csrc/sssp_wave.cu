@@ -26,6 +26,33 @@ uint32_t pow2_at_least(double x) {
 constexpr int32_t kClusterVertices = 1 << 21;
 static_assert((size_t)kClusterVertices / 2 / 16 <= kWaveMaxShared, "pending bits of 16 blocks");
 
+// Side by side the queries advance by hops, and a step costs 20 us and more
+// however few vertices wait.  G(n, m), random directed and power-law graphs take
+// 15 to 42 steps; a small world of 10^6 vertices and 5 10^4 shortcuts takes 76
+// (20 queries: 13.1 ms, 10.3 in turn); boxes, eight-neighbour grids and road maps
+// hundreds to thousands (20 queries on a box of 100^3 vertices of degree 26: 80 ms,
+// 22 in turn; on a road map of 4000^2 crossings: 8400 ms, 193 through the queues).
+// On the largest graphs the arcs make up for more steps.
+uint32_t deep_steps(int64_t m) { return (uint32_t)std::max<int64_t>(48, m >> 20); }
+
+// Then the queries are taken one after the other on the whole grid, up to a
+// number from which on the queue engine is faster, which works on all of them at
+// once but 2 to 5 times as slowly on one.  ms in turn (queues): eight-neighbour
+// grid 1000^2, 5300 arcs a step, 3 queries 19 (23), 6 35 (27); road maps of degree
+// 2.5 with a few crossings of 14 arms, 1500^2 3 30 (35), 6 59 (43), 4000^2 3 109
+// (99).  A warp's several hops make the line later on meshes: grid 1500 x 1450,
+// 17000 arcs a step, 6 34 (48), 10 54 (53), 16 83 (61); grid 4000^2, 41000, 10 188
+// (183).  With more arcs a step the chip is busy with one query: road 4096^2,
+// 220000 arcs a step, 64 queries 324 (534); road 2000^2, 120000, 48 96 (117); the box
+// of degree 26, 124000, 20 22 (38), 48 53 (54); the small world, 109000, 20 10 (11).
+// A box of 100^3 vertices of degree 6, a mesh by its degrees with a wide front: 8
+// 10 (9), 20 24 (16).
+int32_t in_turn_limit(const WaveGraph& g) {
+    const bool thin = thin_graph(std::max(1.0, (double)g.m / (double)g.n), g.max_deg);
+    if (g.steps && g.m < 100000 * g.steps) return thin && !g.wide ? 8 : 3;
+    return !thin ? 24 : g.wide ? 8 : 0x7fffffff;
+}
+
 bool plan_wave(const WaveGraph& g, int32_t nq, int pred_mode, WavePlan* w) {
     const double deg = std::max(1.0, (double)g.m / (double)g.n);
     const bool hubs = g.max_deg > 64.0;
@@ -97,7 +124,7 @@ bool plan_wave(const WaveGraph& g, int32_t nq, int pred_mode, WavePlan* w) {
     // queries leave room for (13 queries on grid 301 x 257: 8 blocks 1690 us,
     // 4: 1880, 1: 2130; 20 queries on grid 900 x 1000 16: 8465, 8: 5820, 4: 6030).
     // A mesh too large for that goes one by one: side by side, by hops, 20 queries
-    // on grid 900 x 1000 take 167 ms.
+    // on grid 900 x 1000 take 167 ms.  So does any graph of many steps.
     const bool mesh = thin && !g.wide;
     if (g.n > kClusterVertices || (!mesh && (g.m > (1 << 21) || (hubs && g.m > (1 << 18))))) {
         // A group of up to 32 queries side by side costs as much as this many
@@ -105,7 +132,12 @@ bool plan_wave(const WaveGraph& g, int32_t nq, int pred_mode, WavePlan* w) {
         // with all arcs 7, G(200K, 2M) 14 (2.6 ms).  Predecessors of the
         // strict-improvement rule cannot be found after the distances and stay
         // with the queues.
-        if (mesh || nq < (g.core ? 6 : hubs ? 8 : 14)) w->kind = kInTurn;
+        // (many steps of one query may be those of its distances: whether the hops
+        // are as many, side by side finds out)
+        const int32_t limit = in_turn_limit(g);
+        const int32_t line = g.core ? 6 : hubs ? 8 : 14;
+        if ((mesh || g.deep) && nq > limit) return false;
+        if (mesh || g.deep || (nq < line && (g.steps <= (int64_t)deep_steps(g.m) || nq <= limit))) w->kind = kInTurn;
         else if (pred_mode != 2 && g.n <= kFanMaxVertices) w->kind = kSideBySide;
         else return false;
         return true;
@@ -184,6 +216,7 @@ void fan_carve(uint32_t* words, uint4* slices, int32_t n, int64_t m, bool pred, 
 }
 
 void fan_graph(const Graph* g, FanParams* p) {
+    p->max_steps = deep_steps(g->m);
     p->span = g->span;
     p->adj = g->adj;
     if (wave_graph(g).core) {
@@ -236,7 +269,8 @@ int run_fan(Graph* g, const int32_t* srcs_host, const int32_t* srcs_dev, int32_t
 }  // namespace
 
 int run_wave(Graph* g, const int32_t* srcs_host, const int32_t* srcs_dev, int32_t src0, int32_t nq, void* dist_out,
-             int32_t* pred_out, cudaStream_t stream, sssp_stats* st_out, bool unit) {
+             int32_t* pred_out, cudaStream_t stream, sssp_stats* st_out, bool unit, int32_t* done) {
+    if (done) *done = 0;
     // unit weights are >= 1: the packed minimum gives the smallest-index parent
     const int pred_mode = pred_out ? (unit ? 1 : pred_mode_for(g)) : 0;
     WavePlan plan;
@@ -250,6 +284,17 @@ int run_wave(Graph* g, const int32_t* srcs_host, const int32_t* srcs_dev, int32_
         sssp_stats sum;
         std::memset(&sum, 0, sizeof(sum));
         for (int32_t q = 0; q < nq; q++) {
+            // what the queries before found out may send the others elsewhere
+            WavePlan rest;
+            if (q && nq - q > 1 && (!plan_wave(wave_graph(g), nq - q, pred_mode, &rest) || rest.kind != kInTurn)) {
+                const size_t at = (size_t)q * (size_t)n;
+                int32_t more = 0;
+                const int rc = run_wave(g, srcs_host + q, srcs_dev ? srcs_dev + q : nullptr, 0, nq - q,
+                                        (uint32_t*)dist_out + at, pred_out ? pred_out + at : nullptr, stream, st_out,
+                                        unit, &more);
+                if (done) *done = q + more;
+                return rc;
+            }
             sssp_stats one;
             const size_t at = (size_t)q * (size_t)n;
             const int rc = run_wave(g, nullptr, nullptr, srcs_host[q], 1, (uint32_t*)dist_out + at,
@@ -342,7 +387,12 @@ int run_wave(Graph* g, const int32_t* srcs_host, const int32_t* srcs_dev, int32_
     const Ctrl& hc = *ws.host_ctrl;
     if (hc.error == kErrWide) {
         g->wide = true;
-        return run_wave(g, srcs_host, srcs_dev, src0, nq, dist_out, pred_out, stream, st_out, unit);
+        return run_wave(g, srcs_host, srcs_dev, src0, nq, dist_out, pred_out, stream, st_out, unit, done);
+    }
+    if (hc.error == kErrDeep) {
+        g->deep = true;
+        grid_lock.unlock();
+        return run_wave(g, srcs_host, srcs_dev, src0, nq, dist_out, pred_out, stream, st_out, unit, done);
     }
     float ms = 0;
     cudaEventElapsedTime(&ms, ws.ev1, ws.ev2);
@@ -358,7 +408,10 @@ int run_wave(Graph* g, const int32_t* srcs_host, const int32_t* srcs_dev, int32_
     st.attempts = 1;
     g->last = st;
     if (st_out) *st_out = st;
-    if (hc.error == kErrNone && hc.finished == nq) return SSSP_OK;
+    if (hc.error == kErrNone && hc.finished == nq) {
+        if (nq == 1 && !unit) note_steps(g, st.rounds);
+        return SSSP_OK;
+    }
     return hc.error == kErrTimeout ? SSSP_E_TIMEOUT : SSSP_E_CUDA;
 }
 

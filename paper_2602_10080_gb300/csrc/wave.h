@@ -27,7 +27,8 @@ struct WavePlan {
 };
 
 // What the plan depends on.  wide: a solve found the front too wide for one
-// cluster.
+// cluster; deep: a batch side by side took too many steps; steps: the most that
+// a single query has taken (0: none yet).
 struct WaveGraph {
     int32_t n;
     int64_t m;
@@ -37,6 +38,8 @@ struct WaveGraph {
     // symmetric, hubs, rows with their light arcs first: for a batch side by
     // side, and (few light arcs) for one query
     bool core, core_one;
+    bool deep;
+    int64_t steps;
 };
 
 constexpr int kTideLogWords = 17;               // the grid kernel spreads the places over at least 2^17 words
@@ -48,6 +51,10 @@ inline bool thin_graph(double deg, double max_deg) {
     return deg <= 6.5 && max_deg <= (2.0 * deg + 1.5 < 11.5 ? 2.0 * deg + 1.5 : 11.5);
 }
 bool plan_wave(const WaveGraph& g, int32_t nq, int pred_mode, WavePlan* w);
+// Steps from which on a batch side by side may give up (see FanParams).
+uint32_t deep_steps(int64_t m);
+// How many queries on a graph of many steps are taken in turn at most.
+int32_t in_turn_limit(const WaveGraph& g);
 // The fields of the parameters that follow from the plan; returns the dynamic
 // shared memory of a block.
 size_t wave_params(const WavePlan& w, const WaveGraph& g, bool f32, bool unit, WaveParams* p);
