@@ -66,14 +66,15 @@ struct Graph {
     int32_t* row_ptr = nullptr;   // [nv + 1]
     uint2* adj = nullptr;         // [mv] (col, weight bits)
     int32_t* owner = nullptr;     // [nv - n]
-    int2* span = nullptr;         // [n] (begin, end) of a real vertex's arcs in adj (a hub's slices are contiguous)
-    // hubs of symmetric graphs (see check_symmetry): rows are laid out with
-    // their light arcs first (weight bits <= light_w), mid[v] ends them
+    int2* span = nullptr;         // [n] (begin, end) of a real vertex's arcs in wave_adj (a hub's slices are contiguous)
+    // symmetric graphs with hubs (see check_symmetry): the arcs once more for the
+    // wavefront kernels, whose rows have their light arcs first (weight bits <=
+    // light_w); mid[v] ends them
     bool symmetric = false;       // every arc has its reverse of equal weight (shown arc by arc)
-    bool light_first = false;     // the current layout's rows are partitioned
     uint32_t light_w = 0;
     double light_share = 0.0;     // of the arcs
-    int32_t* mid = nullptr;       // [n] (light_first)
+    uint2* wadj = nullptr;        // [m], or null
+    int32_t* mid = nullptr;       // [n] (wadj)
     uint4* quads = nullptr;       // [n][2] the first four arcs of every vertex of a thin graph (see WaveParams)
     sssp_features feat{};
     sssp_config defaults{};
@@ -119,10 +120,11 @@ int lane_refs(uint64_t uid, int delta);
 int ensure_layout(Graph* g, int32_t split, cudaStream_t s);
 // The layout (sssp_layout.cu): hubs split into shadow vertices of `split`
 // arcs.  rp0 / adj0 are the validated original arrays (device); on success
-// g->row_ptr / adj / owner describe the layout (rp0 / adj0 are freed when new
-// arrays replaced them), on failure the graph is untouched.
+// g->row_ptr / adj / owner describe the layout (rp0 / adj0 are freed, or adj0
+// kept as g->wadj, when new arrays replaced them), on failure the layout is
+// untouched.
 int build_layout(Graph* g, int32_t* rp0, uint2* adj0, int32_t split, cudaStream_t s);
-// g->span (and g->mid, g->quads) for the current layout.
+// g->span (and g->quads) for the current layout.
 int fill_span(Graph* g, cudaStream_t s);
 // Original arc order from a split layout: row v of rp0 from adj[src_start[v] ..].
 void launch_unsplit(const Graph* g, const int32_t* src_start, const int32_t* rp0, uint2* adj0, cudaStream_t s);
@@ -162,14 +164,16 @@ int run_queries(Graph* g, const int32_t* srcs_host, const int32_t* srcs_dev, int
 
 inline WaveGraph wave_graph(const Graph* g) {
     return WaveGraph{g->n, g->m, g->feat.avg_w, g->feat.max_deg, g->sms, g->wide.load(),
-                     g->light_first && g->light_share >= 0.02 && g->light_share <= 0.4,
-                     g->light_first && g->light_share >= 0.02 && g->light_share <= 0.15,
+                     g->wadj && g->light_share >= 0.02 && g->light_share <= 0.4,
+                     g->wadj && g->light_share >= 0.02 && g->light_share <= 0.15,
                      g->deep.load(), g->steps.load()};
 }
 inline void note_steps(Graph* g, int64_t steps) {
     int64_t had = g->steps.load();
     while (had < steps && !g->steps.compare_exchange_weak(had, steps)) {}
 }
+// The arcs that g->span numbers.
+inline const uint2* wave_adj(const Graph* g) { return g->wadj ? g->wadj : g->adj; }
 // The graph's part of the multi-source kernel's parameters.
 struct FanParams;
 void fan_graph(const Graph* g, FanParams* p);

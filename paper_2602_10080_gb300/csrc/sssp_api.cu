@@ -1115,6 +1115,7 @@ extern "C" int sssp_graph_create(const int32_t* row_ptr, const int32_t* col_idx,
         cudaFree(g->adj);
         cudaFree(g->owner);
         cudaFree(g->span);
+        cudaFree(g->wadj);
         cudaFree(g->mid);
         cudaFree(g->quads);
         delete g;
@@ -1135,6 +1136,7 @@ extern "C" int sssp_graph_destroy(sssp_graph* gh) {
         cudaFree(g->adj);
         cudaFree(g->owner);
         cudaFree(g->span);
+        cudaFree(g->wadj);
         cudaFree(g->mid);
         cudaFree(g->quads);
     }

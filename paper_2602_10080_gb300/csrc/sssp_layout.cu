@@ -1,6 +1,6 @@
 // sssp_layout.cu -- the device layout of a graph: hubs split into shadow
-// vertices, light arcs first in the rows of symmetric graphs with hubs, and
-// where every real vertex's arcs lie.  All of it runs on the device (built on
+// vertices, a second copy of the arcs of symmetric graphs with hubs whose rows
+// have their light arcs first, and where every real vertex's arcs lie.  All of it runs on the device (built on
 // the host, R-MAT-22's layout took 11 of the 17 ms of its creation).
 #include <algorithm>
 #include <cmath>
@@ -124,9 +124,9 @@ __global__ void __launch_bounds__(kScanThreads) split_rows_kernel(const int32_t*
     if (blockIdx.x == 0 && threadIdx.x == 0) rp1[(int64_t)n + all.x] = (int32_t)(m + (int64_t)all.x);
 }
 
-// Copies `count` arcs, those of weight <= light first (both parts in order).
-// T threads, one of them per lane of `rank`: a warp (T = 32) or a block.
-__device__ void copy_row_warp(const uint2* from, uint2* to, int32_t count, uint32_t light) {
+// Copies `count` arcs by one warp, those of weight <= light first (both parts
+// in order).
+__device__ void part_row_warp(const uint2* from, uint2* to, int32_t count, uint32_t light) {
     const uint32_t lane = lane_id();
     int32_t nl = 0;
     for (int32_t b = 0; b < count; b += 32)
@@ -142,10 +142,15 @@ __device__ void copy_row_warp(const uint2* from, uint2* to, int32_t count, uint3
     }
 }
 
-// The rows of up to kBigRow arcs to their places, one warp per vertex; links
-// of every hub.  light: partition bound (all ones: plain copy).
+// Row v of the original arrays (rp0, adj0) and of the split layout (rp1, first, adj1).
+__device__ __forceinline__ int32_t split_at(const int32_t* rp1, const int32_t* first, int64_t v) {
+    return first[v] >= 0 ? rp1[first[v]] : rp1[v];
+}
+
+// The rows to their places in the split layout and the links of every hub, one
+// warp per vertex; rows above kBigRow arcs by the next kernel.
 __global__ void relayout_kernel(const int32_t* rp0, const uint2* adj0, int32_t n, const int32_t* rp1,
-                                const int32_t* first, int32_t split, uint32_t light, uint2* adj1) {
+                                const int32_t* first, int32_t split, uint2* adj1) {
     const int64_t wid = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
     const uint32_t lane = lane_id();
@@ -155,12 +160,26 @@ __global__ void relayout_kernel(const int32_t* rp0, const uint2* adj0, int32_t n
             const int32_t k = (int32_t)split_of(deg, split).x, at = rp1[v];
             for (int32_t j = (int32_t)lane; j < k; j += 32) adj1[at + j] = make_uint2((uint32_t)(s0 + j), 0u);
         }
-        if (deg > 0 && deg <= kBigRow) copy_row_warp(adj0 + b, adj1 + (s0 >= 0 ? rp1[s0] : rp1[v]), deg, light);
+        if (deg > kBigRow) continue;
+        const int32_t to = split_at(rp1, first, v);
+        for (int32_t j = (int32_t)lane; j < deg; j += 32) adj1[to + j] = adj0[b + j];
     }
 }
 
-// The rows above kBigRow arcs, one block per vertex.
-__global__ void __launch_bounds__(kBigThreads) relayout_big_kernel(const int32_t* rp0, const uint2* adj0, int32_t n,
+// Light-first rows out of the split layout, in the original places.
+__global__ void light_first_kernel(const int32_t* rp0, uint2* adj0, int32_t n, const int32_t* rp1,
+                                   const int32_t* first, uint32_t light, const uint2* adj1) {
+    const int64_t wid = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
+    for (int64_t v = wid; v < n; v += nw) {
+        const int32_t b = rp0[v], deg = rp0[v + 1] - b;
+        if (deg > 0 && deg <= kBigRow) part_row_warp(adj1 + split_at(rp1, first, v), adj0 + b, deg, light);
+    }
+}
+
+// The rows above kBigRow arcs of the two kernels above, one block per vertex.
+template <bool LIGHT_FIRST>
+__global__ void __launch_bounds__(kBigThreads) relayout_big_kernel(const int32_t* rp0, uint2* adj0, int32_t n,
                                                                    const int32_t* rp1, const int32_t* first,
                                                                    uint32_t light, uint2* adj1) {
     __shared__ int32_t list[kBigThreads];
@@ -175,20 +194,23 @@ __global__ void __launch_bounds__(kBigThreads) relayout_big_kernel(const int32_t
         for (int i = 0; i < listed; i++) {
             const int32_t u = list[i], b = rp0[u];
             const uint32_t deg = (uint32_t)(rp0[u + 1] - b);
-            const uint2* from = adj0 + b;
-            uint2* to = adj1 + (first[u] >= 0 ? rp1[first[u]] : rp1[u]);
+            uint2 *row0 = adj0 + b, *row1 = adj1 + split_at(rp1, first, u);
+            if (!LIGHT_FIRST) {
+                for (uint32_t e = threadIdx.x; e < deg; e += kBigThreads) row1[e] = row0[e];
+                continue;
+            }
             uint2 mine = make_uint2(0u, 0u), total;
-            for (uint32_t e = threadIdx.x; e < deg; e += kBigThreads) mine.x += from[e].y <= light;
+            for (uint32_t e = threadIdx.x; e < deg; e += kBigThreads) mine.x += row1[e].y <= light;
             block_scan(mine, total);
             uint32_t l = 0u, h = total.x;
             for (uint32_t e0 = 0; e0 < deg; e0 += kBigThreads) {
                 const uint32_t e = e0 + threadIdx.x;
                 const bool in = e < deg;
-                const uint2 a = in ? from[e] : make_uint2(0u, 0u);
+                const uint2 a = in ? row1[e] : make_uint2(0u, 0u);
                 const bool lt = in && a.y <= light;
                 uint2 tile;
                 const uint2 at = block_scan(make_uint2(lt, in && !lt), tile);
-                if (in) to[lt ? l + at.x : h + at.y] = a;
+                if (in) row0[lt ? l + at.x : h + at.y] = a;
                 l += tile.x;
                 h += tile.y;
             }
@@ -349,6 +371,9 @@ __global__ void __launch_bounds__(kBigThreads) symmetry_big_kernel(const int32_t
 }
 
 int warps_grid(const Graph* g) { return g->sms * 8; }
+int span_grid(const Graph* g) {
+    return (int)std::max<int64_t>(1, std::min<int64_t>(((int64_t)g->n + 255) / 256, (int64_t)g->sms * 8));
+}
 
 }  // namespace
 
@@ -383,6 +408,41 @@ int check_symmetry(Graph* g, const int32_t* rp0, const uint2* adj0, cudaStream_t
 
 void launch_unsplit(const Graph* g, const int32_t* src_start, const int32_t* rp0, uint2* adj0, cudaStream_t s) {
     unsplit_kernel<<<warps_grid(g), 256, 0, s>>>(g->adj, src_start, rp0, g->n, adj0);
+}
+
+// The arcs of a symmetric graph with hubs once more, light arcs first, where the
+// original ones were (adj0), for the wavefront kernels; span and mid describe
+// them from now on, in every layout.  The queue engine keeps the original order:
+// with rows partitioned for both it relaxed 43% more arcs (a hub's slices were
+// all light or all heavy), R-MAT-20 1.41 ms -> 1.89, R-MAT-18 1.03 -> 1.29.
+// They only save time: without room, false.
+static bool light_first(Graph* g, const int32_t* rp0, uint2* adj0, const int32_t* rp1, const int32_t* first,
+                        uint2* adj1, cudaStream_t s) {
+    const int32_t n = g->n;
+    unsigned long long *lights = nullptr, h = 0;
+    int32_t* mid = nullptr;
+    if ((!g->span && cudaMalloc((void**)&g->span, sizeof(int2) * (size_t)n) != cudaSuccess) ||
+        cudaMalloc((void**)&mid, sizeof(int32_t) * (size_t)n) != cudaSuccess ||
+        cudaMalloc((void**)&lights, sizeof(*lights)) != cudaSuccess) {
+        cudaGetLastError();
+        cudaFree(mid);
+        return false;
+    }
+    light_first_kernel<<<warps_grid(g), 256, 0, s>>>(rp0, adj0, n, rp1, first, g->light_w, adj1);
+    relayout_big_kernel<true><<<g->sms, kBigThreads, 0, s>>>(rp0, adj0, n, rp1, first, g->light_w, adj1);
+    cudaMemsetAsync(lights, 0, sizeof(*lights), s);
+    span_kernel<<<span_grid(g), 256, 0, s>>>(rp0, adj0, n, g->span, g->light_w, mid, lights);
+    cudaMemcpyAsync(&h, lights, sizeof(h), cudaMemcpyDeviceToHost, s);
+    const bool ok = cudaStreamSynchronize(s) == cudaSuccess;
+    cudaFree(lights);
+    if (!ok) {
+        cudaFree(mid);
+        return false;
+    }
+    g->wadj = adj0;
+    g->mid = mid;
+    g->light_share = (double)h / (double)g->m;
+    return true;
 }
 
 int build_layout(Graph* g, int32_t* rp0, uint2* adj0, int32_t split, cudaStream_t s) {
@@ -427,13 +487,13 @@ int build_layout(Graph* g, int32_t* rp0, uint2* adj0, int32_t split, cudaStream_
         cudaGetLastError();
         rc = SSSP_E_NOMEM;
     }
-    const uint32_t light = g->symmetric ? g->light_w : 0xffffffffu;
     if (rc == SSSP_OK) {
         split_rows_kernel<<<tiles, kScanThreads, 0, s>>>(rp0, n, g->m, split, sums, tiles, rp1, first, owner);
-        relayout_kernel<<<warps_grid(g), 256, 0, s>>>(rp0, adj0, n, rp1, first, split, light, adj1);
-        relayout_big_kernel<<<g->sms, kBigThreads, 0, s>>>(rp0, adj0, n, rp1, first, light, adj1);
+        relayout_kernel<<<warps_grid(g), 256, 0, s>>>(rp0, adj0, n, rp1, first, split, adj1);
+        relayout_big_kernel<false><<<g->sms, kBigThreads, 0, s>>>(rp0, adj0, n, rp1, first, 0u, adj1);
         if (cudaStreamSynchronize(s) != cudaSuccess) rc = SSSP_E_CUDA;
     }
+    const bool keep = rc == SSSP_OK && g->symmetric && !g->wadj && light_first(g, rp0, adj0, rp1, first, adj1, s);
     cudaFree(sums);
     cudaFree(first);
     if (rc != SSSP_OK) {
@@ -443,52 +503,32 @@ int build_layout(Graph* g, int32_t* rp0, uint2* adj0, int32_t split, cudaStream_
         return rc;
     }
     cudaFree(rp0);
-    cudaFree(adj0);
+    if (!keep) cudaFree(adj0);
     g->row_ptr = rp1;
     g->adj = adj1;
     g->owner = owner;
     g->nv = nv;
     g->mv = mv;
     g->split = split;
-    // (rows partitioned once stay so in every later layout)
-    if (g->symmetric) g->light_first = true;
     return SSSP_OK;
 }
 
 int fill_span(Graph* g, cudaStream_t s) {
+    if (g->wadj) return SSSP_OK;   // light_first has filled it
     if (!g->span && cudaMalloc((void**)&g->span, sizeof(int2) * (size_t)g->n) != cudaSuccess) {
         cudaGetLastError();
         return SSSP_E_NOMEM;
     }
-    unsigned long long* lights = nullptr;
-    unsigned long long h = 0;
-    if (g->light_first) {
-        // (without room for them the share of light arcs stays 0, which turns
-        // the core search off)
-        if ((!g->mid && cudaMalloc((void**)&g->mid, sizeof(int32_t) * (size_t)g->n) != cudaSuccess) ||
-            cudaMalloc((void**)&lights, sizeof(*lights)) != cudaSuccess) {
-            cudaGetLastError();
-            lights = nullptr;
-        } else {
-            cudaMemsetAsync(lights, 0, sizeof(*lights), s);
-        }
-    }
-    const int64_t blocks = std::min<int64_t>(((int64_t)g->n + 255) / 256, (int64_t)g->sms * 8);
-    span_kernel<<<(int)std::max<int64_t>(1, blocks), 256, 0, s>>>(g->row_ptr, g->adj, g->n, g->span, g->light_w,
-                                                                  lights ? g->mid : nullptr, lights);
+    span_kernel<<<span_grid(g), 256, 0, s>>>(g->row_ptr, g->adj, g->n, g->span, 0u, nullptr, nullptr);
     if (thin_graph(g->feat.avg_deg, g->feat.max_deg)) {
         if (!g->quads && cudaMalloc((void**)&g->quads, 2 * sizeof(uint4) * (size_t)g->n) != cudaSuccess) {
             // they only save time: without room for them, without them
             cudaGetLastError();
             g->quads = nullptr;
         }
-        if (g->quads) quads_kernel<<<(int)std::max<int64_t>(1, blocks), 256, 0, s>>>(g->span, g->adj, g->n, g->quads);
+        if (g->quads) quads_kernel<<<span_grid(g), 256, 0, s>>>(g->span, g->adj, g->n, g->quads);
     }
-    if (lights) cudaMemcpyAsync(&h, lights, sizeof(h), cudaMemcpyDeviceToHost, s);
-    const cudaError_t e = cudaStreamSynchronize(s);
-    cudaFree(lights);
-    g->light_share = g->m > 0 ? (double)h / (double)g->m : 0.0;
-    return cuda_status(e);
+    return cuda_status(cudaStreamSynchronize(s));
 }
 
 }  // namespace sssp

@@ -976,7 +976,7 @@ int express_launch(sssp_server* s, Lane* L) {
                 e = launch_fan_out(F.pred, g->n, k, reinterpret_cast<uint32_t*>(J->out_p), s->sms, J->stream);
         } else {
             P.span = g->span;
-            P.adj = g->adj;
+            P.adj = wave_adj(g);
             P.quads = g->quads;
             if (plan.core) {
                 P.mid = g->mid;

@@ -218,7 +218,7 @@ void fan_carve(uint32_t* words, uint4* slices, int32_t n, int64_t m, bool pred, 
 void fan_graph(const Graph* g, FanParams* p) {
     p->max_steps = deep_steps(g->m);
     p->span = g->span;
-    p->adj = g->adj;
+    p->adj = wave_adj(g);
     if (wave_graph(g).core) {
         p->mid = g->mid;
         p->light_w = g->light_w;
@@ -346,7 +346,7 @@ int run_wave(Graph* g, const int32_t* srcs_host, const int32_t* srcs_dev, int32_
             P.srcs = ws.srcs;
         }
         P.span = g->span;
-        P.adj = g->adj;
+        P.adj = wave_adj(g);
         P.quads = g->quads;
         P.pull = unit && g->symmetric;
         if (plan.core && !unit) {
