@@ -237,7 +237,8 @@ SSSP_API int sssp_config_default(sssp_config *cfg);
 SSSP_API int sssp_graph_create(const int32_t *row_ptr, const int32_t *col_idx, const void *weights,
                       int32_t n, int64_t m, int32_t wtype, sssp_graph **out);
 
-/* Frees the graph and every device buffer it owns.  NULL is a no-op. */
+/* Frees the graph and every device buffer it owns.  Waits while a server still
+ * runs a cancelled query on it.  NULL is a no-op. */
 SSSP_API int sssp_graph_destroy(sssp_graph *g);
 
 /* Table 2 features of the graph (Section 3.5). */

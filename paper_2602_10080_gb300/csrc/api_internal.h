@@ -115,6 +115,10 @@ int cuda_status(cudaError_t e);
 // Serving lanes per graph uid: adds delta and returns the new count.  A
 // graph whose layout is in use by a lane is not relaid out.
 int lane_refs(uint64_t uid, int delta);
+// Uses of a graph by servers, by its uid: while one of its queries is admitted
+// or running, a cancelled one's rest too, its destruction waits.
+void graph_pin(uint64_t uid, int delta);
+void graph_pins_wait(uint64_t uid);
 // Makes the graph's layout the one for hub split threshold `split` (caller
 // holds g->mu); SSSP_E_BUSY while a serving lane uses the graph.
 int ensure_layout(Graph* g, int32_t split, cudaStream_t s);

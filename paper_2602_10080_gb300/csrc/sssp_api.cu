@@ -6,12 +6,14 @@
 #include <atomic>
 #include <chrono>
 #include <cmath>
+#include <condition_variable>
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
 #include <mutex>
 #include <new>
 #include <thread>
+#include <unordered_map>
 #include <vector>
 
 #include "../../include/sssp.h"
@@ -889,6 +891,24 @@ int lane_refs(uint64_t uid, int delta) {
     return delta > 0 ? delta : 0;
 }
 
+static std::mutex g_pins_mu;
+static std::condition_variable g_pins_cv;
+static std::unordered_map<uint64_t, int> g_pins;
+
+void graph_pin(uint64_t uid, int delta) {
+    std::lock_guard<std::mutex> lk(g_pins_mu);
+    const auto it = g_pins.emplace(uid, 0).first;
+    it->second += delta;
+    if (it->second > 0) return;
+    g_pins.erase(it);
+    g_pins_cv.notify_all();
+}
+
+void graph_pins_wait(uint64_t uid) {
+    std::unique_lock<std::mutex> lk(g_pins_mu);
+    g_pins_cv.wait(lk, [&] { return !g_pins.count(uid); });
+}
+
 int ensure_layout(Graph* g, int32_t split, cudaStream_t s) {
     if (split == g->layout_req) return SSSP_OK;
     // no vertex is split under either threshold: the layout is the same
@@ -1128,6 +1148,7 @@ extern "C" int sssp_graph_create(const int32_t* row_ptr, const int32_t* col_idx,
 extern "C" int sssp_graph_destroy(sssp_graph* gh) {
     if (!gh) return SSSP_OK;
     Graph* g = reinterpret_cast<Graph*>(gh);
+    graph_pins_wait(g->uid);
     {
         std::lock_guard<std::mutex> lk(g->mu);
         cudaSetDevice(g->device);

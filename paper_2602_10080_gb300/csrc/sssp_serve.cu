@@ -270,6 +270,7 @@ struct Lane {
     bool many = false;          // slices while many queries wait (see express_launch)
     std::vector<Job*> jobs;
     uint64_t uid = 0;
+    bool pinned = false;        // the graph is in use (graph_pin); g is read only then
     bool counted = false;       // registered in lane_refs (the graph's layout is pinned)
     int pred_mode = 0;
     LaunchPlan plan;
@@ -396,9 +397,25 @@ void job_destroy(sssp_server* s, Job* J) {
     delete J;
 }
 
+// Caller holds s->mu and knows of a query of the lane's graph that has not ended.
+void lane_pin(Lane* L) {
+    if (!L->pinned) graph_pin(L->uid, 1);
+    L->pinned = true;
+}
+
+// Lanes without work give their graph free.  Worker thread, between its steps.
+void lanes_unpin(sssp_server* s) {
+    for (Lane* L : s->lanes) {
+        if (!L->pinned || L->inflight || L->running + L->draining + L->nadm > 0) continue;
+        L->pinned = false;
+        graph_pin(L->uid, -1);
+    }
+}
+
 void lane_destroy(sssp_server* s, Lane* L) {
     for (Job* J : L->jobs) job_destroy(s, J);
     lane_free_buffers(s, L);
+    if (L->pinned) graph_pin(L->uid, -1);
     if (L->counted) lane_refs(L->uid, -1);
     if (L->k0) cudaEventDestroy(L->k0);
     if (L->k1) cudaEventDestroy(L->k1);
@@ -690,6 +707,12 @@ Lane* find_lane(sssp_server* s, Graph* g, int pred_mode) {
     return nullptr;
 }
 
+// The graph of a query that is being admitted, in use meanwhile.
+struct QueryPin {
+    uint64_t uid;
+    ~QueryPin() { graph_pin(uid, -1); }
+};
+
 // Moves backlog queries into free slots (FIFO per lane).  Worker thread.
 void admit(sssp_server* s) {
     std::vector<Lane*> blocked;
@@ -705,10 +728,11 @@ void admit(sssp_server* s) {
     }
     for (Lane* L : s->lanes) L->prev_running = L->running;
     for (Query* q : work) {
-        {
-            std::lock_guard<std::mutex> lk(s->mu);
-            if (q->cancel) continue;   // already ERROR/CANCELLED
-        }
+        std::unique_lock<std::mutex> ql(s->mu);
+        if (q->cancel) continue;   // already ERROR/CANCELLED: its graph may be gone
+        const QueryPin pin{q->g->uid};
+        graph_pin(pin.uid, 1);
+        ql.unlock();
         const int pm = q->pred_out ? pred_mode_for(q->g) : 0;
         Lane* L = find_lane(s, q->g, pm);
         if (L && (L->inflight || std::find(blocked.begin(), blocked.end(), L) != blocked.end())) {
@@ -774,6 +798,7 @@ void admit(sssp_server* s) {
         {
             std::lock_guard<std::mutex> lk(s->mu);
             if (q->cancel) continue;   // cancelled meanwhile
+            lane_pin(L);
             q->state = SSSP_Q_RUNNING;
             q->t_admit = Clock::now();
             if (L->prev_running > 0) s->stats.joined_running++;
@@ -826,6 +851,7 @@ Job* job_create(sssp_server* s) {
 }
 
 // The lane's waiting queries, oldest first (at most `most`); *all: how many wait.
+// If there are any, the lane's graph is in use from here on.
 std::vector<Query*> express_waiting(sssp_server* s, Lane* L, size_t most, size_t* all) {
     std::vector<Query*> qs;
     *all = 0;
@@ -835,6 +861,7 @@ std::vector<Query*> express_waiting(sssp_server* s, Lane* L, size_t most, size_t
         if (qs.size() < most) qs.push_back(q);
         ++*all;
     }
+    if (*all) lane_pin(L);
     return qs;
 }
 
@@ -872,15 +899,16 @@ int lane_to_slices(sssp_server* s, Lane* L) {
 // road map 1500^2 4 41 (87), 20 220 (131); grid 1500 x 1450 20 108 (162), grid
 // 4000^2 20 356 (441).
 int express_launch(sssp_server* s, Lane* L) {
-    Graph* g = L->g;
-    const size_t n = (size_t)g->n;
-    const bool f32 = g->wtype == SSSP_W_F32, pred = L->pred_mode != 0;
+    const bool pred = L->pred_mode != 0;
     for (;;) {
         const int room = std::min<int>((int)L->cap_limit - L->running, kJobQueries);
         if (room <= 0) return SSSP_OK;
         size_t waiting = 0;
         std::vector<Query*> qs = express_waiting(s, L, (size_t)room, &waiting);
         if (qs.empty()) return SSSP_OK;
+        Graph* g = L->g;
+        const size_t n = (size_t)g->n;
+        const bool f32 = g->wtype == SSSP_W_F32;
         const WaveGraph wg = wave_graph(g);
         WavePlan plan;
         const bool steps = wg.deep || (wg.steps > (int64_t)deep_steps(wg.m) && wg.m < 100000 * wg.steps);
@@ -1213,7 +1241,7 @@ int collect_lane(sssp_server* s, Lane* L) {
                     std::lock_guard<std::mutex> lk(s->mu);
                     std::deque<Query*> keep;
                     for (Query* q : s->backlog) {
-                        if (find_lane(s, q->g, q->pred_out ? pred_mode_for(q->g) : 0) == L &&
+                        if (!q->cancel && find_lane(s, q->g, q->pred_out ? pred_mode_for(q->g) : 0) == L &&
                             q->state == SSSP_Q_QUEUED)
                             finish_query(s, q, SSSP_E_NOMEM);
                         else
@@ -1456,6 +1484,7 @@ void worker_main(sssp_server* s) {
             std::this_thread::sleep_for(std::chrono::microseconds(20));
         }
         if (rc) fail_all(s, rc);
+        lanes_unpin(s);
     }
 }
 

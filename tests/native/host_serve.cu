@@ -1,0 +1,172 @@
+// The server's host code on the fake runtime: kernels end at once (or when the
+// test lets them) and report what the test wants.
+#include <chrono>
+#include <cstdio>
+#include <cstdlib>
+#include <cstring>
+#include <functional>
+#include <string>
+#include <sys/mman.h>
+#include <thread>
+
+#include "api_internal.h"
+#include "fake_cuda.h"
+#include "fan.h"
+
+using namespace sssp;
+
+// ------------------------------------------------------------- launches --
+
+struct Launch {
+    char kind;            // 'W' cluster, 'T' grid, 'F' side by side, 'M' slice
+    const int2* graph;    // its span: tells the graphs apart
+    int nq;
+};
+static std::vector<Launch> launches;
+static std::function<cudaError_t(const Launch&, Ctrl*)> on_launch;
+
+static cudaError_t launched(const Launch& l, Ctrl* ctrl) {
+    std::unique_lock<std::mutex> lk(fake::mu);
+    launches.push_back(l);
+    lk.unlock();
+    if (on_launch) {
+        const cudaError_t e = on_launch(l, ctrl);
+        if (e != cudaSuccess || ctrl->error) return e;
+    }
+    ctrl->finished = l.nq;
+    ctrl->stats[kStIter] = 10;
+    return cudaSuccess;
+}
+static size_t count(char kind, const int2* graph = nullptr) {
+    std::lock_guard<std::mutex> lk(fake::mu);
+    size_t k = 0;
+    for (const Launch& l : launches) k += l.kind == kind && (!graph || l.graph == graph);
+    return k;
+}
+
+namespace sssp {
+cudaError_t launch_wave(int, int, const WaveParams& p, int nq, int, size_t, cudaStream_t) {
+    return launched({'W', p.span, nq}, p.ctrl);
+}
+cudaError_t launch_tide(int, int, const WaveParams& p, int, int, cudaStream_t) { return launched({'T', p.span, 1}, p.ctrl); }
+cudaError_t launch_fan(int, const FanParams& p, int, cudaStream_t) { return launched({'F', p.span, p.nq}, p.ctrl); }
+cudaError_t launch_fan_out(const uint32_t*, int32_t, int32_t, uint32_t*, int, cudaStream_t) { return cudaSuccess; }
+#define INSTANCE(name)                                                                                             \
+    cudaError_t launch_mlmq_##name(const KernelKey&, dim3, dim3, size_t, cudaStream_t, const KParams& p) {         \
+        return launched({'M', nullptr, 0}, p.ctrl);                                                                \
+    }                                                                                                              \
+    cudaError_t occupancy_mlmq_##name(const KernelKey&, int, size_t, int* b) {                                     \
+        *b = 1;                                                                                                    \
+        return cudaSuccess;                                                                                        \
+    }
+INSTANCE(u32)
+INSTANCE(u32x)
+INSTANCE(f32)
+INSTANCE(f32x)
+}  // namespace sssp
+
+// --------------------------------------------------------------- graphs --
+
+// A graph in pages of its own, so that a read after its end faults.
+static Graph* make_graph(int32_t n, int64_t m, double max_deg) {
+    static uint64_t uid = 1000;
+    void* p = mmap(nullptr, sizeof(Graph), PROT_READ | PROT_WRITE, MAP_PRIVATE | MAP_ANONYMOUS, -1, 0);
+    Graph* g = new (p) Graph();
+    g->uid = uid++;
+    g->sms = 152;
+    g->n = g->nv = n;
+    g->m = g->mv = m;
+    g->wtype = SSSP_W_U32;
+    g->feat.avg_w = 4.0;
+    g->feat.min_w = 1.0;
+    g->feat.avg_deg = (double)m / n;
+    g->feat.max_deg = max_deg;
+    g->layout_req = kDefaultSplit;
+    g->span = reinterpret_cast<int2*>(g->uid * 64);
+    sssp_config_default(&g->defaults);
+    return g;
+}
+// hubs and many arcs: one query on the grid, eight or more side by side
+static Graph* grid_graph() { return make_graph(1 << 12, 1 << 20, 900.0); }
+static Graph* small_graph() { return make_graph(1000, 6000, 20.0); }
+static void end_graph(Graph* g) {
+    graph_pins_wait(g->uid);
+    mprotect(g, sizeof(Graph), PROT_NONE);
+}
+static sssp_graph* handle(Graph* g) { return reinterpret_cast<sssp_graph*>(g); }
+
+struct Out {
+    std::vector<uint32_t> d;
+    std::vector<int32_t> p;
+    uint64_t ticket = 0;
+    Out(sssp_server* s, Graph* g, bool pred = false) : d(g->n), p(pred ? g->n : 0) {
+        CHECK(sssp_serve_submit(s, handle(g), 1, d.data(), pred ? p.data() : nullptr, &ticket) == SSSP_OK);
+    }
+};
+static int wait_state(sssp_server* s, const Out& o, int ms = 10000, int32_t* status = nullptr) {
+    int32_t state = -1, st = 0;
+    if (sssp_serve_wait(s, o.ticket, ms, &state, &st) == SSSP_E_TIMEOUT) return -1;
+    if (status) *status = st;
+    return state;
+}
+static sssp_server* server(void (*set)(sssp_serve_options*) = nullptr) {
+    sssp_serve_options opt;
+    sssp_serve_options_default(&opt);
+    if (set) set(&opt);
+    sssp_server* s = nullptr;
+    CHECK(sssp_serve_create(&opt, &s) == SSSP_OK);
+    return s;
+}
+static void sleep_ms(int ms) { std::this_thread::sleep_for(std::chrono::milliseconds(ms)); }
+template <typename F>
+static bool soon(F&& f) {
+    for (int i = 0; i < 5000; i++, sleep_ms(1))
+        if (f()) return true;
+    return false;
+}
+
+// ---------------------------------------------------------------- tests --
+
+// A graph that ended after its queries did is not read again; one whose
+// cancelled query still runs ends after the job.
+static void destroyed() {
+    sssp_server* s = server();
+    Graph *a = grid_graph(), *b = small_graph(), *c = grid_graph();
+    {
+        Out q(s, a);
+        CHECK(wait_state(s, q) == SSSP_Q_DONE);
+        end_graph(a);
+    }
+    for (int i = 0; i < 3; i++) {
+        Out q(s, i % 2 ? c : b);
+        CHECK(wait_state(s, q) == SSSP_Q_DONE);
+    }
+    for (Graph* g : {b, c}) {
+        fake::busy = true;
+        const size_t had = count('W') + count('T');
+        Out q(s, g);
+        CHECK(soon([&] { return count('W') + count('T') > had; }));
+        CHECK(sssp_serve_cancel(s, q.ticket) == SSSP_OK);
+        std::atomic<bool> ended{false};
+        std::thread t([&] {
+            end_graph(g);
+            ended = true;
+        });
+        sleep_ms(50);
+        CHECK(!ended);
+        fake::busy = false;
+        t.join();
+    }
+    Graph* d = grid_graph();
+    Out q(s, d);
+    CHECK(wait_state(s, q) == SSSP_Q_DONE);
+    sssp_serve_destroy(s);
+}
+
+int main(int argc, char** argv) {
+    const std::string what = argc > 1 ? argv[1] : "";
+    if (what == "destroyed") destroyed();
+    else CHECK(!"a test's name");
+    std::puts("ok");
+    return 0;
+}

@@ -44,3 +44,8 @@ def run(tmp_path_factory):
 
 def test_shared_memory_limits_do_not_shrink(run):
     run("host_launch", KERNELS)
+
+
+@pytest.mark.parametrize("what", ["destroyed"])
+def test_server(run, what):
+    run("host_serve", HOST, what)
