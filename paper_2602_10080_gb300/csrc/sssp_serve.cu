@@ -1088,22 +1088,38 @@ int express_collect(sssp_server* s, Lane* L, Job* J) {
     return SSSP_OK;
 }
 
-// Launches one slice on every lane that has work and no slice in flight.
+// The express lanes with waiting queries, the one whose query waits longest
+// first: one job at a time has the grid, and a lane that always has something
+// waiting must not keep it.
+std::vector<Lane*> express_order(sssp_server* s) {
+    std::vector<Lane*> order;
+    std::lock_guard<std::mutex> lk(s->mu);
+    for (Query* q : s->backlog) {
+        if (q->cancel) continue;
+        Lane* L = find_lane(s, q->g, q->pred_out ? pred_mode_for(q->g) : 0);
+        if (L && L->express && std::find(order.begin(), order.end(), L) == order.end()) order.push_back(L);
+    }
+    return order;
+}
+
+// Launches jobs of the express lanes and one slice on every other lane that has
+// work and no slice in flight.
 int launch_ready(sssp_server* s) {
     // the SMs are shared in proportion to each lane's queries in flight
     int total = 0;
     for (Lane* L : s->lanes)
         if (!L->express) total += L->running + L->draining;
-    for (Lane* L : s->lanes) {
+    for (Lane* L : s->lanes)
         if (L->many && !L->inflight && L->running + L->draining + L->nadm == 0) {
             L->express = true;   // those many are done
             L->many = false;
         }
-        if (L->express) {
-            const int rc = express_launch(s, L);
-            if (rc) return rc;
-            continue;
-        }
+    for (Lane* L : express_order(s)) {
+        const int rc = express_launch(s, L);
+        if (rc) return rc;
+    }
+    for (Lane* L : s->lanes) {
+        if (L->express) continue;
         if (L->inflight || L->running + L->draining == 0) continue;
         KParams P = L->plan.P;
         P.nq = (int32_t)L->cap;

@@ -5,6 +5,7 @@
 #include <cstdlib>
 #include <cstring>
 #include <functional>
+#include <memory>
 #include <string>
 #include <sys/mman.h>
 #include <thread>
@@ -163,9 +164,41 @@ static void destroyed() {
     sssp_serve_destroy(s);
 }
 
+// One lane has always queries waiting; a query on another graph, and one on the
+// same graph without predecessors, each get the grid in their turn.
+static void turns() {
+    sssp_server* s = server();
+    Graph *a = grid_graph(), *b = grid_graph(), *c = grid_graph();
+    a->feat.min_w = 0.0;   // strict-improvement predecessors: one by one
+    std::vector<std::unique_ptr<Out>> more;
+    std::atomic<int> left{300};
+    on_launch = [&](const Launch& l, Ctrl*) {
+        if (l.graph == a->span && left > 0) {
+            left--;
+            more.emplace_back(new Out(s, a, true));
+        }
+        return cudaSuccess;
+    };
+    fake::busy = true;
+    for (int i = 0; i < 4; i++) more.emplace_back(new Out(s, a, true));
+    CHECK(soon([&] { return count('T', a->span) == 1; }));
+    Out q1(s, b), q2(s, c, true), q3(s, a);
+    fake::busy = false;
+    CHECK(wait_state(s, q1) == SSSP_Q_DONE && wait_state(s, q2) == SSSP_Q_DONE && wait_state(s, q3) == SSSP_Q_DONE);
+    CHECK(left > 250);
+    left = 0;
+    CHECK(soon([&] {
+        sssp_serve_stats st;
+        sssp_serve_get_stats(s, &st);
+        return st.completed == st.submitted;
+    }));
+    sssp_serve_destroy(s);
+}
+
 int main(int argc, char** argv) {
     const std::string what = argc > 1 ? argv[1] : "";
     if (what == "destroyed") destroyed();
+    else if (what == "turns") turns();
     else CHECK(!"a test's name");
     std::puts("ok");
     return 0;

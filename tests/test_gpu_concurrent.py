@@ -65,3 +65,43 @@ def test_clusters_of_different_sizes_at_once():
 
     in_threads(lambda: solves(0, 60), lambda: solves(1, 600), lambda: solves(1, 600), noalloc)
     [G.close() for G in Gs]
+
+
+def test_a_lane_that_is_never_empty_leaves_the_grid_to_others():
+    """One lane of a server always has queries waiting; queries of another
+    graph, and of the same one without predecessors, are served in between."""
+    a, b = gg.rmat(15, 24, seed=8, wtype="f32"), gg.rmat(15, 20, seed=9)
+    A, B = upload(a), upload(b)
+    total, served = 400, []
+    srv = S.sssp_serve_create()
+    started = threading.Event()
+
+    def feed():
+        d = torch.empty((4, a.n), dtype=torch.int32, device="cuda")
+        p = torch.empty((4, a.n), dtype=torch.int32, device="cuda")
+        open_ = [S.sssp_serve_submit(srv, A.handle, 7, d[i], p[i]) for i in range(4)]
+        for k in range(total):
+            t = open_.pop(0)
+            assert S.sssp_serve_wait(srv, t)[0] == S.Q_DONE
+            served.append(t)
+            open_.append(S.sssp_serve_submit(srv, A.handle, 7, d[k % 4], p[k % 4]))
+            if k == 20:
+                started.set()
+        assert all(S.sssp_serve_wait(srv, t)[0] == S.Q_DONE for t in open_)
+
+    def others():
+        started.wait()
+        db = torch.empty(b.n, dtype=torch.int32, device="cuda")
+        da = torch.empty(a.n, dtype=torch.int32, device="cuda")
+        tb, ta = S.sssp_serve_submit(srv, B.handle, 3, db), S.sssp_serve_submit(srv, A.handle, 7, da)
+        assert S.sssp_serve_wait(srv, tb)[0] == S.Q_DONE and S.sssp_serve_wait(srv, ta)[0] == S.Q_DONE
+        assert len(served) < total // 2, len(served)
+        np.testing.assert_array_equal(db.cpu().numpy().view(np.uint32), oracle_dist(b, 3))
+        np.testing.assert_array_equal(da.cpu().numpy().view(np.uint32), oracle_dist(a, 7))
+
+    try:
+        in_threads(feed, others)
+    finally:
+        S.sssp_serve_destroy(srv)
+    A.close()
+    B.close()
