@@ -220,8 +220,8 @@ extern "C" int sssp_solve_noalloc(const int32_t* row_ptr, const uint32_t* arcs, 
         if (tide_slices(m, P.hub_deg) > P.items_cap) P.has_hubs = 0;
         const bool grid = plan.kind == kWholeGrid;
         if (grid ? (size_t)P.words * 4 * sizeof(uint32_t) > kBitBytes : smem > kWaveMaxShared) return SSSP_E_INVAL;
-        std::unique_lock<std::mutex> grid_lock;
-        if (grid) grid_lock = std::unique_lock<std::mutex>(grid_mutex(dev));
+        GridTurn turn(dev);
+        if (grid) turn.wait();
         const cudaError_t ce = grid ? launch_tide(f32 ? 1 : 0, pred_mode, P, sms, plan.threads, stream)
                                     : launch_wave(f32 ? 1 : 0, pred_mode, P, 1, plan.threads, smem, stream);
         if (ce != cudaSuccess) return SSSP_E_CUDA;

@@ -261,7 +261,7 @@ struct Job {
     size_t out_n = 0, outp_n = 0, work_n = 0, words_n = 0, slices_n = 0;
     size_t bytes = 0;           // charged to the budget
     std::vector<Query*> qs;     // in flight (empty: free)
-    bool grid = false;          // holds the grid mutex
+    bool grid = false;          // has the turn on the grid
 };
 
 struct Lane {
@@ -333,7 +333,10 @@ struct sssp_server {
     sssp_serve_stats stats{};
     std::thread worker;
     // worker-thread state
-    bool grid_job = false;                                  // a job holds the grid mutex
+    bool grid_place = false;                                // a place or the turn on the grid: grid_at
+    bool grid_job = false;                                  // a job has the turn
+    bool grid_wanted = false;                               // a lane waits for the turn
+    uint64_t grid_at = 0;
     std::deque<sssp::Query*> backlog;                       // waiting for a slot
     std::vector<sssp::Lane*> lanes;
 };
@@ -371,11 +374,27 @@ void lane_free_buffers(sssp_server* s, Lane* L) {
     L->nrings = 0;
 }
 
+void grid_leave(sssp_server* s) {
+    if (s->grid_place) grid_turns(s->device).leave(s->grid_at);
+    s->grid_place = false;
+}
+
+// Worker thread: whether a lane may launch on the grid now; if not, the server
+// keeps a place in the order for it.
+bool grid_turn(sssp_server* s) {
+    if (s->grid_job) return false;
+    if (!s->grid_place) s->grid_at = grid_turns(s->device).take();
+    s->grid_place = true;
+    if (grid_turns(s->device).mine(s->grid_at)) return true;
+    s->grid_wanted = true;
+    return false;
+}
+
 // Worker thread, after the job's kernel (or a failure of the device).
 void job_release_grid(sssp_server* s, Job* J) {
     if (!J->grid) return;
-    grid_mutex(s->device).unlock();
     J->grid = s->grid_job = false;
+    grid_leave(s);
 }
 
 void job_destroy(sssp_server* s, Job* J) {
@@ -740,9 +759,9 @@ void admit(sssp_server* s) {
             continue;
         }
         int rc = SSSP_OK;
-        if (!L && s->grid_job) {
+        if (!L && s->grid_place) {
             // lane_create waits for the graph's lock, whose holder may wait
-            // for the grid that this thread's job holds: after the job
+            // for the grid behind this server: after its job
             keep.push_back(q);
             continue;
         }
@@ -926,7 +945,7 @@ int express_launch(sssp_server* s, Lane* L) {
             plan_wave(wg, 1, L->pred_mode, &plan);
         }
         const bool grid = plan.kind != kOneCluster;
-        if (grid && s->grid_job) return SSSP_OK;
+        if (grid && !grid_turn(s)) return SSSP_OK;
         Job* J = nullptr;
         for (Job* j : L->jobs)
             if (j->qs.empty()) J = j;
@@ -969,10 +988,7 @@ int express_launch(sssp_server* s, Lane* L) {
             }
         }
         if (rc) return L->running ? SSSP_OK : lane_to_slices(s, L);
-        if (grid) {
-            if (!grid_mutex(s->device).try_lock()) return SSSP_OK;   // a solve holds the grid
-            J->grid = s->grid_job = true;
-        }
+        if (grid) J->grid = s->grid_job = true;
         {
             std::lock_guard<std::mutex> lk(s->mu);
             const Clock::time_point now = Clock::now();
@@ -1114,10 +1130,12 @@ int launch_ready(sssp_server* s) {
             L->express = true;   // those many are done
             L->many = false;
         }
+    s->grid_wanted = false;
     for (Lane* L : express_order(s)) {
         const int rc = express_launch(s, L);
         if (rc) return rc;
     }
+    if (!s->grid_job && !s->grid_wanted) grid_leave(s);   // nobody waits for it any more
     for (Lane* L : s->lanes) {
         if (L->express) continue;
         if (L->inflight || L->running + L->draining == 0) continue;
@@ -1207,6 +1225,7 @@ void fail_all(sssp_server* s, int status) {
         L->running = 0;
         L->draining = 0;
     }
+    grid_leave(s);
     for (Query* q : s->backlog)
         if (!q->cancel) finish_query(s, q, status);
     s->backlog.clear();
@@ -1493,6 +1512,7 @@ void worker_main(sssp_server* s) {
                 if (waits) std::this_thread::sleep_for(std::chrono::microseconds(20));
             }
             if (rc || any || !inflight) break;
+            if (s->grid_wanted && grid_turns(s->device).mine(s->grid_at)) break;
             if (std::chrono::duration<double, std::micro>(Clock::now() - t0).count() > 250.0) {
                 std::lock_guard<std::mutex> lk(s->mu);
                 if (!s->pending.empty()) break;

@@ -226,9 +226,31 @@ void fan_graph(const Graph* g, FanParams* p) {
     }
 }
 
-std::mutex& grid_mutex(int device) {
-    static std::mutex mu[64];
-    return mu[device & 63];
+GridTurns& grid_turns(int device) {
+    static GridTurns turns[kMaxDevices];
+    return turns[device % kMaxDevices];
+}
+
+uint64_t GridTurns::take() {
+    std::lock_guard<std::mutex> lk(mu_);
+    return next_++;
+}
+
+bool GridTurns::mine(uint64_t place) {
+    std::lock_guard<std::mutex> lk(mu_);
+    return now_ == place;
+}
+
+void GridTurns::wait(uint64_t place) {
+    std::unique_lock<std::mutex> lk(mu_);
+    cv_.wait(lk, [&] { return now_ == place; });
+}
+
+void GridTurns::leave(uint64_t place) {
+    std::lock_guard<std::mutex> lk(mu_);
+    left_.insert(place);
+    while (left_.erase(now_)) now_++;
+    cv_.notify_all();
 }
 
 namespace {
@@ -331,8 +353,8 @@ int run_wave(Graph* g, const int32_t* srcs_host, const int32_t* srcs_dev, int32_
         if ((rc = grow(&ws.out_p, &ws.out_p_n, cells))) return rc;
         pp = ws.out_p;
     }
-    std::unique_lock<std::mutex> grid_lock;
-    if (plan.kind != kOneCluster) grid_lock = std::unique_lock<std::mutex>(grid_mutex(g->device));
+    GridTurn turn(g->device);
+    if (plan.kind != kOneCluster) turn.wait();
     cudaMemsetAsync(ws.ctrl, 0, sizeof(Ctrl), stream);
     if (plan.kind == kSideBySide) {
         cudaEventRecord(ws.ev1, stream);
@@ -391,7 +413,7 @@ int run_wave(Graph* g, const int32_t* srcs_host, const int32_t* srcs_dev, int32_
     }
     if (hc.error == kErrDeep) {
         g->deep = true;
-        grid_lock.unlock();
+        turn.end();
         return run_wave(g, srcs_host, srcs_dev, src0, nq, dist_out, pred_out, stream, st_out, unit, done);
     }
     float ms = 0;

@@ -1,8 +1,10 @@
 // wave.h -- host-side declarations of the cluster wavefront kernel (wave.cuh).
 #pragma once
 
+#include <condition_variable>
 #include <cstddef>
 #include <mutex>
+#include <set>
 
 #include "wave.cuh"
 
@@ -62,9 +64,45 @@ size_t wave_params(const WavePlan& w, const WaveGraph& g, bool f32, bool unit, W
 // kTideChunk arcs.
 uint32_t tide_slices(int64_t m, int32_t hub_deg);
 // The blocks of a whole-grid kernel wait for one another, so that two of them
-// (of two graphs, on two streams) must not share the device half and half:
-// one runs at a time.  Held from the launch to the end of the call.
-std::mutex& grid_mutex(int device);
+// (of two graphs, on two streams) must not share the device half and half: one
+// runs at a time, held from the launch to the end of the call, in the order in
+// which they asked.  Nobody who has a place or the turn waits for a graph's lock
+// or for work that others have queued.
+class GridTurns {
+public:
+    uint64_t take();              // a place in the order
+    bool mine(uint64_t place);    // its turn has come
+    void wait(uint64_t place);
+    void leave(uint64_t place);   // gives up the turn, or the place before it
+
+private:
+    std::mutex mu_;
+    std::condition_variable cv_;
+    uint64_t next_ = 0, now_ = 0;
+    std::set<uint64_t> left_;     // places given up before their turn
+};
+GridTurns& grid_turns(int device);
+
+// A call's turn, until its end.
+class GridTurn {
+public:
+    explicit GridTurn(int device) : turns_(grid_turns(device)) {}
+    ~GridTurn() { end(); }
+    void wait() {
+        place_ = turns_.take();
+        has_ = true;
+        turns_.wait(place_);
+    }
+    void end() {
+        if (has_) turns_.leave(place_);
+        has_ = false;
+    }
+
+private:
+    GridTurns& turns_;
+    uint64_t place_ = 0;
+    bool has_ = false;
+};
 
 // Launches one cluster of 1 << p.log_g blocks per query.
 cudaError_t launch_wave(int wt, int pred, const WaveParams& p, int nq, int threads, size_t smem,

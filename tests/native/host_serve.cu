@@ -195,10 +195,70 @@ static void turns() {
     sssp_serve_destroy(s);
 }
 
+// A server that waits for the grid has its place among the solves that do, and
+// gives it up when nobody waits any more.
+static void places() {
+    sssp_server* s = server();
+    Graph* a = grid_graph();
+    GridTurns& t = grid_turns(0);
+    uint64_t later = 0;
+    on_launch = [&](const Launch&, Ctrl*) {
+        CHECK(!t.mine(later));
+        return cudaSuccess;
+    };
+    for (int i = 0; i < 3; i++) {
+        const uint64_t first = t.take();
+        Out q(s, a);
+        sleep_ms(30);
+        CHECK(count('T') == (size_t)i);
+        later = t.take();
+        t.leave(first);
+        CHECK(wait_state(s, q) == SSSP_Q_DONE && count('T') == (size_t)i + 1);
+        CHECK(soon([&] { return t.mine(later); }));
+        t.leave(later);
+    }
+    on_launch = nullptr;
+    const uint64_t first = t.take();
+    {
+        Out q(s, a);
+        sleep_ms(30);
+        CHECK(sssp_serve_cancel(s, q.ticket) == SSSP_OK);
+    }
+    later = t.take();
+    t.leave(first);
+    CHECK(soon([&] { return t.mine(later); }));
+    t.leave(later);
+    // a place that is given up before its turn is passed over
+    const uint64_t x = t.take(), y = t.take(), z = t.take();
+    t.leave(y);
+    CHECK(t.mine(x) && !t.mine(z));
+    t.leave(x);
+    CHECK(t.mine(z));
+    t.leave(z);
+    // the solves of two threads and a server's queries side by side
+    std::atomic<int> solves{0};
+    std::vector<std::thread> ts;
+    for (int k = 0; k < 2; k++)
+        ts.emplace_back([&] {
+            Graph* g = grid_graph();
+            std::vector<uint32_t> d(g->n);
+            for (int i = 0; i < 200; i++, solves++)
+                CHECK(sssp_solve(handle(g), i, d.data(), nullptr, nullptr, nullptr) == SSSP_OK);
+        });
+    for (int i = 0; i < 50; i++) {
+        Out q(s, a);
+        CHECK(wait_state(s, q) == SSSP_Q_DONE);
+    }
+    for (std::thread& th : ts) th.join();
+    CHECK(solves == 400);
+    sssp_serve_destroy(s);
+}
+
 int main(int argc, char** argv) {
     const std::string what = argc > 1 ? argv[1] : "";
     if (what == "destroyed") destroyed();
     else if (what == "turns") turns();
+    else if (what == "places") places();
     else CHECK(!"a test's name");
     std::puts("ok");
     return 0;
