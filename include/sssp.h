@@ -258,6 +258,10 @@ SSSP_API int sssp_graph_features(const sssp_graph *g, sssp_features *out);
  *             after a wavefront solve, which counts kernel_ms, relax_arcs,
  *             improved and rounds (its steps).
  *   stream    cudaStream_t or NULL.
+ * Solves that take the whole device (graphs of more than 2^19 arcs, but for
+ * meshes) run one at a time on it, whatever their graphs, streams and threads,
+ * in the order in which they reach it; a call waits for the work before it on its
+ * stream first.
  * Returns after completion.  Errors: SSSP_E_INVAL, SSSP_E_TIMEOUT,
  * SSSP_E_NOMEM (queue could not be grown), SSSP_E_CUDA. */
 SSSP_API int sssp_solve(sssp_graph *g, int32_t src, void *dist_out, int32_t *pred_out,

@@ -354,7 +354,13 @@ int run_wave(Graph* g, const int32_t* srcs_host, const int32_t* srcs_dev, int32_
         pp = ws.out_p;
     }
     GridTurn turn(g->device);
-    if (plan.kind != kOneCluster) turn.wait();
+    if (plan.kind != kOneCluster) {
+        // what the caller has queued on its stream is over first: it may take
+        // long, or wait for another thread's solve
+        const cudaError_t se = cudaStreamSynchronize(stream);
+        if (se != cudaSuccess) return cuda_status(se);
+        turn.wait();
+    }
     cudaMemsetAsync(ws.ctrl, 0, sizeof(Ctrl), stream);
     if (plan.kind == kSideBySide) {
         cudaEventRecord(ws.ev1, stream);

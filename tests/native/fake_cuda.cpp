@@ -12,7 +12,7 @@
 
 namespace fake {
 std::atomic<bool> busy{false};
-std::atomic<long> stream_waits{0};
+std::atomic<void*> busy_stream{nullptr};
 std::atomic<size_t> largest_malloc{~(size_t)0};
 std::mutex mu;
 std::map<const void*, int> max_shared;
@@ -44,10 +44,9 @@ cudaError_t cudaPointerGetAttributes(cudaPointerAttributes* a, const void* p) {
 }
 cudaError_t cudaStreamCreateWithFlags(cudaStream_t* s, unsigned) { *s = (cudaStream_t)std::malloc(1); return cudaSuccess; }
 cudaError_t cudaStreamDestroy(cudaStream_t s) { std::free(s); return cudaSuccess; }
-cudaError_t cudaStreamQuery(cudaStream_t) { return fake::busy ? cudaErrorNotReady : cudaSuccess; }
-cudaError_t cudaStreamSynchronize(cudaStream_t) {
-    if (fake::busy) fake::stream_waits++;
-    while (fake::busy) std::this_thread::sleep_for(std::chrono::microseconds(100));
+cudaError_t cudaStreamQuery(cudaStream_t s) { return fake::busy || (s && fake::busy_stream == (void*)s) ? cudaErrorNotReady : cudaSuccess; }
+cudaError_t cudaStreamSynchronize(cudaStream_t s) {
+    while (fake::busy || (s && fake::busy_stream == (void*)s)) std::this_thread::sleep_for(std::chrono::microseconds(100));
     return cudaSuccess;
 }
 cudaError_t cudaEventCreate(cudaEvent_t* e) { *e = (cudaEvent_t)std::malloc(1); return cudaSuccess; }

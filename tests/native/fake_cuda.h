@@ -11,7 +11,7 @@
 namespace fake {
 
 extern std::atomic<bool> busy;             // events are not ready, streams wait
-extern std::atomic<long> stream_waits;     // streams waited for while busy
+extern std::atomic<void*> busy_stream;     // this one alone waits
 extern std::atomic<size_t> largest_malloc; // larger ones fail (device memory)
 extern std::mutex mu;
 extern std::map<const void*, int> max_shared;   // cudaFuncAttributeMaxDynamicSharedMemorySize by function

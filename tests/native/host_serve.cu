@@ -254,11 +254,43 @@ static void places() {
     sssp_serve_destroy(s);
 }
 
+// A solve on a stream that is busy holds up neither another graph's solve nor a
+// server; one whose stream waits for another's solve ends after it.
+static void busy_stream() {
+    Graph *a = grid_graph(), *b = grid_graph(), *c = grid_graph();
+    int mine;
+    const cudaStream_t st = (cudaStream_t)&mine;
+    std::vector<uint32_t> da(a->n), db(b->n);
+    fake::busy_stream = st;
+    std::atomic<bool> done{false};
+    std::thread t([&] {
+        CHECK(sssp_solve(handle(a), 1, da.data(), nullptr, nullptr, st) == SSSP_OK);
+        done = true;
+    });
+    sleep_ms(50);
+    CHECK(!done);
+    std::atomic<bool> other{false};
+    std::thread u([&] {
+        CHECK(sssp_solve(handle(b), 1, db.data(), nullptr, nullptr, nullptr) == SSSP_OK);
+        other = true;
+    });
+    CHECK(soon([&] { return other.load(); }));
+    u.join();
+    sssp_server* s = server();
+    Out q(s, c);
+    CHECK(wait_state(s, q) == SSSP_Q_DONE);
+    sssp_serve_destroy(s);
+    CHECK(!done);
+    fake::busy_stream = nullptr;
+    t.join();
+}
+
 int main(int argc, char** argv) {
     const std::string what = argc > 1 ? argv[1] : "";
     if (what == "destroyed") destroyed();
     else if (what == "turns") turns();
     else if (what == "places") places();
+    else if (what == "busy_stream") busy_stream();
     else CHECK(!"a test's name");
     std::puts("ok");
     return 0;
