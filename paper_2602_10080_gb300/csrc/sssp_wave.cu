@@ -357,8 +357,11 @@ int run_wave(Graph* g, const int32_t* srcs_host, const int32_t* srcs_dev, int32_
     if (plan.kind != kOneCluster) {
         // what the caller has queued on its stream is over first: it may take
         // long, or wait for another thread's solve
-        const cudaError_t se = cudaStreamSynchronize(stream);
-        if (se != cudaSuccess) return cuda_status(se);
+        if (cudaStreamQuery(stream) != cudaSuccess) {
+            cudaGetLastError();
+            const cudaError_t se = cudaStreamSynchronize(stream);
+            if (se != cudaSuccess) return cuda_status(se);
+        }
         turn.wait();
     }
     cudaMemsetAsync(ws.ctrl, 0, sizeof(Ctrl), stream);
