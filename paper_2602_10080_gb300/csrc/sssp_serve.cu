@@ -1207,9 +1207,21 @@ int deliver(Lane* L, uint32_t slot, Query* q) {
 }
 
 void fail_all(sssp_server* s, int status) {
-    // every query anywhere ends with `status` (a sticky CUDA failure)
+    // every query anywhere ends with `status` (a sticky CUDA failure), after
+    // what still runs (a dead device answers at once): it writes to their buffers,
+    // and may have the grid
+    {
+        std::lock_guard<std::mutex> lk(s->mu);
+        s->fatal = status;
+    }
+    for (Lane* L : s->lanes) {
+        for (Job* J : L->jobs) cudaStreamSynchronize(J->stream);
+        cudaStreamSynchronize(L->stream);
+        L->inflight = false;
+        L->nadm = 0;
+    }
+    cudaGetLastError();
     std::lock_guard<std::mutex> lk(s->mu);
-    s->fatal = status;
     for (Lane* L : s->lanes) {
         for (uint32_t k = 0; k < L->cap; k++)
             if (L->slot_q[k]) {

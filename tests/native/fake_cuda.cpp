@@ -14,6 +14,7 @@ namespace fake {
 std::atomic<bool> busy{false};
 std::atomic<void*> busy_stream{nullptr};
 std::atomic<size_t> largest_malloc{~(size_t)0};
+std::atomic<bool> event_fault{false};
 std::mutex mu;
 std::map<const void*, int> max_shared;
 }  // namespace fake
@@ -53,7 +54,9 @@ cudaError_t cudaEventCreate(cudaEvent_t* e) { *e = (cudaEvent_t)std::malloc(1); 
 cudaError_t cudaEventCreateWithFlags(cudaEvent_t* e, unsigned) { return cudaEventCreate(e); }
 cudaError_t cudaEventDestroy(cudaEvent_t e) { std::free(e); return cudaSuccess; }
 cudaError_t cudaEventRecord(cudaEvent_t, cudaStream_t) { return cudaSuccess; }
-cudaError_t cudaEventQuery(cudaEvent_t) { return fake::busy ? cudaErrorNotReady : cudaSuccess; }
+cudaError_t cudaEventQuery(cudaEvent_t) {
+    return fake::event_fault ? cudaErrorLaunchFailure : fake::busy ? cudaErrorNotReady : cudaSuccess;
+}
 cudaError_t cudaEventElapsedTime(float* ms, cudaEvent_t, cudaEvent_t) { *ms = 0.1f; return cudaSuccess; }
 cudaError_t cudaGetLastError(void) { return cudaSuccess; }
 const char* cudaGetErrorString(cudaError_t) { return "fake"; }

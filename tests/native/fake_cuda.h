@@ -13,6 +13,7 @@ namespace fake {
 extern std::atomic<bool> busy;             // events are not ready, streams wait
 extern std::atomic<void*> busy_stream;     // this one alone waits
 extern std::atomic<size_t> largest_malloc; // larger ones fail (device memory)
+extern std::atomic<bool> event_fault;      // events report a device fault
 extern std::mutex mu;
 extern std::map<const void*, int> max_shared;   // cudaFuncAttributeMaxDynamicSharedMemorySize by function
 

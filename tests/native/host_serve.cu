@@ -285,12 +285,52 @@ static void busy_stream() {
     t.join();
 }
 
+// After a device fault every query ends with it, and the server can be destroyed:
+// jobs, slices and the grid's turn are given up.
+static void fault() {
+    for (const bool slices : {false, true}) {
+        sssp_server* s = slices ? server([](sssp_serve_options* o) { o->query_timeout_ms = 1000000; }) : server();
+        Graph *a = grid_graph(), *b = small_graph();
+        launches.clear();
+        if (slices) {
+            on_launch = [](const Launch&, Ctrl*) {
+                fake::busy = true;   // (a lane is opened on a quiet stream)
+                return cudaSuccess;
+            };
+        } else {
+            fake::busy = true;
+        }
+        Out q1(s, a);
+        CHECK(soon([&] { return count(slices ? 'M' : 'T') == 1; }));
+        Out q2(s, b), q3(s, a);
+        on_launch = nullptr;
+        fake::event_fault = true;
+        sleep_ms(20);
+        // what still runs is waited for
+        CHECK(wait_state(s, q1, 0) == -1 && wait_state(s, q2, 0) == -1);
+        fake::busy = false;
+        int32_t status = 0;
+        for (Out* q : {&q1, &q2, &q3})
+            CHECK(wait_state(s, *q, 10000, &status) == SSSP_Q_ERROR && status == SSSP_E_CUDA);
+        fake::event_fault = false;
+        uint64_t t;
+        CHECK(sssp_serve_submit(s, handle(b), 0, q2.d.data(), nullptr, &t) == SSSP_E_CUDA);
+        sssp_serve_destroy(s);
+        const uint64_t place = grid_turns(0).take();
+        CHECK(grid_turns(0).mine(place));
+        grid_turns(0).leave(place);
+        end_graph(a);
+        end_graph(b);
+    }
+}
+
 int main(int argc, char** argv) {
     const std::string what = argc > 1 ? argv[1] : "";
     if (what == "destroyed") destroyed();
     else if (what == "turns") turns();
     else if (what == "places") places();
     else if (what == "busy_stream") busy_stream();
+    else if (what == "fault") fault();
     else CHECK(!"a test's name");
     std::puts("ok");
     return 0;

@@ -46,6 +46,6 @@ def test_shared_memory_limits_do_not_shrink(run):
     run("host_launch", KERNELS)
 
 
-@pytest.mark.parametrize("what", ["destroyed", "turns", "places", "busy_stream"])
+@pytest.mark.parametrize("what", ["destroyed", "turns", "places", "busy_stream", "fault"])
 def test_server(run, what):
     run("host_serve", HOST, what)
