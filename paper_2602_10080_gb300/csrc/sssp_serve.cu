@@ -397,24 +397,37 @@ void job_release_grid(sssp_server* s, Job* J) {
     grid_leave(s);
 }
 
-void job_destroy(sssp_server* s, Job* J) {
-    if (J->stream) cudaStreamSynchronize(J->stream);
-    cudaFree(J->ctrl);
-    cudaFree(J->srcs);
+// The job's buffers that job_room made (no launch in flight).
+void job_drop_rooms(sssp_server* s, Job* J) {
     cudaFree(J->out_d);
     cudaFree(J->out_p);
     cudaFree(J->work);
     cudaFree(J->words);
     cudaFree(J->slices);
+    J->out_d = J->words = nullptr;
+    J->out_p = nullptr;
+    J->work = nullptr;
+    J->slices = nullptr;
+    J->out_n = J->outp_n = J->work_n = J->words_n = J->slices_n = 0;
+    s->used -= J->bytes;
+    J->bytes = 0;
+}
+
+void job_destroy(sssp_server* s, Job* J) {
+    if (J->stream) cudaStreamSynchronize(J->stream);
+    job_drop_rooms(s, J);
+    cudaFree(J->ctrl);
+    cudaFree(J->srcs);
     if (J->ctrl_h) cudaFreeHost(J->ctrl_h);
     if (J->srcs_h) cudaFreeHost(J->srcs_h);
     if (J->k0) cudaEventDestroy(J->k0);
     if (J->k1) cudaEventDestroy(J->k1);
     if (J->done) cudaEventDestroy(J->done);
     if (J->stream) cudaStreamDestroy(J->stream);
-    s->used -= J->bytes;
     delete J;
 }
+
+bool lane_idle(const Lane* L) { return !L->inflight && L->running + L->draining + L->nadm == 0; }
 
 // Caller holds s->mu and knows of a query of the lane's graph that has not ended.
 void lane_pin(Lane* L) {
@@ -425,7 +438,7 @@ void lane_pin(Lane* L) {
 // Lanes without work give their graph free.  Worker thread, between its steps.
 void lanes_unpin(sssp_server* s) {
     for (Lane* L : s->lanes) {
-        if (!L->pinned || L->inflight || L->running + L->draining + L->nadm > 0) continue;
+        if (!L->pinned || !lane_idle(L)) continue;
         L->pinned = false;
         graph_pin(L->uid, -1);
     }
@@ -726,6 +739,19 @@ Lane* find_lane(sssp_server* s, Graph* g, int pred_mode) {
     return nullptr;
 }
 
+// Gives back what idle lanes other than `but` hold.
+void free_idle_lanes(sssp_server* s, const Lane* but) {
+    for (size_t i = 0; i < s->lanes.size();) {
+        Lane* o = s->lanes[i];
+        if (o != but && lane_idle(o)) {
+            lane_destroy(s, o);
+            s->lanes.erase(s->lanes.begin() + (long)i);
+        } else {
+            i++;
+        }
+    }
+}
+
 // The graph of a query that is being admitted, in use meanwhile.
 struct QueryPin {
     uint64_t uid;
@@ -778,15 +804,7 @@ void admit(sssp_server* s) {
             rc = lane_grow_slots(s, L, want);
             if (rc == SSSP_E_NOMEM && L->cap == 0) {
                 // free idle lanes and try once more
-                for (size_t i = 0; i < s->lanes.size();) {
-                    Lane* o = s->lanes[i];
-                    if (o != L && !o->inflight && o->running == 0 && o->draining == 0 && o->nadm == 0) {
-                        lane_destroy(s, o);
-                        s->lanes.erase(s->lanes.begin() + (long)i);
-                    } else {
-                        i++;
-                    }
-                }
+                free_idle_lanes(s, L);
                 rc = lane_grow_slots(s, L, want);
             }
         }
@@ -895,36 +913,95 @@ void job_requeue(sssp_server* s, const std::vector<Query*>& qs) {
     }
 }
 
-// The lane runs slices from now on (no job in flight).
+// The lane runs slices from now on (no job in flight).  SSSP_E_NOMEM: without
+// room for their results it stays as it is.
 int lane_to_slices(sssp_server* s, Lane* L) {
     for (Job* J : L->jobs) job_destroy(s, J);
     L->jobs.clear();
-    L->express = false;
     if (L->pred_mode && !L->out_d) {
         const size_t n = (size_t)L->g->n;
-        if (dev_alloc(&L->out_d, n) || dev_alloc(&L->out_p, n)) return SSSP_E_NOMEM;
+        if (dev_alloc(&L->out_d, n) || dev_alloc(&L->out_p, n)) {
+            cudaFree(L->out_d);
+            L->out_d = nullptr;
+            return SSSP_E_NOMEM;
+        }
         L->bytes += n * 8;
         s->used += n * 8;
     }
+    L->express = false;
     return SSSP_OK;
 }
 
+// A lane for whose next job there is no room, or that the device did not launch:
+// what runs ends first, then slices take its queries, and without room for those
+// either they wait for the other lanes, or fail.  Other lanes are not concerned.
+void express_stuck(sssp_server* s, Lane* L) {
+    if (L->running || lane_to_slices(s, L) == SSSP_OK) return;
+    for (Lane* o : s->lanes)
+        if (o != L && !lane_idle(o)) return;
+    std::lock_guard<std::mutex> lk(s->mu);
+    std::deque<Query*> keep;
+    for (Query* q : s->backlog) {
+        if (!q->cancel && find_lane(s, q->g, q->pred_out ? pred_mode_for(q->g) : 0) == L)
+            finish_query(s, q, SSSP_E_NOMEM);
+        else
+            keep.push_back(q);
+    }
+    s->backlog.swap(keep);
+    s->cv_done.notify_all();
+}
+
+// The buffers and the parameters of a job of k queries.
+int job_prepare(sssp_server* s, Job* J, const Graph* g, int pred_mode, const WaveGraph& wg, const WavePlan& plan, int32_t k,
+                WaveParams* P, FanParams* F, size_t* smem) {
+    const size_t cells = (size_t)k * (size_t)g->n;
+    const bool pred = pred_mode != 0;
+    std::memset(P, 0, sizeof(*P));
+    std::memset(F, 0, sizeof(*F));
+    int rc = job_room(s, J, &J->out_d, &J->out_n, cells);
+    if (!rc && pred) rc = job_room(s, J, &J->out_p, &J->outp_n, cells);
+    if (!rc && plan.kind == kSideBySide) {
+        rc = job_room(s, J, &J->words, &J->words_n, fan_words(g->n, pred));
+        if (!rc) rc = job_room(s, J, &J->slices, &J->slices_n, fan_slices(g->n, g->m));
+        if (!rc) fan_carve(J->words, J->slices, g->n, g->m, pred, F);
+        return rc;
+    }
+    *smem = wave_params(plan, wg, g->wtype == SSSP_W_F32, false, P);
+    P->wide = kInfU32;   // (a job does not start over)
+    if (*smem > kWaveMaxShared) return SSSP_E_NOMEM;
+    if (!rc && pred) rc = job_room(s, J, &J->work, &J->work_n, cells);
+    if (!rc && plan.kind == kWholeGrid) {
+        const size_t sync_words = sizeof(TideSync) / sizeof(uint32_t);
+        rc = job_room(s, J, &J->words, &J->words_n, sync_words + 4 * (size_t)P->words);
+        if (!rc && P->has_hubs) {
+            P->items_cap = tide_slices(g->m, P->hub_deg);
+            rc = job_room(s, J, &J->slices, &J->slices_n, 2 * (size_t)P->items_cap);
+            P->items = J->slices;
+        }
+        if (!rc) {
+            P->sync = reinterpret_cast<TideSync*>(J->words);
+            P->bits = J->words + sync_words;
+        }
+    }
+    return rc;
+}
+
 // Starts jobs for the lane's waiting queries as far as slots, jobs and the
-// grid are free.  Without memory for a job the lane goes back to slices (and
-// to their rules when that does not fit either).  Where a graph takes many steps,
-// so that queries are taken in turn, and many wait, slices are faster: three
-// times as many as in a batch, since slices are slower than a batch.  ms one by
-// one (slices): eight-neighbour grid 1000^2 4 queries 25 (71), 20 140 (94);
-// road map 1500^2 4 41 (87), 20 220 (131); grid 1500 x 1450 20 108 (162), grid
-// 4000^2 20 356 (441).
-int express_launch(sssp_server* s, Lane* L) {
+// grid are free.  Without memory for a job it takes fewer queries, then what idle
+// lanes hold, and then the lane goes back to slices (express_stuck).  Where a
+// graph takes many steps, so that queries are taken in turn, and many wait, slices
+// are faster: three times as many as in a batch, since slices are slower than a
+// batch.  ms one by one (slices): eight-neighbour grid 1000^2 4 queries 25 (71), 20
+// 140 (94); road map 1500^2 4 41 (87), 20 220 (131); grid 1500 x 1450 20 108 (162),
+// grid 4000^2 20 356 (441).
+void express_launch(sssp_server* s, Lane* L) {
     const bool pred = L->pred_mode != 0;
     for (;;) {
         const int room = std::min<int>((int)L->cap_limit - L->running, kJobQueries);
-        if (room <= 0) return SSSP_OK;
+        if (room <= 0) return;
         size_t waiting = 0;
         std::vector<Query*> qs = express_waiting(s, L, (size_t)room, &waiting);
-        if (qs.empty()) return SSSP_OK;
+        if (qs.empty()) return;
         Graph* g = L->g;
         const size_t n = (size_t)g->n;
         const bool f32 = g->wtype == SSSP_W_F32;
@@ -933,61 +1010,52 @@ int express_launch(sssp_server* s, Lane* L) {
         const bool steps = wg.deep || (wg.steps > (int64_t)deep_steps(wg.m) && wg.m < 100000 * wg.steps);
         if (steps && (int64_t)waiting > 3ll * in_turn_limit(wg) &&
             (!plan_wave(wg, (int32_t)qs.size(), L->pred_mode, &plan) || plan.kind == kInTurn)) {
-            if (L->running) return SSSP_OK;
-            L->many = true;
-            return lane_to_slices(s, L);
-        }
-        plan = WavePlan();
-        if (qs.size() > 1 && (!plan_wave(wg, (int32_t)qs.size(), L->pred_mode, &plan) || plan.kind == kInTurn))
-            qs.resize(1);
-        if (qs.size() == 1) {
-            plan = WavePlan();
-            plan_wave(wg, 1, L->pred_mode, &plan);
-        }
-        const bool grid = plan.kind != kOneCluster;
-        if (grid && !grid_turn(s)) return SSSP_OK;
-        Job* J = nullptr;
-        for (Job* j : L->jobs)
-            if (j->qs.empty()) J = j;
-        if (!J) {
-            if (L->jobs.size() == kLaneJobs) return SSSP_OK;
-            J = job_create(s);
-            if (J) L->jobs.push_back(J);
-        }
-        const int32_t k = (int32_t)qs.size();
-        const size_t cells = (size_t)k * n;
-        WaveParams P;
-        std::memset(&P, 0, sizeof(P));
-        FanParams F;
-        std::memset(&F, 0, sizeof(F));
-        size_t smem = 0;
-        int rc = J ? SSSP_OK : SSSP_E_NOMEM;
-        if (!rc) rc = job_room(s, J, &J->out_d, &J->out_n, cells);
-        if (!rc && pred) rc = job_room(s, J, &J->out_p, &J->outp_n, cells);
-        if (!rc && plan.kind == kSideBySide) {
-            rc = job_room(s, J, &J->words, &J->words_n, fan_words(g->n, pred));
-            if (!rc) rc = job_room(s, J, &J->slices, &J->slices_n, fan_slices(g->n, g->m));
-            if (!rc) fan_carve(J->words, J->slices, g->n, g->m, pred, &F);
-        } else if (!rc) {
-            smem = wave_params(plan, wg, f32, false, &P);
-            P.wide = kInfU32;   // (a job does not start over)
-            if (smem > kWaveMaxShared) rc = SSSP_E_NOMEM;
-            if (!rc && pred) rc = job_room(s, J, &J->work, &J->work_n, cells);
-            if (!rc && grid) {
-                const size_t sync_words = sizeof(TideSync) / sizeof(uint32_t);
-                rc = job_room(s, J, &J->words, &J->words_n, sync_words + 4 * (size_t)P.words);
-                if (!rc && P.has_hubs) {
-                    P.items_cap = tide_slices(g->m, P.hub_deg);
-                    rc = job_room(s, J, &J->slices, &J->slices_n, 2 * (size_t)P.items_cap);
-                    P.items = J->slices;
-                }
-                if (!rc) {
-                    P.sync = reinterpret_cast<TideSync*>(J->words);
-                    P.bits = J->words + sync_words;
-                }
+            if (L->running) return;
+            if (lane_to_slices(s, L) == SSSP_OK) {
+                L->many = true;
+                return;
             }
         }
-        if (rc) return L->running ? SSSP_OK : lane_to_slices(s, L);
+        Job* J = nullptr;
+        WaveParams P;
+        FanParams F;
+        size_t smem = 0;
+        bool grid = false, freed = false;
+        int rc;
+        for (;;) {
+            plan = WavePlan();
+            if (qs.size() > 1 && (!plan_wave(wg, (int32_t)qs.size(), L->pred_mode, &plan) || plan.kind == kInTurn))
+                qs.resize(1);
+            if (qs.size() == 1) {
+                plan = WavePlan();
+                plan_wave(wg, 1, L->pred_mode, &plan);
+            }
+            grid = plan.kind != kOneCluster;
+            if (grid && !grid_turn(s)) return;
+            for (Job* j : L->jobs)
+                if (j->qs.empty()) J = j;
+            if (!J) {
+                if (L->jobs.size() == kLaneJobs) return;
+                J = job_create(s);
+                if (J) L->jobs.push_back(J);
+            }
+            rc = J ? job_prepare(s, J, g, L->pred_mode, wg, plan, (int32_t)qs.size(), &P, &F, &smem) : SSSP_E_NOMEM;
+            if (!rc) break;
+            if (J) job_drop_rooms(s, J);
+            if (qs.size() > 1) {
+                qs.resize(qs.size() / 2);
+            } else if (!freed) {
+                free_idle_lanes(s, L);
+                freed = true;
+            } else {
+                break;
+            }
+        }
+        if (rc) {
+            express_stuck(s, L);
+            return;
+        }
+        const int32_t k = (int32_t)qs.size();
         if (grid) J->grid = s->grid_job = true;
         {
             std::lock_guard<std::mutex> lk(s->mu);
@@ -1038,9 +1106,11 @@ int express_launch(sssp_server* s, Lane* L) {
         if (e != cudaSuccess) {
             // no room for the cluster or the cooperative grid on this device
             cudaGetLastError();
+            cudaStreamSynchronize(J->stream);   // what was launched before it
             job_release_grid(s, J);
             job_requeue(s, qs);
-            return L->running ? cuda_status(e) : lane_to_slices(s, L);
+            express_stuck(s, L);
+            return;
         }
         J->qs = qs;
         L->running += k;
@@ -1126,15 +1196,13 @@ int launch_ready(sssp_server* s) {
     for (Lane* L : s->lanes)
         if (!L->express) total += L->running + L->draining;
     for (Lane* L : s->lanes)
-        if (L->many && !L->inflight && L->running + L->draining + L->nadm == 0) {
+        if (L->many && lane_idle(L)) {
             L->express = true;   // those many are done
             L->many = false;
         }
     s->grid_wanted = false;
-    for (Lane* L : express_order(s)) {
-        const int rc = express_launch(s, L);
-        if (rc) return rc;
-    }
+    for (Lane* L : express_order(s))
+        if (std::find(s->lanes.begin(), s->lanes.end(), L) != s->lanes.end()) express_launch(s, L);
     if (!s->grid_job && !s->grid_wanted) grid_leave(s);   // nobody waits for it any more
     for (Lane* L : s->lanes) {
         if (L->express) continue;

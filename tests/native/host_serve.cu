@@ -285,6 +285,80 @@ static void busy_stream() {
     t.join();
 }
 
+// A lane without memory concerns its own queries: they wait for the lanes that
+// are at work, then fail; the server and its other lanes go on.
+static void no_memory() {
+    sssp_server* s = server();
+    Graph *a = grid_graph(), *b = small_graph();
+    fake::busy = true;
+    Out qb(s, b);
+    CHECK(soon([&] { return count('W') == 1; }));
+    fake::largest_malloc = 8 << 10;
+    Out qa(s, a, true);
+    sleep_ms(50);
+    CHECK(wait_state(s, qa, 0) == -1);
+    fake::busy = false;
+    CHECK(wait_state(s, qb) == SSSP_Q_DONE);
+    int32_t status = 0;
+    CHECK(wait_state(s, qa, 10000, &status) == SSSP_Q_ERROR && status == SSSP_E_NOMEM);
+    Out again(s, b);
+    CHECK(wait_state(s, again) == SSSP_Q_DONE);
+    fake::largest_malloc = ~(size_t)0;
+    Out qc(s, a, true), qd(s, a);
+    CHECK(wait_state(s, qc) == SSSP_Q_DONE && wait_state(s, qd) == SSSP_Q_DONE);
+    CHECK(count('M') == 0);
+    sssp_serve_destroy(s);
+}
+
+// A job of 32 queries that finds no room becomes smaller ones.
+static void smaller_jobs() {
+    sssp_server* s = server();
+    Graph* a = make_graph(1 << 20, 1 << 22, 900.0);
+    fake::busy = true;
+    std::vector<std::unique_ptr<Out>> qs;
+    qs.emplace_back(new Out(s, a));
+    CHECK(soon([&] { return count('T') == 1; }));
+    fake::largest_malloc = (size_t)100 << 20;   // the rows of a group are 134 MB
+    for (int i = 0; i < 40; i++) qs.emplace_back(new Out(s, a));
+    fake::busy = false;
+    for (auto& q : qs) CHECK(wait_state(s, *q) == SSSP_Q_DONE);
+    CHECK(count('F') == 0 && count('M') == 0 && count('T') == 41);
+    fake::largest_malloc = ~(size_t)0;
+    sssp_serve_destroy(s);
+}
+
+// Launches that the device refuses beside a running job wait for its end; refused
+// with nothing running they go by slices.
+static void refused_launches() {
+    for (const bool always : {false, true}) {
+        sssp_server* s = server();
+        Graph* a = small_graph();
+        launches.clear();
+        std::atomic<bool> refuse{false};
+        on_launch = [&](const Launch& l, Ctrl*) {
+            return refuse && l.kind == 'W' ? cudaErrorLaunchOutOfResources : cudaSuccess;
+        };
+        fake::busy = true;
+        Out q1(s, a);
+        CHECK(soon([&] { return count('W') == 1; }));
+        refuse = true;
+        Out q2(s, a);
+        if (!always) {
+            // (the refused launch waits for its stream first)
+            std::thread t([&] { sleep_ms(50); refuse = false; fake::busy = false; });
+            CHECK(wait_state(s, q2) == SSSP_Q_DONE);
+            t.join();
+        } else {
+            sleep_ms(20);
+            fake::busy = false;
+            CHECK(wait_state(s, q2) == SSSP_Q_DONE && count('M') > 0);
+        }
+        CHECK(wait_state(s, q1) == SSSP_Q_DONE);
+        sssp_serve_destroy(s);
+    }
+    on_launch = nullptr;
+}
+
 // After a device fault every query ends with it, and the server can be destroyed:
 // jobs, slices and the grid's turn are given up.
 static void fault() {
@@ -330,6 +404,9 @@ int main(int argc, char** argv) {
     else if (what == "turns") turns();
     else if (what == "places") places();
     else if (what == "busy_stream") busy_stream();
+    else if (what == "no_memory") no_memory();
+    else if (what == "smaller_jobs") smaller_jobs();
+    else if (what == "refused_launches") refused_launches();
     else if (what == "fault") fault();
     else CHECK(!"a test's name");
     std::puts("ok");

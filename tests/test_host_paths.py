@@ -46,6 +46,7 @@ def test_shared_memory_limits_do_not_shrink(run):
     run("host_launch", KERNELS)
 
 
-@pytest.mark.parametrize("what", ["destroyed", "turns", "places", "busy_stream", "fault"])
+@pytest.mark.parametrize("what", ["destroyed", "turns", "places", "busy_stream", "no_memory", "smaller_jobs", "refused_launches",
+                                  "fault"])
 def test_server(run, what):
     run("host_serve", HOST, what)
