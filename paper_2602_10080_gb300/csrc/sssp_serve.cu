@@ -268,6 +268,7 @@ struct Lane {
     Graph* g = nullptr;
     bool express = false;       // wavefront jobs instead of slices
     bool many = false;          // slices while many queries wait (see express_launch)
+    bool slow = false;          // a job ran into the kernels' time limit: slices, which have none, are next
     std::vector<Job*> jobs;
     uint64_t uid = 0;
     bool pinned = false;        // the graph is in use (graph_pin); g is read only then
@@ -996,12 +997,14 @@ int job_prepare(sssp_server* s, Job* J, const Graph* g, int pred_mode, const Wav
 // grid 4000^2 20 356 (441).
 void express_launch(sssp_server* s, Lane* L) {
     const bool pred = L->pred_mode != 0;
+    if (L->slow && L->running) return;
     for (;;) {
         const int room = std::min<int>((int)L->cap_limit - L->running, kJobQueries);
         if (room <= 0) return;
         size_t waiting = 0;
         std::vector<Query*> qs = express_waiting(s, L, (size_t)room, &waiting);
         if (qs.empty()) return;
+        if (L->slow && lane_to_slices(s, L) == SSSP_OK) return;
         Graph* g = L->g;
         const size_t n = (size_t)g->n;
         const bool f32 = g->wtype == SSSP_W_F32;
@@ -1128,9 +1131,11 @@ int express_collect(sssp_server* s, Lane* L, Job* J) {
     cudaEventElapsedTime(&ms, J->k0, J->k1);
     const Ctrl& hc = *J->ctrl_h;
     int status = SSSP_OK;
-    if (hc.error == kErrDeep) {
-        // too many steps side by side: the queries take another way
-        {
+    if (hc.error == kErrDeep || hc.error == kErrTimeout) {
+        // too many steps side by side, or too long a run for one launch: the
+        // queries take another way
+        if (hc.error == kErrTimeout) L->slow = true;
+        else {
             std::lock_guard<std::mutex> lk(s->mu);
             for (Query* q : J->qs)
                 if (!q->cancel) q->g->deep = true;
@@ -1140,8 +1145,7 @@ int express_collect(sssp_server* s, Lane* L, Job* J) {
         J->qs.clear();
         return SSSP_OK;
     }
-    if (hc.error != kErrNone || hc.finished != (int)J->qs.size())
-        status = hc.error == kErrTimeout ? SSSP_E_TIMEOUT : SSSP_E_CUDA;
+    if (hc.error != kErrNone || hc.finished != (int)J->qs.size()) status = SSSP_E_CUDA;
     std::vector<Query*> out;
     {
         std::lock_guard<std::mutex> lk(s->mu);

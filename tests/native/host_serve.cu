@@ -359,6 +359,24 @@ static void refused_launches() {
     on_launch = nullptr;
 }
 
+// A job that runs into its kernels' time limit is not the query's end: a server
+// without a limit of its own goes on in slices.
+static void time_limit() {
+    sssp_server* s = server();
+    for (Graph* a : {grid_graph(), small_graph()}) {
+        launches.clear();
+        on_launch = [&](const Launch& l, Ctrl* c) {
+            if (l.kind == 'W' || l.kind == 'T') c->error = kErrTimeout;
+            return cudaSuccess;
+        };
+        Out q1(s, a), q2(s, a, true);
+        CHECK(wait_state(s, q1) == SSSP_Q_DONE && wait_state(s, q2) == SSSP_Q_DONE);
+        CHECK(count('M') >= 2);
+    }
+    on_launch = nullptr;
+    sssp_serve_destroy(s);
+}
+
 // After a device fault every query ends with it, and the server can be destroyed:
 // jobs, slices and the grid's turn are given up.
 static void fault() {
@@ -408,6 +426,7 @@ int main(int argc, char** argv) {
     else if (what == "smaller_jobs") smaller_jobs();
     else if (what == "refused_launches") refused_launches();
     else if (what == "fault") fault();
+    else if (what == "time_limit") time_limit();
     else CHECK(!"a test's name");
     std::puts("ok");
     return 0;
