@@ -273,6 +273,7 @@ int run_fan(Graph* g, const int32_t* srcs_host, const int32_t* srcs_dev, int32_t
     fan_graph(g, &P);
     P.ctrl = ws.ctrl;
     P.timeout_ns = 20000ull * 1000000ull;
+    cudaEventRecord(ws.ev1, stream);   // kernel_ms: without the allocations
     const int32_t groups = (nq + 31) / 32, per = (nq + groups - 1) / groups;
     for (int32_t q0 = 0; q0 < nq; q0 += per) {
         P.nq = std::min(per, nq - q0);
@@ -305,29 +306,35 @@ int run_wave(Graph* g, const int32_t* srcs_host, const int32_t* srcs_dev, int32_
     if (plan.kind == kInTurn) {
         sssp_stats sum;
         std::memset(&sum, 0, sizeof(sum));
-        for (int32_t q = 0; q < nq; q++) {
-            // what the queries before found out may send the others elsewhere
-            WavePlan rest;
-            if (q && nq - q > 1 && (!plan_wave(wave_graph(g), nq - q, pred_mode, &rest) || rest.kind != kInTurn)) {
-                const size_t at = (size_t)q * (size_t)n;
-                int32_t more = 0;
-                const int rc = run_wave(g, srcs_host + q, srcs_dev ? srcs_dev + q : nullptr, 0, nq - q,
-                                        (uint32_t*)dist_out + at, pred_out ? pred_out + at : nullptr, stream, st_out,
-                                        unit, &more);
-                if (done) *done = q + more;
-                return rc;
-            }
-            sssp_stats one;
-            const size_t at = (size_t)q * (size_t)n;
-            const int rc = run_wave(g, nullptr, nullptr, srcs_host[q], 1, (uint32_t*)dist_out + at,
-                                    pred_out ? pred_out + at : nullptr, stream, &one, unit);
-            if (rc) return rc;
+        auto add = [&](sssp_stats one) {
             one.kernel_ms += sum.kernel_ms;
             one.total_ms += sum.total_ms;
             one.relax_arcs += sum.relax_arcs;
             one.improved += sum.improved;
             one.rounds += sum.rounds;
             sum = one;
+        };
+        for (int32_t q = 0; q < nq; q++) {
+            // what the queries before found out may send the others elsewhere
+            WavePlan rest;
+            if (q && nq - q > 1 && (!plan_wave(wave_graph(g), nq - q, pred_mode, &rest) || rest.kind != kInTurn)) {
+                const size_t at = (size_t)q * (size_t)n;
+                int32_t more = 0;
+                sssp_stats others;
+                const int rc = run_wave(g, srcs_host + q, srcs_dev ? srcs_dev + q : nullptr, 0, nq - q,
+                                        (uint32_t*)dist_out + at, pred_out ? pred_out + at : nullptr, stream, &others,
+                                        unit, &more);
+                if (done) *done = q + more;
+                if (rc) return rc;
+                add(others);
+                break;
+            }
+            sssp_stats one;
+            const size_t at = (size_t)q * (size_t)n;
+            const int rc = run_wave(g, nullptr, nullptr, srcs_host[q], 1, (uint32_t*)dist_out + at,
+                                    pred_out ? pred_out + at : nullptr, stream, &one, unit);
+            if (rc) return rc;
+            add(one);
         }
         g->last = sum;
         if (st_out) *st_out = sum;
@@ -366,7 +373,6 @@ int run_wave(Graph* g, const int32_t* srcs_host, const int32_t* srcs_dev, int32_
     }
     cudaMemsetAsync(ws.ctrl, 0, sizeof(Ctrl), stream);
     if (plan.kind == kSideBySide) {
-        cudaEventRecord(ws.ev1, stream);
         if ((rc = run_fan(g, srcs_host, srcs_dev, nq, dd, pp, stream))) return rc;
     } else {
         if (pred_mode && (rc = grow(&ws.d64, &ws.d64_n, cells))) return rc;

@@ -54,7 +54,7 @@ cudaError_t launch_fan(int, const FanParams& p, int, cudaStream_t) { return laun
 cudaError_t launch_fan_out(const uint32_t*, int32_t, int32_t, uint32_t*, int, cudaStream_t) { return cudaSuccess; }
 #define INSTANCE(name)                                                                                             \
     cudaError_t launch_mlmq_##name(const KernelKey&, dim3, dim3, size_t, cudaStream_t, const KParams& p) {         \
-        return launched({'M', nullptr, 0}, p.ctrl);                                                                \
+        return launched({'M', nullptr, p.nq}, p.ctrl);                                                             \
     }                                                                                                              \
     cudaError_t occupancy_mlmq_##name(const KernelKey&, int, size_t, int* b) {                                     \
         *b = 1;                                                                                                    \
@@ -377,6 +377,32 @@ static void time_limit() {
     sssp_serve_destroy(s);
 }
 
+// The engines are timed alike: a first launch that takes long (memory, loading)
+// does not make the wavefront kernels the slower ones.
+static void autotune() {
+    Graph* a = grid_graph();
+    bool first = true;
+    on_launch = [&](const Launch& l, Ctrl*) {
+        sleep_ms(l.kind == 'M' ? 3 : first ? 40 : 0);
+        if (l.kind != 'M') first = false;
+        return cudaSuccess;
+    };
+    std::vector<int32_t> srcs(20, 1);
+    sssp_config c;
+    CHECK(sssp_autotune(handle(a), srcs.data(), 1, 30, &c) == SSSP_OK);
+    CHECK(!first && !a->tuned_queues);
+    first = true;
+    CHECK(sssp_autotune_batch(handle(a), srcs.data(), 20, 30, &c) == SSSP_OK);
+    CHECK(!first && count('F') == 2 && a->batch_tuned.size() == 1 && !a->batch_tuned[0].queues);
+    on_launch = [&](const Launch& l, Ctrl*) {   // and the other way round
+        sleep_ms(l.kind == 'M' ? 0 : 10);
+        return cudaSuccess;
+    };
+    CHECK(sssp_autotune(handle(a), srcs.data(), 1, 30, &c) == SSSP_OK && a->tuned_queues);
+    CHECK(sssp_autotune_batch(handle(a), srcs.data(), 20, 30, &c) == SSSP_OK && a->batch_tuned[0].queues);
+    on_launch = nullptr;
+}
+
 // After a device fault every query ends with it, and the server can be destroyed:
 // jobs, slices and the grid's turn are given up.
 static void fault() {
@@ -426,6 +452,7 @@ int main(int argc, char** argv) {
     else if (what == "smaller_jobs") smaller_jobs();
     else if (what == "refused_launches") refused_launches();
     else if (what == "fault") fault();
+    else if (what == "autotune") autotune();
     else if (what == "time_limit") time_limit();
     else CHECK(!"a test's name");
     std::puts("ok");

@@ -105,3 +105,20 @@ def test_a_lane_that_is_never_empty_leaves_the_grid_to_others():
         S.sssp_serve_destroy(srv)
     A.close()
     B.close()
+
+
+def test_tuned_graphs_keep_the_faster_engine():
+    """Both engines are timed warm: where the wavefront kernels are several times
+    faster, a call without a configuration stays with them after tuning."""
+    g = gg.rmat(17, 16, seed=4)
+    srcs = gg.giant_sources(g, 40)[0]
+    G = upload(g)
+    G.autotune(srcs[:1], 150)
+    d = torch.empty(40 * g.n, dtype=torch.int32, device="cuda")
+    G.solve(int(srcs[0]), d)
+    assert by_wavefront(G)
+    G.autotune_batch(srcs, 150)
+    G.solve_batch(srcs, d)
+    assert by_wavefront(G)
+    np.testing.assert_array_equal(d.cpu().numpy().view(np.uint32)[:g.n], oracle_dist(g, int(srcs[0])))
+    G.close()
