@@ -199,9 +199,15 @@ extern "C" int sssp_solve_noalloc(const int32_t* row_ptr, const uint32_t* arcs, 
     const double avg_w = m > 0 ? hf.sum_w / (double)m : 1.0;
     WaveGraph wg{n, m, avg_w, (double)hf.max_deg, sms, false, false, false, false, 0};
     Ctrl hc;
+    bool clusters = true;
     for (;;) {
         WavePlan plan;
         plan_wave(wg, 1, pred_mode, &plan);
+        if (!clusters) {
+            plan.kind = kWholeGrid;
+            plan.log_g = 0;
+            plan.threads = 1024;
+        }
         WaveParams P;
         std::memset(&P, 0, sizeof(P));
         const size_t smem = wave_params(plan, wg, f32, false, &P);
@@ -224,6 +230,12 @@ extern "C" int sssp_solve_noalloc(const int32_t* row_ptr, const uint32_t* arcs, 
         if (grid) turn.wait();
         const cudaError_t ce = grid ? launch_tide(f32 ? 1 : 0, pred_mode, P, sms, plan.threads, stream)
                                     : launch_wave(f32 ? 1 : 0, pred_mode, P, 1, plan.threads, smem, stream);
+        if (ce != cudaSuccess && !grid) {
+            // no room for a cluster on this device (a part of one): the grid needs none
+            cudaGetLastError();
+            clusters = false;
+            continue;
+        }
         if (ce != cudaSuccess) return SSSP_E_CUDA;
         if (cudaMemcpyAsync(&hc, L.ctrl, sizeof(Ctrl), cudaMemcpyDeviceToHost, stream) != cudaSuccess ||
             cudaStreamSynchronize(stream) != cudaSuccess)

@@ -403,6 +403,21 @@ static void autotune() {
     on_launch = nullptr;
 }
 
+// Where the device has no room for a cluster, the fixed scratch serves the grid.
+static void noalloc_without_clusters() {
+    std::vector<int32_t> rp(1001), d(1000), p(1000);
+    std::vector<uint32_t> arcs(12000);
+    on_launch = [&](const Launch& l, Ctrl*) { return l.kind == 'W' ? cudaErrorLaunchOutOfResources : cudaSuccess; };
+    for (int32_t* pred : {p.data(), (int32_t*)nullptr}) {
+        launches.clear();
+        CHECK(sssp_solve_noalloc(rp.data(), arcs.data(), 1000, 6000, SSSP_W_U32, 3, d.data(), pred, nullptr) == SSSP_OK);
+        CHECK(count('W') == 1 && count('T') == 1);
+    }
+    on_launch = [&](const Launch&, Ctrl*) { return cudaErrorLaunchOutOfResources; };
+    CHECK(sssp_solve_noalloc(rp.data(), arcs.data(), 1000, 6000, SSSP_W_U32, 3, d.data(), nullptr, nullptr) == SSSP_E_CUDA);
+    on_launch = nullptr;
+}
+
 // After a device fault every query ends with it, and the server can be destroyed:
 // jobs, slices and the grid's turn are given up.
 static void fault() {
@@ -452,6 +467,7 @@ int main(int argc, char** argv) {
     else if (what == "smaller_jobs") smaller_jobs();
     else if (what == "refused_launches") refused_launches();
     else if (what == "fault") fault();
+    else if (what == "noalloc_without_clusters") noalloc_without_clusters();
     else if (what == "autotune") autotune();
     else if (what == "time_limit") time_limit();
     else CHECK(!"a test's name");
