@@ -29,6 +29,7 @@ def big():
     arcs[:, 1] = 100
     arcs[M - TAIL:, 0] = torch.arange(N - 128, N - 64, dtype=torch.int32, device="cuda")
     arcs[M - TAIL:, 1] = 7
+    torch.cuda.synchronize()
     yield rp, arcs
 
 
@@ -76,7 +77,10 @@ def test_noalloc_with_the_most_arcs(big):
 def test_graph_with_the_most_arcs(big):
     """One query, a batch side by side and levels on a graph handle."""
     rp, arcs = big
-    G = S.Graph(rp, arcs[:, 0].contiguous(), arcs[:, 1].contiguous(), "u32")
+    col, w = arcs[:, 0].contiguous(), arcs[:, 1].contiguous()
+    torch.cuda.synchronize()   # creation reads them on a stream of its own
+    G = S.Graph(rp, col, w, "u32")
+    del col, w
     d = torch.empty(N, dtype=torch.int32, device="cuda")
     p = torch.empty(N, dtype=torch.int32, device="cuda")
     G.solve(77, d, p)
