@@ -968,7 +968,6 @@ int job_prepare(sssp_server* s, Job* J, const Graph* g, int pred_mode, const Wav
         return rc;
     }
     *smem = wave_params(plan, wg, g->wtype == SSSP_W_F32, false, P);
-    P->wide = kInfU32;   // (a job does not start over)
     if (*smem > kWaveMaxShared) return SSSP_E_NOMEM;
     if (!rc && pred) rc = job_room(s, J, &J->work, &J->work_n, cells);
     if (!rc && plan.kind == kWholeGrid) {
@@ -1131,14 +1130,14 @@ int express_collect(sssp_server* s, Lane* L, Job* J) {
     cudaEventElapsedTime(&ms, J->k0, J->k1);
     const Ctrl& hc = *J->ctrl_h;
     int status = SSSP_OK;
-    if (hc.error == kErrDeep || hc.error == kErrTimeout) {
-        // too many steps side by side, or too long a run for one launch: the
-        // queries take another way
+    if (hc.error == kErrWide || hc.error == kErrDeep || hc.error == kErrTimeout) {
+        // too wide a front for a cluster, too many steps side by side, or too
+        // long a run for one launch: the queries take another way
         if (hc.error == kErrTimeout) L->slow = true;
         else {
             std::lock_guard<std::mutex> lk(s->mu);
             for (Query* q : J->qs)
-                if (!q->cancel) q->g->deep = true;
+                if (!q->cancel) (hc.error == kErrWide ? q->g->wide : q->g->deep) = true;
         }
         L->running -= (int)J->qs.size();
         job_requeue(s, J->qs);

@@ -418,6 +418,24 @@ static void noalloc_without_clusters() {
     on_launch = nullptr;
 }
 
+// A front that is too wide for a cluster sends a job to the grid, and the graph
+// remembers it.
+static void wide_fronts() {
+    sssp_server* s = server();
+    Graph* a = make_graph(200000, 800000, 4.0);
+    on_launch = [&](const Launch& l, Ctrl* c) {
+        if (l.kind == 'W') c->error = kErrWide;
+        return cudaSuccess;
+    };
+    for (int i = 0; i < 2; i++) {
+        Out q(s, a);
+        CHECK(wait_state(s, q) == SSSP_Q_DONE);
+        CHECK(a->wide && count('W') == 1 && count('T') == (size_t)i + 1);
+    }
+    on_launch = nullptr;
+    sssp_serve_destroy(s);
+}
+
 // After a device fault every query ends with it, and the server can be destroyed:
 // jobs, slices and the grid's turn are given up.
 static void fault() {
@@ -467,6 +485,7 @@ int main(int argc, char** argv) {
     else if (what == "smaller_jobs") smaller_jobs();
     else if (what == "refused_launches") refused_launches();
     else if (what == "fault") fault();
+    else if (what == "wide_fronts") wide_fronts();
     else if (what == "noalloc_without_clusters") noalloc_without_clusters();
     else if (what == "autotune") autotune();
     else if (what == "time_limit") time_limit();

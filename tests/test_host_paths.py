@@ -48,6 +48,6 @@ def test_shared_memory_limits_do_not_shrink(run):
 
 @pytest.mark.parametrize("what", ["destroyed", "turns", "places", "busy_stream", "no_memory", "smaller_jobs", "refused_launches",
                                   "fault", "time_limit", "autotune",
-                                  "noalloc_without_clusters"])
+                                  "noalloc_without_clusters", "wide_fronts"])
 def test_server(run, what):
     run("host_serve", HOST, what)
