@@ -776,15 +776,16 @@ void admit(sssp_server* s) {
     for (Query* q : work) {
         std::unique_lock<std::mutex> ql(s->mu);
         if (q->cancel) continue;   // already ERROR/CANCELLED: its graph may be gone
-        const QueryPin pin{q->g->uid};
-        graph_pin(pin.uid, 1);
-        ql.unlock();
         const int pm = q->pred_out ? pred_mode_for(q->g) : 0;
         Lane* L = find_lane(s, q->g, pm);
-        if (L && (L->inflight || std::find(blocked.begin(), blocked.end(), L) != blocked.end())) {
+        // (an express lane's next job takes it)
+        if (L && (L->express || L->inflight || std::find(blocked.begin(), blocked.end(), L) != blocked.end())) {
             keep.push_back(q);
             continue;
         }
+        const QueryPin pin{q->g->uid};
+        graph_pin(pin.uid, 1);
+        ql.unlock();
         int rc = SSSP_OK;
         if (!L && s->grid_place) {
             // lane_create waits for the graph's lock, whose holder may wait
@@ -797,7 +798,7 @@ void admit(sssp_server* s) {
             if (L) s->lanes.push_back(L);
         }
         if (L && L->express) {
-            keep.push_back(q);   // its next job takes it
+            keep.push_back(q);
             continue;
         }
         if (L && L->free_slots.empty()) {
