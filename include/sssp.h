@@ -231,6 +231,10 @@ SSSP_API int sssp_config_default(sssp_config *cfg);
  * The graph's default configuration is the feature prior: the Table 2
  * features pick a family (power-law, mesh or road) and its settings
  * (Section 3.5).
+ * Device memory: 8 bytes an arc and 4 a vertex; 8 a vertex for the wavefront
+ * kernels, and for them, where there is room, 32 more a vertex of a mesh or road
+ * map (its first four arcs at a fixed place), or on a symmetric graph with split
+ * hubs a second copy of the arcs (light ones first) and 4 more a vertex.
  * Errors: SSSP_E_INVAL (NULL/negative sizes), SSSP_E_BADGRAPH (validation),
  * SSSP_E_NOMEM, SSSP_E_CUDA, SSSP_E_NODEV.  Cites: Section 2.1 (G(V,E,W)),
  * Listing 2 (edge_list / edge_weight). */
@@ -275,8 +279,9 @@ SSSP_API int sssp_solve(sssp_graph *g, int32_t src, void *dist_out, int32_t *pre
  * nq * 2^ceil(log2 n) must not exceed 2^32 (the element key packs the query
  * index above the vertex bits).  With cfg NULL the library picks the kernels
  * as for sssp_solve (on a small graph or a mesh a cluster of blocks for every
- * query, on a larger one groups of 32 queries side by side); in the queue
- * engine the batch uses the configuration sssp_autotune_batch cached for its size class, if any.
+ * query, on a larger one groups of 32 queries side by side; where a search takes
+ * many steps, few queries one after the other and many by the queue engine); in
+ * the queue engine the batch uses the configuration sssp_autotune_batch cached for its size class, if any.
  * Otherwise, when the library picks delta (cfg NULL, or a zero delta), the
  * batch uses delta / min(16, max(1, nq / 32)) with bnum <= 4: the queries
  * supply the parallelism, and narrower buckets cut out-of-order work.
@@ -331,7 +336,7 @@ SSSP_API int sssp_autotune_batch(sssp_graph *g, const int32_t *srcs, int32_t nq,
  *
  * It runs the wavefront kernels of sssp_solve, keeping every piece of scratch
  * state (control block, pending bits, hub slices, packed
- * distance/predecessor words) in one array of about 25 MiB that is part of
+ * distance/predecessor words) in one array of about 26 MiB that is part of
  * the library image: every GPU that loads the library holds it until the
  * process exits.  The first call on a device resolves that array's device
  * address.  All calls share the array and it keeps the last call's contents;
@@ -386,8 +391,9 @@ SSSP_API int sssp_solve_sampled(sssp_graph *g, int32_t src, void *dist_out, int3
  *              (host or device memory).
  *   pred_out   [n] int32 or NULL: the smallest-index parent one level up,
  *              pred[src] = src, -1 when unreachable.
- *   cfg        NULL = the graph's configuration with delta 1 (one bucket
- *              per level); a given cfg with delta 0 also means 1.
+ *   cfg        NULL = the wavefront kernels, level by level (several levels a
+ *              step on a mesh); a given cfg runs the queue engine, its delta 0
+ *              meaning 1 (one bucket per level).
  * Errors as for sssp_solve. */
 SSSP_API int sssp_bfs(sssp_graph *g, int32_t src, uint32_t *level_out, int32_t *pred_out,
                       const sssp_config *cfg, void *stream);
@@ -406,17 +412,22 @@ SSSP_API int sssp_bfs(sssp_graph *g, int32_t src, uint32_t *level_out, int32_t *
  * while earlier ones are still running.  A query admitted while the
  * lane's bucket window is at W has its buckets shifted by W, so its work
  * is ordered with the work already in flight.  A lane uses a quarter of the
- * graph's delta (it holds many queries under load).  Lanes of different graphs
- * run concurrently on their own streams, sharing the SMs.
+ * graph's delta (it holds many queries under load).  Lanes in slices run
+ * concurrently on their own streams, sharing the SMs.
  *
  * Queries that the wavefront kernels finish within a few slices are run to
- * their end instead (without per-query timeouts and test flags): on a graph
- * of at most 2^19 arcs, and on a mesh unless slice_us is below its default, a
- * cluster of blocks each, the waiting ones in one launch beside those that
+ * their end instead, as jobs (without per-query timeouts and test flags): on a
+ * graph of at most 2^19 arcs, and on a mesh unless slice_us is below its default,
+ * a cluster of blocks each, the waiting ones in one launch beside those that
  * run; on a larger graph up to 32 waiting ones side by side, or one by one,
- * with the whole device. */
+ * with the whole device.  One such job runs at a time: the lane whose query has
+ * waited longest is next, in turn with the solves of other threads that take the
+ * whole device.  Many waiting queries on a graph of many steps, a query of more
+ * than 20 s, and a lane whose jobs find no memory take slices.  Without memory
+ * for those either, the lane's queries wait for the lanes at work, or end with
+ * SSSP_E_NOMEM. */
 typedef struct sssp_serve_options {
-    size_t  mem_budget_bytes;  /* device bytes for distance slices and L2 rings of all lanes
+    size_t  mem_budget_bytes;  /* device bytes for distance slices, L2 rings and jobs of all lanes
                                   (0 = a quarter of the free device memory at creation) */
     int32_t max_slots;         /* concurrent queries per lane, 1..4096 (default 128: with five
                                   resident graphs at 2000 q/s, 256 filled every lane and served

@@ -14,7 +14,7 @@
 // outgrew the rings failed.
 //
 // The array is a file-scope __device__ variable: every GPU that loads the
-// library holds it (kNoAllocBytes, about 25 MiB) until the process exits.
+// library holds it (kNoAllocBytes, about 26 MiB) until the process exits.
 // Host code cannot use the array's name as a device address, so the first
 // call on each device resolves it with cudaGetSymbolAddress (with that device
 // current).  All calls share the array and it keeps the previous call's

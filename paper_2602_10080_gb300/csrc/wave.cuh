@@ -27,7 +27,8 @@
 // breadth-first on it 2.12 -> 0.34.  wave_kernel is bound by the chain of a hop
 // (two trips to L2, 460 + 540 cycles, and 400 to 950 of instructions between
 // them), tide_kernel by steps: two thirds of its stalls are the barriers of the
-// block and the grid, L2 and L1 run at 20 to 40%, DRAM at 4 to 11%.
+// block and the grid, L2 and L1 run at 20 to 40%, DRAM at 4% (R-MAT-20) to 25%
+// (R-MAT-22) of its rate.
 #pragma once
 
 #include "mlmq.cuh"
