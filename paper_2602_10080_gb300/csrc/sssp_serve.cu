@@ -892,8 +892,10 @@ Job* job_create(sssp_server* s) {
     return J;
 }
 
-// The lane's waiting queries, oldest first (at most `most`); *all: how many wait.
-// If there are any, the lane's graph is in use from here on.
+constexpr size_t kWaitingCount = 128;   // above every line that the number of waiting queries is compared with
+
+// The lane's waiting queries, oldest first (at most `most`); *all: how many wait
+// (at most kWaitingCount: a long backlog is not walked for it).  If there are any, the lane's graph is in use from here on.
 std::vector<Query*> express_waiting(sssp_server* s, Lane* L, size_t most, size_t* all) {
     std::vector<Query*> qs;
     *all = 0;
@@ -901,7 +903,7 @@ std::vector<Query*> express_waiting(sssp_server* s, Lane* L, size_t most, size_t
     for (Query* q : s->backlog) {
         if (q->cancel || q->g->uid != L->uid || (q->pred_out ? pred_mode_for(q->g) : 0) != L->pred_mode) continue;
         if (qs.size() < most) qs.push_back(q);
-        ++*all;
+        if (++*all == kWaitingCount) break;
     }
     if (*all) lane_pin(L);
     return qs;
@@ -1000,14 +1002,16 @@ int job_prepare(sssp_server* s, Job* J, const Graph* g, int pred_mode, const Wav
 // grid 4000^2 20 356 (441).
 void express_launch(sssp_server* s, Lane* L) {
     const bool pred = L->pred_mode != 0;
-    if (L->slow && L->running) return;
     for (;;) {
         const int room = std::min<int>((int)L->cap_limit - L->running, kJobQueries);
         if (room <= 0) return;
         size_t waiting = 0;
         std::vector<Query*> qs = express_waiting(s, L, (size_t)room, &waiting);
         if (qs.empty()) return;
-        if (L->slow && lane_to_slices(s, L) == SSSP_OK) return;
+        if (L->slow) {
+            express_stuck(s, L);
+            return;
+        }
         Graph* g = L->g;
         const size_t n = (size_t)g->n;
         const bool f32 = g->wtype == SSSP_W_F32;
@@ -1017,7 +1021,8 @@ void express_launch(sssp_server* s, Lane* L) {
         if (steps && (int64_t)waiting > 3ll * in_turn_limit(wg) &&
             (!plan_wave(wg, (int32_t)qs.size(), L->pred_mode, &plan) || plan.kind == kInTurn)) {
             if (L->running) return;
-            if (lane_to_slices(s, L) == SSSP_OK) {
+            // (slices whose memory others hold now would keep the queries waiting)
+            if (lane_slices_fit(s, L) && lane_to_slices(s, L) == SSSP_OK) {
                 L->many = true;
                 return;
             }
@@ -1186,8 +1191,11 @@ int express_collect(sssp_server* s, Lane* L, Job* J) {
 // waiting must not keep it.
 std::vector<Lane*> express_order(sssp_server* s) {
     std::vector<Lane*> order;
+    size_t lanes = 0;
+    for (Lane* L : s->lanes) lanes += L->express;
     std::lock_guard<std::mutex> lk(s->mu);
     for (Query* q : s->backlog) {
+        if (order.size() == lanes) break;
         if (q->cancel) continue;
         Lane* L = find_lane(s, q->g, q->pred_out ? pred_mode_for(q->g) : 0);
         if (L && L->express && std::find(order.begin(), order.end(), L) == order.end()) order.push_back(L);

@@ -373,6 +373,18 @@ static void time_limit() {
         CHECK(wait_state(s, q1) == SSSP_Q_DONE && wait_state(s, q2) == SSSP_Q_DONE);
         CHECK(count('M') >= 2);
     }
+    // without room for slices the query ends, and is not run over and over
+    Graph* b = grid_graph();
+    launches.clear();
+    on_launch = [&](const Launch& l, Ctrl* c) {
+        if (l.kind == 'T') c->error = kErrTimeout;
+        fake::largest_malloc = 8 << 10;
+        return cudaSuccess;
+    };
+    Out q(s, b, true);
+    int32_t status = 0;
+    CHECK(wait_state(s, q, 10000, &status) == SSSP_Q_ERROR && status == SSSP_E_NOMEM && count('T') == 1);
+    fake::largest_malloc = ~(size_t)0;
     on_launch = nullptr;
     sssp_serve_destroy(s);
 }
