@@ -37,20 +37,30 @@ uint32_t deep_steps(int64_t m) { return (uint32_t)std::max<int64_t>(48, m >> 20)
 
 // Then the queries are taken one after the other on the whole grid, up to a
 // number from which on the queue engine is faster, which works on all of them at
-// once but 2 to 5 times as slowly on one.  ms in turn (queues): eight-neighbour
-// grid 1000^2, 5300 arcs a step, 3 queries 19 (23), 6 35 (27); road maps of degree
-// 2.5 with a few crossings of 14 arms, 1500^2 3 30 (35), 6 59 (43), 4000^2 3 109
-// (99).  A warp's several hops make the line later on meshes: grid 1500 x 1450,
-// 17000 arcs a step, 6 34 (48), 10 54 (53), 16 83 (61); grid 4000^2, 41000, 10 188
-// (183).  With more arcs a step the chip is busy with one query: road 4096^2,
-// 220000 arcs a step, 64 queries 324 (534); road 2000^2, 120000, 48 96 (117); the box
-// of degree 26, 124000, 20 22 (38), 48 53 (54); the small world, 109000, 20 10 (11).
+// once but 2 to 7 times as slowly on one.  The more arcs a step has, the busier
+// the chip is with one query, and the later the line: from 10^5 arcs a step on
+// there is next to none on a mesh.  ms in turn (queues), arcs a step in thousands:
+//   eight-neighbour grid 1000^2, 5: 3 queries 19 (23), 4 25 (25), 6 35 (27); 2500^2,
+//     12: 4 72 (79), 5 89 (83)
+//   road maps of degree 2.5 with a few crossings of 14 arms, 1500^2, 2: 3 30 (36), 4
+//     40 (39); 4000^2, 6: 2 75 (89), 3 109 (99)
+//   small worlds of 10^6 vertices, 17: 4 11 (12), 8 21 (16); 50: 6 6.5 (7.8), 12 13
+//     (11); 79: 12 8.6 (8.8), 20 14 (12); 109: 20 10 (11)
+//   boxes of degree 26, whose arcs cost the queues more: 60^3, 49: 8 4.4 (14), 20 12
+//     (20); 100^3, 124: 20 23 (36), 48 53 (56); 150^3, 311: 20 43 (74)
+//   meshes, where a warp takes several hops a step: grid 1500 x 1450, 17: 8 44 (51),
+//     12 65 (56); 2500^2, 25: 9 88 (91), 12 118 (101); 4000^2, 41: 9 169 (176), 11 205
+//     (190); road maps 2000^2, 34: 12 64 (65), 20 104 (85); 1450^2, 45: 20 43 (43), 48
+//     104 (76); 1500^2, 76: 20 28 (36), 48 67 (69); 4096^2, 220: 64 324 (534)
 // A box of 100^3 vertices of degree 6, a mesh by its degrees with a wide front: 8
 // 10 (9), 20 24 (16).
 int32_t in_turn_limit(const WaveGraph& g) {
-    const bool thin = thin_graph(std::max(1.0, (double)g.m / (double)g.n), g.max_deg);
-    if (g.steps && g.m < 100000 * g.steps) return thin && !g.wide ? 8 : 3;
-    return !thin ? 24 : g.wide ? 8 : 0x7fffffff;
+    const double deg = std::max(1.0, (double)g.m / (double)g.n);
+    const bool thin = thin_graph(deg, g.max_deg);
+    const int32_t most = !thin ? 24 : g.wide ? 8 : 0x7fffffff;
+    const double busy = g.steps ? (double)g.m / (1e5 * (double)g.steps) : 1.0;
+    if (busy >= 1.0) return most;
+    return (int32_t)std::min((double)most, (thin && !g.wide ? 7.0 : deg > 12.0 && g.max_deg <= 64.0 ? 0.44 * deg : 3.55) / (1.0 - busy));
 }
 
 bool plan_wave(const WaveGraph& g, int32_t nq, int pred_mode, WavePlan* w) {
