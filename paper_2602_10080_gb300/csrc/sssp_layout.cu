@@ -91,10 +91,11 @@ __global__ void __launch_bounds__(1024) split_scan_kernel(uint2* sums, int tiles
 
 // Row offsets of the split layout: real vertices first (a hub's row links its
 // shadows), then the shadows in vertex order; first[v] = a hub's first shadow
-// or -1.
+// or -1.  at0 (or null): where row v lies without the links, hubs last.
 __global__ void __launch_bounds__(kScanThreads) split_rows_kernel(const int32_t* rp, int32_t n, int64_t m,
                                                                   int32_t split, const uint2* sums, int tiles,
-                                                                  int32_t* rp1, int32_t* first, int32_t* owner) {
+                                                                  int32_t* rp1, int32_t* first, int32_t* owner,
+                                                                  int32_t* at0) {
     const uint2 all = sums[tiles];
     const int64_t shadows0 = m - (int64_t)all.y + (int64_t)all.x;   // where the shadows' arcs begin
     const int64_t base = (int64_t)blockIdx.x * kScanTile + (int64_t)threadIdx.x * kScanItems;
@@ -114,6 +115,7 @@ __global__ void __launch_bounds__(kScanThreads) split_rows_kernel(const int32_t*
         const uint2 k = split_of(rp[v + 1] - rp[v], split);
         rp1[v] = (int32_t)((int64_t)rp[v] - at.y + at.x);
         first[v] = k.x ? (int32_t)(n + (int64_t)at.x) : -1;
+        if (at0) at0[v] = (int32_t)(k.x ? m - (int64_t)all.y + at.y : (int64_t)rp[v] - at.y);
         for (uint32_t j = 0; j < k.x; j++) {
             owner[at.x + j] = (int32_t)v;
             rp1[(int64_t)n + at.x + j] = (int32_t)(shadows0 + at.y + (int64_t)j * split);
@@ -166,14 +168,14 @@ __global__ void relayout_kernel(const int32_t* rp0, const uint2* adj0, int32_t n
     }
 }
 
-// Light-first rows out of the split layout, in the original places.
+// Light-first rows out of the split layout, at their places at0.
 __global__ void light_first_kernel(const int32_t* rp0, uint2* adj0, int32_t n, const int32_t* rp1,
-                                   const int32_t* first, uint32_t light, const uint2* adj1) {
+                                   const int32_t* first, const int32_t* at0, uint32_t light, const uint2* adj1) {
     const int64_t wid = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
     for (int64_t v = wid; v < n; v += nw) {
-        const int32_t b = rp0[v], deg = rp0[v + 1] - b;
-        if (deg > 0 && deg <= kBigRow) part_row_warp(adj1 + split_at(rp1, first, v), adj0 + b, deg, light);
+        const int32_t deg = rp0[v + 1] - rp0[v];
+        if (deg > 0 && deg <= kBigRow) part_row_warp(adj1 + split_at(rp1, first, v), adj0 + at0[v], deg, light);
     }
 }
 
@@ -181,7 +183,7 @@ __global__ void light_first_kernel(const int32_t* rp0, uint2* adj0, int32_t n, c
 template <bool LIGHT_FIRST>
 __global__ void __launch_bounds__(kBigThreads) relayout_big_kernel(const int32_t* rp0, uint2* adj0, int32_t n,
                                                                    const int32_t* rp1, const int32_t* first,
-                                                                   uint32_t light, uint2* adj1) {
+                                                                   const int32_t* at0, uint32_t light, uint2* adj1) {
     __shared__ int32_t list[kBigThreads];
     __shared__ int listed;
     const int64_t step = (int64_t)gridDim.x * kBigThreads;
@@ -192,9 +194,9 @@ __global__ void __launch_bounds__(kBigThreads) relayout_big_kernel(const int32_t
         if (v < n && rp0[v + 1] - rp0[v] > kBigRow) list[atomicAdd(&listed, 1)] = (int32_t)v;
         __syncthreads();
         for (int i = 0; i < listed; i++) {
-            const int32_t u = list[i], b = rp0[u];
-            const uint32_t deg = (uint32_t)(rp0[u + 1] - b);
-            uint2 *row0 = adj0 + b, *row1 = adj1 + split_at(rp1, first, u);
+            const int32_t u = list[i];
+            const uint32_t deg = (uint32_t)(rp0[u + 1] - rp0[u]);
+            uint2 *row0 = adj0 + (LIGHT_FIRST ? at0[u] : rp0[u]), *row1 = adj1 + split_at(rp1, first, u);
             if (!LIGHT_FIRST) {
                 for (uint32_t e = threadIdx.x; e < deg; e += kBigThreads) row1[e] = row0[e];
                 continue;
@@ -220,15 +222,19 @@ __global__ void __launch_bounds__(kBigThreads) relayout_big_kernel(const int32_t
 }
 
 // Where the arcs of every real vertex lie: its row, or (a split hub, whose row
-// links its shadows) the shadows' rows, which follow one another.  mid (or
-// null): the end of the light arcs; their count is added to *lights.
-__global__ void span_kernel(const int32_t* rp, const uint2* adj, int32_t n, int2* span, uint32_t light, int32_t* mid,
-                            unsigned long long* lights) {
+// links its shadows) the shadows' rows, which follow one another; with at0, rows
+// of these lengths from at0[v] on.  mid (with at0): the end of the light arcs;
+// their count is added to *lights.
+__global__ void span_kernel(const int32_t* rp, const uint2* adj, int32_t n, int2* span, const int32_t* at0,
+                            uint32_t light, int32_t* mid, unsigned long long* lights) {
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     unsigned long long count = 0;
     for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < n; v += stride) {
         int32_t b = rp[v], e = rp[v + 1];
-        if (e > b) {
+        if (at0) {
+            e = at0[v] + (e - b);
+            b = at0[v];
+        } else if (e > b) {
             const uint32_t first = adj[b].x;
             if (first >= (uint32_t)n) {
                 const int32_t k = e - b;
@@ -410,14 +416,15 @@ void launch_unsplit(const Graph* g, const int32_t* src_start, const int32_t* rp0
     unsplit_kernel<<<warps_grid(g), 256, 0, s>>>(g->adj, src_start, rp0, g->n, adj0);
 }
 
-// The arcs of a symmetric graph with hubs once more, light arcs first, where the
-// original ones were (adj0), for the wavefront kernels; span and mid describe
+// The arcs of a symmetric graph with hubs once more, light arcs first, in the
+// array of the original ones (adj0; hubs last: with them in between, 64 queries on
+// R-MAT-18 f32 took 1 to 3% longer), for the wavefront kernels; span and mid describe
 // them from now on, in every layout.  The queue engine keeps the original order:
 // with rows partitioned for both it relaxed 43% more arcs (a hub's slices were
 // all light or all heavy), R-MAT-20 1.41 ms -> 1.89, R-MAT-18 1.03 -> 1.29.
 // They only save time: without room, false.
 static bool light_first(Graph* g, const int32_t* rp0, uint2* adj0, const int32_t* rp1, const int32_t* first,
-                        uint2* adj1, cudaStream_t s) {
+                        const int32_t* at0, uint2* adj1, cudaStream_t s) {
     const int32_t n = g->n;
     unsigned long long *lights = nullptr, h = 0;
     int32_t* mid = nullptr;
@@ -428,10 +435,10 @@ static bool light_first(Graph* g, const int32_t* rp0, uint2* adj0, const int32_t
         cudaFree(mid);
         return false;
     }
-    light_first_kernel<<<warps_grid(g), 256, 0, s>>>(rp0, adj0, n, rp1, first, g->light_w, adj1);
-    relayout_big_kernel<true><<<g->sms, kBigThreads, 0, s>>>(rp0, adj0, n, rp1, first, g->light_w, adj1);
+    light_first_kernel<<<warps_grid(g), 256, 0, s>>>(rp0, adj0, n, rp1, first, at0, g->light_w, adj1);
+    relayout_big_kernel<true><<<g->sms, kBigThreads, 0, s>>>(rp0, adj0, n, rp1, first, at0, g->light_w, adj1);
     cudaMemsetAsync(lights, 0, sizeof(*lights), s);
-    span_kernel<<<span_grid(g), 256, 0, s>>>(rp0, adj0, n, g->span, g->light_w, mid, lights);
+    span_kernel<<<span_grid(g), 256, 0, s>>>(rp0, adj0, n, g->span, at0, g->light_w, mid, lights);
     cudaMemcpyAsync(&h, lights, sizeof(h), cudaMemcpyDeviceToHost, s);
     const bool ok = cudaStreamSynchronize(s) == cudaSuccess;
     cudaFree(lights);
@@ -477,7 +484,7 @@ int build_layout(Graph* g, int32_t* rp0, uint2* adj0, int32_t split, cudaStream_
     }
     const int32_t nv = (int32_t)(n + ns);
     const int64_t mv = g->m + ns;   // every hub's arcs move, and a link per shadow comes
-    int32_t *rp1 = nullptr, *first = nullptr, *owner = nullptr;
+    int32_t *rp1 = nullptr, *first = nullptr, *owner = nullptr, *at0 = nullptr;
     uint2* adj1 = nullptr;
     int rc = SSSP_OK;
     if (cudaMalloc((void**)&rp1, sizeof(int32_t) * ((size_t)nv + 1)) != cudaSuccess ||
@@ -488,12 +495,17 @@ int build_layout(Graph* g, int32_t* rp0, uint2* adj0, int32_t split, cudaStream_
         rc = SSSP_E_NOMEM;
     }
     if (rc == SSSP_OK) {
-        split_rows_kernel<<<tiles, kScanThreads, 0, s>>>(rp0, n, g->m, split, sums, tiles, rp1, first, owner);
+        if (g->symmetric && !g->wadj && cudaMalloc((void**)&at0, sizeof(int32_t) * (size_t)n) != cudaSuccess) {
+            cudaGetLastError();   // (only saves time)
+            at0 = nullptr;
+        }
+        split_rows_kernel<<<tiles, kScanThreads, 0, s>>>(rp0, n, g->m, split, sums, tiles, rp1, first, owner, at0);
         relayout_kernel<<<warps_grid(g), 256, 0, s>>>(rp0, adj0, n, rp1, first, split, adj1);
-        relayout_big_kernel<false><<<g->sms, kBigThreads, 0, s>>>(rp0, adj0, n, rp1, first, 0u, adj1);
+        relayout_big_kernel<false><<<g->sms, kBigThreads, 0, s>>>(rp0, adj0, n, rp1, first, nullptr, 0u, adj1);
         if (cudaStreamSynchronize(s) != cudaSuccess) rc = SSSP_E_CUDA;
     }
-    const bool keep = rc == SSSP_OK && g->symmetric && !g->wadj && light_first(g, rp0, adj0, rp1, first, adj1, s);
+    const bool keep = rc == SSSP_OK && at0 && light_first(g, rp0, adj0, rp1, first, at0, adj1, s);
+    cudaFree(at0);
     cudaFree(sums);
     cudaFree(first);
     if (rc != SSSP_OK) {
@@ -519,7 +531,7 @@ int fill_span(Graph* g, cudaStream_t s) {
         cudaGetLastError();
         return SSSP_E_NOMEM;
     }
-    span_kernel<<<span_grid(g), 256, 0, s>>>(g->row_ptr, g->adj, g->n, g->span, 0u, nullptr, nullptr);
+    span_kernel<<<span_grid(g), 256, 0, s>>>(g->row_ptr, g->adj, g->n, g->span, nullptr, 0u, nullptr, nullptr);
     if (thin_graph(g->feat.avg_deg, g->feat.max_deg)) {
         if (!g->quads && cudaMalloc((void**)&g->quads, 2 * sizeof(uint4) * (size_t)g->n) != cudaSuccess) {
             // they only save time: without room for them, without them
